@@ -115,13 +115,18 @@ def _normal(g, *shape):
     return torch.randn(shape, generator=g, device=DEVICE).half()
 
 
-def _layer(g, N, K, bits, group):
-    """A layer of random integers over the full range whose product keeps the variance of its input."""
+def _weights(g, N, K, bits, group):
+    """Random integers over the full range and scales with which the product keeps the variance of its input."""
     lo, hi = (-8, 8) if bits == 4 else (-127, 128)
     q = torch.randint(lo, hi, (N, K), generator=g, device=DEVICE, dtype=torch.int8)
     rms = math.sqrt((hi - lo) ** 2 / 12.0)
     s = (torch.rand((N, K // group if group else 1), generator=g, device=DEVICE) + 0.5) / (rms * math.sqrt(K))
-    return P.QLinear.from_weights(q.cpu().numpy(), s.clamp_min(6.2e-5).half().cpu().numpy(), bits, group, device=DEVICE)
+    return q, s.clamp_min(6.2e-5).half()
+
+
+def _layer(g, N, K, bits, group):
+    q, s = _weights(g, N, K, bits, group)
+    return P.QLinear.from_weights(q.cpu().numpy(), s.cpu().numpy(), bits, group, device=DEVICE)
 
 
 def _projections(case):
@@ -152,15 +157,16 @@ def _captured(step):
     return graph, out
 
 
-def prepare(case, seed):
+def _inputs(case, seed, layer, cache):
+    """The state of a case; layer(g, N, K, bits, group) and cache(heads, positions, d_h) make what holds weights and keys."""
     g = _generator(seed)
     kind = case["kind"]
     st = {"case": case}
     if kind == "linear":
-        st["layer"] = _layer(g, case["N"], case["K"], case["bits"], case["group"])
+        st["layer"] = layer(g, case["N"], case["K"], case["bits"], case["group"])
         st["x"] = _normal(g, case["M"], case["K"])
     elif kind in ("block", "a8"):
-        st["blocks"] = [{n: _layer(g, N, K, b, gr) for n, N, K, b, gr in _projections(case)} for _ in range(case.get("layers", 1))]
+        st["blocks"] = [{n: layer(g, N, K, b, gr) for n, N, K, b, gr in _projections(case)} for _ in range(case.get("layers", 1))]
         M, h = case["M"], case["hidden"]
         st["x"] = _normal(g, M, h)
         if kind == "a8":
@@ -179,7 +185,7 @@ def prepare(case, seed):
         R = new * case["group"]
         st["layers"] = []
         for _ in range(case["layers"]):
-            kv = P.KVHeads(H, T, d, device=DEVICE)
+            kv = cache(H, T, d)
             if case["filled"]:
                 kv.append(_normal(g, H, case["filled"], d), _normal(g, H, case["filled"], d))
             # (the softmax between the two products is the caller's: its result is an input here)
@@ -188,10 +194,15 @@ def prepare(case, seed):
             prob[:, :, :n] = torch.softmax(2.0 * torch.randn((H, R, n), generator=g, device=DEVICE), -1).half()
             st["layers"].append({"kv": kv, "k": _normal(g, H, new, d), "v": _normal(g, H, new, d), "q": _normal(g, H, R, d), "prob": prob})
     else:
-        st["table"] = _layer(g, case["vocab"], case["hidden"], 4, 32)
+        st["table"] = layer(g, case["vocab"], case["hidden"], 4, 32)
         st["ids"] = torch.randint(0, case["vocab"], (case["tokens"],), generator=g, device=DEVICE).int()
         st["x"] = _normal(g, case["rows"], case["hidden"])
         st["norm"] = (1.0 + 0.1 * torch.randn(case["hidden"], generator=g, device=DEVICE)).half()
+    return st
+
+
+def prepare(case, seed):
+    st = _inputs(case, seed, _layer, lambda heads, positions, d_h: P.KVHeads(heads, positions, d_h, device=DEVICE))
     if _is_captured(case):
         st["graph"], st["out"] = _captured(lambda: _step(st))
     return st
@@ -286,3 +297,82 @@ def tolerance(case):
     # rounds to fp16 after every operator, 1.6e-3 over two blocks; the value scales of a cache are folded into fp16
     # probabilities, whose product is subnormal over long caches, 1.1e-3.
     return {"rel": {"linear": 1.2e-3, "block": 6.4e-3, "a8": 1.2e-3, "kv": 4.5e-3, "ends": 1.2e-3}[case["kind"]]}
+
+
+# ------------------------------------------------------------------------------------------------ the same in 64 bits
+def _weights64(g, N, K, bits, group):
+    q, s = _weights(g, N, K, bits, group)
+    return lambda: (q.double().view(N, -1, group or K) * s.double()[:, :, None]).view(N, K)
+
+
+class _Cache64:
+    """Keys and values quantised to int8 with one fp16 scale per token (decided in fp32, as the cache defines it)."""
+
+    def __init__(self, heads, positions, d_h):
+        self.k, self.v = (torch.zeros((heads, positions, d_h), device=DEVICE, dtype=torch.float64) for _ in range(2))
+        self.length = 0
+
+    def append(self, k, v):
+        at = slice(self.length, self.length + k.shape[1])
+        for store, x in ((self.k, k.float()), (self.v, v.float())):
+            s = (x.abs().amax(-1, keepdim=True) / 127.0).half().float()
+            store[:, at] = (torch.round(x / s).clamp(-127, 127) * s).double()
+        self.length = at.stop
+
+
+def _norm64(h, gamma):
+    return h / (h.square().mean(-1, keepdim=True) + 1e-5).sqrt() * gamma.double()
+
+
+def _block64(st):
+    case, out = st["case"], []
+    M, hq, hkv, d = case["M"], case["q_heads"], case["kv_heads"], case["d_h"]
+    B, S, gq = st["batch"], case["M"] // st["batch"], case["q_heads"] // case["kv_heads"]
+    cos, sin = (st[n].double()[st["pos"].long()][:, None, :] for n in ("cos", "sin"))
+
+    def rotate(x, heads):
+        lo, hi = x.view(M, heads, d).split(d // 2, -1)
+        return torch.cat([lo * cos - hi * sin, hi * cos + lo * sin], -1)
+
+    def per_kv_head(x, n):                               # [B S, h_kv n, d] -> [B h_kv, S n, d]
+        return x.reshape(B, S, hkv, n, d).permute(0, 2, 1, 3, 4).reshape(B * hkv, S * n, d)
+    h, delta = 0.0, st["x"].double()
+    for w in st["blocks"]:
+        h = h + delta
+        y = _norm64(h, w["norm1"])
+        q, k, v = (y @ w[n]().T for n in "qkv")
+        out += [per_kv_head(rotate(k, hkv), 1), per_kv_head(v.view(M, hkv, d), 1)]
+        h = h + per_kv_head(rotate(q, hq), gq).reshape(M, hq * d) @ w["o"]().T
+        y = _norm64(h, w["norm2"])
+        gate = y @ w["gate"]().T
+        gate = torch.nn.functional.silu(gate) if case["act"] == "silu" else torch.nn.functional.gelu(gate, approximate="tanh")
+        delta = (gate * (y @ w["up"]().T)) @ w["down"]().T
+    return out + [h, delta]
+
+
+def _a8_64(x, w):
+    """Activations quantised per token (decided in fp32, as the call defines it), then the product."""
+    amax = x.float().abs().amax(-1, keepdim=True)
+    xq = torch.round(x.float() * (127.0 / amax)).clamp(-127, 127)
+    return (xq.double() @ w.T) * (amax / 127.0).double()
+
+
+def exact(case, seed):
+    st = _inputs(case, seed, _weights64, _Cache64)
+    kind, out = case["kind"], []
+    if kind == "linear":
+        return st["x"].double() @ st["layer"]().T
+    if kind == "block":
+        return _block64(st)
+    if kind == "a8":
+        w = st["blocks"][0]
+        return [_a8_64(st["attn"] if n == "o" else st["inner"] if n == "down" else st["x"], w[n]()) for n in ("q", "k", "v", "o", "gate", "up", "down")]
+    if kind == "kv":
+        for layer in st["layers"]:
+            kv, prob = layer["kv"], layer["prob"].double()
+            kv.append(layer["k"], layer["v"])
+            o = prob @ kv.v
+            out += [layer["q"].double() @ kv.k.transpose(1, 2), o if case["new"] * case["group"] <= 8 else list(o)]
+        return out
+    table = st["table"]()
+    return [table[st["ids"].long()], _norm64(st["x"].double(), st["norm"]) @ table.T]
