@@ -30,6 +30,7 @@ __device__ unsigned int* g_status_host;
 #include "gemv_a8.cuh"
 #include "kv.cuh"
 #include "gemm.cuh"
+#include "gemm_mid.cuh"
 #include "gemm_pair.cuh"
 #include "gemm_pair_ta.cuh"
 #include "norm.cuh"
@@ -52,6 +53,7 @@ struct Config {
     int warps_per_sm;        // QLINEAR_GEMV_WARPS_PER_SM: residency target of the cluster decode kernel
     bool oversubscribe;      // QLINEAR_GEMV_OVERSUBSCRIBE=0: the group-scaled int4 decode kernel never takes more CTAs than fit at once
     int force_ks;            // QLINEAR_GEMV_KS: forced K split of the cluster decode kernel (0 = planned)
+    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M served by the kernel for a batch of tokens (0: never)
     bool xdirect;            // QLINEAR_GEMV_XDIRECT: x fragments straight from global memory
     int kernel;              // QLINEAR_GEMV_KERNEL: 0 / 1 cluster kernel (default), 2 streaming kernel
     int stream_ctas_per_sm, stream_stages;
@@ -70,6 +72,7 @@ void load_config()
     c.warps_per_sm = env_int("QLINEAR_GEMV_WARPS_PER_SM", 32);
     c.oversubscribe = env_int("QLINEAR_GEMV_OVERSUBSCRIBE", 1) != 0;
     c.force_ks = env_int("QLINEAR_GEMV_KS", 0);
+    c.mid_max_m = env_int("QLINEAR_MID_MAX_M", 32);
     c.xdirect = env_int("QLINEAR_GEMV_XDIRECT", 1) != 0;
     const char* kc = std::getenv("QLINEAR_GEMV_KERNEL");
     c.kernel = !kc ? 0 : !std::strcmp(kc, "cluster") ? 1 : !std::strcmp(kc, "stream") ? 2 : 0;
@@ -364,6 +367,69 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
+template <int BITS, bool GROUPED, int NT, bool GATED, bool KSCALE>
+cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, cudaStream_t st)
+{
+    using S = MidSmem<BITS, GROUPED, NT>;
+    static std::atomic<bool> attr_set[kMaxDevices];
+    auto kern = gemm_mid_kernel<BITS, GROUPED, NT, GATED, KSCALE>;
+    cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, S::kTotal);
+    if (e != cudaSuccess) return e;
+    prm.n_tb = (prm.M + S::kTokens - 1) / S::kTokens;
+    prm.n_steps = (prm.n_kc + 1) / 2;
+    // K parts per tile: what the busiest SM has to do, in stages (two CTAs per SM at once, and about 4 stages' time for the
+    // ramp at the start of a CTA and the sums at its end)
+    const int tiles = units * prm.n_tb, slots = 2 * h->num_sms;
+    double best = 1e30;
+    prm.cl = 1;
+    for (int cl = 1; cl <= 8 && cl <= prm.n_steps; ++cl) {
+        const double cost = std::ceil((double)tiles * cl / slots) * ((double)prm.n_steps / cl + 4.0 + (cl > 1 ? 1.0 : 0.0));
+        if (cost < best) { best = cost; prm.cl = cl; }
+    }
+    return launch(kern, prm, dim3((unsigned)(tiles * prm.cl)), dim3(kMidThreads), S::kTotal, st, prm.cl, h->pdl);
+}
+
+// Up to 32 tokens (Config::mid_max_m): beyond, the MMAs of this kernel take longer than the 256-token tiles of the prefill
+// kernel on wide layers (48 tokens: Llama gate + up 59 us against 49).
+template <int BITS, bool GROUPED, bool GATED, bool KSCALE = false>
+cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, cudaStream_t st)
+{
+    if (prm.M <= 16) return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, st);
+    if (prm.M <= 24) return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, st);
+    if (prm.M <= 32) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, st);
+    return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, st);
+}
+
+// n layers that share K and scheme, layer i on xs[i]; act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
+// kscales != nullptr (int8 layers): layer i's input is multiplied by kscales[i][0 .. K).
+ql_status forward_mid(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st, int act = -1,
+                      const void* const* kscales = nullptr)
+{
+    const qlinear_s* h = hs[0];
+    const Layout& L = h->L;
+    MidParams prm{};
+    int units = 0;
+    for (int i = 0; i < n; ++i) {
+        const Layout& Li = hs[i]->L;
+        prm.body[i] = hs[i]->blob + Li.body_offset;
+        prm.chan_scales[i] = Li.grouped ? nullptr : reinterpret_cast<const __half*>(hs[i]->blob + Li.chan_scale_offset);
+        prm.x[i] = static_cast<const __half*>(xs[i]);
+        prm.kscale[i] = static_cast<const __half*>(kscales ? kscales[i] : nullptr);
+        prm.y[i] = static_cast<__half*>(ys[act >= 0 ? 0 : i]);
+        prm.N[i] = Li.N;
+        units += Li.n_rsb;
+        prm.unit_end[i] = units;
+    }
+    if (act >= 0) units = (L.N + 63) / 64;                               // half super-blocks of one layer
+    prm.n_layers = n; prm.M = M; prm.K = L.K; prm.n_kc = L.n_kc; prm.act = act >= 0 ? act : 0;
+    cudaError_t e;
+    if (kscales) e = launch_mid<8, false, false, true>(h, prm, units, st);
+    else if (act >= 0) e = L.bits == 8 ? launch_mid<8, false, true>(h, prm, units, st) : L.grouped ? launch_mid<4, true, true>(h, prm, units, st) : launch_mid<4, false, true>(h, prm, units, st);
+    else e = L.bits == 8 ? launch_mid<8, false, false>(h, prm, units, st) : L.grouped ? launch_mid<4, true, false>(h, prm, units, st) : launch_mid<4, false, false>(h, prm, units, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
 // y = act(g) * u, element-wise (the unfused form of the gating, for shapes the fused kernels do not take).
 __global__ void __launch_bounds__(256) gate_mul_kernel(const __half* g, const __half* u, __half* y, int64_t n, int act)
 {
@@ -591,6 +657,7 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
     if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (M <= h->gemv_max_m) return h->use_stream ? forward_gemv_stream(h, x, y, M, st) : forward_gemv(&h, 1, x, &y, M, st);
+    if (M <= config().mid_max_m) return forward_mid(&h, 1, &x, &y, M, st);
     {
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_ok ? &h->wmap : nullptr;
@@ -616,6 +683,13 @@ extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const
         DeviceGuard guard(hs[0]->device);
         if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
         return forward_gemv(const_cast<qlinear_s* const*>(hs), n, x, ys, M, static_cast<cudaStream_t>(stream));
+    }
+    if (n > 1 && M > hs[0]->gemv_max_m && M <= config().mid_max_m) {
+        DeviceGuard guard(hs[0]->device);
+        if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
+        const void* xs[kGemvMaxGroup];
+        for (int i = 0; i < n; ++i) xs[i] = x;
+        return forward_mid(const_cast<const qlinear_s* const*>(hs), n, xs, ys, M, static_cast<cudaStream_t>(stream));
     }
     if (n > 1 && M > hs[0]->gemv_max_m) {                                // prefill: one launch of the CTA-pair kernel
         bool pair_ok = true;
@@ -681,6 +755,9 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
         void* ys[2] = {y, y};
         const ql_status s = forward_gemv(hs, 2, x, ys, M, st, act);
         if (s != QL_ERR_UNSUPPORTED) return s;
+    } else if (M > hg->gemv_max_m && M <= config().mid_max_m) {
+        const void* xs[2] = {x, x};
+        return forward_mid(hs, 2, xs, &y, M, st, act);
     } else if (M > hg->gemv_max_m && gemm_pair_applicable(a, M)) {       // prefill: both accumulators of the CTA-pair kernel
         GemmPairLayers set{};
         set.n = 2;
@@ -889,6 +966,14 @@ extern "C" ql_status qlinear_kv_output(qlinear_t hv, const void* prob, const voi
     if (!((reinterpret_cast<uintptr_t>(prob) | reinterpret_cast<uintptr_t>(v_scale)) & 15)) {
         const ql_status s = qlinear_kv_output_heads(&hv, 1, prob, &v_scale, out, R, stream);
         if (s != QL_ERR_UNSUPPORTED) return s;
+        // more rows: the kernel that takes any number of tokens against few channels, with the scales folded in on the way
+        if (R > hv->gemv_max_m) {
+            if (device_timed_out(hv)) return QL_ERR_DEVICE_TIMEOUT;
+            DeviceGuard guard(hv->device);
+            if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
+            const qlinear_s* h = hv;
+            return forward_mid(&h, 1, &prob, &out, R, static_cast<cudaStream_t>(stream), -1, &v_scale);
+        }
     }
     {
         DeviceGuard guard(hv->device);
