@@ -62,6 +62,7 @@ struct GemvParamsT {
     int32_t x_stride;                    // halves between tokens in the shared x slab
     int32_t x_bytes;                     // bytes of the x slab (the warp rings follow it)
     int32_t act;                         // gated form only: activation of the gate branch (QL_ACT_*)
+    int32_t late;                        // the weights may come from the previous kernel (a KV cache): nothing of them is read before griddepcontrol.wait
 };
 using GemvParams = GemvParamsT<kGemvMaxGroup>;
 
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
 
     // Weights do not depend on the previous kernel: fill the ring before waiting for it.
+    if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (GROUPED) copy16(sbuf_u32, wsrc + s_off, kc0 + (lane >> 2) < kc1);
 #pragma unroll
     for (int d = 0; d < kGemvRing; ++d) {                                // one commit group per pair of chunks

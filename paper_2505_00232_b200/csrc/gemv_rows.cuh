@@ -29,6 +29,7 @@ struct GemvRowsParams {
     int32_t N[kGemvMaxBatch];
     int32_t rsb_end[kGemvMaxBatch];              // row super-blocks of layers 0..i
     int32_t n_layers, M, K, n_rsb, block_bytes;
+    int32_t late;                                // as in GemvParamsT
 };
 
 // NKC: chunks of 32 along K (K = 32 * NKC).
@@ -62,6 +63,7 @@ __global__ void __launch_bounds__(kGemvThreads, NKC <= 4 ? 4 : 3) gemv_rows_kern
     };
 
     int sb = blockIdx.x, stage = 0;
+    if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
     issue(sb, 0);                                                       // weights do not depend on the previous kernel
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

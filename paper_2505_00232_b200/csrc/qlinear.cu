@@ -126,7 +126,7 @@ std::mutex g_dev_mutex;
 }  // namespace
 
 struct qlinear_s {
-    // Immutable after qlinear_create.
+    // Immutable after qlinear_create (but for `cache`).
     Layout L;
     const uint8_t* blob;
     int device;
@@ -141,9 +141,21 @@ struct qlinear_s {
     CUtensorMap wmap_i8;       // the same with the integer form's box (128 k per step)
     bool wmap_ok, wmap_i8_ok;
     DeviceState* dev;
+    // Set by the first append: the blob is a KV cache, and the kernel before a reader in the stream may be writing it.  The
+    // decode kernels then read it only after griddepcontrol.wait; every other kernel is launched without the programmatic edge.
+    // (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
+    std::atomic<bool> cache{false};
+    bool early() const { return pdl && !cache.load(std::memory_order_relaxed); }
 };
 
 namespace {
+
+bool any_cache(const qlinear_s* const* hs, int n)
+{
+    for (int i = 0; i < n; ++i)
+        if (hs[i]->cache.load(std::memory_order_relaxed)) return true;
+    return false;
+}
 
 constexpr int kGemvMaxSmem = 96 * 1024;
 
@@ -288,6 +300,7 @@ void fill_gemv_params(GemvParamsT<NG>& prm, qlinear_s* const* hs, int n, const v
     }
     prm.n_layers = n;
     prm.act = gated ? act : 0;
+    prm.late = any_cache(hs, n);
     prm.x = static_cast<const __half*>(xs ? xs[0] : x);
     for (int i = 0; i < NG; ++i) {
         prm.xl[i] = static_cast<const __half*>(xs ? xs[i < n ? i : 0] : x);
@@ -343,6 +356,7 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
             rp.rsb_end[i] = n_rsb;
         }
         if (n_rsb > 4 * h->num_sms) {
+            rp.late = any_cache(hs, n);
             rp.n_layers = n; rp.M = M; rp.K = L.K; rp.n_rsb = n_rsb; rp.block_bytes = L.block_bytes;
             const cudaError_t e = L.n_kc == 2 ? launch_gemv_rows<2>(h, rp, st) : L.n_kc == 4 ? launch_gemv_rows<4>(h, rp, st) : launch_gemv_rows<8>(h, rp, st);
             return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
@@ -368,7 +382,7 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
 }
 
 template <int BITS, bool GROUPED, int NT, bool GATED, bool KSCALE>
-cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, cudaStream_t st)
+cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pdl, cudaStream_t st)
 {
     using S = MidSmem<BITS, GROUPED, NT>;
     static std::atomic<bool> attr_set[kMaxDevices];
@@ -386,18 +400,18 @@ cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, cudaStr
         const double cost = std::ceil((double)tiles * cl / slots) * ((double)prm.n_steps / cl + 4.0 + (cl > 1 ? 1.0 : 0.0));
         if (cost < best) { best = cost; prm.cl = cl; }
     }
-    return launch(kern, prm, dim3((unsigned)(tiles * prm.cl)), dim3(kMidThreads), S::kTotal, st, prm.cl, h->pdl);
+    return launch(kern, prm, dim3((unsigned)(tiles * prm.cl)), dim3(kMidThreads), S::kTotal, st, prm.cl, pdl);
 }
 
 // Up to 32 tokens (Config::mid_max_m): beyond, the MMAs of this kernel take longer than the 256-token tiles of the prefill
 // kernel on wide layers (48 tokens: Llama gate + up 59 us against 49).
 template <int BITS, bool GROUPED, bool GATED, bool KSCALE = false>
-cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, cudaStream_t st)
+cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, bool pdl, cudaStream_t st)
 {
-    if (prm.M <= 16) return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, st);
-    if (prm.M <= 24) return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, st);
-    if (prm.M <= 32) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, st);
-    return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, st);
+    if (prm.M <= 16) return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, pdl, st);
+    if (prm.M <= 24) return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, pdl, st);
+    if (prm.M <= 32) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
+    return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
 }
 
 // n layers that share K and scheme, layer i on xs[i]; act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
@@ -422,10 +436,11 @@ ql_status forward_mid(const qlinear_s* const* hs, int n, const void* const* xs, 
     }
     if (act >= 0) units = (L.N + 63) / 64;                               // half super-blocks of one layer
     prm.n_layers = n; prm.M = M; prm.K = L.K; prm.n_kc = L.n_kc; prm.act = act >= 0 ? act : 0;
+    const bool pdl = h->pdl && !any_cache(hs, n);
     cudaError_t e;
-    if (kscales) e = launch_mid<8, false, false, true>(h, prm, units, st);
-    else if (act >= 0) e = L.bits == 8 ? launch_mid<8, false, true>(h, prm, units, st) : L.grouped ? launch_mid<4, true, true>(h, prm, units, st) : launch_mid<4, false, true>(h, prm, units, st);
-    else e = L.bits == 8 ? launch_mid<8, false, false>(h, prm, units, st) : L.grouped ? launch_mid<4, true, false>(h, prm, units, st) : launch_mid<4, false, false>(h, prm, units, st);
+    if (kscales) e = launch_mid<8, false, false, true>(h, prm, units, pdl, st);
+    else if (act >= 0) e = L.bits == 8 ? launch_mid<8, false, true>(h, prm, units, pdl, st) : L.grouped ? launch_mid<4, true, true>(h, prm, units, pdl, st) : launch_mid<4, false, true>(h, prm, units, pdl, st);
+    else e = L.bits == 8 ? launch_mid<8, false, false>(h, prm, units, pdl, st) : L.grouped ? launch_mid<4, true, false>(h, prm, units, pdl, st) : launch_mid<4, false, false>(h, prm, units, pdl, st);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
@@ -445,7 +460,7 @@ cudaError_t launch_stream_ns(const qlinear_s* h, const StreamParams& prm, cudaSt
     auto kern = gemv_stream_kernel<BITS, GROUPED, NS>;
     cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, NS * StreamStage<BITS>::kBytes);
     if (e != cudaSuccess) return e;
-    return launch(kern, prm, dim3(prm.P), dim3(kStreamThreads), (size_t)NS * StreamStage<BITS>::kBytes, st, 1, h->pdl);
+    return launch(kern, prm, dim3(prm.P), dim3(kStreamThreads), (size_t)NS * StreamStage<BITS>::kBytes, st, 1, h->early());
 }
 
 template <int BITS, bool GROUPED>
@@ -661,10 +676,10 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
     {
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_ok ? &h->wmap : nullptr;
-        const ql_status s = gemm_pair_forward_auto(set, x, M, st, h->device, h->pdl, h->num_sms, h->dev->gemm_scratch, h->dev->gemm_counters);
+        const ql_status s = gemm_pair_forward_auto(set, x, M, st, h->device, h->early(), h->num_sms, h->dev->gemm_scratch, h->dev->gemm_counters);
         if (s != QL_ERR_UNSUPPORTED) return s;                           // (an odd number of row super-blocks: the single-CTA kernel)
     }
-    return gemm_forward(h->L, h->blob, x, y, M, st, h->device, h->pdl, h->num_sms);
+    return gemm_forward(h->L, h->blob, x, y, M, st, h->device, h->early(), h->num_sms);
 }
 
 extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const void* x, void* const* ys, int32_t M, void* stream)
@@ -703,7 +718,7 @@ extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const
                 set.L[i] = &hs[i]->L; set.blob[i] = hs[i]->blob; set.y[i] = ys[i];
                 set.wmap[i] = hs[i]->wmap_ok ? &hs[i]->wmap : nullptr;
             }
-            const ql_status s = gemm_pair_forward_auto(set, x, M, static_cast<cudaStream_t>(stream), hs[0]->device, hs[0]->pdl, hs[0]->num_sms,
+            const ql_status s = gemm_pair_forward_auto(set, x, M, static_cast<cudaStream_t>(stream), hs[0]->device, hs[0]->pdl && !any_cache(hs, n), hs[0]->num_sms,
                                                        hs[0]->dev->gemm_scratch, hs[0]->dev->gemm_counters);
             if (s != QL_ERR_UNSUPPORTED) return s;
         }
@@ -763,8 +778,8 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
         set.n = 2;
         set.L[0] = &hg->L; set.blob[0] = hg->blob; set.y[0] = y; set.wmap[0] = hg->wmap_ok ? &hg->wmap : nullptr;
         set.L[1] = &hu->L; set.blob[1] = hu->blob; set.y[1] = y; set.wmap[1] = hu->wmap_ok ? &hu->wmap : nullptr;
-        if (gemm_pair_ta_applicable(set, M, hg->num_sms, true)) return gemm_pair_ta_forward_gated(set, x, M, act, st, hg->device, hg->pdl, hg->num_sms);
-        return gemm_pair_forward_gated(set, x, M, act, st, hg->device, hg->pdl, hg->num_sms);
+        if (gemm_pair_ta_applicable(set, M, hg->num_sms, true)) return gemm_pair_ta_forward_gated(set, x, M, act, st, hg->device, hg->pdl && !any_cache(hs, 2), hg->num_sms);
+        return gemm_pair_forward_gated(set, x, M, act, st, hg->device, hg->pdl && !any_cache(hs, 2), hg->num_sms);
     }
     // Unfused: the two projections into the device's shared scratch, then the element-wise product.
     const int64_t n = (int64_t)M * a.N;
@@ -787,7 +802,7 @@ cudaError_t launch_a8(const qlinear_s* h, const GemvA8Params& prm, const GemvPla
     auto kern = gemv_a8_kernel<BITS, GROUPED>;
     cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, kGemvMaxSmem);
     if (e != cudaSuccess) return e;
-    return launch(kern, prm, dim3(pl.grid), dim3(kGemvThreads), pl.smem_bytes, st, pl.cl, h->pdl);
+    return launch(kern, prm, dim3(pl.grid), dim3(kGemvThreads), pl.smem_bytes, st, pl.cl, h->early());
 }
 }  // namespace
 
@@ -816,8 +831,8 @@ extern "C" ql_status qlinear_forward_a8(qlinear_t h, const void* x, void* y, int
         if (cudaGetLastError() != cudaSuccess) return QL_ERR_CUDA;
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_i8_ok ? &h->wmap_i8 : nullptr;
-        if (gemm_pair_ta_i8_applicable(set, M, h->num_sms)) return gemm_pair_ta_forward_i8(set, xq, sx, rs, M, st, h->device, h->pdl, h->num_sms);
-        return gemm_pair_forward_i8(set, xq, sx, rs, M, st, h->device, h->pdl, h->num_sms);
+        if (gemm_pair_ta_i8_applicable(set, M, h->num_sms)) return gemm_pair_ta_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms);
+        return gemm_pair_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms);
     }
     const GemvPlan pl = plan_gemv(L, h->n_rb, M, h->num_sms, false, true);
     if (pl.grid <= 0) return QL_ERR_UNSUPPORTED;
@@ -882,6 +897,8 @@ extern "C" ql_status qlinear_kv_append_heads(const qlinear_t* hk, const qlinear_
         prm.k_scales[i] = reinterpret_cast<__half*>(kb + K.chan_scale_offset);
         prm.v_body[i] = vb + V.body_offset;
         prm.v_scale[i] = static_cast<__half*>(v_scales[i]);
+        hk[i]->cache.store(true, std::memory_order_relaxed);
+        hv[i]->cache.store(true, std::memory_order_relaxed);
     }
     prm.k_new = static_cast<const __half*>(k_new);
     prm.v_new = static_cast<const __half*>(v_new);

@@ -180,3 +180,40 @@ def test_small_launches_are_planned_without_clusters(P, torch):
     assert plan(v, 4)["cl"] == 1
     big = P.QLinear(P.Desc(4096, 14336, 8, 0), torch.zeros(P.qlinear_packed_size(P.Desc(4096, 14336, 8, 0)), dtype=torch.uint8, device="cuda"))
     assert plan(big, 1)["cl"] > 1
+
+
+@pytest.mark.parametrize("R", [GROUP, 64, 256])
+def test_products_see_the_tokens_appended_just_before(P, torch, R):
+    """append, scores, output enqueued back to back (a captured graph, replayed on new tokens), against the same calls with the
+    host waiting in between: the products request cache bytes ahead of their stream dependency, so the append may not let
+    them start before its bytes are written."""
+    n_heads, T = 8, 1000
+    k0, v0 = tensors(1700, T)
+    start = torch.from_numpy(np.stack([k0] * n_heads)).cuda(), torch.from_numpy(np.stack([v0] * n_heads)).cuda()
+    pair = [P.KVHeads(n_heads, CACHE, DH) for _ in range(2)]
+    for kv in pair:
+        kv.append(*start)
+    q = torch.randn((n_heads, R, DH), device="cuda").half()
+    prob = torch.full((n_heads, R, CACHE), 2.0 ** -10, dtype=torch.float16, device="cuda")
+    kn, vn = (torch.zeros((n_heads, 5, DH), dtype=torch.float16, device="cuda") for _ in range(2))
+
+    def step(kv, wait):
+        kv.length = T
+        kv.append(kn, vn)
+        wait()
+        sc = kv.scores(q)
+        wait()
+        return sc, [c.output(prob[i]) for i, c in enumerate(kv.heads)]
+    step(pair[0], lambda: None)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sc, out = step(pair[0], lambda: None)
+    for _ in range(20):
+        kn.copy_(torch.randn_like(kn) * 3)
+        vn.copy_(torch.randn_like(vn) * 3)
+        graph.replay()
+        torch.cuda.synchronize()
+        sc_w, out_w = step(pair[1], torch.cuda.synchronize)
+        torch.cuda.synchronize()
+        assert torch.equal(sc, sc_w) and all(torch.equal(a, b) for a, b in zip(out, out_w))
