@@ -25,6 +25,7 @@ __device__ unsigned int* g_status_host;
 #include "dequant.cuh"
 #include "embed.cuh"
 #include "gemv.cuh"
+#include "gemv_cols.cuh"
 #include "gemv_rows.cuh"
 #include "gemv_stream.cuh"
 #include "gemv_a8.cuh"
@@ -254,37 +255,33 @@ cudaError_t ensure_smem_attr(Kern kern, std::atomic<bool>* flags, int device, in
     return e;
 }
 
-template <int BITS, bool GROUPED, bool XDIRECT, bool GATED = false, bool XSCALE = false, int NG = kGemvMaxGroup>
+template <int BITS, bool GROUPED, bool XDIRECT, bool GATED = false, int NG = kGemvMaxGroup>
 cudaError_t launch_gemv_x(const qlinear_s* h, const GemvParamsT<NG>& prm, const GemvPlan& pl, cudaStream_t st)
 {
     static std::atomic<bool> attr_set[kMaxDevices];
-    auto kern = gemv_kernel<BITS, GROUPED, XDIRECT, GATED, XSCALE, NG>;
+    auto kern = gemv_kernel<BITS, GROUPED, XDIRECT, GATED, NG>;
     cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, kGemvMaxSmem);
     if (e != cudaSuccess) return e;
     return launch(kern, prm, dim3(pl.grid), dim3(kGemvThreads), pl.smem_bytes, st, pl.cl, h->pdl);
 }
 
 template <int BITS, bool GROUPED>
-cudaError_t launch_gemv(const qlinear_s* h, const GemvParams& prm, const GemvPlan& pl, cudaStream_t st, bool gated = false, bool xscale = false)
+cudaError_t launch_gemv(const qlinear_s* h, const GemvParams& prm, const GemvPlan& pl, cudaStream_t st, bool gated = false)
 {
-    if constexpr (BITS == 8 && !GROUPED) {
-        if (xscale) return launch_gemv_x<8, false, true, false, true>(h, prm, pl, st);   // (int8, direct x: checked by the caller)
-    }
     if (gated) return launch_gemv_x<BITS, GROUPED, true, true>(h, prm, pl, st);     // (planned only with direct x)
     return prm.x_bytes == 0 ? launch_gemv_x<BITS, GROUPED, true>(h, prm, pl, st)
                             : launch_gemv_x<BITS, GROUPED, false>(h, prm, pl, st);
 }
 // The wide form (5 to 8 layers, each with its own input read straight from global memory): int8 layers, the KV heads of
 // an attention layer.
-cudaError_t launch_gemv_wide(const qlinear_s* h, const GemvParamsT<kGemvMaxBatch>& prm, const GemvPlan& pl, cudaStream_t st, bool xscale)
+cudaError_t launch_gemv_wide(const qlinear_s* h, const GemvParamsT<kGemvMaxBatch>& prm, const GemvPlan& pl, cudaStream_t st)
 {
-    return xscale ? launch_gemv_x<8, false, true, false, true, kGemvMaxBatch>(h, prm, pl, st)
-                  : launch_gemv_x<8, false, true, false, false, kGemvMaxBatch>(h, prm, pl, st);
+    return launch_gemv_x<8, false, true, false, kGemvMaxBatch>(h, prm, pl, st);
 }
 
 template <int NG>
 void fill_gemv_params(GemvParamsT<NG>& prm, qlinear_s* const* hs, int n, const void* x, void* const* ys, int M, int n_rb, const GemvPlan& pl,
-                      int act, const void* const* xs, const void* const* xscales)
+                      int act, const void* const* xs)
 {
     const Layout& L = hs[0]->L;
     const bool gated = act >= 0;
@@ -302,10 +299,7 @@ void fill_gemv_params(GemvParamsT<NG>& prm, qlinear_s* const* hs, int n, const v
     prm.act = gated ? act : 0;
     prm.late = any_cache(hs, n);
     prm.x = static_cast<const __half*>(xs ? xs[0] : x);
-    for (int i = 0; i < NG; ++i) {
-        prm.xl[i] = static_cast<const __half*>(xs ? xs[i < n ? i : 0] : x);
-        prm.xscale[i] = static_cast<const __half*>(xscales ? xscales[i < n ? i : 0] : nullptr);
-    }
+    for (int i = 0; i < NG; ++i) prm.xl[i] = static_cast<const __half*>(xs ? xs[i < n ? i : 0] : x);
     prm.M = M; prm.K = L.K;
     prm.n_rb = n_rb;
     prm.n_kc = L.n_kc;
@@ -326,14 +320,39 @@ cudaError_t launch_gemv_rows(const qlinear_s* h, const GemvRowsParams& prm, cuda
     return launch(kern, prm, dim3(grid), dim3(kGemvThreads), smem, st, 1, h->pdl);
 }
 
+// The value product over a KV cache (gemv_cols.cuh): int8 layers of equal shape, every layer with its own input and input scales.
+ql_status forward_gemv_cols(qlinear_s* const* hs, int n, const void* const* xs, const void* const* xscales, void* const* ys, int M, cudaStream_t st)
+{
+    const qlinear_s* h = hs[0];
+    const Layout& L = h->L;
+    GemvColsParams p{};
+    for (int i = 0; i < n; ++i) {
+        p.body[i] = hs[i]->blob + L.body_offset;
+        p.chan_scales[i] = reinterpret_cast<const __half*>(hs[i]->blob + L.chan_scale_offset);
+        p.x[i] = static_cast<const __half*>(xs[i]);
+        p.xscale[i] = static_cast<const __half*>(xscales[i]);
+        p.y[i] = static_cast<__half*>(ys[i]);
+    }
+    p.n_layers = n; p.M = M; p.N = L.N; p.K = L.K; p.n_rb = h->n_rb; p.n_kc = L.n_kc;
+    p.late = any_cache(hs, n);
+    // one CTA per SM; a K split only while every warp keeps at least 4 chunks
+    p.cl = 1;
+    while (p.cl < 8 && n * h->n_rb * p.cl * 2 <= h->num_sms && L.n_kc >= kColsWarps * p.cl * 2 * 4) p.cl *= 2;
+    p.cps = (L.n_kc + kColsWarps * p.cl - 1) / (kColsWarps * p.cl);
+    static std::atomic<bool> attr_set[kMaxDevices];
+    cudaError_t e = ensure_smem_attr(gemv_cols_kernel, attr_set, h->device, kColsSmem);
+    if (e == cudaSuccess) e = launch(gemv_cols_kernel, p, dim3(n * h->n_rb * p.cl), dim3(kColsThreads), kColsSmem, st, p.cl, h->pdl);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
 // One launch for n layers that read the same x (n == 1: the plain forward).  The plan of a group is made per
 // call (integer arithmetic only); nothing is written to a handle.
 // act >= 0: the gated form (n == 2: gate, up; ys[0] the output; the row-blocks of the two layers alternate).
 // xs != nullptr: the batched form, layer i reads xs[i] (x is then ignored); needs the kernel form that reads x straight
-// from global memory; int8 layers may come up to kGemvMaxBatch at a time.  xscales != nullptr (with xs, int8 layers):
-// layer i's input is multiplied by xscales[i][0 .. K).
+// from global memory; int8 layers may come up to kGemvMaxBatch at a time.
 ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* ys, int M, cudaStream_t st, int act = -1,
-                       const void* const* xs = nullptr, const void* const* xscales = nullptr)
+                       const void* const* xs = nullptr)
 {
     const qlinear_s* h = hs[0];
     const Layout& L = h->L;
@@ -344,7 +363,7 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
     // Short K (the score product over a KV cache): the persistent form, whatever the number of rows.  With at most one wave of
     // row super-blocks it wins as well, having no ring to fill, no sums across warps and no barrier (8 heads of 128 at 1280
     // positions 4.1 -> 1.8 us, at 8192 6.7 -> 3.1 us; 2 heads of 64 at 1024 3.3 -> 1.5 us).
-    if (xs && !xscales && !gated && n <= kGemvMaxBatch && L.bits == 8 && (L.K % 32) == 0 && (L.n_kc == 2 || L.n_kc == 4 || L.n_kc == 8)) {
+    if (xs && !gated && n <= kGemvMaxBatch && L.bits == 8 && (L.K % 32) == 0 && (L.n_kc == 2 || L.n_kc == 4 || L.n_kc == 8)) {
         GemvRowsParams rp{};
         int n_rsb = 0;
         for (int i = 0; i < n; ++i) {
@@ -364,18 +383,17 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
     }
     const GemvPlan pl = gated ? plan_gemv(L, n_rb, M, h->num_sms, true) : n == 1 ? h->gemv[M] : plan_gemv(L, n_rb, M, h->num_sms);
     if ((gated || xs) && (pl.grid <= 0 || pl.x_bytes != 0)) return QL_ERR_UNSUPPORTED;
-    if (xscales && (!xs || L.bits != 8)) return QL_ERR_UNSUPPORTED;
     if (n > kGemvMaxGroup && (n > kGemvMaxBatch || !xs || L.bits != 8)) return QL_ERR_UNSUPPORTED;
     cudaError_t e;
     if (pl.grid <= 0) return QL_ERR_UNSUPPORTED;
     if (n > kGemvMaxGroup) {
         GemvParamsT<kGemvMaxBatch> wide{};
-        fill_gemv_params(wide, hs, n, x, ys, M, n_rb, pl, act, xs, xscales);
-        return launch_gemv_wide(h, wide, pl, st, xscales != nullptr) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+        fill_gemv_params(wide, hs, n, x, ys, M, n_rb, pl, act, xs);
+        return launch_gemv_wide(h, wide, pl, st) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
     }
     GemvParams prm{};
-    fill_gemv_params(prm, hs, n, x, ys, M, n_rb, pl, act, xs, xscales);
-    if (L.bits == 8) e = launch_gemv<8, false>(h, prm, pl, st, gated, xscales != nullptr);
+    fill_gemv_params(prm, hs, n, x, ys, M, n_rb, pl, act, xs);
+    if (L.bits == 8) e = launch_gemv<8, false>(h, prm, pl, st, gated);
     else if (L.grouped) e = launch_gemv<4, true>(h, prm, pl, st, gated);
     else e = launch_gemv<4, false>(h, prm, pl, st, gated);
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
@@ -967,7 +985,7 @@ extern "C" ql_status qlinear_kv_output_heads(const qlinear_t* hv, int32_t n_head
             xs[i] = static_cast<const __half*>(prob) + (h0 + i) * xs_stride;
             ys[i] = static_cast<__half*>(out) + (h0 + i) * ys_stride;
         }
-        const ql_status s = forward_gemv(const_cast<qlinear_s* const*>(hv + h0), n, nullptr, ys, R, static_cast<cudaStream_t>(stream), -1, xs, v_scales + h0);
+        const ql_status s = forward_gemv_cols(const_cast<qlinear_s* const*>(hv + h0), n, xs, v_scales + h0, ys, R, static_cast<cudaStream_t>(stream));
         if (s != QL_OK) return s;
     }
     return QL_OK;

@@ -217,3 +217,24 @@ def test_products_see_the_tokens_appended_just_before(P, torch, R):
         sc_w, out_w = step(pair[1], torch.cuda.synchronize)
         torch.cuda.synchronize()
         assert torch.equal(sc, sc_w) and all(torch.equal(a, b) for a, b in zip(out, out_w))
+
+
+@pytest.mark.parametrize("n_heads,d_h,cache,R", [(1, 64, 32, 1), (1, 64, 992, 8), (3, 128, 2048, 5), (8, 128, 4128, 4), (2, 256, 8192, 7)])
+def test_value_product_over_slices_of_any_length(P, torch, n_heads, d_h, cache, R):
+    """The decode kernel of the value product: fewer chunks than warps, a ring that is not a multiple of the slice, slices that
+    end early, with and without a split over a cluster."""
+    rng = np.random.default_rng(cache + R)
+    v = (rng.standard_normal((n_heads, cache, d_h)) * rng.uniform(0.2, 3.0, size=(n_heads, cache, 1))).astype(np.float16)
+    prob = (rng.random((n_heads, R, cache)) / cache).astype(np.float16)
+    heads = P.KVHeads(n_heads, cache, d_h)
+    vd = torch.from_numpy(v).cuda()
+    heads.append(vd, vd)
+    out = heads.output(torch.from_numpy(prob).cuda())
+    torch.cuda.synchronize()
+    assert heads.heads[0].v.device_status() == (0, 0)
+    for h in range(n_heads):
+        v_q, v_s = O.kv_quantize_rows(v[h])
+        folded = (prob[h].astype(np.float32) * v_s.astype(np.float32)).astype(np.float16)
+        y64, A, _ = O.kv_output(folded, np.ascontiguousarray(v_q.T), np.ones(d_h, np.float16))
+        ok, rel, worst = O.check_against(out[h].cpu().numpy(), y64, A)
+        assert ok, (h, rel, worst)
