@@ -577,12 +577,15 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         for (int g = my_turn; g < total_steps && ok; g += 3) {
             while (g >= tile_g0 + n_steps) { ++tile_j; tile_g0 += n_steps; }
             // an earlier tile still holds the accumulator: run its epilogue once it is complete, or, at the latest,
-            // after `forced` steps of this tile have been dequantised
-            if (epi_warp && next_epi < tile_j && (g - tile_g0 >= forced || tile_complete(next_epi))) {
+            // after `forced` steps of this tile have been dequantised, or before any step of the tile after next (a warp's
+            // steps of a short tile may all lie before `forced`): the slots it would wait for belong to tiles whose MMAs wait
+            // for this epilogue
+            while (epi_warp && next_epi < tile_j && (next_epi + 1 < tile_j || g - tile_g0 >= forced || tile_complete(next_epi))) {
                 epilogue(next_epi);
                 ++next_epi;
                 if (!ok) break;
             }
+            if (!ok) break;
             uint32_t r[16];
             // A weight stage whose ring length is not a multiple of the 3 turns is served by a different turn every time
             // round, so this warp has not seen the stage's previous phase: the load of step g - NW may still be in flight

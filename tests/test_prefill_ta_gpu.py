@@ -197,3 +197,29 @@ def test_back_to_back_multi_layer_launches_keep_their_bits(P, torch, form):
             assert torch.equal(y.view(torch.int16), f.view(torch.int16)), f"round {rnd}"
     torch.cuda.synchronize()
     assert lins[0].device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("N,K,M,bits,group", [(9216, 512, 777, 4, 32), (8192, 128, 2048, 8, 0), (8192, 64, 1500, 4, 32), (9216, 256, 1024, 4, 0), (9216, 544, 1030, 8, 0)])
+def test_many_tiles_of_few_k_steps_per_cluster(P, torch, N, K, M, bits, group):
+    """Several tiles per CTA pair with fewer k-steps than a dequantise warp needs to reach the step that forces the previous
+    tile's epilogue: every warp still runs it before the tile after next.  Plain and gated, launched back to back."""
+    layer = C.LayerSpec("t", N, K, bits, group, *((-8, 7) if bits == 4 else (-128, 127)))
+    w = [C.layer_weights(8800 + K + i, layer) for i in range(2)]
+    x = C.layer_activations(8800 + M, layer, M)
+    lins = [P.QLinear.from_weights(q, s, bits, group, device="cuda:0") for q, s in w]
+    xd = torch.from_numpy(x).cuda()
+    first = P.qlinear_forward_group(lins, xd)
+    gated = P.qlinear_forward_gated(lins[0], lins[1], xd, "silu")
+    for _ in range(20):
+        again = P.qlinear_forward_group(lins, xd)
+    torch.cuda.synchronize()
+    assert lins[0].device_status() == (0, 0)
+    assert all(torch.equal(a, b) for a, b in zip(first, again))
+    rows = np.r_[0:64, N - 64:N]                        # (channels of the first and the last tiles)
+    for y, (q, s) in zip(first, w):
+        y64, A, _ = O.linear(x, q[rows], s[rows], group)
+        ok, rel, worst = O.check_against(y.cpu().numpy()[:, rows], y64, A)
+        assert ok, (rel, worst)
+    g64, bound, _ = O.gated_linear(x, w[0][0][rows], w[0][1][rows], w[1][0][rows], w[1][1][rows], group, "silu")
+    ok, rel, worst = O.check_gated(gated.cpu().numpy()[:, rows], g64, bound)
+    assert ok, (rel, worst)
