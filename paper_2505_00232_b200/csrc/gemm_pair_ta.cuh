@@ -77,7 +77,7 @@ struct GemmTaSmem {
 };
 
 struct TaMaps {
-    CUtensorMap x;                       // [M, K] fp16, box 64 k x 128 tokens, 128-byte swizzle
+    CUtensorMap x;                       // [M, K] fp16, box 64 k x half a tile's tokens, 128-byte swizzle
     CUtensorMap w[kGemmMaxGroup];        // packed body of each layer as rows of 64 bytes, 64-byte swizzle
 };
 
@@ -220,7 +220,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     static_assert(!I8 || (!GATED && !GROUPED), "the integer form: per-channel scales, plain output");
     using S = GemmTaSmem<BITS, I8>;
     constexpr int NX = S::kXStages, NW = S::kWStages, NA = S::kASlots;
-    constexpr int BN = 256;
+    const int bn = p.bn;                                                 // tokens per tile: a multiple of 32, at most 256
     constexpr int W_BOX_BYTES = I8 ? S::kWBytes : BITS == 4 ? (GROUPED ? kWeightBlockBytes + kScaleBlockBytes : kWeightBlockBytes) : 2 * kWeightBlockBytes;
     extern __shared__ unsigned char smem_dyn[];
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -244,7 +244,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();                             // 0 = leader
-    const int n_mblk = (p.M + BN - 1) / BN;
+    const int n_mblk = (p.M + bn - 1) / bn;
     const int first_tile = blockIdx.x >> 1, tile_stride = gridDim.x >> 1;   // tile = (rsb pair, token block)
     // K split (p.split = 2 or 4 parts per tile; launches with so few tiles that every cluster then has ONE unit of work):
     // work unit v = tile * split + part, this cluster's part covers k-steps [it_base, it_base + n_steps) of its tile
@@ -337,17 +337,18 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             }
         }
     } else if (warp == 2) {
-        // ------------------------------------------------------------------ x producer (each CTA loads its 128 tokens)
+        // ------------------------------------------------------------------ x producer (each CTA loads its half of the tokens)
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.x) : "memory");
             asm volatile("griddepcontrol.wait;" ::: "memory");           // x may come from the previous kernel
             abort_flag[2] = 1;                                           // from here on, waiting counts against the time limit
             abort_flag[3] = 1;
+            const uint32_t x_bytes = (uint32_t)(bn >> 1) * 128;
             int s = 0, g = 0;
             bool ok = true;
             int tile, gl;
             for (int j = 0; ok && unit(j, tile, gl); ++j) {
-                const int m0 = (tile % n_mblk) * BN + 128 * (int)rank;   // this CTA's 128 tokens
+                const int m0 = (tile % n_mblk) * bn + (bn >> 1) * (int)rank;   // this CTA's half of the tokens
                 for (int it = 0; it < n_steps; ++it, ++g) {
                     // stage s was last used by step g - NX, whose MMAs signal A-slot barrier (g - NX) % NA; by then the
                     // afull barrier of step g's slot has completed its previous phase (step g - NA was issued earlier)
@@ -355,7 +356,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                         const int ao = (g - NX) % NA;
                         if (!mbar_wait(aempty_bar(ao), (uint32_t)((g - NX) / NA) & 1, abort_flag, 0x180 + ao)) { ok = false; break; }
                     }
-                    mbar_expect_tx(afull_bar(g % NA), S::kXBytes);
+                    mbar_expect_tx(afull_bar(g % NA), x_bytes);
                     tma_load_2d(xs_addr(s), &maps.x, (it_base + it) * S::kKStep, m0, afull_bar(g % NA));
                     if (++s == NX) s = 0;
                 }
@@ -370,9 +371,9 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         // The whole warp runs the loop (warp-uniform control flow, so counters and descriptors can stay in uniform
         // registers); one elected lane issues.
         if (rank == 0) {
-            // f16 x f16 -> f32, both operands K-major (A from tensor memory), M = 256 per pair, N = 256
+            // f16 x f16 -> f32, both operands K-major (A from tensor memory), M = 256 per pair, N = bn
             // (integer form: u8 weights x s8 activations -> s32)
-            const uint32_t idesc = (I8 ? (2u << 4) | (1u << 10) : (1u << 4)) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+            const uint32_t idesc = (I8 ? (2u << 4) | (1u << 10) : (1u << 4)) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
             const uint32_t b_lo0 = umma_desc_lo(xs_addr(0));
             int s = 0, a = 0;
             uint32_t apar = 0;
@@ -422,6 +423,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         const uint32_t out_addr = base + S::kOutOffset;
         unsigned char* out_ptr = base_ptr + S::kOutOffset;
         const int grp_thread = quarter * 32 + lane;                      // 0..127 inside the group of four warps
+        const int n_cols = max(0, min(64, bn - 64 * wi));                // columns (tokens) of this warp: 0, 32 or 64
         // K-split tile: every part parks its fp32 accumulator in the device's scratch ([token][channel], a warp writes
         // 128 contiguous bytes per token), frees the accumulator and counts itself in; the part that arrives last adds all
         // parts in part order (fixed order, no float atomics, nobody waits) and stores y.
@@ -429,16 +431,16 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             int rsb = 2 * (tile / n_mblk) + (int)rank;
             const int ly = pair_layer(p, rsb);
             const int N = p.lN[ly];
-            const int m0 = (tile % n_mblk) * BN + 64 * wi;
-            float* slab0 = p.scratch + ((int64_t)((tile * P) * 2 + (int)rank) * BN + 64 * wi) * 128 + grp_thread;   // part 0
-            const int64_t part_stride = (int64_t)2 * BN * 128;
+            const int m0 = (tile % n_mblk) * bn + 64 * wi;
+            float* slab0 = p.scratch + ((int64_t)((tile * P) * 2 + (int)rank) * bn + 64 * wi) * 128 + grp_thread;   // part 0
+            const int64_t part_stride = (int64_t)2 * bn * 128;
             unsigned int* cnt = p.counters + ((tile * 2 + (int)rank) * 4 + wi) * 4 + quarter;
             if (!mbar_wait(tfull_bar, (uint32_t)(j & 1), abort_flag, 0x500)) { ok = false; return; }
             tc_fence_after();
             const uint32_t taddr = tmem_base + lane_base + (uint32_t)(64 * wi);
             float* mine = slab0 + part * part_stride;
 #pragma unroll 1
-            for (int cc = 0; cc < 64; cc += 16) {
+            for (int cc = 0; cc < n_cols; cc += 16) {
                 uint32_t r[16];
                 tmem_ld16(taddr + (uint32_t)cc, r);
 #pragma unroll
@@ -456,7 +458,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             float scale = 1.f;
             if (!GROUPED && n < N) scale = __half2float(p.lscales[ly][n]);
             __half* yrow = p.ly[ly] + (int64_t)m0 * N + n;
-            const int m_left = min(64, p.M - m0);
+            const int m_left = min(n_cols, p.M - m0);
 #pragma unroll 1
             for (int cc = 0; cc < m_left; cc += 8) {
                 float acc[8];
@@ -484,7 +486,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             int rsb = 2 * (tile / n_mblk) + (int)rank;
             const int ly = GATED ? 0 : pair_layer(p, rsb);
             const int N = p.lN[ly];
-            const int m0 = (tile % n_mblk) * BN + 64 * wi;
+            const int m0 = (tile % n_mblk) * bn + 64 * wi;
             const uint32_t gpar = (uint32_t)(GATED ? j >> 1 : j) & 1;   // phase of the group barriers: once per output tile
             bool live = true;
             if (!GATED || gl == 0) {
@@ -502,19 +504,22 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                 if (!GROUPED && n < N) scale = __half2float(p.lscales[GATED ? gl : ly][n]);
                 const uint32_t taddr = tmem_base + lane_base + (uint32_t)(64 * wi);
                 __half* orow = reinterpret_cast<__half*>(out_ptr + (64 * wi) * 256) + grp_thread;
+                auto release = [&] {                                     // accumulator read: the next tile's MMAs may start
+                    // RELAXED arrive, like the relay's: what must precede the leader's next MMA is the completion of
+                    // this warp's tensor-memory loads, which tcgen05.wait::ld (inside tmem_ld32) has already waited
+                    // for; nothing in shared or global memory is handed over.  With release semantics at cluster
+                    // scope the arrive sat on the critical path of every tile boundary (Llama gate: 179 -> 176 us).
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_remote_relaxed(tempty_bar, 0);
+                };
+                if (n_cols == 0) release();
 #pragma unroll
                 for (int cc = 0; cc < 64; cc += 32) {
+                    if (cc >= n_cols) break;
                     uint32_t r[32];
                     tmem_ld32(taddr + (uint32_t)cc, r);
-                    if (cc == 32) {                                      // accumulator read: the next tile's MMAs may start
-                        // RELAXED arrive, like the relay's: what must precede the leader's next MMA is the completion of
-                        // this warp's tensor-memory loads, which tcgen05.wait::ld (inside tmem_ld32) has already waited
-                        // for; nothing in shared or global memory is handed over.  With release semantics at cluster
-                        // scope the arrive sat on the critical path of every tile boundary (Llama gate: 179 -> 176 us).
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_remote_relaxed(tempty_bar, 0);
-                    }
+                    if (cc + 32 >= n_cols) release();
                     if (I8) {
                         // acc = sum (q + off) * xq: remove off * (sum of the token's quantised row), then both scales; the 32
                         // tokens' scales and row sums come as whole lines (the arrays are padded to whole tiles)
@@ -551,7 +556,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             __syncwarp();
             if (lane == 0) mbar_arrive(grp_bar(wi, 1));
             live = mbar_wait(grp_bar(wi, 1), gpar, abort_flag, 0xC10 + wi) && live;
-            if (live && grp_thread < 64 && m0 + grp_thread < p.M) {
+            if (live && grp_thread < n_cols && m0 + grp_thread < p.M) {
                 const int n0 = rsb * kRsbRows;
                 const uint32_t bytes = (uint32_t)min(kRsbRows, N - n0) * 2;
                 bulk_copy_s2g(p.ly[ly] + (int64_t)(m0 + grp_thread) * N + n0, out_addr + (uint32_t)(64 * wi + grp_thread) * 256, bytes);
@@ -617,7 +622,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     }
 }
 
-// The tensor-memory form: 256-token tiles, whole tiles dealt out round-robin, or (fewer tiles than half the CTA pairs)
+// The tensor-memory form: tiles of up to 256 tokens, whole tiles dealt out round-robin, or (fewer tiles than half the CTA pairs)
 // 2 or 4 K parts per tile that meet in the device's scratch.
 // K parts per tile for a launch of `tiles` tiles: 1 unless the tiles would leave half of the CTA pairs (or more) idle.
 inline int gemm_pair_ta_split(int tiles, int n_ksteps, int num_sms, bool have_scratch)
@@ -644,7 +649,11 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const void* x, int M, c
     using S = GemmTaSmem<BITS, I8>;
     const Layout& L = *set.L[0];
     TaMaps maps;
-    if (!x_tensor_map(x, L.K, M, 128, &maps.x, I8 ? 1 : 2)) return QL_ERR_CUDA;
+    // Tokens per tile: M in as few blocks of at most 256 as it takes, all of the same width (the MMA's N, a multiple of 32).  A
+    // narrower tile costs the same dequantisation and less tensor-core time, x traffic and epilogue
+    // (a Llama block at 100 tokens 145.9 -> 136.9 us, at 300 224.9 -> 211.1).
+    const int n_mblk = (M + 255) / 256, bn = ((M + n_mblk - 1) / n_mblk + 31) / 32 * 32;
+    if (!x_tensor_map(x, L.K, M, bn / 2, &maps.x, I8 ? 1 : 2)) return QL_ERR_CUDA;
     for (int i = 0; i < kGemmMaxGroup; ++i) maps.w[i] = *set.wmap[i < set.n ? i : 0];
     auto kern = gemm_pair_ta_kernel<BITS, GROUPED, GATED, I8>;
     static std::atomic<bool> attr_set[64];
@@ -673,7 +682,8 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const void* x, int M, c
     prm.n_ksteps = (L.K + S::kKStep - 1) / S::kKStep;
     prm.a8_scale = a8_scale; prm.a8_rowsum = a8_rowsum;
     prm.n_rsb = n_rsb;
-    prm.n_tiles = (n_rsb / 2) * ((M + 255) / 256);
+    prm.bn = bn;
+    prm.n_tiles = (n_rsb / 2) * n_mblk;
     prm.split = (GATED || I8) ? 1 : gemm_pair_ta_split(prm.n_tiles, prm.n_ksteps, num_sms, scratch && counters);
     prm.scratch = scratch;
     prm.counters = counters;
