@@ -54,7 +54,7 @@ struct Config {
     int warps_per_sm;        // QLINEAR_GEMV_WARPS_PER_SM: residency target of the cluster decode kernel
     bool oversubscribe;      // QLINEAR_GEMV_OVERSUBSCRIBE=0: the group-scaled int4 decode kernel never takes more CTAs than fit at once
     int force_ks;            // QLINEAR_GEMV_KS: forced K split of the cluster decode kernel (0 = planned)
-    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M served by the kernel for a batch of tokens (0: never)
+    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M served by the kernel for a batch of tokens (0: never); see takes_mid
     bool xdirect;            // QLINEAR_GEMV_XDIRECT: x fragments straight from global memory
     int kernel;              // QLINEAR_GEMV_KERNEL: 0 / 1 cluster kernel (default), 2 streaming kernel
     int stream_ctas_per_sm, stream_stages;
@@ -73,7 +73,7 @@ void load_config()
     c.warps_per_sm = env_int("QLINEAR_GEMV_WARPS_PER_SM", 32);
     c.oversubscribe = env_int("QLINEAR_GEMV_OVERSUBSCRIBE", 1) != 0;
     c.force_ks = env_int("QLINEAR_GEMV_KS", 0);
-    c.mid_max_m = env_int("QLINEAR_MID_MAX_M", 32);
+    c.mid_max_m = env_int("QLINEAR_MID_MAX_M", 64);
     c.xdirect = env_int("QLINEAR_GEMV_XDIRECT", 1) != 0;
     const char* kc = std::getenv("QLINEAR_GEMV_KERNEL");
     c.kernel = !kc ? 0 : !std::strcmp(kc, "cluster") ? 1 : !std::strcmp(kc, "stream") ? 2 : 0;
@@ -421,14 +421,27 @@ cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pd
     return launch(kern, prm, dim3((unsigned)(tiles * prm.cl)), dim3(kMidThreads), S::kTotal, st, prm.cl, pdl);
 }
 
-// Up to 32 tokens (Config::mid_max_m): beyond, the MMAs of this kernel take longer than the 256-token tiles of the prefill
-// kernel on wide layers (48 tokens: Llama gate + up 59 us against 49).
+// Which launches take this kernel: up to 32 tokens all of them, up to 64 those with at most 48 million weights.  Beyond, its
+// MMAs take longer than the prefill kernel, which does not depend on M below 256 tokens but has fewer and larger tiles.
+// Measured at 64 tokens, this kernel / the prefill kernel: 117 M weights (Llama gate + up) 59 / 49 us, 59 M (down) 29.8 /
+// 29.3, 42 M (Gemma2-2B gate + up) 19.4 / 21.5, 21 M (its down) 20.9 / 22.0, 17 M (Llama o) 12.7 / 17.6, 9 M 10.0 / 15.7.
+bool takes_mid(const qlinear_s* const* hs, int n, int M)
+{
+    const int max_m = config().mid_max_m;
+    if (M <= max_m / 2) return true;
+    if (M > max_m) return false;
+    int64_t weights = 0;
+    for (int i = 0; i < n; ++i) weights += (int64_t)hs[i]->L.N * hs[i]->L.K;
+    return weights <= 48000000;
+}
+
 template <int BITS, bool GROUPED, bool GATED, bool KSCALE = false>
 cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, bool pdl, cudaStream_t st)
 {
     if (prm.M <= 16) return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, pdl, st);
     if (prm.M <= 24) return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, pdl, st);
     if (prm.M <= 32) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
+    if (prm.M <= 48) return launch_mid_nt<BITS, GROUPED, 6, GATED, KSCALE>(h, prm, units, pdl, st);
     return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
 }
 
@@ -690,7 +703,7 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
     if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (M <= h->gemv_max_m) return h->use_stream ? forward_gemv_stream(h, x, y, M, st) : forward_gemv(&h, 1, x, &y, M, st);
-    if (M <= config().mid_max_m) return forward_mid(&h, 1, &x, &y, M, st);
+    if (takes_mid(&h, 1, M)) return forward_mid(&h, 1, &x, &y, M, st);
     {
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_ok ? &h->wmap : nullptr;
@@ -717,7 +730,7 @@ extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const
         if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
         return forward_gemv(const_cast<qlinear_s* const*>(hs), n, x, ys, M, static_cast<cudaStream_t>(stream));
     }
-    if (n > 1 && M > hs[0]->gemv_max_m && M <= config().mid_max_m) {
+    if (n > 1 && M > hs[0]->gemv_max_m && takes_mid(hs, n, M)) {
         DeviceGuard guard(hs[0]->device);
         if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
         const void* xs[kGemvMaxGroup];
@@ -788,7 +801,7 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
         void* ys[2] = {y, y};
         const ql_status s = forward_gemv(hs, 2, x, ys, M, st, act);
         if (s != QL_ERR_UNSUPPORTED) return s;
-    } else if (M > hg->gemv_max_m && M <= config().mid_max_m) {
+    } else if (M > hg->gemv_max_m && takes_mid(hs, 2, M)) {
         const void* xs[2] = {x, x};
         return forward_mid(hs, 2, xs, &y, M, st, act);
     } else if (M > hg->gemv_max_m && gemm_pair_applicable(a, M)) {       // prefill: both accumulators of the CTA-pair kernel

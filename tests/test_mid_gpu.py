@@ -1,4 +1,4 @@
-"""The kernel for a batch of tokens (9 to 32) and for the value product of many query rows, against the CPU oracle, on a
+"""The kernel for a batch of tokens (9 to 64) and for the value product of many query rows, against the CPU oracle, on a
 B200: edges of its token blocks, of the 128-channel super-blocks and of its two-chunk stages, with and without a K split."""
 import numpy as np
 import pytest
@@ -28,7 +28,7 @@ def spec(N, K, bits, group):
 
 
 @pytest.mark.parametrize("bits,group", [(4, 32), (4, 0), (4, 128), (8, 0)])
-@pytest.mark.parametrize("M", [9, 16, 17, 24, 25, 32])
+@pytest.mark.parametrize("M", [9, 16, 17, 24, 25, 32, 33, 48, 64])
 @pytest.mark.parametrize("N,K", [(8, 128), (136, 384), (264, 2048), (640, 1152)])
 def test_layer_group_and_gated_match_the_oracle(P, torch, M, N, K, bits, group):
     """One layer, three layers in one launch (of different widths), and the gated pair; K not a whole number of stages
