@@ -45,6 +45,7 @@ struct MidParams {
     int32_t N[kMidMaxLayers];
     int32_t unit_end[kMidMaxLayers];             // row units of layers 0..i
     int32_t n_layers, M, K, n_kc, n_steps, n_tb, cl, act;
+    int32_t late;                                // the weights may come from the previous kernel (a KV cache): nothing of them is read before griddepcontrol.wait
 };
 
 template <int BITS, bool GROUPED, int NT>
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(kMidThreads, 2) gemm_mid_kernel(const MidParam
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
 
     // Weights do not depend on the previous kernel: those of the first stages are requested before waiting for it.
+    if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll
     for (int s = 0; s < NS - 1; ++s)
         if (st0 + s < st1) load_weights(st0 + s, s);

@@ -32,6 +32,7 @@ __device__ unsigned int* g_status_host;
 #include "kv.cuh"
 #include "gemm.cuh"
 #include "gemm_mid.cuh"
+#include "gemm_rows.cuh"
 #include "gemm_pair.cuh"
 #include "gemm_pair_ta.cuh"
 #include "norm.cuh"
@@ -143,8 +144,8 @@ struct qlinear_s {
     bool wmap_ok, wmap_i8_ok;
     DeviceState* dev;
     // Set by the first append: the blob is a KV cache, and the kernel before a reader in the stream may be writing it.  The
-    // decode kernels then read it only after griddepcontrol.wait; every other kernel is launched without the programmatic edge.
-    // (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
+    // decode and batch kernels then read it only after griddepcontrol.wait; the prefill kernels are launched without the programmatic
+    // edge.  (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
     std::atomic<bool> cache{false};
     bool early() const { return pdl && !cache.load(std::memory_order_relaxed); }
 };
@@ -441,6 +442,8 @@ cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, bool pdl, 
     if (prm.M <= 16) return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, pdl, st);
     if (prm.M <= 24) return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, pdl, st);
     if (prm.M <= 32) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
+    // (more tokens than that: the value product.  Tiles of 32 tokens where those of 64 would leave every SM with one CTA.)
+    if (prm.M > 64 && units * ((prm.M + 63) / 64) * 8 <= 2 * h->num_sms) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
     if (prm.M <= 48) return launch_mid_nt<BITS, GROUPED, 6, GATED, KSCALE>(h, prm, units, pdl, st);
     return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
 }
@@ -467,11 +470,56 @@ ql_status forward_mid(const qlinear_s* const* hs, int n, const void* const* xs, 
     }
     if (act >= 0) units = (L.N + 63) / 64;                               // half super-blocks of one layer
     prm.n_layers = n; prm.M = M; prm.K = L.K; prm.n_kc = L.n_kc; prm.act = act >= 0 ? act : 0;
-    const bool pdl = h->pdl && !any_cache(hs, n);
+    prm.late = any_cache(hs, n);
+    const bool pdl = h->pdl;
     cudaError_t e;
     if (kscales) e = launch_mid<8, false, false, true>(h, prm, units, pdl, st);
     else if (act >= 0) e = L.bits == 8 ? launch_mid<8, false, true>(h, prm, units, pdl, st) : L.grouped ? launch_mid<4, true, true>(h, prm, units, pdl, st) : launch_mid<4, false, true>(h, prm, units, pdl, st);
     else e = L.bits == 8 ? launch_mid<8, false, false>(h, prm, units, pdl, st) : L.grouped ? launch_mid<4, true, false>(h, prm, units, pdl, st) : launch_mid<4, false, false>(h, prm, units, pdl, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
+template <int NKC, int NT>
+cudaError_t launch_gemm_rows_nt(const qlinear_s* h, GemmRowsParams& prm, int n_rsb, bool pdl, cudaStream_t st)
+{
+    using S = GemmRowsSmem<NKC, NT>;
+    static std::atomic<bool> attr_set[kMaxDevices];
+    auto kern = gemm_rows_kernel<NKC, NT>;
+    cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, S::kTotal);
+    if (e != cudaSuccess) return e;
+    prm.n_tb = (prm.M + S::kTokens - 1) / S::kTokens;
+    prm.n_tiles = n_rsb * prm.n_tb;
+    return launch(kern, prm, dim3(std::min(prm.n_tiles, 2 * h->num_sms)), dim3(256), S::kTotal, st, 1, pdl);
+}
+template <int NKC>
+cudaError_t launch_gemm_rows(const qlinear_s* h, GemmRowsParams& prm, int n_rsb, bool pdl, cudaStream_t st)
+{
+    if (prm.M <= 16) return launch_gemm_rows_nt<NKC, 2>(h, prm, n_rsb, pdl, st);
+    if (prm.M <= 32) return launch_gemm_rows_nt<NKC, 4>(h, prm, n_rsb, pdl, st);
+    return launch_gemm_rows_nt<NKC, 8>(h, prm, n_rsb, pdl, st);
+}
+// The layers gemm_rows.cuh takes: int8, K of 64, 128 or 256 (the head dimensions of a K cache), any number of rows and tokens.
+bool takes_gemm_rows(const Layout& L) { return L.bits == 8 && (L.n_kc == 2 || L.n_kc == 4 || L.n_kc == 8) && L.K == 32 * L.n_kc; }
+ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st)
+{
+    const qlinear_s* h = hs[0];
+    GemmRowsParams prm{};
+    int n_rsb = 0;
+    for (int i = 0; i < n; ++i) {
+        const Layout& Li = hs[i]->L;
+        prm.body[i] = hs[i]->blob + Li.body_offset;
+        prm.chan_scales[i] = reinterpret_cast<const __half*>(hs[i]->blob + Li.chan_scale_offset);
+        prm.x[i] = static_cast<const __half*>(xs[i]);
+        prm.y[i] = static_cast<__half*>(ys[i]);
+        prm.N[i] = Li.N;
+        n_rsb += Li.n_rsb;
+        prm.rsb_end[i] = n_rsb;
+    }
+    prm.n_layers = n; prm.M = M;
+    const bool pdl = h->pdl;                                             // (every byte is read after griddepcontrol.wait)
+    const int n_kc = h->L.n_kc;
+    const cudaError_t e = n_kc == 2 ? launch_gemm_rows<2>(h, prm, n_rsb, pdl, st) : n_kc == 4 ? launch_gemm_rows<4>(h, prm, n_rsb, pdl, st) : launch_gemm_rows<8>(h, prm, n_rsb, pdl, st);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
@@ -703,6 +751,7 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
     if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (M <= h->gemv_max_m) return h->use_stream ? forward_gemv_stream(h, x, y, M, st) : forward_gemv(&h, 1, x, &y, M, st);
+    if (takes_gemm_rows(h->L)) return forward_gemm_rows(&h, 1, &x, &y, M, st);
     if (takes_mid(&h, 1, M)) return forward_mid(&h, 1, &x, &y, M, st);
     {
         GemmPairLayers set{};
@@ -776,6 +825,11 @@ extern "C" ql_status qlinear_forward_batch(const qlinear_t* hs, int32_t n, const
         if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
         const ql_status s = forward_gemv(const_cast<qlinear_s* const*>(hs), n, nullptr, ys, M, static_cast<cudaStream_t>(stream), -1, xs);
         if (s != QL_ERR_UNSUPPORTED) return s;
+    }
+    if (n > 1 && M > hs[0]->gemv_max_m && takes_gemm_rows(hs[0]->L)) {   // (the K caches of a prompt's attention)
+        DeviceGuard guard(hs[0]->device);
+        if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
+        return forward_gemm_rows(hs, n, xs, ys, M, static_cast<cudaStream_t>(stream));
     }
     for (int i = 0; i < n; ++i) {                                        // anything else: one call per layer
         const ql_status s = qlinear_forward(hs[i], xs[i], ys[i], M, stream);

@@ -238,3 +238,25 @@ def test_value_product_over_slices_of_any_length(P, torch, n_heads, d_h, cache, 
         y64, A, _ = O.kv_output(folded, np.ascontiguousarray(v_q.T), np.ones(d_h, np.float16))
         ok, rel, worst = O.check_against(out[h].cpu().numpy(), y64, A)
         assert ok, (h, rel, worst)
+
+
+@pytest.mark.parametrize("n_heads,d_h,cache,T,R", [(3, 64, 96, 90, 9), (1, 256, 992, 992, 17), (8, 128, 1280, 1031, 33), (11, 128, 160, 130, 100), (2, 64, 8192, 8000, 65), (2, 128, 4096, 3256, 1024)])
+def test_scores_of_many_rows(P, torch, n_heads, d_h, cache, T, R):
+    """The kernel of the score product for more than 8 query rows: token blocks of 16, 32 and 64 with a remainder, a last
+    super-block that is not full, CTAs whose range of tiles spans heads; per head and all heads in one launch agree."""
+    rng = np.random.default_rng(cache + R)
+    k = (rng.standard_normal((n_heads, T, d_h)) * rng.uniform(0.2, 3.0, size=(n_heads, T, 1))).astype(np.float16)
+    q = rng.standard_normal((n_heads, R, d_h)).astype(np.float16)
+    heads = P.KVHeads(n_heads, cache, d_h)
+    kd, qd = torch.from_numpy(k).cuda(), torch.from_numpy(q).cuda()
+    heads.append(kd, kd)
+    sc = heads.scores(qd)
+    torch.cuda.synchronize()
+    assert heads.heads[0].k.device_status() == (0, 0)
+    assert (sc[:, :, T:] == 0).all()
+    for h in range(n_heads):
+        assert torch.equal(sc[h], heads.heads[h].scores(qd[h]))
+        k_q, k_s = O.kv_quantize_rows(k[h])
+        y64, A, _ = O.linear(q[h], k_q, k_s.reshape(-1, 1), 0)
+        ok, rel, worst = O.check_against(sc[h, :, :T].cpu().numpy(), y64, A)
+        assert ok, (h, rel, worst)
