@@ -880,14 +880,22 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
 }
 
 namespace {
-template <int BITS, bool GROUPED>
-cudaError_t launch_a8(const qlinear_s* h, const GemvA8Params& prm, const GemvPlan& pl, cudaStream_t st)
+template <int BITS, bool GROUPED, int T>
+cudaError_t launch_a8_t(const qlinear_s* h, const GemvA8Params& prm, const GemvPlan& pl, cudaStream_t st)
 {
     static std::atomic<bool> attr_set[kMaxDevices];
-    auto kern = gemv_a8_kernel<BITS, GROUPED>;
+    auto kern = gemv_a8_kernel<BITS, GROUPED, T>;
     cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, kGemvMaxSmem);
     if (e != cudaSuccess) return e;
     return launch(kern, prm, dim3(pl.grid), dim3(kGemvThreads), pl.smem_bytes, st, pl.cl, h->early());
+}
+template <int BITS, bool GROUPED>
+cudaError_t launch_a8(const qlinear_s* h, const GemvA8Params& prm, const GemvPlan& pl, cudaStream_t st)
+{
+    if (prm.M == 1) return launch_a8_t<BITS, GROUPED, 1>(h, prm, pl, st);
+    if (prm.M == 2) return launch_a8_t<BITS, GROUPED, 2>(h, prm, pl, st);
+    if (prm.M <= 4) return launch_a8_t<BITS, GROUPED, 4>(h, prm, pl, st);
+    return launch_a8_t<BITS, GROUPED, 8>(h, prm, pl, st);
 }
 }  // namespace
 

@@ -74,6 +74,18 @@ def test_a8_decode_parity(P, torch, M, N, K, bits, group):
     assert torch.equal(y, lin.forward_a8(xd))         # run-to-run identical
 
 
+@pytest.mark.parametrize("M,K,bits,group", [(1, 16384, 4, 32), (1, 16416, 8, 0), (2, 8192, 4, 0), (2, 8224, 8, 0), (4, 4096, 8, 0), (3, 4160, 4, 32), (8, 2048, 4, 32), (6, 2080, 8, 0)])
+def test_a8_decode_rows_at_the_edge_of_what_registers_keep(P, torch, M, K, bits, group):
+    """The longest rows a CTA keeps in registers between the two quantisation steps, and the next longer ones."""
+    q, s, x = rand_case(7300 + K + M, M, 136, K, bits, group)
+    x *= np.linspace(0.5, 3.0, M, dtype=np.float16)[:, None]
+    lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
+    y = lin.forward_a8(torch.from_numpy(x).cuda())
+    torch.cuda.synchronize()
+    assert lin.device_status() == (0, 0)
+    assert_a8(y.cpu().numpy(), x, q, s, group)
+
+
 @pytest.mark.parametrize("bits,group", [(8, 0), (4, 32), (4, 0)])
 def test_a8_integer_path_is_bit_exact_when_no_rounding_is_left(P, torch, bits, group):
     """Power-of-two scales and x on the int8 grid: every fp32 operation of the dequantisation is exact, so the
