@@ -169,11 +169,37 @@ def qlinear_unpack(desc: Desc, packed: np.ndarray):
 
 
 # ---------------------------------------------------------------------------- device calls
-def _stream_ptr(stream) -> ctypes.c_void_p:
+# A small layer takes the GPU a few microseconds, less than these calls took the host: so the raw handle of the current
+# stream is asked for without building a Stream object, pointers go to ctypes as plain integers (the argument types are
+# declared), and a tensor's properties are checked in one expression.  Measured: QLinear.forward at one token 11.8 -> 7.0 us.
+_torch = _half = _raw_stream = _device = None
+
+
+def _bind_torch() -> None:
+    """torch is imported with the first device object, not with the package (packing needs none of it)."""
+    global _torch, _half, _raw_stream, _device
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    _torch, _half, _raw_stream, _device = torch, torch.float16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
+def _stream_ptr(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if _torch is None:
+        _bind_torch()
+    return _raw_stream(_device())                                        # the current stream of the current device
+
+
+def _is_out(out, M: int, N: int) -> bool:
+    return tuple(out.shape) == (M, N) and out.dtype == _half and out.is_contiguous()
+
+
+def _is_x(x, K: int) -> bool:
+    """A contiguous fp16 CUDA tensor [M, K]."""
+    if _half is None:
+        _bind_torch()
+    shape = x.shape
+    return len(shape) == 2 and shape[1] == K and x.dtype == _half and x.is_cuda and x.is_contiguous()
 
 
 def qlinear_decode_static(desc: Desc, packed, x, out=None, stream=None):
@@ -190,8 +216,8 @@ def qlinear_decode_static(desc: Desc, packed, x, out=None, stream=None):
         out = torch.empty((M, desc.N), dtype=torch.float16, device=x.device)
     elif out.shape != (M, desc.N) or out.dtype != torch.float16 or not out.is_contiguous() or out.device != x.device:
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_decode_static (bad out tensor)")
-    _check(lib.qlinear_decode_static(ctypes.byref(desc.c()), ctypes.c_void_p(packed.data_ptr()),
-                                     ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(out.data_ptr()), M,
+    _check(lib.qlinear_decode_static(ctypes.byref(desc.c()), packed.data_ptr(),
+                                     x.data_ptr(), out.data_ptr(), M,
                                      x.device.index or 0, _stream_ptr(stream)), "qlinear_decode_static")
     return out
 
@@ -200,16 +226,16 @@ def qlinear_forward_group_raw(lins, x_ptr: int, y_ptrs, M: int, stream=None) -> 
     """qlinear_forward_group on raw device pointers: the layers `lins` applied to one x."""
     n = len(lins)
     hs = (ctypes.c_void_p * n)(*[l._h for l in lins])
-    ys = (ctypes.c_void_p * n)(*[ctypes.c_void_p(int(p)) for p in y_ptrs])
-    _check(lib.qlinear_forward_group(hs, n, ctypes.c_void_p(x_ptr), ys, M, _stream_ptr(stream)), "qlinear_forward_group")
+    ys = (ctypes.c_void_p * n)(*map(int, y_ptrs))
+    _check(lib.qlinear_forward_group(hs, n, x_ptr, ys, M, _stream_ptr(stream)), "qlinear_forward_group")
 
 
 def qlinear_forward_batch_raw(lins, x_ptrs, y_ptrs, M: int, stream=None) -> None:
     """qlinear_forward_batch on raw device pointers: layer i applied to its own input x_ptrs[i]."""
     n = len(lins)
     hs = (ctypes.c_void_p * n)(*[l._h for l in lins])
-    xs = (ctypes.c_void_p * n)(*[ctypes.c_void_p(int(p)) for p in x_ptrs])
-    ys = (ctypes.c_void_p * n)(*[ctypes.c_void_p(int(p)) for p in y_ptrs])
+    xs = (ctypes.c_void_p * n)(*map(int, x_ptrs))
+    ys = (ctypes.c_void_p * n)(*map(int, y_ptrs))
     _check(lib.qlinear_forward_batch(hs, n, xs, ys, M, _stream_ptr(stream)), "qlinear_forward_batch")
 
 
@@ -223,9 +249,9 @@ def qlinear_forward_batch(lins, xs, outs=None, stream=None):
         if x.dim() != 2 or tuple(x.shape) != (M, K) or x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous():
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_batch (every x must be contiguous fp16 CUDA [M, K])")
     if outs is None:
-        outs = [torch.empty((M, l.desc.N), dtype=torch.float16, device=xs[0].device) for l in lins]
+        outs = [xs[0].new_empty((M, l.desc.N)) for l in lins]
     for l, o in zip(lins, outs):
-        if o.shape != (M, l.desc.N) or o.dtype != torch.float16 or not o.is_contiguous():
+        if not _is_out(o, M, l.desc.N):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_batch (bad out tensor)")
     qlinear_forward_batch_raw(lins, [x.data_ptr() for x in xs], [o.data_ptr() for o in outs], M, stream)
     return outs
@@ -238,37 +264,35 @@ def kv_scores_batch(caches, q_rows, stream=None):
 
 def qlinear_forward_group(lins, x, outs=None, stream=None):
     """x: fp16 CUDA tensor [M, K] -> list of fp16 [M, N_i], one per layer (one launch for M <= 8)."""
-    import torch
     K = lins[0].desc.K
-    if x.dim() != 2 or x.shape[1] != K or x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous():
+    if not _is_x(x, K):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_group (x must be contiguous fp16 CUDA [M, K])")
     M = x.shape[0]
     if outs is None:
-        outs = [torch.empty((M, l.desc.N), dtype=torch.float16, device=x.device) for l in lins]
+        outs = [x.new_empty((M, l.desc.N)) for l in lins]
     for l, o in zip(lins, outs):
-        if o.shape != (M, l.desc.N) or o.dtype != torch.float16 or not o.is_contiguous():
+        if not _is_out(o, M, l.desc.N):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_group (bad out tensor)")
     qlinear_forward_group_raw(lins, x.data_ptr(), [o.data_ptr() for o in outs], M, stream)
     return outs
 
 
 def qlinear_forward_gated_raw(gate, up, x_ptr: int, y_ptr: int, M: int, act: str, stream=None) -> None:
-    _check(lib.qlinear_forward_gated(gate._h, up._h, ctypes.c_void_p(x_ptr), ctypes.c_void_p(y_ptr), M, ACTIVATIONS[act],
+    _check(lib.qlinear_forward_gated(gate._h, up._h, x_ptr, y_ptr, M, ACTIVATIONS[act],
                                      _stream_ptr(stream)), "qlinear_forward_gated")
 
 
 def qlinear_forward_gated(gate, up, x, act: str = "silu", out=None, stream=None):
     """y = act(x . W_gate^T) * (x . W_up^T) as fp16 [M, N], from one fused launch where the shape allows."""
-    import torch
     K, N = gate.desc.K, gate.desc.N
-    if x.dim() != 2 or x.shape[1] != K or x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous():
+    if not _is_x(x, K):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_gated (x must be contiguous fp16 CUDA [M, K])")
     if act not in ACTIVATIONS:
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_gated (unknown activation)")
     M = x.shape[0]
     if out is None:
-        out = torch.empty((M, N), dtype=torch.float16, device=x.device)
-    elif out.shape != (M, N) or out.dtype != torch.float16 or not out.is_contiguous():
+        out = x.new_empty((M, N))
+    elif not _is_out(out, M, N):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_gated (bad out tensor)")
     qlinear_forward_gated_raw(gate, up, x.data_ptr(), out.data_ptr(), M, act, stream)
     return out
@@ -282,7 +306,7 @@ def qlinear_quantize_activations(x, stream=None):
     M, K = x.shape
     xq = torch.empty((M, K), dtype=torch.int8, device=x.device)
     scale = torch.empty((M,), dtype=torch.float32, device=x.device)
-    _check(lib.qlinear_quantize_activations(ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(xq.data_ptr()), ctypes.c_void_p(scale.data_ptr()),
+    _check(lib.qlinear_quantize_activations(x.data_ptr(), xq.data_ptr(), scale.data_ptr(),
                                             M, K, x.device.index or 0, _stream_ptr(stream)), "qlinear_quantize_activations")
     return xq, scale
 
@@ -290,24 +314,26 @@ def qlinear_quantize_activations(x, stream=None):
 def qlinear_residual_rmsnorm(x, residual, gamma, eps: float, gamma_offset: float = 0.0, h_out=None, y_out=None, want_h=True, stream=None):
     """x, residual (or None) fp16 CUDA [M, K], gamma fp16 [K] -> (h, y): h = x + residual, y = rmsnorm(h) * (gamma_offset + gamma).
     h_out / y_out may be given (h_out may be x or residual: in place); want_h=False skips the h output (h is then None)."""
-    import torch
+    if _half is None:
+        _bind_torch()
+    dev = x.get_device()
     def ok(t, shape):
-        return t.dtype == torch.float16 and t.is_cuda and t.is_contiguous() and tuple(t.shape) == shape and t.device == x.device
+        return t.dtype == _half and t.get_device() == dev and t.is_cuda and t.is_contiguous() and tuple(t.shape) == shape
     if x.dim() != 2 or not ok(x, tuple(x.shape)) or x.shape[1] % 8 or x.shape[1] < 8:
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_residual_rmsnorm (x must be contiguous fp16 CUDA [M, K], K % 8 == 0)")
     M, K = x.shape
     if (residual is not None and not ok(residual, (M, K))) or not ok(gamma, (K,)):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_residual_rmsnorm (residual [M, K] / gamma [K] fp16 on x's device)")
-    if y_out is None:
-        y_out = torch.empty_like(x)
-    if h_out is None and want_h:
-        h_out = torch.empty_like(x)
-    if not ok(y_out, (M, K)) or (h_out is not None and not ok(h_out, (M, K))):
+    if (y_out is not None and not ok(y_out, (M, K))) or (h_out is not None and not ok(h_out, (M, K))):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_residual_rmsnorm (bad output tensor)")
-    _check(lib.qlinear_residual_rmsnorm(ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(residual.data_ptr() if residual is not None else None),
-                                        ctypes.c_void_p(gamma.data_ptr()), float(eps), float(gamma_offset),
-                                        ctypes.c_void_p(h_out.data_ptr() if h_out is not None else None), ctypes.c_void_p(y_out.data_ptr()),
-                                        M, K, x.device.index or 0, _stream_ptr(stream)), "qlinear_residual_rmsnorm")
+    if y_out is None:
+        y_out = x.new_empty((M, K))
+    if h_out is None and want_h:
+        h_out = x.new_empty((M, K))
+    _check(lib.qlinear_residual_rmsnorm(x.data_ptr(), residual.data_ptr() if residual is not None else None,
+                                        gamma.data_ptr(), float(eps), float(gamma_offset),
+                                        h_out.data_ptr() if h_out is not None else None, y_out.data_ptr(),
+                                        M, K, dev, _stream_ptr(stream)), "qlinear_residual_rmsnorm")
     return h_out, y_out
 
 
@@ -316,19 +342,20 @@ def qlinear_rope_qkv(q, k, v, pos, cos, sin, B: int, S: int, h_q: int, h_kv: int
     -> (q_out [B*h_kv, S*h_q/h_kv, d_h], k_out [B*h_kv, S, d_h], v_out [B*h_kv, S, d_h]): rotary embedding + layout change."""
     import torch
     T = B * S
+    dev = q.get_device()
     def ok(t, dtype, shape):
-        return t.dtype == dtype and t.is_cuda and t.is_contiguous() and tuple(t.shape) == shape and t.device == q.device
+        return t.dtype == dtype and t.get_device() == dev and t.is_cuda and t.is_contiguous() and tuple(t.shape) == shape
     if h_kv < 1 or h_q % h_kv or d_h % 16 or not ok(q, torch.float16, (T, h_q * d_h)) or not ok(k, torch.float16, (T, h_kv * d_h)) \
             or not ok(v, torch.float16, (T, h_kv * d_h)) or not ok(pos, torch.int32, (T,)) or cos.dim() != 2 \
             or not ok(cos, torch.float32, (cos.shape[0], d_h // 2)) or not ok(sin, torch.float32, tuple(cos.shape)):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_rope_qkv (shapes / dtypes: see the header)")
     g = h_q // h_kv
-    q_out = torch.empty((B * h_kv, S * g, d_h), dtype=torch.float16, device=q.device)
-    k_out = torch.empty((B * h_kv, S, d_h), dtype=torch.float16, device=q.device)
-    v_out = torch.empty((B * h_kv, S, d_h), dtype=torch.float16, device=q.device)
-    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    q_out = q.new_empty((B * h_kv, S * g, d_h))
+    k_out = q.new_empty((B * h_kv, S, d_h))
+    v_out = q.new_empty((B * h_kv, S, d_h))
+    p = lambda t: t.data_ptr()
     _check(lib.qlinear_rope_qkv(p(q), p(k), p(v), p(pos), p(cos), p(sin), cos.shape[0], p(q_out), p(k_out), p(v_out), B, S, h_q, h_kv, d_h,
-                                q.device.index or 0, _stream_ptr(stream)), "qlinear_rope_qkv")
+                                dev, _stream_ptr(stream)), "qlinear_rope_qkv")
     return q_out, k_out, v_out
 
 
@@ -337,6 +364,7 @@ class QLinear:
 
     def __init__(self, desc: Desc, packed, device=None):
         import torch
+        _bind_torch()
         self.desc = desc
         if isinstance(packed, np.ndarray):
             dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
@@ -348,7 +376,7 @@ class QLinear:
         self.packed = packed                      # keeps the device memory alive
         self.device = packed.device
         h = ctypes.c_void_p()
-        _check(lib.qlinear_create(ctypes.byref(desc.c()), ctypes.c_void_p(packed.data_ptr()),
+        _check(lib.qlinear_create(ctypes.byref(desc.c()), packed.data_ptr(),
                                   self.device.index or 0, ctypes.byref(h)), "qlinear_create")
         self._h = h
 
@@ -359,36 +387,34 @@ class QLinear:
 
     def forward(self, x, out=None, stream=None):
         """x: fp16 CUDA tensor [M, K] -> y fp16 [M, N] (qlinear_forward on the current stream)."""
-        import torch
-        if x.dim() != 2 or x.shape[1] != self.desc.K or x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous():
+        if not _is_x(x, self.desc.K):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward (x must be contiguous fp16 CUDA [M, K])")
         M = x.shape[0]
         if out is None:
-            out = torch.empty((M, self.desc.N), dtype=torch.float16, device=x.device)
-        elif out.shape != (M, self.desc.N) or out.dtype != torch.float16 or not out.is_contiguous():
+            out = x.new_empty((M, self.desc.N))
+        elif not _is_out(out, M, self.desc.N):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward (bad out tensor)")
         self.forward_raw(x.data_ptr(), out.data_ptr(), M, stream)
         return out
 
     def forward_a8(self, x, out=None, stream=None):
         """The decode call with int8 activations quantised inside the kernel (qlinear_forward_a8), M <= 8."""
-        import torch
-        if x.dim() != 2 or x.shape[1] != self.desc.K or x.dtype != torch.float16 or not x.is_cuda or not x.is_contiguous():
+        if not _is_x(x, self.desc.K):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_a8 (x must be contiguous fp16 CUDA [M, K])")
         M = x.shape[0]
         if out is None:
-            out = torch.empty((M, self.desc.N), dtype=torch.float16, device=x.device)
-        elif out.shape != (M, self.desc.N) or out.dtype != torch.float16 or not out.is_contiguous():
+            out = x.new_empty((M, self.desc.N))
+        elif not _is_out(out, M, self.desc.N):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_a8 (bad out tensor)")
-        _check(lib.qlinear_forward_a8(self._h, ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(out.data_ptr()), M, _stream_ptr(stream)),
+        _check(lib.qlinear_forward_a8(self._h, x.data_ptr(), out.data_ptr(), M, _stream_ptr(stream)),
                "qlinear_forward_a8")
         return out
 
     def forward_a8_raw(self, x_ptr: int, y_ptr: int, M: int, stream=None) -> None:
-        _check(lib.qlinear_forward_a8(self._h, ctypes.c_void_p(x_ptr), ctypes.c_void_p(y_ptr), M, _stream_ptr(stream)), "qlinear_forward_a8")
+        _check(lib.qlinear_forward_a8(self._h, x_ptr, y_ptr, M, _stream_ptr(stream)), "qlinear_forward_a8")
 
     def forward_raw(self, x_ptr: int, y_ptr: int, M: int, stream=None) -> None:
-        _check(lib.qlinear_forward(self._h, ctypes.c_void_p(x_ptr), ctypes.c_void_p(y_ptr), M, _stream_ptr(stream)),
+        _check(lib.qlinear_forward(self._h, x_ptr, y_ptr, M, _stream_ptr(stream)),
                "qlinear_forward")
 
     def embed(self, ids, out=None, stream=None):
@@ -401,7 +427,7 @@ class QLinear:
             out = torch.empty((n, self.desc.K), dtype=torch.float16, device=ids.device)
         elif out.shape != (n, self.desc.K) or out.dtype != torch.float16 or not out.is_contiguous():
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_embed (bad out tensor)")
-        _check(lib.qlinear_embed(self._h, ctypes.c_void_p(ids.data_ptr()), n, ctypes.c_void_p(out.data_ptr()),
+        _check(lib.qlinear_embed(self._h, ids.data_ptr(), n, out.data_ptr(),
                                  _stream_ptr(stream)), "qlinear_embed")
         return out
 
@@ -411,7 +437,7 @@ class QLinear:
     def debug_unpack(self, stream=None):
         import torch
         q = torch.empty((self.desc.N, self.desc.K), dtype=torch.int8, device=self.device)
-        _check(lib.qlinear_debug_unpack_device(self._h, ctypes.c_void_p(q.data_ptr()), _stream_ptr(stream)),
+        _check(lib.qlinear_debug_unpack_device(self._h, q.data_ptr(), _stream_ptr(stream)),
                "qlinear_debug_unpack_device")
         return q
 
@@ -461,29 +487,27 @@ class KVCache:
         n = k_new.shape[0]
         if v_new.shape[0] != n:
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_append (k_new and v_new differ in length)")
-        _check(lib.qlinear_kv_append(self.k._h, self.v._h, ctypes.c_void_p(k_new.data_ptr()), ctypes.c_void_p(v_new.data_ptr()),
-                                     ctypes.c_void_p(self.v_scale.data_ptr()), self.length, n, _stream_ptr(stream)), "qlinear_kv_append")
+        _check(lib.qlinear_kv_append(self.k._h, self.v._h, k_new.data_ptr(), v_new.data_ptr(),
+                                     self.v_scale.data_ptr(), self.length, n, _stream_ptr(stream)), "qlinear_kv_append")
         self.length += n
 
     def scores(self, q_rows, stream=None):
         """q_rows fp16 [R, d_h] -> fp16 [R, cache_size] (positions beyond `length` score 0)."""
-        import torch
-        if q_rows.dim() != 2 or q_rows.shape[1] != self.d_h or q_rows.dtype != torch.float16 or not q_rows.is_cuda or not q_rows.is_contiguous():
+        if not _is_x(q_rows, self.d_h):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_scores (q_rows must be contiguous fp16 CUDA [R, d_h])")
-        out = torch.empty((q_rows.shape[0], self.cache_size), dtype=torch.float16, device=q_rows.device)
-        _check(lib.qlinear_kv_scores(self.k._h, ctypes.c_void_p(q_rows.data_ptr()), ctypes.c_void_p(out.data_ptr()), q_rows.shape[0],
+        out = q_rows.new_empty((q_rows.shape[0], self.cache_size))
+        _check(lib.qlinear_kv_scores(self.k._h, q_rows.data_ptr(), out.data_ptr(), q_rows.shape[0],
                                      _stream_ptr(stream)), "qlinear_kv_scores")
         return out
 
     def output(self, prob, stream=None):
         """prob fp16 [R, cache_size] -> fp16 [R, d_h]."""
-        import torch
-        if prob.dim() != 2 or prob.shape[1] != self.cache_size or prob.dtype != torch.float16 or not prob.is_cuda or not prob.is_contiguous():
+        if not _is_x(prob, self.cache_size):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_output (prob must be contiguous fp16 CUDA [R, cache_size])")
-        tmp = torch.empty_like(prob)
-        out = torch.empty((prob.shape[0], self.d_h), dtype=torch.float16, device=prob.device)
-        _check(lib.qlinear_kv_output(self.v._h, ctypes.c_void_p(prob.data_ptr()), ctypes.c_void_p(self.v_scale.data_ptr()),
-                                     ctypes.c_void_p(tmp.data_ptr()), ctypes.c_void_p(out.data_ptr()), prob.shape[0], _stream_ptr(stream)),
+        tmp = prob.new_empty(prob.shape)
+        out = prob.new_empty((prob.shape[0], self.d_h))
+        _check(lib.qlinear_kv_output(self.v._h, prob.data_ptr(), self.v_scale.data_ptr(),
+                                     tmp.data_ptr(), out.data_ptr(), prob.shape[0], _stream_ptr(stream)),
                "qlinear_kv_output")
         return out
 
@@ -498,10 +522,10 @@ class KVHeads:
         arr = ctypes.c_void_p * n_heads
         self._hk = arr(*[c.k._h for c in self.heads])
         self._hv = arr(*[c.v._h for c in self.heads])
-        self._vs = arr(*[ctypes.c_void_p(c.v_scale.data_ptr()) for c in self.heads])
+        self._vs = arr(*[c.v_scale.data_ptr() for c in self.heads])
 
     def append_raw(self, k_ptr: int, v_ptr: int, head_stride: int, token_stride: int, n_new: int, stream=None) -> None:
-        _check(lib.qlinear_kv_append_heads(self._hk, self._hv, self.n, ctypes.c_void_p(k_ptr), ctypes.c_void_p(v_ptr), head_stride, token_stride,
+        _check(lib.qlinear_kv_append_heads(self._hk, self._hv, self.n, k_ptr, v_ptr, head_stride, token_stride,
                                            self._vs, self.length, n_new, _stream_ptr(stream)), "qlinear_kv_append_heads")
         self.length += n_new
         for c in self.heads:
@@ -519,7 +543,7 @@ class KVHeads:
         self.append_raw(k_new.data_ptr(), v_new.data_ptr(), n_new * self.d_h, self.d_h, n_new, stream)
 
     def scores_raw(self, q_ptr: int, out_ptr: int, R: int, stream=None) -> None:
-        _check(lib.qlinear_kv_scores_heads(self._hk, self.n, ctypes.c_void_p(q_ptr), ctypes.c_void_p(out_ptr), R, _stream_ptr(stream)),
+        _check(lib.qlinear_kv_scores_heads(self._hk, self.n, q_ptr, out_ptr, R, _stream_ptr(stream)),
                "qlinear_kv_scores_heads")
 
     def scores(self, q_rows, stream=None):
@@ -527,12 +551,12 @@ class KVHeads:
         import torch
         if q_rows.dim() != 3 or q_rows.shape[0] != self.n or q_rows.shape[2] != self.d_h or q_rows.dtype != torch.float16 or not q_rows.is_cuda or not q_rows.is_contiguous():
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_scores_heads (q_rows must be contiguous fp16 CUDA [n_heads, R, d_h])")
-        out = torch.empty((self.n, q_rows.shape[1], self.cache_size), dtype=torch.float16, device=q_rows.device)
+        out = q_rows.new_empty((self.n, q_rows.shape[1], self.cache_size))
         self.scores_raw(q_rows.data_ptr(), out.data_ptr(), q_rows.shape[1], stream)
         return out
 
     def output_raw(self, prob_ptr: int, out_ptr: int, R: int, stream=None) -> None:
-        _check(lib.qlinear_kv_output_heads(self._hv, self.n, ctypes.c_void_p(prob_ptr), self._vs, ctypes.c_void_p(out_ptr), R, _stream_ptr(stream)),
+        _check(lib.qlinear_kv_output_heads(self._hv, self.n, prob_ptr, self._vs, out_ptr, R, _stream_ptr(stream)),
                "qlinear_kv_output_heads")
 
     def output(self, prob, stream=None):
@@ -540,6 +564,6 @@ class KVHeads:
         import torch
         if prob.dim() != 3 or prob.shape[0] != self.n or prob.shape[2] != self.cache_size or prob.dtype != torch.float16 or not prob.is_cuda or not prob.is_contiguous():
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_output_heads (prob must be contiguous fp16 CUDA [n_heads, R, cache_size])")
-        out = torch.empty((self.n, prob.shape[1], self.d_h), dtype=torch.float16, device=prob.device)
+        out = prob.new_empty((self.n, prob.shape[1], self.d_h))
         self.output_raw(prob.data_ptr(), out.data_ptr(), prob.shape[1], stream)
         return out
