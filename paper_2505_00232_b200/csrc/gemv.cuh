@@ -66,7 +66,15 @@ using GemvParams = GemvParamsT<kGemvMaxGroup>;
 // alternately, so that a CTA (which then holds an even number of row-blocks, no cluster) has both branches of
 // every output channel it owns; the epilogue writes y[0] = act(gate) * up (paper Section 3.6: element-wise
 // operators of two branches fused with a fully connected operator).
-template <int BITS, bool GROUPED, bool XDIRECT, bool GATED = false, int NG = kGemvMaxGroup>
+// ONE: a single token (group-scaled layers): only column 0 of the MMA is ever stored, so the group scales are applied to the
+// two accumulator registers of the even columns alone.
+//
+// The loop is bound by its instruction stream as much as by HBM (with the math taken out LM head would take 47 us, Llama
+// gate + up 12.5, down 7.0), so what is not arithmetic is kept out of it: the block size is a constant for int4, per-thread
+// addresses pass through an empty asm statement so that the compiler does not form them again from the lane number at the
+// register limit, and int8 refills are predicated copies.  Before / after, one token: LM head (295 MB) 55.5 / 53.4 us, gate +
+// up 17.3 / 15.4, down 10.2 / 9.9, Llama q + k + v (int8) 6.1 / 5.9, o 5.4 / 5.1, Gemma2-2B q + k + v 3.95 / 3.64.
+template <int BITS, bool GROUPED, bool XDIRECT, bool GATED = false, int NG = kGemvMaxGroup, bool ONE = false>
 __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT<NG> p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -77,6 +85,7 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, c = lane & 3;
     constexpr int CHUNK_K = BITS == 4 ? 64 : 32;
+    const int BB = BITS == 4 ? kWeightBlockBytes + (GROUPED ? kScaleBlockBytes : 0) : p.block_bytes;
 
     // No integer division on the way in: ks_cta is a power of two, and the position inside the cluster
     // comes from the special registers (without a cluster launch they read rank 0, cluster id = block id).
@@ -111,15 +120,23 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
     constexpr int WARP_SMEM = kGemvRing * 512 + (GROUPED ? 2 * 512 : 0);
     unsigned char* ring = smem_raw + p.x_bytes + warp * WARP_SMEM;
     unsigned char* sbuf = ring + kGemvRing * 512;
-    const uint32_t ring_u32 = (uint32_t)__cvta_generic_to_shared(ring) + lane * 16;
-    const uint32_t sbuf_u32 = (uint32_t)__cvta_generic_to_shared(sbuf) + lane * 16;
-    const uint8_t* blk = p.body[layer] + ((int64_t)(rb >> 3) * p.n_kc + kc0) * p.block_bytes;
+    uint32_t ring_u32 = (uint32_t)__cvta_generic_to_shared(ring) + lane * 16;
+    if (BITS == 4) asm volatile("" : "+r"(ring_u32));
+    const uint32_t sbuf_u32 = ring_u32 + kGemvRing * 512;
+    const uint8_t* blk = p.body[layer] + ((int64_t)(rb >> 3) * p.n_kc + kc0) * BB;
     const uint8_t* wsrc = blk + (rb & 7) * 512 + lane * 16;
     // lane L copies part (L & 3) of the scales of chunk (pass start + L / 4); the address is kept relative
     // to the weight address of the pass's first chunk (wsrc at the top of a pass)
-    const int s_off = (lane >> 2) * p.block_bytes + kWeightBlockBytes - (rb & 7) * 448 + (lane & 3) * 16 - lane * 16;
+    int s_off = (lane >> 2) * BB + kWeightBlockBytes - (rb & 7) * 448 + (lane & 3) * 16 - lane * 16;
 
-    auto copy16 = [](uint32_t dst, const void* src, bool in_range) {     // out of range: reads nothing, writes zeros
+    if (GROUPED) asm volatile("" : "+r"(s_off));
+    // Out of range: int8 copies nothing (a predicated copy; no such slot reaches the math), int4 reads nothing and writes zeros
+    // (there the size operand, formed ahead of time, is the cheaper form: Llama gate + up 15.4 us against 16.0).
+    auto copy16 = [](uint32_t dst, const void* src, bool in_range) {
+        if (BITS == 8) {
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p cp.async.cg.shared.global [%0], [%1], 16;\n\t}" ::"r"(dst), "l"(src), "r"((int)in_range) : "memory");
+            return;
+        }
         const uint32_t sz = in_range ? 16u : 0u;
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(sz) : "memory");
     };
@@ -132,7 +149,7 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
     for (int d = 0; d < kGemvRing; ++d) {                                // one commit group per pair of chunks
         copy16(ring_u32 + d * 512, wsrc, kc0 + d < kc1);
         if (d & 1) commit();
-        wsrc += p.block_bytes;
+        wsrc += BB;
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // Per-channel scales are weights too: the (at most 4) this thread will apply when it stores outputs are requested
@@ -202,7 +219,8 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
         asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
         return v;
     };
-    const uint32_t sc_u32 = sbuf_u32 - lane * 16 + g * 8;                // this lane's scales inside a pass buffer
+    uint32_t sc_u32 = sbuf_u32 - lane * 16 + g * 8;                // this lane's scales inside a pass buffer
+    if (GROUPED) asm volatile("" : "+r"(sc_u32));
     int sflip = 0;                                                       // scale buffer of the current pass
 
     // one chunk: unpack in registers, feed the tensor core, apply the group scales in fp32
@@ -224,9 +242,11 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
                     const float sg = h == 0 ? __low2float(s_lo) : __high2float(s_lo);
                     const float sg8 = h == 0 ? __low2float(s_hi) : __high2float(s_hi);
                     total[0] = fmaf(sg, acc[0], total[0]);
-                    total[1] = fmaf(sg, acc[1], total[1]);
                     total[2] = fmaf(sg8, acc[2], total[2]);
-                    total[3] = fmaf(sg8, acc[3], total[3]);
+                    if (!ONE) {
+                        total[1] = fmaf(sg, acc[1], total[1]);
+                        total[3] = fmaf(sg8, acc[3], total[3]);
+                    }
                 } else {
                     unpack_int4_word(ww[2 * h], a);
                     mma_16816_pure(total, a, xv.x, xv.y);
@@ -271,9 +291,9 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
                 sc1 = lds64(sc_u32 + sflip * 512 + (d + 1) * 64);
             }
             copy16(ring_u32 + d * 512, wsrc, !checked || kc + d + kGemvRing < kc1);      // refill the slots just read
-            copy16(ring_u32 + (d + 1) * 512, wsrc + p.block_bytes, !checked || kc + d + 1 + kGemvRing < kc1);
+            copy16(ring_u32 + (d + 1) * 512, wsrc + BB, !checked || kc + d + 1 + kGemvRing < kc1);
             commit();                                                    // (one group per pair)
-            wsrc += 2 * (int64_t)p.block_bytes;
+            wsrc += 2 * (int64_t)BB;
             if (two) {
                 chunk_math(w0, sc0, x00, x01);
                 chunk_math(w1, sc1, x10, x11);

@@ -256,11 +256,14 @@ cudaError_t ensure_smem_attr(Kern kern, std::atomic<bool>* flags, int device, in
     return e;
 }
 
-template <int BITS, bool GROUPED, bool XDIRECT, bool GATED = false, int NG = kGemvMaxGroup>
+template <int BITS, bool GROUPED, bool XDIRECT, bool GATED = false, int NG = kGemvMaxGroup, bool ONE = false>
 cudaError_t launch_gemv_x(const qlinear_s* h, const GemvParamsT<NG>& prm, const GemvPlan& pl, cudaStream_t st)
 {
+    if constexpr (GROUPED && !ONE) {
+        if (prm.M == 1) return launch_gemv_x<BITS, GROUPED, XDIRECT, GATED, NG, true>(h, prm, pl, st);
+    }
     static std::atomic<bool> attr_set[kMaxDevices];
-    auto kern = gemv_kernel<BITS, GROUPED, XDIRECT, GATED, NG>;
+    auto kern = gemv_kernel<BITS, GROUPED, XDIRECT, GATED, NG, ONE>;
     cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, kGemvMaxSmem);
     if (e != cudaSuccess) return e;
     return launch(kern, prm, dim3(pl.grid), dim3(kGemvThreads), pl.smem_bytes, st, pl.cl, h->pdl);
