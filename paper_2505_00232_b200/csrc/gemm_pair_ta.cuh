@@ -32,6 +32,11 @@
 // the leader across the SM pair -- which is why both cross-SM signals on that path (the relay's and the epilogue's)
 // are relaxed arrives.
 //
+// The dequantise loop is held to the instructions it needs: per-thread constants are kept from being recomputed at the
+// register limit, the addresses of the step's stage, barriers and slot are advanced instead of formed from an index, and tile
+// bookkeeping runs at the few steps where something changes (1714 -> 1326 warp instructions per k-step and SM of grouped
+// int4; Llama gate + up, fused, 2048 tokens 395 -> 363 us, 777 tokens 196 -> 166, Gemma2-2B's 777 tokens 63 -> 57).
+//
 // Forms of the kernel (template flags): the plain product, whole tiles dealt out round-robin or, for launches with
 // few tiles, 2 or 4 K parts per tile that meet in the device scratch; GATED (y = act(gate) * up, Section 3.6); I8
 // (int8 activations, kind::i8 on the stored weight bytes, Section 3.7).
@@ -122,33 +127,41 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t addr)
     return v;
 }
 
+// (pin: the members pass through an empty asm statement.  The kernel is at its register limit, and the compiler otherwise
+// computes them again from the lane number on every k-step.  The integer form has next to no arithmetic and a larger epilogue:
+// there the registers are worth more, 327 us of projections at 1024 tokens against 349 pinned.)
 struct DequantRowTa {
     int off[4];                  // byte offset, inside the packed block, of piece c of the row's 64-byte line (64-byte swizzle:
                                  // piece c sits at position c ^ ((line / 2) & 3))
     int s_off;                   // grouped int4: byte offset of the row's scale of group 0 (group 1: + 2)
     uint32_t mask, mul, add;     // int4: nibble mask and the exact fp16 fix-up of the chosen nibbles
     uint32_t sel;                // int8: byte pair of the chosen row
-    __device__ DequantRowTa(int quarter, int lane)
+    // half_bytes, half_scale: what the warp's half h of the k-step adds to the packed addresses
+    __device__ DequantRowTa(int quarter, int lane, int half_bytes, int half_scale, bool pin)
     {
         const int rb = 2 * quarter + (lane >> 4), g = lane & 7, hi = (lane >> 3) & 1;
-        for (int c = 0; c < 4; ++c) off[c] = (rb * 8 + g) * 64 + ((c ^ ((g >> 1) & 3)) << 4);
+        for (int c = 0; c < 4; ++c) off[c] = (rb * 8 + g) * 64 + ((c ^ ((g >> 1) & 3)) << 4) + half_bytes;
         // scales: 64-byte line 64 + rb of the block (swizzle term (rb >> 1) & 3 = quarter), piece g / 2
-        s_off = kWeightBlockBytes + rb * 64 + (((g >> 1) ^ quarter) << 4) + (g & 1) * 8 + hi * 4;
+        s_off = kWeightBlockBytes + rb * 64 + (((g >> 1) ^ quarter) << 4) + (g & 1) * 8 + hi * 4 + half_scale;
         mask = hi ? 0x00F000F0u : 0x000F000Fu;
         mul = hi ? 0x2C002C00u : 0x3C003C00u;                            // {1/16, 1/16} or {1, 1}
         add = hi ? 0xD480D480u : 0xE408E408u;                            // {-72, -72} or {-1032, -1032}
         sel = hi ? 0x4342u : 0x4140u;
+        if (pin) {
+            for (int c = 0; c < 4; ++c) asm volatile("" : "+r"(off[c]));
+            asm volatile("" : "+r"(s_off), "+r"(mask), "+r"(mul), "+r"(add), "+r"(sel));
+        }
     }
     // 32 consecutive k of the row (half h of the 64-k step) -> 16 registers = 16 columns of the row's TMEM lane.
     // Same arithmetic as unpack_int4_word / unpack_int8_words (exact integers, then one multiplication by the scale).
     template <int BITS, bool GROUPED, bool I8 = false>
-    __device__ __forceinline__ void convert(uint32_t wp, int h, uint32_t r[16]) const   // wp: shared-window address of the stage
+    __device__ __forceinline__ void convert(uint32_t wp, uint32_t r[16]) const   // wp: shared-window address of the stage
     {
         if (I8) {
             // integer form: 64 consecutive k of the row (half h of the 128-k step) as the stored unsigned bytes
             // (q + 8 or q + 128), 4 per column: no arithmetic, only the choice of nibbles / bytes and their order
             if (BITS == 4) {
-                const uint32_t rp = wp + h * kWeightBlockBytes;                              // packed block h of the step
+                const uint32_t rp = wp;                                                      // packed block h of the step
                 const uint32_t sh = mask == 0x000F000Fu ? 0u : 4u;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
@@ -163,7 +176,7 @@ struct DequantRowTa {
                 const uint32_t bsel = sel == 0x4140u ? 0x5410u : 0x7632u;                    // this row's byte pair of two words
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {                                                // blocks 2h, 2h + 1: 32 k each
-                    const uint32_t rp = wp + (2 * h + b) * kWeightBlockBytes;
+                    const uint32_t rp = wp + b * kWeightBlockBytes;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         const uint4 w = lds_u128(rp + off[c]);
@@ -175,7 +188,7 @@ struct DequantRowTa {
             return;
         }
         if (BITS == 4) {
-            const uint32_t rp = wp + 8 * h;
+            const uint32_t rp = wp;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const uint2 w = lds_u64(rp + off[c]);
@@ -185,13 +198,13 @@ struct DequantRowTa {
                 r[4 * c + 3] = h2_fma(lop3_and_or(w.y >> 8, mask, 0x64006400u), mul, add);   // k 8c + 6, 7
             }
             if (GROUPED) {
-                const uint32_t s = lds_u16(wp + s_off + 2 * h);
+                const uint32_t s = lds_u16(wp + s_off);
                 const uint32_t s2 = s | (s << 16);
 #pragma unroll
                 for (int i = 0; i < 16; ++i) r[i] = h2_mul(r[i], s2);
             }
         } else {
-            const uint32_t rp = wp + h * kWeightBlockBytes;                                  // chunk h of the step
+            const uint32_t rp = wp;                                                          // chunk h of the step
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const uint4 w = lds_u128(rp + off[c]);
@@ -220,10 +233,11 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     static_assert(!I8 || (!GATED && !GROUPED), "the integer form: per-channel scales, plain output");
     using S = GemmTaSmem<BITS, I8>;
     constexpr int NX = S::kXStages, NW = S::kWStages, NA = S::kASlots;
-    const int bn = p.bn;                                                 // tokens per tile: a multiple of 32, at most 256
+    const int bn = I8 ? 256 : p.bn;                                                 // tokens per tile: a multiple of 32, at most 256
     constexpr int W_BOX_BYTES = I8 ? S::kWBytes : BITS == 4 ? (GROUPED ? kWeightBlockBytes + kScaleBlockBytes : kWeightBlockBytes) : 2 * kWeightBlockBytes;
     extern __shared__ unsigned char smem_dyn[];
-    const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    if (!I8) asm volatile("" : "+r"(base));                                     // (computed once: see DequantRowTa)
     unsigned char* base_ptr = smem_dyn + (base - smem_u32(smem_dyn));
     auto xs_addr = [&](int s) { return base + s * S::kXBytes; };
     auto wpk_addr = [&](int s) { return base + S::kWOffset + s * S::kWBytes; };
@@ -288,7 +302,8 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     __syncthreads();
     cluster_sync_all();                                                  // both CTAs' barriers exist before any remote arrive
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    uint32_t tmem_base = *tmem_slot;
+    if (!I8) asm volatile("" : "+r"(tmem_base));
     // The next kernel in the stream may move onto SMs this grid has left (the last, partial round of tiles) and set up
     // there; whatever it reads of this grid's output comes after its own griddepcontrol.wait.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -412,7 +427,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         const int quarter = warp & 3, wi = (warp - kTaFirstDequantWarp) >> 2;
         const int half = wi & 1, my_turn = wi >> 1;                      // 32-k half of the step; this warp takes every third step
         const bool epi_warp = wi < 4;                                    // the first 16 warps also run the epilogue (64 tokens each)
-        const DequantRowTa dq(quarter, lane);
+        const DequantRowTa dq(quarter, lane, half * (I8 ? (BITS == 4 ? 1 : 2) * kWeightBlockBytes : BITS == 4 ? 8 : kWeightBlockBytes), 2 * half, !I8);
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         bool ok = true;
 
@@ -423,7 +438,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         const uint32_t out_addr = base + S::kOutOffset;
         unsigned char* out_ptr = base_ptr + S::kOutOffset;
         const int grp_thread = quarter * 32 + lane;                      // 0..127 inside the group of four warps
-        const int n_cols = max(0, min(64, bn - 64 * wi));                // columns (tokens) of this warp: 0, 32 or 64
+        const int n_cols = I8 ? 64 : max(0, min(64, bn - 64 * wi));                // columns (tokens) of this warp: 0, 32 or 64
         // K-split tile: every part parks its fp32 accumulator in the device's scratch ([token][channel], a warp writes
         // 128 contiguous bytes per token), frees the accumulator and counts itself in; the part that arrives last adds all
         // parts in part order (fixed order, no float atomics, nobody waits) and stores y.
@@ -575,39 +590,59 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
 
         // The k-steps of all tiles of this cluster are numbered through (g); this warp takes g = my_turn, my_turn + 3, ...
         const int forced = min(S::kEarlySteps, n_steps - 1);
-        int s = my_turn, a = my_turn;                                    // W stage and A slot of step g (my_turn < NW, NA)
+        // Addresses of the step's weight stage, barriers and A slot are kept and advanced, not computed from an index (the integer
+        // form, short of registers in its epilogue, does form them from the indices s, a: 328 us against 332, see DequantRowTa).
+        [[maybe_unused]] int s = my_turn, a = my_turn;
+        uint32_t wst = wpk_addr(my_turn), wbar = wfull_bar(my_turn), abar = afull_bar(my_turn);   // my_turn < NW, NA
+        uint32_t slot = tmem_base + lane_base + (uint32_t)(kTaAccCols + my_turn * kTaSlotCols + 16 * half);
+        const uint32_t wbar_end = wfull_bar(NW), abar_end = afull_bar(NA);
         uint32_t wpar = 0, apar = 1;                                     // A slots start out free
         int tile_j = 0, tile_g0 = 0;                                     // tile of step g and its first step
         int next_epi = 0;                                                // tiles leave through the epilogue in order
-        for (int g = my_turn; g < total_steps && ok; g += 3) {
-            while (g >= tile_g0 + n_steps) { ++tile_j; tile_g0 += n_steps; }
-            // an earlier tile still holds the accumulator: run its epilogue once it is complete, or, at the latest,
-            // after `forced` steps of this tile have been dequantised, or before any step of the tile after next (a warp's
-            // steps of a short tile may all lie before `forced`): the slots it would wait for belong to tiles whose MMAs wait
-            // for this epilogue
-            while (epi_warp && next_epi < tile_j && (next_epi + 1 < tile_j || g - tile_g0 >= forced || tile_complete(next_epi))) {
-                epilogue(next_epi);
-                ++next_epi;
+        int event = n_steps;                                             // first step at which the tile or the epilogue has to be looked at
+        for (int g = my_turn; g < total_steps; g += 3) {
+            if (I8 || g >= event) {
+                while (g >= tile_g0 + n_steps) { ++tile_j; tile_g0 += n_steps; }
+                // an earlier tile still holds the accumulator: run its epilogue once it is complete, or, at the latest,
+                // after `forced` steps of this tile have been dequantised, or before any step of the tile after next (a warp's
+                // steps of a short tile may all lie before `forced`): the slots it would wait for belong to tiles whose MMAs wait
+                // for this epilogue
+                while (epi_warp && next_epi < tile_j && (next_epi + 1 < tile_j || g - tile_g0 >= forced || tile_complete(next_epi))) {
+                    epilogue(next_epi);
+                    ++next_epi;
+                    if (!ok) break;
+                }
                 if (!ok) break;
+                event = epi_warp && next_epi < tile_j ? g + 1 : tile_g0 + n_steps;
             }
-            if (!ok) break;
+            if (I8) {
+                wst = wpk_addr(s); wbar = wfull_bar(s); abar = afull_bar(a);
+                slot = tmem_base + lane_base + (uint32_t)(kTaAccCols + a * kTaSlotCols + 16 * half);
+            }
             uint32_t r[16];
             // A weight stage whose ring length is not a multiple of the 3 turns is served by a different turn every time
             // round, so this warp has not seen the stage's previous phase: the load of step g - NW may still be in flight
             // (bulk copies complete in any order), and a parity test alone would then take that phase for this one.  The
             // producer issues the load of step g only after step g - NW's warps have released the stage: wait for that first.
-            if (NW % 3 != 0 && !mbar_wait(wempty_bar(s), wpar ^ 1, abort_flag, 0x480 + s)) { ok = false; break; }
-            if (!mbar_wait(wfull_bar(s), wpar, abort_flag, 0x400 + s)) { ok = false; break; }
-            dq.template convert<BITS, GROUPED, I8>(wpk_addr(s), half, r);
-            // the MMAs that read slot a (step g - NA) have retired
-            if (!mbar_wait(aempty_bar(a), apar, abort_flag, 0xB00 + a)) { ok = false; break; }
+            if (NW % 3 != 0 && !mbar_wait(wbar + 8 * NW, wpar ^ 1, abort_flag, 0x480)) { ok = false; break; }
+            if (!mbar_wait(wbar, wpar, abort_flag, 0x400)) { ok = false; break; }
+            dq.template convert<BITS, GROUPED, I8>(wst, r);
+            // the MMAs that read the slot (step g - NA) have retired
+            if (!mbar_wait(abar + 8 * NA, apar, abort_flag, 0xB00)) { ok = false; break; }
             tc_fence_after();
-            tmem_st16(tmem_base + lane_base + (uint32_t)(kTaAccCols + a * kTaSlotCols + 16 * half), r);
+            tmem_st16(slot, r);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) { mbar_arrive(wempty_bar(s)); mbar_arrive(afull_bar(a)); }
-            s += 3; if (s >= NW) { s -= NW; wpar ^= 1; }
-            a += 3; if (a >= NA) { a -= NA; apar ^= 1; }
+            if (lane == 0) { mbar_arrive(wbar + 8 * NW); mbar_arrive(abar); }
+            if (I8) {
+                s += 3; if (s >= NW) { s -= NW; wpar ^= 1; }
+                a += 3; if (a >= NA) { a -= NA; apar ^= 1; }
+                continue;
+            }
+            wst += 3 * S::kWBytes; wbar += 24;
+            if (wbar >= wbar_end) { wst -= NW * S::kWBytes; wbar -= 8 * NW; wpar ^= 1; }
+            abar += 24; slot += 3 * kTaSlotCols;
+            if (abar >= abar_end) { abar -= 8 * NA; slot -= NA * kTaSlotCols; apar ^= 1; }
         }
         while (epi_warp && ok && next_epi < n_units) { epilogue(next_epi); ++next_epi; }
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // y written before the kernel ends
@@ -652,7 +687,8 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const void* x, int M, c
     // Tokens per tile: M in as few blocks of at most 256 as it takes, all of the same width (the MMA's N, a multiple of 32).  A
     // narrower tile costs the same dequantisation and less tensor-core time, x traffic and epilogue
     // (a Llama block at 100 tokens 145.9 -> 136.9 us, at 300 224.9 -> 211.1).
-    const int n_mblk = (M + 255) / 256, bn = ((M + n_mblk - 1) / n_mblk + 31) / 32 * 32;
+    // The integer form keeps 256: it gains nothing at 300 tokens, and its epilogue is short of registers.
+    const int n_mblk = (M + 255) / 256, bn = I8 ? 256 : ((M + n_mblk - 1) / n_mblk + 31) / 32 * 32;
     if (!x_tensor_map(x, L.K, M, bn / 2, &maps.x, I8 ? 1 : 2)) return QL_ERR_CUDA;
     for (int i = 0; i < kGemmMaxGroup; ++i) maps.w[i] = *set.wmap[i < set.n ? i : 0];
     auto kern = gemm_pair_ta_kernel<BITS, GROUPED, GATED, I8>;
