@@ -590,59 +590,76 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
 
         // The k-steps of all tiles of this cluster are numbered through (g); this warp takes g = my_turn, my_turn + 3, ...
         const int forced = min(S::kEarlySteps, n_steps - 1);
-        // Addresses of the step's weight stage, barriers and A slot are kept and advanced, not computed from an index (the integer
-        // form, short of registers in its epilogue, does form them from the indices s, a: 328 us against 332, see DequantRowTa).
-        [[maybe_unused]] int s = my_turn, a = my_turn;
-        uint32_t wst = wpk_addr(my_turn), wbar = wfull_bar(my_turn), abar = afull_bar(my_turn);   // my_turn < NW, NA
-        uint32_t slot = tmem_base + lane_base + (uint32_t)(kTaAccCols + my_turn * kTaSlotCols + 16 * half);
-        const uint32_t wbar_end = wfull_bar(NW), abar_end = afull_bar(NA);
-        uint32_t wpar = 0, apar = 1;                                     // A slots start out free
+        // When the next epilogue runs: an earlier tile still holds the accumulator; its epilogue runs once it is complete, or, at the
+        // latest, after `forced` steps of this tile have been dequantised, or before any step of the tile after next (a warp's
+        // steps of a short tile may all lie before `forced`): the slots it would wait for belong to tiles whose MMAs wait
+        // for this epilogue.
+        // Why the weight stage is waited for twice: a stage whose ring length is not a multiple of the 3 turns is served by a
+        // different turn every time round, so this warp has not seen the stage's previous phase: the load of step g - NW may
+        // still be in flight (bulk copies complete in any order), and a parity test alone would then take that phase for this
+        // one.  The producer issues the load of step g only after step g - NW's warps have released the stage.
         int tile_j = 0, tile_g0 = 0;                                     // tile of step g and its first step
         int next_epi = 0;                                                // tiles leave through the epilogue in order
-        int event = n_steps;                                             // first step at which the tile or the epilogue has to be looked at
-        for (int g = my_turn; g < total_steps; g += 3) {
-            if (I8 || g >= event) {
+        uint32_t wpar = 0, apar = 1;                                     // A slots start out free
+        if constexpr (I8) {
+            // The integer form has a loop of its own: it converts with next to no arithmetic and has a larger epilogue, so the
+            // registers that the other loop keeps addresses in are worth more here (with both in one loop 60 bytes of spills instead of 8).
+            int s = my_turn, a = my_turn;                                // W stage and A slot of step g (my_turn < NW, NA)
+            for (int g = my_turn; g < total_steps;) {
                 while (g >= tile_g0 + n_steps) { ++tile_j; tile_g0 += n_steps; }
-                // an earlier tile still holds the accumulator: run its epilogue once it is complete, or, at the latest,
-                // after `forced` steps of this tile have been dequantised, or before any step of the tile after next (a warp's
-                // steps of a short tile may all lie before `forced`): the slots it would wait for belong to tiles whose MMAs wait
-                // for this epilogue
-                while (epi_warp && next_epi < tile_j && (next_epi + 1 < tile_j || g - tile_g0 >= forced || tile_complete(next_epi))) {
+                if (epi_warp && next_epi < tile_j && (next_epi + 1 < tile_j || g - tile_g0 >= forced || tile_complete(next_epi))) {
                     epilogue(next_epi);
                     ++next_epi;
                     if (!ok) break;
+                    continue;                                            // (tiles of a few steps: the one after it may be due as well)
                 }
-                if (!ok) break;
-                event = epi_warp && next_epi < tile_j ? g + 1 : tile_g0 + n_steps;
-            }
-            if (I8) {
-                wst = wpk_addr(s); wbar = wfull_bar(s); abar = afull_bar(a);
-                slot = tmem_base + lane_base + (uint32_t)(kTaAccCols + a * kTaSlotCols + 16 * half);
-            }
-            uint32_t r[16];
-            // A weight stage whose ring length is not a multiple of the 3 turns is served by a different turn every time
-            // round, so this warp has not seen the stage's previous phase: the load of step g - NW may still be in flight
-            // (bulk copies complete in any order), and a parity test alone would then take that phase for this one.  The
-            // producer issues the load of step g only after step g - NW's warps have released the stage: wait for that first.
-            if (NW % 3 != 0 && !mbar_wait(wbar + 8 * NW, wpar ^ 1, abort_flag, 0x480)) { ok = false; break; }
-            if (!mbar_wait(wbar, wpar, abort_flag, 0x400)) { ok = false; break; }
-            dq.template convert<BITS, GROUPED, I8>(wst, r);
-            // the MMAs that read the slot (step g - NA) have retired
-            if (!mbar_wait(abar + 8 * NA, apar, abort_flag, 0xB00)) { ok = false; break; }
-            tc_fence_after();
-            tmem_st16(slot, r);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) { mbar_arrive(wbar + 8 * NW); mbar_arrive(abar); }
-            if (I8) {
+                uint32_t r[16];
+                if (NW % 3 != 0 && !mbar_wait(wempty_bar(s), wpar ^ 1, abort_flag, 0x480)) { ok = false; break; }
+                if (!mbar_wait(wfull_bar(s), wpar, abort_flag, 0x400)) { ok = false; break; }
+                dq.template convert<BITS, GROUPED, I8>(wpk_addr(s), r);
+                // the MMAs that read the slot (step g - NA) have retired
+                if (!mbar_wait(aempty_bar(a), apar, abort_flag, 0xB00)) { ok = false; break; }
+                tc_fence_after();
+                tmem_st16(tmem_base + lane_base + (uint32_t)(kTaAccCols + a * kTaSlotCols + 16 * half), r);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) { mbar_arrive(wempty_bar(s)); mbar_arrive(afull_bar(a)); }
                 s += 3; if (s >= NW) { s -= NW; wpar ^= 1; }
                 a += 3; if (a >= NA) { a -= NA; apar ^= 1; }
-                continue;
+                g += 3;
             }
-            wst += 3 * S::kWBytes; wbar += 24;
-            if (wbar >= wbar_end) { wst -= NW * S::kWBytes; wbar -= 8 * NW; wpar ^= 1; }
-            abar += 24; slot += 3 * kTaSlotCols;
-            if (abar >= abar_end) { abar -= 8 * NA; slot -= NA * kTaSlotCols; apar ^= 1; }
+        } else {
+            // The addresses of the step's weight stage, barriers and A slot are kept and advanced, not formed from an index.
+            uint32_t wst = wpk_addr(my_turn), wbar = wfull_bar(my_turn), abar = afull_bar(my_turn);   // my_turn < NW, NA
+            uint32_t slot = tmem_base + lane_base + (uint32_t)(kTaAccCols + my_turn * kTaSlotCols + 16 * half);
+            const uint32_t wbar_end = wfull_bar(NW), abar_end = afull_bar(NA);
+            int event = n_steps;                                         // first step at which the tile or the epilogue has to be looked at
+            for (int g = my_turn; g < total_steps; g += 3) {
+                if (g >= event) {
+                    while (g >= tile_g0 + n_steps) { ++tile_j; tile_g0 += n_steps; }
+                    while (epi_warp && next_epi < tile_j && (next_epi + 1 < tile_j || g - tile_g0 >= forced || tile_complete(next_epi))) {
+                        epilogue(next_epi);
+                        ++next_epi;
+                        if (!ok) break;
+                    }
+                    if (!ok) break;
+                    event = epi_warp && next_epi < tile_j ? g + 1 : tile_g0 + n_steps;
+                }
+                uint32_t r[16];
+                if (NW % 3 != 0 && !mbar_wait(wbar + 8 * NW, wpar ^ 1, abort_flag, 0x480)) { ok = false; break; }
+                if (!mbar_wait(wbar, wpar, abort_flag, 0x400)) { ok = false; break; }
+                dq.template convert<BITS, GROUPED, I8>(wst, r);
+                if (!mbar_wait(abar + 8 * NA, apar, abort_flag, 0xB00)) { ok = false; break; }
+                tc_fence_after();
+                tmem_st16(slot, r);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) { mbar_arrive(wbar + 8 * NW); mbar_arrive(abar); }
+                wst += 3 * S::kWBytes; wbar += 24;
+                if (wbar >= wbar_end) { wst -= NW * S::kWBytes; wbar -= 8 * NW; wpar ^= 1; }
+                abar += 24; slot += 3 * kTaSlotCols;
+                if (abar >= abar_end) { abar -= 8 * NA; slot -= NA * kTaSlotCols; apar ^= 1; }
+            }
         }
         while (epi_warp && ok && next_epi < n_units) { epilogue(next_epi); ++next_epi; }
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // y written before the kernel ends

@@ -131,6 +131,23 @@ def test_a8_prefill_parity(P, torch, M, N, K, bits):
     assert torch.equal(y, lin.forward_a8(xd))
 
 
+@pytest.mark.parametrize("M,N,K,bits", [(1500, 4864, 128, 8), (2048, 5120, 256, 4), (1100, 9728, 384, 8), (1024, 9728, 896, 4)])
+def test_a8_prefill_many_tiles_of_few_k_steps(P, torch, M, N, K, bits):
+    """Several tiles of 1, 2, 3 and 7 k-steps per CTA pair: a warp's own steps then skip whole tiles, and it has more than one
+    epilogue to run before a step.  Back to back, same bits."""
+    q, s, x = rand_case(7600 + N + K + M, M, N, K, bits, 0)
+    lin = P.QLinear.from_weights(q, s, bits, 0, device="cuda:0")
+    xd = torch.from_numpy(x).cuda()
+    y = lin.forward_a8(xd)
+    for _ in range(20):
+        again = lin.forward_a8(xd)
+    torch.cuda.synchronize()
+    assert lin.device_status() == (0, 0)
+    assert torch.equal(y, again)
+    rows = np.r_[0:64, N - 64:N]
+    assert_a8(y.cpu().numpy()[:, rows], x, q[rows], s[rows], 0)
+
+
 @pytest.mark.parametrize("bits,N", [(8, 256), (4, 256), (8, 9728), (4, 9728)])
 def test_a8_prefill_integer_path_is_bit_exact_when_no_rounding_is_left(P, torch, bits, N):
     M, K = 300, 512
