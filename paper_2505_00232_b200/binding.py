@@ -172,20 +172,23 @@ def qlinear_unpack(desc: Desc, packed: np.ndarray):
 # A small layer takes the GPU a few microseconds, less than these calls took the host: so the raw handle of the current
 # stream is asked for without building a Stream object, pointers go to ctypes as plain integers (the argument types are
 # declared), and a tensor's properties are checked in one expression.  Measured: QLinear.forward at one token 11.8 -> 7.0 us.
-_torch = _half = _raw_stream = _device = None
+_half = _raw_stream = _device = None
 
 
 def _bind_torch() -> None:
     """torch is imported with the first device object, not with the package (packing needs none of it)."""
-    global _torch, _half, _raw_stream, _device
+    global _half, _raw_stream, _device
     import torch
-    _torch, _half, _raw_stream, _device = torch, torch.float16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    # (a torch without CUDA has neither entry point: its own error comes from the calls that need a device)
+    _device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+    _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", lambda device: torch.cuda.current_stream(device).cuda_stream)
+    _half = torch.float16
 
 
 def _stream_ptr(stream) -> int:
     if stream is not None:
         return stream.cuda_stream
-    if _torch is None:
+    if _raw_stream is None:
         _bind_torch()
     return _raw_stream(_device())                                        # the current stream of the current device
 

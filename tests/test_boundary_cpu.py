@@ -151,3 +151,25 @@ def test_environment_is_read_once(P, monkeypatch):
     d = P.Desc(16, 64, 8, 0).c()
     P.lib.qlinear_create(ctypes.byref(d), ctypes.c_void_p(256), 0, ctypes.byref(h))   # fails without a device; reads nothing new
     assert P.lib.qlinear_debug_config_reads() == 1
+
+
+def test_torch_without_cuda_says_so_itself(P, monkeypatch):
+    """A handle cannot exist without a device: what a program sees is torch's own error, also from a torch that was built
+    without CUDA and has none of its entry points."""
+    import torch
+    from paper_2505_00232_b200 import binding
+    if torch.cuda.is_available():
+        pytest.skip("this machine has a device")
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    for name in ("_half", "_raw_stream", "_device"):
+        monkeypatch.setattr(binding, name, None)
+    with pytest.raises(Exception) as own:
+        torch.cuda.current_device()
+    d = P.Desc(8, 32, 8, 0)
+    blob = P.qlinear_pack(d, np.zeros((8, 32), np.int8), np.ones((8, 1), np.float16))
+    with pytest.raises(type(own.value)) as seen:
+        P.QLinear(d, blob)
+    assert str(seen.value) == str(own.value)
+    with pytest.raises(P.QLinearError):
+        P.qlinear_residual_rmsnorm(torch.zeros((1, 8)).half(), None, torch.ones(8).half(), 1e-5)
