@@ -196,12 +196,18 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_a8_kernel(const GemvA8Pa
     };
     const int vec_span = span >> 3;
     if (keep) {
-        // vectors beyond K (a last chunk of int4 that is half padding) are zeros in u where they exist at all
-        const int v_first = k_cta0 >> 3;
+        // (a thread whose vectors all lie beyond the row has loaded nothing into u: nothing of it is stored)
+        const int v_first = k_cta0 >> 3, v_end = max(0, min(vec_span, vec_per_row - v_first));
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = i / T, m = i % T, v = (int)threadIdx.x + j * kGemvThreads - v_first;
-            if (m < p.M && j * kGemvThreads < v_first + vec_span && (j + 1) * kGemvThreads > v_first) quantise8(u[i], recip[m], m, v, v >= 0 && v < vec_span);
+            if (m < p.M && j * kGemvThreads < v_first + vec_span && (j + 1) * kGemvThreads > v_first) quantise8(u[i], recip[m], m, v, v >= 0 && v < v_end);
+        }
+        // the last chunk of int4 can be half padding: 32 k of zeros, which the MMAs multiply by whatever the blob holds there
+        if (BITS == 4 && v_end < vec_span && (int)threadIdx.x < 4 * p.M) {   // (whole chunks: v_end = vec_span - 4)
+            const int m = threadIdx.x >> 2, v = v_end + (threadIdx.x & 3);
+            *reinterpret_cast<uint2*>(xq + m * p.xq_stride + v * 8) = make_uint2(0, 0);
+            if ((threadIdx.x & 3) == 0) sg[(v >> 2) * 8 + m] = 0;
         }
     } else {
         constexpr int LOG = T == 8 ? 3 : T == 4 ? 2 : T == 2 ? 1 : 0;

@@ -86,6 +86,26 @@ def test_a8_decode_rows_at_the_edge_of_what_registers_keep(P, torch, M, K, bits,
     assert_a8(y.cpu().numpy(), x, q, s, group)
 
 
+@pytest.mark.parametrize("M,K", [(1, 96), (1, 1056), (2, 1056), (4, 352), (8, 96), (8, 1056)])
+def test_a8_decode_takes_nothing_from_beyond_the_row(P, torch, M, K):
+    """int4 with a last chunk that is half padding: the quantised activations there are zeros, so whatever the padding of the
+    blob holds has no part in the result (the packer leaves zeros in it, which would hide activations that are not)."""
+    q, s, x = rand_case(7900 + K + M, M, 136, K, 4, 0)
+    lin = P.QLinear.from_weights(q, s, 4, 0, device="cuda:0")
+    blob = lin.packed.cpu().numpy().copy()
+    n_kc, n_rsb = (K + 63) // 64, 2
+    body = blob[256:256 + n_rsb * n_kc * 4096].reshape(n_rsb, n_kc, 8 * 32, 16)
+    body[:, -1, :, 8:] = np.random.default_rng(K).integers(0, 256, size=(n_rsb, 8 * 32, 8))   # k 32 .. 63 of the last chunk
+    other = P.QLinear(lin.desc, torch.from_numpy(blob).cuda())
+    assert torch.equal(lin.debug_unpack(), other.debug_unpack())         # the same layer
+    xd = torch.from_numpy(x).cuda()
+    for _ in range(20):
+        lin.forward_a8(torch.randn((8, 4096 - 32), device="cuda").half()[:M, :K].contiguous() * 100)   # (other values in the registers)
+        y, y2 = lin.forward_a8(xd), other.forward_a8(xd)
+        assert torch.equal(y, y2)
+    assert_a8(y.cpu().numpy(), x, q, s, 0)
+
+
 @pytest.mark.parametrize("bits,group", [(8, 0), (4, 32), (4, 0)])
 def test_a8_integer_path_is_bit_exact_when_no_rounding_is_left(P, torch, bits, group):
     """Power-of-two scales and x on the int8 grid: every fp32 operation of the dequantisation is exact, so the
