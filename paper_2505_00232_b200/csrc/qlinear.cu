@@ -1082,6 +1082,7 @@ extern "C" ql_status qlinear_kv_output(qlinear_t hv, const void* prob, const voi
         if (s != QL_ERR_UNSUPPORTED) return s;
         // more rows: the kernel that takes any number of tokens against few channels, with the scales folded in on the way
         if (R > hv->gemv_max_m) {
+            if ((int64_t)R * hv->L.N > INT32_MAX) return QL_ERR_INVALID_ARG;   // (the limit of qlinear_forward)
             if (device_timed_out(hv)) return QL_ERR_DEVICE_TIMEOUT;
             DeviceGuard guard(hv->device);
             if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }

@@ -88,3 +88,14 @@ def test_value_product_of_many_rows(P, torch, d_h, cache, T, R):
     y64, A, _ = O.kv_output(folded, np.ascontiguousarray(v_q.T), np.ones(d_h, np.float16))
     ok, rel, worst = O.check_against(out.cpu().numpy(), y64, A)
     assert ok, (rel, worst)
+
+
+def test_value_product_keeps_the_limit_on_its_output(P, torch):
+    """2^31 output elements: refused like a forward call of that size (the buffers have the full size all the same)."""
+    kv = P.KVCache(32, 65536)
+    R = 32768
+    prob = torch.zeros((R, 32), dtype=torch.float16, device="cuda")
+    with pytest.raises(P.QLinearError) as err:
+        kv.output(prob)
+    assert err.value.status == P.QL_ERR_INVALID_ARG
+    assert kv.output(prob[:100]).shape == (100, 65536)
