@@ -350,6 +350,10 @@ ql_status forward_gemv_cols(qlinear_s* const* hs, int n, const void* const* xs, 
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
+// The layers that gemv_rows.cuh (decode) and gemm_rows.cuh (more tokens) take: int8, K of 64, 128 or 256 (the head dimensions of a K
+// cache), any number of rows.
+bool takes_rows(const Layout& L) { return L.bits == 8 && (L.n_kc == 2 || L.n_kc == 4 || L.n_kc == 8) && L.K == 32 * L.n_kc; }
+
 // One launch for n layers that read the same x (n == 1: the plain forward).  The plan of a group is made per
 // call (integer arithmetic only); nothing is written to a handle.
 // act >= 0: the gated form (n == 2: gate, up; ys[0] the output; the row-blocks of the two layers alternate).
@@ -366,8 +370,9 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
     if (gated) n_rb = 2 * hs[0]->n_rb;
     // Short K (the score product over a KV cache): the persistent form, whatever the number of rows.  With at most one wave of
     // row super-blocks it wins as well, having no ring to fill, no sums across warps and no barrier (8 heads of 128 at 1280
-    // positions 4.1 -> 1.8 us, at 8192 6.7 -> 3.1 us; 2 heads of 64 at 1024 3.3 -> 1.5 us).
-    if (xs && !gated && n <= kGemvMaxBatch && L.bits == 8 && (L.K % 32) == 0 && (L.n_kc == 2 || L.n_kc == 4 || L.n_kc == 8)) {
+    // positions 4.1 -> 1.8 us, at 8192 6.7 -> 3.1 us; 2 heads of 64 at 1024 3.3 -> 1.5 us).  One layer as well, a cache or not
+    // (a head of 128, 4 rows, 4096 positions 3.7 -> 1.6 us; 32768 x 256 weights, 8 tokens 3.8 -> 3.5 us).
+    if (xs && !gated && n <= kGemvMaxBatch && takes_rows(L)) {
         GemvRowsParams rp{};
         int n_rsb = 0;
         for (int i = 0; i < n; ++i) {
@@ -503,8 +508,6 @@ cudaError_t launch_gemm_rows(const qlinear_s* h, GemmRowsParams& prm, int n_rsb,
     if (prm.M <= 32) return launch_gemm_rows_nt<NKC, 4>(h, prm, n_rsb, pdl, st);
     return launch_gemm_rows_nt<NKC, 8>(h, prm, n_rsb, pdl, st);
 }
-// The layers gemm_rows.cuh takes: int8, K of 64, 128 or 256 (the head dimensions of a K cache), any number of rows and tokens.
-bool takes_gemm_rows(const Layout& L) { return L.bits == 8 && (L.n_kc == 2 || L.n_kc == 4 || L.n_kc == 8) && L.K == 32 * L.n_kc; }
 ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st)
 {
     const qlinear_s* h = hs[0];
@@ -754,8 +757,11 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
     DeviceGuard guard(h->device);
     if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (M <= h->gemv_max_m) return h->use_stream ? forward_gemv_stream(h, x, y, M, st) : forward_gemv(&h, 1, x, &y, M, st);
-    if (takes_gemm_rows(h->L)) return forward_gemm_rows(&h, 1, &x, &y, M, st);
+    if (M <= h->gemv_max_m) {
+        if (h->use_stream) return forward_gemv_stream(h, x, y, M, st);
+        return forward_gemv(&h, 1, x, &y, M, st, -1, takes_rows(h->L) ? &x : nullptr);   // (short K: the persistent form, see there)
+    }
+    if (takes_rows(h->L)) return forward_gemm_rows(&h, 1, &x, &y, M, st);
     if (takes_mid(&h, 1, M)) return forward_mid(&h, 1, &x, &y, M, st);
     {
         GemmPairLayers set{};
@@ -830,7 +836,7 @@ extern "C" ql_status qlinear_forward_batch(const qlinear_t* hs, int32_t n, const
         const ql_status s = forward_gemv(const_cast<qlinear_s* const*>(hs), n, nullptr, ys, M, static_cast<cudaStream_t>(stream), -1, xs);
         if (s != QL_ERR_UNSUPPORTED) return s;
     }
-    if (n > 1 && M > hs[0]->gemv_max_m && takes_gemm_rows(hs[0]->L)) {   // (the K caches of a prompt's attention)
+    if (n > 1 && M > hs[0]->gemv_max_m && takes_rows(hs[0]->L)) {   // (the K caches of a prompt's attention)
         DeviceGuard guard(hs[0]->device);
         if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
         return forward_gemm_rows(hs, n, xs, ys, M, static_cast<cudaStream_t>(stream));

@@ -260,3 +260,22 @@ def test_scores_of_many_rows(P, torch, n_heads, d_h, cache, T, R):
         y64, A, _ = O.linear(q[h], k_q, k_s.reshape(-1, 1), 0)
         ok, rel, worst = O.check_against(sc[h, :, :T].cpu().numpy(), y64, A)
         assert ok, (h, rel, worst)
+
+
+@pytest.mark.parametrize("d_h,cache,R", [(64, 96, 1), (128, 1280, 4), (256, 992, 8), (256, 9632, 5)])
+def test_scores_of_one_head_are_those_of_all_heads(P, torch, d_h, cache, R):
+    """One head's scores come from the kernel that serves all heads, K undivided: the same bits at every head dimension."""
+    rng = np.random.default_rng(d_h + cache + R)
+    k = rng.standard_normal((2, cache, d_h)).astype(np.float16)
+    q = rng.standard_normal((2, R, d_h)).astype(np.float16)
+    heads = P.KVHeads(2, cache, d_h)
+    kd, qd = torch.from_numpy(k).cuda(), torch.from_numpy(q).cuda()
+    heads.append(kd, kd)
+    sc = heads.scores(qd)
+    for h in range(2):
+        assert torch.equal(sc[h], heads.heads[h].scores(qd[h]))
+        k_q, k_s = O.kv_quantize_rows(k[h])
+        y64, A, _ = O.linear(q[h], k_q, k_s.reshape(-1, 1), 0)
+        ok, rel, worst = O.check_against(sc[h].cpu().numpy(), y64, A)
+        assert ok, (h, rel, worst)
+    assert heads.heads[0].k.device_status() == (0, 0)
