@@ -362,8 +362,11 @@ uint32_t qlinear_version(void);
  * tokens {kernel (1 cluster, 3 streaming), grid CTAs, CTAs per cluster, K slices per CTA, chunks per slice,
  * 1000 x (work of the busiest SM / mean), row-blocks, chunks along K} and returns how many it wrote (0 on bad
  * arguments).  qlinear_debug_config_reads returns how many times the QLINEAR_* environment has been read by
- * this process (1 after the first call, for good). */
+ * this process (1 after the first call, for good).  qlinear_debug_plan_kv_output does for the (first) launch of
+ * qlinear_kv_output_heads over n_heads caches like h_v what qlinear_debug_plan does for the other decode launches: {CTAs per
+ * cluster, chunks per warp, clusters of the launch, clusters that run at once}. */
 int32_t qlinear_debug_plan(qlinear_t h, int32_t M, int32_t* out, int32_t n_out);
+int32_t qlinear_debug_plan_kv_output(qlinear_t h_v, int32_t n_heads, int32_t* out, int32_t n_out);
 uint32_t qlinear_debug_config_reads(void);
 
 #ifdef __cplusplus

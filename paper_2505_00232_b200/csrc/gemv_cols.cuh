@@ -9,7 +9,7 @@
 // Here a CTA of 16 warps takes ONE row-block (16 rows), a warp a contiguous slice of K, and everything a chunk needs
 // (weights, x, scales) travels in one ring of cp.async slots, kColsRing chunks per warp ahead: x and weights miss
 // together, once.  One CTA per SM; K is split over a cluster only where the row-blocks leave SMs idle and the slices
-// stay at least 4 chunks long.  Sums: tensor core, then the 16 warps in order, then the cluster's ranks in order.
+// keep 2 chunks per warp (cols_split in qlinear.cu).  Sums: tensor core, then the 16 warps in order, then the cluster's ranks in order.
 //
 // Measured, append + scores + values of one layer (8 heads of 128, 4 query rows each, caches rotated past L2): 6.3 -> 5.6 us
 // at 1280 positions, 10.2 -> 9.2 at 8192, 26.7 -> 22.0 at 32768.

@@ -324,6 +324,46 @@ cudaError_t launch_gemv_rows(const qlinear_s* h, const GemvRowsParams& prm, cuda
     return launch(kern, prm, dim3(grid), dim3(kGemvThreads), smem, st, 1, h->pdl);
 }
 
+// Clusters of `cl` CTAs of the value product's kernel (one CTA per SM) that run at once on `device`: a cluster lies inside one GPC, so
+// fewer fit than the SMs alone would hold (148 SMs: 33 of 4, 15 of 8).
+int cols_clusters_at_once(int device, int cl)
+{
+    static std::atomic<int> known[kMaxDevices][4];
+    std::atomic<int>& k = known[device][cl == 8 ? 3 : cl == 4 ? 2 : cl == 2 ? 1 : 0];
+    int n = k.load(std::memory_order_relaxed);
+    if (n) return n;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = cl;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(cl);
+    cfg.blockDim = dim3(kColsThreads);
+    cfg.dynamicSmemBytes = kColsSmem;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, gemv_cols_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    k.store(n, std::memory_order_relaxed);
+    return n;
+}
+
+// K parts of the value product (CTAs per cluster) for n_rb row-blocks of all its layers: a K of more than 64 chunks is split as far as all
+// clusters run at once and every warp keeps 4 chunks, or 2 where the clusters fill no more than half of the GPU (the kernel before
+// still holds SMs when these start).  Measured, us undivided / 2 / 4 / 8 parts: 8 row-blocks (a head of 128) at 2048 positions 2.5 / 2.8 /
+// 2.7 / 2.8, at 4096 3.5 / 3.2 / 2.8 / 2.8, at 8192 5.0 / 4.4 / 3.2 / 3.0, at 32768 13.9 / 8.8 / 5.9 / 4.4; 16 row-blocks at 32768 14.1 / 8.9 / 5.9 /
+// 8.3, 64 of them 14.7 / 10.0 / 12.9 / 21.9 (a second wave of clusters costs more than the split gains); 32 row-blocks at 4096, alone
+// 3.5 / 3.2 / 3.1 / 7.4, behind append and scores 6.7 us as 2 parts and 7.3 as 4.
+int cols_split(int device, int n_rb, int n_kc)
+{
+    int cl = 1;
+    while (cl < 8 && n_kc > 64) {
+        const int at_once = cols_clusters_at_once(device, cl * 2);
+        if (n_rb > at_once || n_kc < kColsWarps * cl * 2 * (n_rb * 2 <= at_once ? 2 : 4)) break;
+        cl *= 2;
+    }
+    return cl;
+}
+
 // The value product over a KV cache (gemv_cols.cuh): int8 layers of equal shape, every layer with its own input and input scales.
 ql_status forward_gemv_cols(qlinear_s* const* hs, int n, const void* const* xs, const void* const* xscales, void* const* ys, int M, cudaStream_t st)
 {
@@ -339,13 +379,12 @@ ql_status forward_gemv_cols(qlinear_s* const* hs, int n, const void* const* xs, 
     }
     p.n_layers = n; p.M = M; p.N = L.N; p.K = L.K; p.n_rb = h->n_rb; p.n_kc = L.n_kc;
     p.late = any_cache(hs, n);
-    // one CTA per SM; a K split only while every warp keeps at least 4 chunks
-    p.cl = 1;
-    while (p.cl < 8 && n * h->n_rb * p.cl * 2 <= h->num_sms && L.n_kc >= kColsWarps * p.cl * 2 * 4) p.cl *= 2;
-    p.cps = (L.n_kc + kColsWarps * p.cl - 1) / (kColsWarps * p.cl);
     static std::atomic<bool> attr_set[kMaxDevices];
     cudaError_t e = ensure_smem_attr(gemv_cols_kernel, attr_set, h->device, kColsSmem);
-    if (e == cudaSuccess) e = launch(gemv_cols_kernel, p, dim3(n * h->n_rb * p.cl), dim3(kColsThreads), kColsSmem, st, p.cl, h->pdl);
+    if (e != cudaSuccess) { cudaGetLastError(); return QL_ERR_CUDA; }
+    p.cl = cols_split(h->device, n * h->n_rb, L.n_kc);
+    p.cps = (L.n_kc + kColsWarps * p.cl - 1) / (kColsWarps * p.cl);
+    e = launch(gemv_cols_kernel, p, dim3(n * h->n_rb * p.cl), dim3(kColsThreads), kColsSmem, st, p.cl, h->pdl);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
@@ -1385,6 +1424,18 @@ extern "C" int32_t qlinear_debug_plan(qlinear_t h, int32_t M, int32_t* out, int3
     const int32_t v[8] = {h->use_stream ? 3 : 1, h->gemv[M].grid, h->gemv[M].cl, h->gemv[M].ks_cta, h->gemv[M].cps,
                           (int32_t)(1000 * h->gemv[M].max_over_mean), h->n_rb, h->L.n_kc};
     int n = n_out < 8 ? n_out : 8;
+    for (int i = 0; i < n; ++i) out[i] = v[i];
+    return n;
+}
+
+extern "C" int32_t qlinear_debug_plan_kv_output(qlinear_t h, int32_t n_heads, int32_t* out, int32_t n_out)
+{
+    if (!h || h->L.bits != 8 || n_heads < 1 || n_heads > kKvMaxHeads || !out) return 0;
+    DeviceGuard guard(h->device);
+    if (!guard.ok || cudaFuncSetAttribute(gemv_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kColsSmem) != cudaSuccess) { cudaGetLastError(); return 0; }
+    const int heads = std::min(n_heads, (int32_t)kGemvMaxBatch), cl = cols_split(h->device, heads * h->n_rb, h->L.n_kc);
+    const int32_t v[4] = {cl, (h->L.n_kc + kColsWarps * cl - 1) / (kColsWarps * cl), heads * h->n_rb, cl > 1 ? cols_clusters_at_once(h->device, cl) : h->num_sms};
+    const int n = n_out < 4 ? n_out : 4;
     for (int i = 0; i < n; ++i) out[i] = v[i];
     return n;
 }

@@ -279,3 +279,22 @@ def test_scores_of_one_head_are_those_of_all_heads(P, torch, d_h, cache, R):
         ok, rel, worst = O.check_against(sc[h].cpu().numpy(), y64, A)
         assert ok, (h, rel, worst)
     assert heads.heads[0].k.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("n_heads,d_h,cache", [(1, 64, 32), (8, 128, CACHE), (1, 128, 2048), (1, 128, 8192), (2, 128, 32768), (1, 256, 32768), (3, 128, 32768), (8, 128, 32768), (8, 256, 16384), (11, 64, 16384)])
+def test_value_product_is_planned_for_one_wave(P, torch, n_heads, d_h, cache):
+    """The launch that the value product makes: no clusters for a cache of up to 2048 positions, a split beyond where the row-blocks
+    leave SMs idle, and never more clusters than run at once (a second wave of them costs more than the split gains)."""
+    import ctypes
+    desc = P.Desc(d_h, cache, 8, 0)
+    v = P.QLinear(desc, torch.zeros(P.qlinear_packed_size(desc), dtype=torch.uint8, device="cuda"))
+    out = (ctypes.c_int32 * 4)()
+    assert P.lib.qlinear_debug_plan_kv_output(v._h, n_heads, out, 4) == 4
+    cl, cps, clusters, at_once = out
+    assert clusters == min(n_heads, 8) * d_h // 16
+    assert cl == 1 or clusters <= at_once
+    assert cps * 16 * cl >= cache // 32 and (cl == 1 or cps >= 2)        # (16 warps per CTA)
+    if cache <= 2048 or clusters * 2 > torch.cuda.get_device_properties(0).multi_processor_count:
+        assert cl == 1
+    elif cache >= 8192 and clusters <= 16:
+        assert cl >= 4
