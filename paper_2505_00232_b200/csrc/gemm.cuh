@@ -50,6 +50,7 @@ struct GemmParams {
     int32_t n_rsb, n_tiles;                  // work units of the grid (pair kernel: tiles x split)
     int32_t split;                           // pair kernel: K parts of the tiles that are split (1 = none are)
     int32_t bn;                              // tensor-memory form: tokens per tile, a multiple of 32 up to 256
+    int32_t late;                            // as in GemvParamsT
     int32_t n_whole;                         // pair kernel: units [0, n_whole) are whole tiles, the rest are parts
     float* scratch;                          // pair kernel, split > 1: fp32 partial tiles [tile][part][rank][256][128]
     unsigned int* counters;                  // pair kernel, split > 1: arrivals per (tile, rank, quarter), zero between launches
@@ -224,6 +225,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const GemmParams p)
             int s = 0, issued = 0;
             uint32_t par = 1;                                            // first pass: stages start out free
             bool waited_dep = false, ok = true;
+            auto wait_dep = [&] {
+                if (waited_dep) return;
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                waited_dep = true;
+                abort_flag[2] = 1;                                       // from here on, waiting counts against the time limit
+                abort_flag[3] = 1;
+            };
             for (int t = first_tile; t < p.n_tiles && ok; t += tile_stride) {
                 const int rsb = t % p.n_rsb, m0 = (t / p.n_rsb) * BN;
                 const uint8_t* wsrc = p.body + (int64_t)rsb * p.n_kc * p.block_bytes;
@@ -233,13 +241,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const GemmParams p)
                     const int nblk = min(CHUNKS, p.n_kc - kc);
                     const uint32_t wbytes = (uint32_t)nblk * p.block_bytes;
                     mbar_expect_tx(full_bar(s), wbytes + S::kXBytes);
+                    if (p.late) wait_dep();
                     bulk_copy_g2s(wpk_addr(s), wsrc + (int64_t)kc * p.block_bytes, wbytes, full_bar(s));
-                    if (!waited_dep) {                                   // x may come from the previous kernel
-                        asm volatile("griddepcontrol.wait;" ::: "memory");
-                        waited_dep = true;
-                        abort_flag[2] = 1;                               // from here on, waiting counts against the time limit
-                        abort_flag[3] = 1;
-                    }
+                    wait_dep();                                          // x may come from the previous kernel
                     tma_load_2d(xs_addr(s), &x_map, it * kGemmKStep, m0, full_bar(s));
                     ++issued;
                     if (++s == NS) { s = 0; par ^= 1; }
@@ -421,7 +425,7 @@ inline int gemm_pick_bn(const Layout& L, int M, int num_sms)
 }
 
 template <int BITS, bool GROUPED, int BN>
-ql_status gemm_launch(const Layout& L, const uint8_t* blob, const void* x, void* y, int M, cudaStream_t st, int device, bool pdl, int num_sms)
+ql_status gemm_launch(const Layout& L, const uint8_t* blob, const void* x, void* y, int M, cudaStream_t st, int device, bool pdl, int num_sms, bool late)
 {
     using S = GemmSmem<BITS, BN>;
     static_assert(S::kStages >= 2, "pipeline needs at least two stages");
@@ -446,6 +450,7 @@ ql_status gemm_launch(const Layout& L, const uint8_t* blob, const void* x, void*
     prm.n_ksteps = (L.K + kGemmKStep - 1) / kGemmKStep;
     prm.n_rsb = L.n_rsb;
     prm.n_tiles = L.n_rsb * ((M + BN - 1) / BN);
+    prm.late = late;
 
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(prm.n_tiles < num_sms ? prm.n_tiles : num_sms);
@@ -466,24 +471,24 @@ ql_status gemm_launch(const Layout& L, const uint8_t* blob, const void* x, void*
 
 template <int BITS, bool GROUPED>
 ql_status gemm_dispatch_bn(int bn, const Layout& L, const uint8_t* blob, const void* x, void* y, int M, cudaStream_t st,
-                           int device, bool pdl, int num_sms)
+                           int device, bool pdl, int num_sms, bool late)
 {
     switch (bn) {
-        case 32: return gemm_launch<BITS, GROUPED, 32>(L, blob, x, y, M, st, device, pdl, num_sms);
-        case 64: return gemm_launch<BITS, GROUPED, 64>(L, blob, x, y, M, st, device, pdl, num_sms);
-        case 128: return gemm_launch<BITS, GROUPED, 128>(L, blob, x, y, M, st, device, pdl, num_sms);
-        case 256: return gemm_launch<BITS, GROUPED, 256>(L, blob, x, y, M, st, device, pdl, num_sms);
+        case 32: return gemm_launch<BITS, GROUPED, 32>(L, blob, x, y, M, st, device, pdl, num_sms, late);
+        case 64: return gemm_launch<BITS, GROUPED, 64>(L, blob, x, y, M, st, device, pdl, num_sms, late);
+        case 128: return gemm_launch<BITS, GROUPED, 128>(L, blob, x, y, M, st, device, pdl, num_sms, late);
+        case 256: return gemm_launch<BITS, GROUPED, 256>(L, blob, x, y, M, st, device, pdl, num_sms, late);
     }
     return QL_ERR_INVALID_ARG;
 }
 
 inline ql_status gemm_forward(const Layout& L, const uint8_t* blob, const void* x, void* y, int M,
-                              cudaStream_t st, int device, bool pdl, int num_sms)
+                              cudaStream_t st, int device, bool pdl, int num_sms, bool late)
 {
     const int bn = gemm_pick_bn(L, M, num_sms);
-    if (L.bits == 8) return gemm_dispatch_bn<8, false>(bn, L, blob, x, y, M, st, device, pdl, num_sms);
-    if (L.grouped) return gemm_dispatch_bn<4, true>(bn, L, blob, x, y, M, st, device, pdl, num_sms);
-    return gemm_dispatch_bn<4, false>(bn, L, blob, x, y, M, st, device, pdl, num_sms);
+    if (L.bits == 8) return gemm_dispatch_bn<8, false>(bn, L, blob, x, y, M, st, device, pdl, num_sms, late);
+    if (L.grouped) return gemm_dispatch_bn<4, true>(bn, L, blob, x, y, M, st, device, pdl, num_sms, late);
+    return gemm_dispatch_bn<4, false>(bn, L, blob, x, y, M, st, device, pdl, num_sms, late);
 }
 
 }  // namespace ql

@@ -158,6 +158,13 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const GemmParams p)
             int s = 0, issued = 0;
             uint32_t par = 1;
             bool waited_dep = false, ok = true;
+            auto wait_dep = [&] {                                        // x may come from the previous kernel
+                if (waited_dep) return;
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                waited_dep = true;
+                abort_flag[2] = 1;                                       // from here on, waiting counts against the time limit
+                abort_flag[3] = 1;
+            };
             int t, gl;
             for (int j = 0; tile_of(j, t, gl) && ok; ++j) {
                 const PairUnit u = pair_unit(t, p);
@@ -172,13 +179,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const GemmParams p)
                     const int nblk = min(CHUNKS, p.n_kc - kc);
                     const uint32_t wbytes = (uint32_t)nblk * p.block_bytes;
                     mbar_expect_tx(full_bar(s), wbytes + S::kXBytes);
+                    if (p.late) wait_dep();
                     bulk_copy_g2s(wpk_addr(s), wsrc + (int64_t)kc * p.block_bytes, wbytes, full_bar(s));
-                    if (!waited_dep) {
-                        asm volatile("griddepcontrol.wait;" ::: "memory");
-                        waited_dep = true;
-                        abort_flag[2] = 1;                               // from here on, waiting counts against the time limit
-                        abort_flag[3] = 1;
-                    }
+                    wait_dep();
 #pragma unroll
                     for (int tb = 0; tb < TB; ++tb)
                         tma_load_2d(xs_addr(s) + tb * S::kXBlockBytes, &x_map, (step0 + it) * S::kKStep, m0 + tb * BN, full_bar(s));
@@ -494,6 +497,7 @@ struct GemmPairLayers {
     const uint8_t* blob[kGemmMaxGroup];
     void* y[kGemmMaxGroup];
     const CUtensorMap* wmap[kGemmMaxGroup];      // packed body as 64-byte rows (tensor-memory form), or nullptr
+    bool late;                                   // as in GemvParamsT
     int n_rsb() const { int t = 0; for (int i = 0; i < n; ++i) t += L[i]->n_rsb; return t; }
 };
 
@@ -542,6 +546,7 @@ ql_status gemm_pair_launch(const GemmPairLayers& set, const void* x, int M, cuda
     // (splitting the tail of a multi-round schedule was measured and does not pay: the exposed scratch
     // reduction costs what the shorter last round saves; only single-round layers are split)
     const int tail = tiles < clusters ? tiles : 0;
+    prm.late = set.late;
     prm.split = (TB == 1 && !GATED && !I8) ? gemm_pair_split(tail, prm.n_ksteps, num_sms, scratch != nullptr) : 1;
     prm.n_whole = prm.split > 1 ? tiles - tail : tiles;
     prm.scratch = scratch;

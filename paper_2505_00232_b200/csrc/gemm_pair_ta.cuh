@@ -329,6 +329,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         // ------------------------------------------------------------------ weight producer (each CTA feeds itself)
         if (lane == 0) {
             constexpr int CHUNKS = S::kWBlocks;                          // packed blocks per k-step
+            if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
             int s = 0, issued = 0;
             uint32_t par = 1;
             bool ok = true;
@@ -736,6 +737,7 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const void* x, int M, c
     prm.a8_scale = a8_scale; prm.a8_rowsum = a8_rowsum;
     prm.n_rsb = n_rsb;
     prm.bn = bn;
+    prm.late = set.late;
     prm.n_tiles = (n_rsb / 2) * n_mblk;
     prm.split = (GATED || I8) ? 1 : gemm_pair_ta_split(prm.n_tiles, prm.n_ksteps, num_sms, scratch && counters);
     prm.scratch = scratch;

@@ -143,9 +143,9 @@ struct qlinear_s {
     CUtensorMap wmap_i8;       // the same with the integer form's box (128 k per step)
     bool wmap_ok, wmap_i8_ok;
     DeviceState* dev;
-    // Set by the first append: the blob is a KV cache, and the kernel before a reader in the stream may be writing it.  The
-    // decode and batch kernels then read it only after griddepcontrol.wait; the prefill kernels are launched without the programmatic
-    // edge.  (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
+    // Set by the first append: the blob is a KV cache, and the kernel before a reader in the stream may be writing it.  Its readers
+    // then touch it only after griddepcontrol.wait (`late` in their parameters), or are launched without the programmatic edge
+    // (early(): int8 activations, the streaming kernel).  (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
     std::atomic<bool> cache{false};
     bool early() const { return pdl && !cache.load(std::memory_order_relaxed); }
 };
@@ -805,10 +805,11 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
     {
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_ok ? &h->wmap : nullptr;
-        const ql_status s = gemm_pair_forward_auto(set, x, M, st, h->device, h->early(), h->num_sms, h->dev->gemm_scratch, h->dev->gemm_counters);
+        set.late = any_cache(&h, 1);
+        const ql_status s = gemm_pair_forward_auto(set, x, M, st, h->device, h->pdl, h->num_sms, h->dev->gemm_scratch, h->dev->gemm_counters);
         if (s != QL_ERR_UNSUPPORTED) return s;                           // (an odd number of row super-blocks: the single-CTA kernel)
     }
-    return gemm_forward(h->L, h->blob, x, y, M, st, h->device, h->early(), h->num_sms);
+    return gemm_forward(h->L, h->blob, x, y, M, st, h->device, h->pdl, h->num_sms, any_cache(&h, 1));
 }
 
 extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const void* x, void* const* ys, int32_t M, void* stream)
@@ -843,11 +844,12 @@ extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const
             if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
             GemmPairLayers set{};
             set.n = n;
+            set.late = any_cache(hs, n);
             for (int i = 0; i < n; ++i) {
                 set.L[i] = &hs[i]->L; set.blob[i] = hs[i]->blob; set.y[i] = ys[i];
                 set.wmap[i] = hs[i]->wmap_ok ? &hs[i]->wmap : nullptr;
             }
-            const ql_status s = gemm_pair_forward_auto(set, x, M, static_cast<cudaStream_t>(stream), hs[0]->device, hs[0]->pdl && !any_cache(hs, n), hs[0]->num_sms,
+            const ql_status s = gemm_pair_forward_auto(set, x, M, static_cast<cudaStream_t>(stream), hs[0]->device, hs[0]->pdl, hs[0]->num_sms,
                                                        hs[0]->dev->gemm_scratch, hs[0]->dev->gemm_counters);
             if (s != QL_ERR_UNSUPPORTED) return s;
         }
@@ -910,10 +912,11 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
     } else if (M > hg->gemv_max_m && gemm_pair_applicable(a, M)) {       // prefill: both accumulators of the CTA-pair kernel
         GemmPairLayers set{};
         set.n = 2;
+        set.late = any_cache(hs, 2);
         set.L[0] = &hg->L; set.blob[0] = hg->blob; set.y[0] = y; set.wmap[0] = hg->wmap_ok ? &hg->wmap : nullptr;
         set.L[1] = &hu->L; set.blob[1] = hu->blob; set.y[1] = y; set.wmap[1] = hu->wmap_ok ? &hu->wmap : nullptr;
-        if (gemm_pair_ta_applicable(set, M, hg->num_sms, true)) return gemm_pair_ta_forward_gated(set, x, M, act, st, hg->device, hg->pdl && !any_cache(hs, 2), hg->num_sms);
-        return gemm_pair_forward_gated(set, x, M, act, st, hg->device, hg->pdl && !any_cache(hs, 2), hg->num_sms);
+        if (gemm_pair_ta_applicable(set, M, hg->num_sms, true)) return gemm_pair_ta_forward_gated(set, x, M, act, st, hg->device, hg->pdl, hg->num_sms);
+        return gemm_pair_forward_gated(set, x, M, act, st, hg->device, hg->pdl, hg->num_sms);
     }
     // Unfused: the two projections into the device's shared scratch, then the element-wise product.
     const int64_t n = (int64_t)M * a.N;

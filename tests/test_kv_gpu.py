@@ -298,3 +298,33 @@ def test_value_product_is_planned_for_one_wave(P, torch, n_heads, d_h, cache):
         assert cl == 1
     elif cache >= 8192 and clusters <= 16:
         assert cl >= 4
+
+
+@pytest.mark.parametrize("d_h,R", [(96, 200), (512, 100), (512, 200), (384, 300)])
+def test_prefill_kernels_see_the_tokens_appended_just_before(P, torch, d_h, R):
+    """Scores of many rows at the head dimensions that the prefill kernels serve (single CTA, CTA pair split along K): append and
+    scores back to back, on tokens that change every time, against the same calls with the host waiting in between."""
+    T, n_new = 700, 5
+    caches = [P.KVCache(768, d_h) for _ in range(2)]
+    start = torch.randn((T, d_h), device="cuda").half()
+    for c in caches:
+        c.append(start, start)
+    q = torch.randn((R, d_h), device="cuda").half()
+    for _ in range(30):
+        kn = (torch.randn((n_new, d_h), device="cuda") * 3).half()
+        torch.cuda.synchronize()
+        got = []
+        for c, wait in zip(caches, (lambda: None, torch.cuda.synchronize)):
+            for factor in (0.5, 2.0, 1.0):
+                c.length = T
+                c.append(kn * factor, kn)
+                wait()
+                sc = c.scores(q)
+            torch.cuda.synchronize()
+            got.append(sc)
+        assert torch.equal(*got)
+    assert caches[0].k.device_status() == (0, 0)
+    k_q, k_s = O.kv_quantize_rows(kn.cpu().numpy())
+    y64, A, _ = O.linear(q.cpu().numpy(), k_q, k_s.reshape(-1, 1), 0)
+    ok, rel, worst = O.check_against(got[0][:, T:T + n_new].cpu().numpy(), y64, A)
+    assert ok, (rel, worst)
