@@ -1118,6 +1118,18 @@ extern "C" ql_status qlinear_kv_output_heads(const qlinear_t* hv, int32_t n_head
     return QL_OK;
 }
 
+namespace {
+// Value products of many rows for which the scales as a pass of their own and the prefill kernel win: heads of more than 256 (whose
+// layers the CTA-pair kernel takes), from a size on at which the batch kernel's warp-level MMAs cost more than that pass.  Measured,
+// us batch kernel / pass and prefill kernel: 512 channels, 4096 positions, 1024 rows 23 / 32, 2048 rows 41 / 41, 4096 rows 76 / 61; 1024
+// channels, 4096 positions, 512 rows 23 / 29, 1024 rows 41 / 34, 4096 rows 148 / 61; 1024 positions, 2048 rows 22 / 25, 4096 rows 42 / 23;
+// 256 positions, 2048 rows 9 / 12, 4096 rows 16 / 13.  256 channels, 4096 positions, 4096 rows 41 / 58.
+bool value_product_is_large(const Layout& V, int R)
+{
+    return V.n_rsb % 2 == 0 && V.N > 256 && (int64_t)R * (V.N - 256) * (V.K + 1024) > 3350000000ll;
+}
+}  // namespace
+
 extern "C" ql_status qlinear_kv_output(qlinear_t hv, const void* prob, const void* v_scale, void* tmp, void* out, int32_t R, void* stream)
 {
     if (!hv || !prob || !v_scale || !tmp || !out || R < 1 || hv->L.bits != 8) return QL_ERR_INVALID_ARG;
@@ -1129,7 +1141,7 @@ extern "C" ql_status qlinear_kv_output(qlinear_t hv, const void* prob, const voi
         const ql_status s = qlinear_kv_output_heads(&hv, 1, prob, &v_scale, out, R, stream);
         if (s != QL_ERR_UNSUPPORTED) return s;
         // more rows: the kernel that takes any number of tokens against few channels, with the scales folded in on the way
-        if (R > hv->gemv_max_m) {
+        if (R > hv->gemv_max_m && !value_product_is_large(hv->L, R)) {
             if ((int64_t)R * hv->L.N > INT32_MAX) return QL_ERR_INVALID_ARG;   // (the limit of qlinear_forward)
             if (device_timed_out(hv)) return QL_ERR_DEVICE_TIMEOUT;
             DeviceGuard guard(hv->device);

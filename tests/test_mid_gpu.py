@@ -99,3 +99,28 @@ def test_value_product_keeps_the_limit_on_its_output(P, torch):
         kv.output(prob)
     assert err.value.status == P.QL_ERR_INVALID_ARG
     assert kv.output(prob[:100]).shape == (100, 65536)
+
+
+@pytest.mark.parametrize("d_h,cache,R,large", [(512, 2048, 4096, False), (512, 4096, 4096, True), (1024, 256, 4096, True), (1024, 1024, 2048, False), (1024, 4096, 1024, True), (640, 4096, 4096, False)])
+def test_value_product_on_both_sides_of_the_prefill_kernel(P, torch, d_h, cache, R, large):
+    """Wide heads and many rows: the scales as a pass of their own (into the scratch argument) and the prefill kernel, where that is
+    faster; 640 channels are an odd number of super-blocks.  Both routes against the oracle, on some of the rows."""
+    import ctypes
+    kv = P.KVCache(cache, d_h)
+    v = (gen.normal_fp16(6500 + cache, 2, (cache, d_h)) * gen.normal_fp16(6500 + cache, 4, (cache, 1))).astype(np.float16)
+    vd = torch.from_numpy(v).cuda()
+    kv.append(vd, vd)
+    prob = (torch.rand((R, cache), device="cuda") / cache).half()
+    tmp = torch.full((R, cache), 7.0, dtype=torch.float16, device="cuda")
+    out = torch.empty((R, d_h), dtype=torch.float16, device="cuda")
+    vp = ctypes.c_void_p
+    assert P.lib.qlinear_kv_output(kv.v._h, vp(prob.data_ptr()), vp(kv.v_scale.data_ptr()), vp(tmp.data_ptr()), vp(out.data_ptr()), R, vp(torch.cuda.current_stream().cuda_stream)) == 0
+    torch.cuda.synchronize()
+    assert kv.v.device_status() == (0, 0)
+    assert bool((tmp == 7).all()) != large
+    rows = [0, 1, 63, 64, 255, 256, R - 1]
+    v_q, v_s = O.kv_quantize_rows(v)
+    folded = (prob[rows].cpu().numpy().astype(np.float32) * v_s.astype(np.float32)).astype(np.float16)
+    y64, A, _ = O.kv_output(folded, np.ascontiguousarray(v_q.T), np.ones(d_h, np.float16))
+    ok, rel, worst = O.check_against(out[rows].cpu().numpy(), y64, A)
+    assert ok, (rel, worst)
