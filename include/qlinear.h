@@ -364,9 +364,11 @@ uint32_t qlinear_version(void);
  * arguments).  qlinear_debug_config_reads returns how many times the QLINEAR_* environment has been read by
  * this process (1 after the first call, for good).  qlinear_debug_plan_kv_output does for the (first) launch of
  * qlinear_kv_output_heads over n_heads caches like h_v what qlinear_debug_plan does for the other decode launches: {CTAs per
- * cluster, chunks per warp, clusters of the launch, clusters that run at once}. */
+ * cluster, chunks per warp, clusters of the launch, clusters that run at once}.  qlinear_debug_takes_batch_kernel returns 1 if a
+ * forward call (n = 1), a group or a gated pair (n = 2) of these layers on M tokens runs on the kernel for a batch of tokens. */
 int32_t qlinear_debug_plan(qlinear_t h, int32_t M, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_plan_kv_output(qlinear_t h_v, int32_t n_heads, int32_t* out, int32_t n_out);
+int32_t qlinear_debug_takes_batch_kernel(const qlinear_t* hs, int32_t n, int32_t M);
 uint32_t qlinear_debug_config_reads(void);
 
 #ifdef __cplusplus

@@ -55,7 +55,7 @@ struct Config {
     int warps_per_sm;        // QLINEAR_GEMV_WARPS_PER_SM: residency target of the cluster decode kernel
     bool oversubscribe;      // QLINEAR_GEMV_OVERSUBSCRIBE=0: the group-scaled int4 decode kernel never takes more CTAs than fit at once
     int force_ks;            // QLINEAR_GEMV_KS: forced K split of the cluster decode kernel (0 = planned)
-    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M served by the kernel for a batch of tokens (0: never); see takes_mid
+    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M of a forward call that the kernel for a batch of tokens may serve (0: none; at most 64); see takes_mid
     bool xdirect;            // QLINEAR_GEMV_XDIRECT: x fragments straight from global memory
     int kernel;              // QLINEAR_GEMV_KERNEL: 0 / 1 cluster kernel (default), 2 streaming kernel
     int stream_ctas_per_sm, stream_stages;
@@ -470,18 +470,25 @@ cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pd
     return launch(kern, prm, dim3((unsigned)(tiles * prm.cl)), dim3(kMidThreads), S::kTotal, st, prm.cl, pdl);
 }
 
-// Which launches take this kernel: up to 32 tokens all of them, up to 64 those with at most 48 million weights.  Beyond, its
-// MMAs take longer than the prefill kernel, which does not depend on M below 256 tokens but has fewer and larger tiles.
-// Measured at 64 tokens, this kernel / the prefill kernel: 117 M weights (Llama gate + up) 59 / 49 us, 59 M (down) 29.8 /
-// 29.3, 42 M (Gemma2-2B gate + up) 19.4 / 21.5, 21 M (its down) 20.9 / 22.0, 17 M (Llama o) 12.7 / 17.6, 9 M 10.0 / 15.7.
+// Which launches take this kernel: up to 32 tokens all of them, up to 48 those with at most 48 million weights, up to 64 those with at most
+// 30 million (int8: 24).  Beyond, its MMAs take longer than the prefill kernel, whose tiles of these widths cost the same dequantisation
+// whatever M is.  Measured, us this kernel / the prefill kernel, int4 in groups (int8: 3 to 12 % less in its favour):
+//   weights                     32 tokens    48           64
+//     9 M (Gemma2-2B q + k + v)  6.8 / 11.4   8.7 / 13.8  11.1 / 15.6
+//    21 M (its down)            12.7 / 16.7  16.7 / 19.3  20.9 / 21.4
+//    25 M (Llama q + k + v)     11.9 / 15.5  15.4 / 17.4  18.3 / 18.7     (int8 12.4 / 15.2, 16.8 / 16.9, 19.8 / 18.2)
+//    34 M (32768 x 1024)        11.1 / 15.4  14.5 / 15.8  17.5 / 15.9
+//    42 M (its gate + up)       13.1 / 18.7  16.5 / 19.0  19.6 / 19.6
+//    59 M (Llama down)          18.8 / 23.1  24.3 / 25.8  30.0 / 27.9     (14336 x 4096: 20.2 / 21.8, 26.3 / 22.1, 32.2 / 22.2)
+//   117 M (Llama gate + up)     36.9 / 42.1  47.7 / 43.1  59.0 / 43.8
+// QLINEAR_MID_MAX_M lowers the number of tokens up to which this holds (0: never).
 bool takes_mid(const qlinear_s* const* hs, int n, int M)
 {
-    const int max_m = config().mid_max_m;
-    if (M <= max_m / 2) return true;
-    if (M > max_m) return false;
+    if (M > 64 || M > config().mid_max_m) return false;
+    if (M <= 32) return true;
     int64_t weights = 0;
     for (int i = 0; i < n; ++i) weights += (int64_t)hs[i]->L.N * hs[i]->L.K;
-    return weights <= 48000000;
+    return weights <= (M <= 48 ? 48000000 : hs[0]->L.bits == 4 ? 30000000 : 24000000);
 }
 
 template <int BITS, bool GROUPED, bool GATED, bool KSCALE = false>
@@ -1453,6 +1460,14 @@ extern "C" int32_t qlinear_debug_plan_kv_output(qlinear_t h, int32_t n_heads, in
     const int n = n_out < 4 ? n_out : 4;
     for (int i = 0; i < n; ++i) out[i] = v[i];
     return n;
+}
+
+extern "C" int32_t qlinear_debug_takes_batch_kernel(const qlinear_t* hs, int32_t n, int32_t M)
+{
+    if (!hs || n < 1 || n > kGemvMaxGroup || M < 1) return 0;
+    for (int i = 0; i < n; ++i)
+        if (!hs[i]) return 0;
+    return M > hs[0]->gemv_max_m && !(n == 1 && takes_rows(hs[0]->L)) && takes_mid(hs, n, M);
 }
 
 extern "C" uint32_t qlinear_debug_config_reads(void) { config(); return g_getenv_reads.load(); }

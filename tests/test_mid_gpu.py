@@ -124,3 +124,26 @@ def test_value_product_on_both_sides_of_the_prefill_kernel(P, torch, d_h, cache,
     y64, A, _ = O.kv_output(folded, np.ascontiguousarray(v_q.T), np.ones(d_h, np.float16))
     ok, rel, worst = O.check_against(out[rows].cpu().numpy(), y64, A)
     assert ok, (rel, worst)
+
+
+# (N, K, bits, group, M, whether the batch kernel takes it): both sides of each line of the rule
+LINES = [(12000, 4096, 4, 32, 48, False), (11584, 4096, 4, 32, 48, True), (7424, 4096, 4, 32, 64, False), (7168, 4096, 4, 32, 64, True),
+         (5888, 4096, 8, 0, 49, False), (5632, 4096, 8, 0, 49, True), (14336, 4096, 4, 0, 32, True), (2304, 2304, 8, 0, 65, False)]
+
+
+@pytest.mark.parametrize("N,K,bits,group,M,mid", LINES)
+def test_lines_between_the_batch_kernel_and_the_prefill_kernel(P, torch, N, K, bits, group, M, mid):
+    """The shape picks the kernel that was measured to be faster; both give the layer."""
+    import ctypes
+    layer = spec(N, K, bits, group)
+    q, s = C.layer_weights(6600 + N, layer)
+    x = C.layer_activations(6600 + M, layer, M)
+    lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
+    assert P.lib.qlinear_debug_takes_batch_kernel((ctypes.c_void_p * 1)(lin._h), 1, M) == mid
+    y = lin.forward(torch.from_numpy(x).cuda())
+    torch.cuda.synchronize()
+    assert lin.device_status() == (0, 0)
+    rows = np.r_[0:64, N - 64:N]
+    y64, A, _ = O.linear(x, q[rows], s[rows], group)
+    ok, rel, worst = O.check_against(y.cpu().numpy()[:, rows], y64, A)
+    assert ok, (rel, worst)
