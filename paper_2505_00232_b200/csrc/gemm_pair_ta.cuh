@@ -615,11 +615,11 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                     continue;                                            // (tiles of a few steps: the one after it may be due as well)
                 }
                 uint32_t r[16];
-                if (NW % 3 != 0 && !mbar_wait(wempty_bar(s), wpar ^ 1, abort_flag, 0x480)) { ok = false; break; }
-                if (!mbar_wait(wfull_bar(s), wpar, abort_flag, 0x400)) { ok = false; break; }
+                if (NW % 3 != 0 && !mbar_wait(wempty_bar(s), wpar ^ 1, abort_flag, 0x480 + s)) { ok = false; break; }
+                if (!mbar_wait(wfull_bar(s), wpar, abort_flag, 0x400 + s)) { ok = false; break; }
                 dq.template convert<BITS, GROUPED, I8>(wpk_addr(s), r);
                 // the MMAs that read the slot (step g - NA) have retired
-                if (!mbar_wait(aempty_bar(a), apar, abort_flag, 0xB00)) { ok = false; break; }
+                if (!mbar_wait(aempty_bar(a), apar, abort_flag, 0xB00 + a)) { ok = false; break; }
                 tc_fence_after();
                 tmem_st16(tmem_base + lane_base + (uint32_t)(kTaAccCols + a * kTaSlotCols + 16 * half), r);
                 tc_fence_before();
@@ -647,10 +647,10 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                     event = epi_warp && next_epi < tile_j ? g + 1 : tile_g0 + n_steps;
                 }
                 uint32_t r[16];
-                if (NW % 3 != 0 && !mbar_wait(wbar + 8 * NW, wpar ^ 1, abort_flag, 0x480)) { ok = false; break; }
-                if (!mbar_wait(wbar, wpar, abort_flag, 0x400)) { ok = false; break; }
+                if (NW % 3 != 0 && !mbar_wait(wbar + 8 * NW, wpar ^ 1, abort_flag, 0x480 + ((wbar - wfull_bar(0)) >> 3))) { ok = false; break; }
+                if (!mbar_wait(wbar, wpar, abort_flag, 0x400 + ((wbar - wfull_bar(0)) >> 3))) { ok = false; break; }
                 dq.template convert<BITS, GROUPED, I8>(wst, r);
-                if (!mbar_wait(abar + 8 * NA, apar, abort_flag, 0xB00)) { ok = false; break; }
+                if (!mbar_wait(abar + 8 * NA, apar, abort_flag, 0xB00 + ((abar - afull_bar(0)) >> 3))) { ok = false; break; }
                 tc_fence_after();
                 tmem_st16(slot, r);
                 tc_fence_before();
