@@ -199,8 +199,8 @@ GemvPlan plan_gemv(const Layout& L, int n_rb, int M, int num_sms, bool gated = f
             // the launch itself still gains but the step that contains it loses 1 to 3 % (the next launch gets its SMs later).
             if (warps > target) score += (cfg.oversubscribe && M == 1 && L.grouped && cl == 1 && warps <= 1.55 * target && cps >= 16) ? 0.25 : -2.0;
             // a cluster launch and its two cluster-wide barriers cost a microsecond or two (the CTAs of a cluster start
-            // together and leave together): more than a launch of a few MB gains from the extra warps (V-cache product of 8
-            // heads at 1280 positions: 4.2 us with clusters of 5, 3.1 us without; one 2304 x 2304 int8 layer: 4.0 / 3.7 us).
+            // together and leave together): more than a launch of a few MB gains from the extra warps (one 2304 x 2304 int8 layer:
+            // 4.0 us with a cluster, 3.7 without).
             // Larger launches keep their clusters: timed alone they look better without (Llama o, 16.8 MB: 5.9 / 4.6 us),
             // but inside the step the under-filled grid costs the launches around it more than it saves.
             if (cl > 1 && (double)n_rb * L.n_kc * 512.0 < 6.0e6) score -= 0.75;

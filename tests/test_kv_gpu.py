@@ -168,8 +168,9 @@ def test_scores_over_a_long_cache_match_the_per_head_calls(P, torch, d_h, cache,
 
 
 def test_small_launches_are_planned_without_clusters(P, torch):
-    """A cluster launch with its cluster-wide barriers costs about a microsecond: launches of a few MB (the V-cache
-    product at the protocol length) are planned without one, large layers with a long K still take clusters."""
+    """A cluster launch with its cluster-wide barriers costs about a microsecond: a forward call on a layer of a few MB is planned
+    without one, large layers with a long K still take clusters.  (The value product over a cache has a plan of its own,
+    test_value_product_is_planned_for_one_wave.)"""
     import ctypes
 
     def plan(lin, M):

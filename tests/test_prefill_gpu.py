@@ -1,4 +1,8 @@
 """Prefill kernel (M > 8, tcgen05) against the CPU oracle, through the C-ABI, on a B200."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -6,6 +10,7 @@ from oracle import qlinear_oracle as O
 from workloads import configs as C
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -65,7 +70,8 @@ def rand_case(seed, M, N, K, bits, group):
 
 
 SMALL = [
-    # (M, N, K, bits, group): every tile width, ragged M / N / K tails, every scheme
+    # (M, N, K, bits, group): ragged M / N / K tails, every scheme.  Up to 64 tokens these run on the kernel for a batch of tokens;
+    # test_narrow_tiles runs them on the single-CTA kernel's tiles of 32 and 64 tokens.
     (9, 8, 32, 8, 0), (16, 128, 64, 4, 32), (17, 136, 160, 8, 0), (33, 200, 352, 4, 32), (64, 256, 512, 4, 0),
     (127, 264, 2304, 4, 32), (128, 128, 1056, 8, 0), (129, 384, 1024, 4, 32), (300, 520, 1056, 8, 0),
     (256, 40, 256, 4, 64), (257, 16, 384, 4, 128), (512, 1000, 96, 8, 0), (1024, 256, 2304, 4, 32),
@@ -80,6 +86,63 @@ def test_parity_small_and_ragged(P, torch, M, N, K, bits, group):
     q, s, x = rand_case(2000 + N + K + M, M, N, K, bits, group)
     lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
     assert_parity(forward(P, torch, lin, x), x, q, s, group)
+
+
+# The single-CTA kernel's narrow tiles: reached by default only by layers of more weights than the batch kernel takes (64-token tiles), so
+# a child process leaves that kernel out.  Rows: token counts around both widths; the last three as gated pairs (unfused there).
+NARROW = [c for c in SMALL if c[0] <= 64] + [(32, 640, 96, 4, 0), (31, 136, 2304, 4, 32), (40, 384, 1056, 8, 0), (63, 8, 4096, 4, 128)]
+NARROW_GATED = [(24, 264, 256, 4, 32), (50, 384, 544, 8, 0), (9, 136, 1024, 4, 0)]
+CHILD = """
+import ctypes, sys, numpy as np, torch
+sys.path.insert(0, {root!r})
+import paper_2505_00232_b200 as P
+from tests.test_prefill_gpu import NARROW, NARROW_GATED, one_hot, rand_case
+out = {{}}
+def layer(q, s, bits, group, M):
+    lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
+    assert P.lib.qlinear_debug_takes_batch_kernel((ctypes.c_void_p * 1)(lin._h), 1, M) == 0
+    return lin
+for i, (M, N, K, bits, group) in enumerate(NARROW):
+    q, s, x = rand_case(2000 + N + K + M, M, N, K, bits, group)
+    lin = layer(q, s, bits, group, M)
+    out[f"plain{{i}}"] = lin.forward(torch.from_numpy(x).cuda()).cpu().numpy()
+    if M >= 16:
+        out[f"hot{{i}}"] = lin.forward(torch.from_numpy(one_hot(M, K)[0]).cuda()).cpu().numpy()
+    torch.cuda.synchronize()
+    assert lin.device_status() == (0, 0)
+for i, (M, N, K, bits, group) in enumerate(NARROW_GATED):
+    (qg, sg, x), (qu, su, _) = (rand_case(2500 + j + N + K + M, M, N, K, bits, group) for j in range(2))
+    pair = layer(qg, sg, bits, group, M), layer(qu, su, bits, group, M)
+    out[f"gated{{i}}"] = P.qlinear_forward_gated(*pair, torch.from_numpy(x).cuda(), "silu").cpu().numpy()
+np.savez({out!r}, **out)
+"""
+
+
+def one_hot(M, K):
+    ks = np.random.default_rng(M + K).integers(0, K, size=M)
+    ks[:3] = 0, K - 1, 31
+    x = np.zeros((M, K), np.float16)
+    x[np.arange(M), ks] = 1.0
+    return x, ks
+
+
+def test_narrow_tiles(P, tmp_path):
+    path = str(tmp_path / "narrow.npz")
+    env = dict(os.environ, QLINEAR_MID_MAX_M="0")
+    subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, out=path)], check=True, env=env, cwd=ROOT, timeout=600)
+    got = np.load(path)
+    for i, (M, N, K, bits, group) in enumerate(NARROW):
+        q, s, x = rand_case(2000 + N + K + M, M, N, K, bits, group)
+        assert_parity(got[f"plain{i}"], x, q, s, group)
+        if M >= 16:                                      # a row of the product is a weight column, rounded once
+            ks = one_hot(M, K)[1]
+            want = (s[:, ks // (group or K)].astype(np.float64) * q[:, ks].astype(np.float64)).astype(np.float16).T
+            assert (got[f"hot{i}"].view(np.uint16) == want.view(np.uint16)).all(), (M, N, K)
+    for i, (M, N, K, bits, group) in enumerate(NARROW_GATED):
+        (qg, sg, x), (qu, su, _) = (rand_case(2500 + j + N + K + M, M, N, K, bits, group) for j in range(2))
+        g64, bound, _ = O.gated_linear(x, qg, sg, qu, su, group, "silu")
+        ok, rel, worst = O.check_gated(got[f"gated{i}"], g64, bound)
+        assert ok, (M, N, K, rel, worst)
 
 
 @pytest.mark.parametrize("N,K,bits,group", [(136, 160, 8, 0), (200, 352, 4, 32), (264, 2304, 4, 32), (128, 1024, 4, 0)])
@@ -136,7 +199,7 @@ def test_run_to_run_deterministic_and_stage_boundary(P, torch):
     a = lin.forward(xd).clone()
     for _ in range(3):
         assert torch.equal(a, lin.forward(xd))
-    # M = 8 takes the decode kernel, M = 9 the prefill kernel: both within tolerance of the oracle
+    # M = 8 takes the decode kernel, M = 9 the kernel for a batch of tokens: both within tolerance of the oracle
     assert lin.path_for(8) == P.QL_PATH_GEMV and lin.path_for(9) == P.QL_PATH_GEMM
     y8 = lin.forward(xd[:8].contiguous()).cpu().numpy()
     assert_parity(y8, x[:8], q, s, 0)

@@ -89,6 +89,46 @@ def test_bit_identical_to_the_shared_memory_form(P, torch, tmp_path):
         assert np.array_equal(y.view(np.uint16), ref[str(i)].view(np.uint16)), f"case {c}"
 
 
+# Tiles of 32, 64, 96 and 128 tokens (one block of at most 128): whole along K, in two and in four parts.  A child process leaves the kernel
+# for a batch of tokens out, which takes most launches of up to 64 tokens before this one sees them.
+WIDTHS = [(M, N, K, bits, group) for M in (20, 33, 40, 64, 65, 96, 100, 128)
+          for N, K, bits, group in ((512, 448, 4, 32), (504, 1024, 8, 0), (248, 2304, 4, 0), (768, 2304, 4, 32), (256, 4096, 8, 0))]
+WIDTHS_CHILD = """
+import sys, numpy as np, torch
+sys.path.insert(0, {root!r})
+import paper_2505_00232_b200 as P
+from tests.test_prefill_ta_gpu import WIDTHS, case, run
+out = {{str(i): run(P, torch, *c, 7700 + c[0] + c[1])[3] for i, c in enumerate(WIDTHS)}}
+for M in (20, 40, 96, 128):                             # two layers in one launch
+    w = [case(7800 + i, M, 512, 2304, 4, 32) for i in range(2)]
+    lins = [P.QLinear.from_weights(q, s, 4, 32, device="cuda:0") for q, s, _ in w]
+    for i, y in enumerate(P.qlinear_forward_group(lins, torch.from_numpy(w[0][2]).cuda())):
+        out[f"group{{M}}_{{i}}"] = y.cpu().numpy()
+np.savez({out!r}, **out)
+"""
+
+
+def test_tile_widths_up_to_128_tokens(P, torch, tmp_path):
+    out = str(tmp_path / "widths.npz")
+    env = dict(os.environ, QLINEAR_MID_MAX_M="0")
+    subprocess.run([sys.executable, "-c", WIDTHS_CHILD.format(root=ROOT, out=out)], check=True, env=env, cwd=ROOT, timeout=600)
+    got = np.load(out)
+    for i, c in enumerate(WIDTHS):
+        M, N, K, bits, group = c
+        q, s, x = case(7700 + M + N, M, N, K, bits, group)
+        y64, A, _ = O.linear(x, q, s, group)
+        ok, rel, worst = O.check_against(got[str(i)], y64, A)
+        assert ok, (c, rel, worst)
+        if M > 64:                                       # the same kernel without the switch
+            assert np.array_equal(run(P, torch, *c, 7700 + M + N)[3].view(np.uint16), got[str(i)].view(np.uint16)), c
+    for M in (20, 40, 96, 128):
+        w = [case(7800 + i, M, 512, 2304, 4, 32) for i in range(2)]
+        for i, (q, s, _) in enumerate(w):
+            y64, A, _ = O.linear(w[0][2], q, s, 32)
+            ok, rel, worst = O.check_against(got[f"group{M}_{i}"], y64, A)
+            assert ok, (M, i, rel, worst)
+
+
 def test_guard_band_around_y(P, torch):
     """The output tile leaves through bulk copies of whole 256-byte rows: nothing outside [M, N] may be written."""
     M, N, K, bits, group = 300, 19448, 128, 4, 32                        # ragged last row super-block (120 channels)
