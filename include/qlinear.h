@@ -13,15 +13,17 @@
  * memory layout the kernels read (Section 3.4, "weights conversion"; Section
  * 3.1, weight layouts); every forward call then picks the kernel for its stage
  * from the shape of the input (Section 3.7: a memory-bound fully-connected
- * kernel for decode, a compute-bound matrix-multiply kernel for prefill), both
- * reading the same resident weights.  Quantisation schemes: Section 4.2 (q8 =
+ * kernel for decode, a compute-bound matrix-multiply kernel for prefill, and
+ * between the two a kernel for a batch of tokens), all reading the same resident weights.  Quantisation schemes: Section 4.2 (q8 =
  * int8 per channel; 8/4/4 = int8 attention, int4 feed-forward/embedding).
  *
- * Threads and streams.  A handle is immutable after qlinear_create, so any
+ * Threads and streams.  A handle is immutable after qlinear_create (the KV-cache
+ * appends mark theirs as caches, once), so any
  * number of host threads may call the forward functions on it.  The kernels of
  * two calls may overlap on the GPU (different streams) unless one of them is a
- * prefill call the library splits along K (a layer, or group of layers, with
- * fewer 256 x 256 output tiles than half the SM count): those calls meet in one
+ * prefill call the library splits along K (a layer, or group of layers, that the
+ * prefill kernel serves and that has fewer tiles of 256 channels x 256 tokens than
+ * half the SM count): those calls meet in one
  * per-device scratch area and must be ordered against each other by the caller
  * (same stream, or events).  qlinear_decode_static has its own rule, stated
  * there.
@@ -72,7 +74,7 @@ typedef struct {
     int32_t N, K, bits, group;
 } qlinear_desc;
 
-/* Which kernel a forward call with M tokens runs (Section 3.7, stage-aware selection). */
+/* The stage of a forward call with M tokens (Section 3.7): QL_PATH_GEMV the decode kernels, QL_PATH_GEMM the batch and prefill kernels. */
 typedef enum { QL_PATH_GEMV = 1, QL_PATH_GEMM = 2 } ql_path;
 
 /* Bytes of the packed blob for this layer; 0 if the descriptor is invalid or unsupported. */
@@ -109,7 +111,10 @@ ql_status qlinear_create(const qlinear_desc* desc, const void* packed_dev, int d
  *   x_dev  device, fp16 [M, K] row-major contiguous, 16-byte aligned, read-only during the call.
  *   y_dev  device, fp16 [M, N] row-major contiguous, 16-byte aligned, must not overlap x_dev.
  * Asynchronous: returns after the launch; allocates nothing; never synchronises.  M <= 8 runs the
- * decode kernel, larger M the prefill kernel (Section 3.7); see qlinear_path_for.
+ * decode kernel, larger M a matrix-multiply kernel (Section 3.7; qlinear_path_for): the kernel for a batch of tokens up to
+ * 32 tokens, up to 48 for layers (or groups) of at most 48 million weights and up to 64 for at most 30 million (int8: 24), the
+ * prefill kernel beyond.  The environment variable QLINEAR_MID_MAX_M lowers the token count up to which the batch kernel is used (0:
+ * never).  int8 layers of K = 64, 128 or 256 have kernels of their own, for M <= 8 and for any larger M.
  * Errors: QL_ERR_INVALID_ARG (null / misaligned pointers, M < 1, M*K or M*N beyond 2^31-1 elements),
  * QL_ERR_CUDA (launch failure, reported synchronously), QL_ERR_DEVICE_TIMEOUT (an earlier kernel of this
  * library on the handle's DEVICE gave up a bounded wait: its output is invalid; nothing is launched, and every
@@ -125,7 +130,7 @@ ql_status qlinear_forward(qlinear_t h, const void* x_dev, void* y_dev, int32_t M
  * the same reason: launch overhead and memory-bound work).  Every output is bit-identical to what
  * qlinear_forward gives for that layer only if the K split chosen for the group equals the layer's own;
  * it always meets the same tolerance, and is run-to-run deterministic.  For larger M the layers share
- * one launch of the prefill kernel when every layer qualifies for its
+ * one launch of the batch kernel (sizes: qlinear_forward), or one launch of the prefill kernel when every layer qualifies for its
  * CTA-pair form (a multiple of 256 output channels after padding to 128); the tiles of all layers then
  * fill the persistent grid together.  Otherwise they run one after the other.
  *   hs      host array of n handles; ys_dev host array of n device pointers (fp16 [M, N_i], 16-byte
@@ -139,8 +144,8 @@ ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const void* x_de
  * case in mind is the attention products over the KV cache held as weights (paper Section 3.8): every KV head has its
  * own cache handle and its own query rows, and a launch per head and product is launch-bound.  Same requirements on the
  * handles as qlinear_forward_group (one device, equal K, bits and group).  For M <= 8 and K a whole number of chunks the
- * call is one decode launch (more than 4 layers: int8 layers only); otherwise it is n calls of qlinear_forward, in
- * order.  Pointers as for qlinear_forward. */
+ * call is one decode launch (more than 4 layers: int8 layers only); int8 layers of K = 64, 128 or 256 (K caches) share one launch
+ * at any larger M too; otherwise it is n calls of qlinear_forward, in order.  Pointers as for qlinear_forward. */
 ql_status qlinear_forward_batch(const qlinear_t* handles, int32_t n, const void* const* xs_dev, void* const* ys_dev, int32_t M, void* cuda_stream);
 
 /* Activation of the gate branch in qlinear_forward_gated. */
@@ -151,11 +156,12 @@ typedef enum { QL_ACT_IDENTITY = 0, QL_ACT_SILU = 1, QL_ACT_GELU_TANH = 2 } ql_a
  *     y[m,n] = fp16( act(gate[m,n]) * up[m,n] ),   gate = x . W_gate^T,  up = x . W_up^T   (both in fp32)
  * with act = identity, SiLU g / (1 + exp(-g)) (the Llama family) or the tanh form of GELU (the Gemma family);
  * the paper names no activation.  Neither projection is written to memory: for M <= 8 one decode launch
- * holds both branches of every output channel in the same CTA; for M > 128 (and layers of a multiple of 256
+ * holds both branches of every output channel in the same CTA, and so does one launch of the batch kernel for the token counts and
+ * weights (of both layers) stated at qlinear_forward; for M > 128 (and layers of a multiple of 256
  * channels after padding to 128) the CTA-pair prefill kernel keeps the two projections of a tile in its two
  * tensor-memory accumulators and the epilogue writes only their product, which halves the write-back.
- * Shapes outside those two cases (9 <= M <= 128, other channel counts, K not a multiple of the decode chunk)
- * run the two projections into the device's shared scratch and a small element-wise kernel after them: same
+ * Shapes outside those cases (up to 128 tokens of more weights than the batch kernel takes, other channel counts at more tokens, K not a
+ * multiple of the decode chunk at M <= 8) run the two projections into the device's shared scratch and a small element-wise kernel after them: same
  * result, no saving; such calls must be ordered against K-split prefill calls like those among themselves.
  *   h_gate, h_up  two layers on one device with the same N, K, bits and group
  *   x_dev, y_dev  as in qlinear_forward; y_dev is fp16 [M, N]
@@ -211,9 +217,11 @@ ql_status qlinear_quantize_activations(const void* x_dev, int8_t* xq_dev, float*
  *     out[r, d] = sum_t (prob[r, t] * s_v[t]) * q_v[t, d].
  * These are the only calls that write to a blob; they must be ordered against forward calls on the same handles.
  * qlinear_kv_scores:  scores_dev [R, cache positions] = q_rows_dev [R, d_h] . K^T   (= qlinear_forward on h_k).
- * qlinear_kv_output:  out_dev [R, d_h] from prob_dev fp16 [R, cache positions]; tmp_dev is caller-owned scratch of
- *                     the same shape as prob_dev (it receives prob * s_v rounded to fp16 where that product needs a
- *                     pass of its own: R > 8, or a cache length that is not a multiple of 32).
+ * qlinear_kv_output:  out_dev [R, d_h] from prob_dev fp16 [R, cache positions].  The product prob * s_v, rounded to fp16, is formed
+ *                     on the way to the tensor core; tmp_dev is caller-owned scratch of the same shape as prob_dev, which
+ *                     receives it where it needs a pass of its own: prob_dev not 16-byte aligned, QLINEAR_GEMV_KERNEL=stream at
+ *                     R <= 8, or more than 256 channels and R (d_h - 256) (cache positions + 1024) > 3.35e9 (then
+ *                     the prefill kernel serves the product, with its rule on ordering).
  * k_new_dev, v_new_dev, v_scale_dev, prob_dev, tmp_dev, out_dev: 16-byte aligned.
  * Masking and the softmax between the two are the caller's.  Asynchronous, allocate nothing.
  * Errors: QL_ERR_INVALID_ARG (null / misaligned pointers, handles that are not an int8 cache pair of matching
@@ -237,10 +245,10 @@ ql_status qlinear_kv_output(qlinear_t h_v, const void* prob_dev, const void* v_s
  *                            qlinear_kv_output) is formed inside the decode kernel on the way to the tensor core, so
  *                            there is no scratch buffer and no pass of its own.  Other shapes: QL_ERR_UNSUPPORTED
  *                            (use qlinear_kv_output per head).
- * All device pointers 16-byte aligned, R * d_h and R * cache positions multiples of 8.  Results are bit-identical to
- * the per-head calls wherever those take K undivided (d_h <= 128) and meet the same tolerance everywhere.  Score
- * products of more than four row super-blocks per SM (long caches; R <= 8, d_h = 64, 128 or 256) run on a persistent
- * kernel of their own (csrc/gemv_rows.cuh).  Asynchronous, allocate nothing.  Errors as above. */
+ * All device pointers 16-byte aligned, R * d_h and R * cache positions multiples of 8.  Scores are
+ * bit-identical to the per-head calls at d_h = 64, 128 and 256 (csrc/gemv_rows.cuh for R <= 8, gemm_rows.cuh beyond).  The value product
+ * splits K by the number of heads in the launch, so beyond 2048 cache positions its bits may depend on that number (at most 8 heads
+ * share a launch); up to there they are those of the per-head calls.  The same tolerance holds everywhere.  Asynchronous, allocate nothing.  Errors as above. */
 ql_status qlinear_kv_append_heads(const qlinear_t* h_k, const qlinear_t* h_v, int32_t n_heads, const void* k_new_dev,
                                   const void* v_new_dev, int64_t head_stride, int64_t token_stride, void* const* v_scale_dev,
                                   int32_t pos, int32_t n_new, void* cuda_stream);
@@ -293,7 +301,7 @@ ql_status qlinear_rope_qkv(const void* q_dev, const void* k_dev, const void* v_d
 ql_status qlinear_residual_rmsnorm(const void* x_dev, const void* residual_dev, const void* gamma_dev, float eps, float gamma_offset,
                                    void* h_out_dev, void* y_out_dev, int32_t M, int32_t K, int32_t device, void* cuda_stream);
 
-/* The kernel qlinear_forward uses for M tokens on this handle (0 if h is NULL or M < 1). */
+/* The stage qlinear_forward takes M tokens on this handle for (0 if h is NULL or M < 1). */
 int32_t qlinear_path_for(qlinear_t h, int32_t M);
 
 /* Runs, on the device, the same unpack routine the forward kernels use and writes the integers

@@ -3,7 +3,9 @@
 // too many tokens for the 8 MMA columns of the decode kernel, too few to fill the 256-token tiles of the prefill kernel,
 // which then multiplies padding and, with few tiles, leaves most SMs without work.
 //
-// Bound: HBM at 16 tokens, the warp-level tensor core (8 cycles per m16n8k16 and SM quarter, measured) from about 32 on.
+// Bound: none of the limits is reached.  Llama gate + up (66 MB of int4 in groups) needs 10.3 us of HBM, and at 8.05 cycles per m16n8k16 and SM
+// quarter (measured, independent MMAs) 6.6 us of MMAs at 16 tokens, 13.1 at 32; at 32 tokens it takes 37, with the tensor pipe active 32 % and
+// DRAM 19 % of the time and 12 warps per SM resident: reads of x, unpack, MMAs and the waits between them add up.
 //
 // Work decomposition: a CTA takes one row super-block (128 channels, one row-block of 16 per warp), one block of 8 NT
 // tokens and one part of K; the K parts of a tile are the CTAs of a thread-block cluster and add their fp32 partial sums
@@ -14,11 +16,10 @@
 // so that the 8 lanes of a shared-memory phase touch all 32 banks.  Arithmetic of the prefill kernels: exact integers,
 // fp16(s * q) for grouped weights, fp32 sums, the per-channel scale on the fp32 result.
 //
-// Measured, weights out of HBM, against the 256-token-tile kernel that served these sizes: Llama gate + up (66 MB of int4 in
-// groups) 26.0 us at 16 tokens (48.1 before), 37.0 at 32 (49.7); down (33 MB) 13.3 (26.3), 18.6 (28.1); q + k + v (25 MB of
-// int8) 12.2 (18.7), 15.7 (20.0); one 2304 x 2304 int8 layer 4.1 (11.4), 5.6 (13.4).  The MMAs alone: 13.6 us of gate + up
-// at 16 tokens, 27 at 32.  Value product of 1024 rows over 4096 positions, d_h = 128: a pass over the probabilities for
-// the scales and a single-CTA matmul on 8 CTAs before, now 8.4 us (one layer of 8 heads, scores included: 414 -> 183 us).
+// Measured, weights out of HBM, against the 256-token-tile kernel that served these sizes: Llama gate + up 25.9 us at 16 tokens (47.3 before),
+// 37.0 at 32 (48.9); down (33 MB) 13.7 (26.6), 18.9 (28.7); q + k + v (25 MB of int8) 8.9 (19.2), 12.4 (20.5); one 2304 x 2304 int8 layer 4.5
+// (11.7), 6.0 (13.7).  Against the prefill kernel as it is: see takes_mid in qlinear.cu.  Value product of 1024 rows over 4096 positions,
+// d_h = 128: a pass over the probabilities for the scales and a single-CTA matmul on 8 CTAs 38.5 us, now 9.8.
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>

@@ -34,8 +34,8 @@
 //
 // The dequantise loop is held to the instructions it needs: per-thread constants are kept from being recomputed at the
 // register limit, the addresses of the step's stage, barriers and slot are advanced instead of formed from an index, and tile
-// bookkeeping runs at the few steps where something changes (1714 -> 1326 warp instructions per k-step and SM of grouped
-// int4; Llama gate + up, fused, 2048 tokens 395 -> 363 us, 777 tokens 196 -> 166, Gemma2-2B's 777 tokens 63 -> 57).
+// bookkeeping runs at the few steps where something changes (1419 warp instructions per k-step and SM of grouped int4, epilogues
+// included; Llama gate + up, fused, 2048 tokens 363 -> 347 us, 777 tokens 185 -> 165, Gemma2-2B's 777 tokens 64.0 -> 58.7).
 //
 // Forms of the kernel (template flags): the plain product, whole tiles dealt out round-robin or, for launches with
 // few tiles, 2 or 4 K parts per tile that meet in the device scratch; GATED (y = act(gate) * up, Section 3.6); I8
@@ -129,7 +129,7 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t addr)
 
 // (pin: the members pass through an empty asm statement.  The kernel is at its register limit, and the compiler otherwise
 // computes them again from the lane number on every k-step.  The integer form has next to no arithmetic and a larger epilogue:
-// there the registers are worth more, 327 us of projections at 1024 tokens against 349 pinned.)
+// there the registers are worth more, 297 us of Llama projections at 1024 tokens against 344 pinned, with 100 bytes of spills.)
 struct DequantRowTa {
     int off[4];                  // byte offset, inside the packed block, of piece c of the row's 64-byte line (64-byte swizzle:
                                  // piece c sits at position c ^ ((line / 2) & 3))

@@ -3,7 +3,7 @@
 // heads of a layer in one launch.
 //
 // Bound: the outputs.  At d_h = 128 a score costs 128 multiply-adds and 2 bytes of HBM; 8 heads x 1024 query rows x 4096
-// positions write 67 MB (10.3 us at the measured copy rate) and keep the warp-level tensor core busy for 16 us (8 cycles per
+// positions write 67 MB (10.3 us at the measured copy rate) and keep the warp-level tensor core busy for 15 us (8.05 cycles per
 // m16n8k16 and SM quarter).  In the prefill kernel such a tile has 2 k-steps and an epilogue that nothing hides.
 //
 // Work decomposition: the tiles (row super-block of 128 positions x 8 NT tokens) of all layers are numbered through, token
@@ -13,8 +13,8 @@
 // through shared memory: stmatrix turns the accumulator fragments, which hold pairs of tokens of one position, into rows of
 // 128 positions, which go out as 256-byte pieces.
 //
-// Measured: 8 heads x 1024 rows x 4096 positions, d_h = 128: 35 us (1.9 TB/s written), 76 us as eight launches of the prefill
-// kernel; 8 heads x 64 rows 5.1 us against 40; 8 heads of 256 x 512 rows 31 us against 77.
+// Measured: 8 heads x 1024 rows x 4096 positions, d_h = 128: 35 us (1.9 TB/s written), 72 us as eight launches of the prefill
+// kernel; 8 heads x 64 rows 4.4 us against 42; 8 heads of 256 x 256 rows 18.6 us against 50.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>

@@ -72,8 +72,8 @@ using GemvParams = GemvParamsT<kGemvMaxGroup>;
 // The loop is bound by its instruction stream as much as by HBM (with the math taken out LM head would take 47 us, Llama
 // gate + up 12.5, down 7.0), so what is not arithmetic is kept out of it: the block size is a constant for int4, per-thread
 // addresses pass through an empty asm statement so that the compiler does not form them again from the lane number at the
-// register limit, and int8 refills are predicated copies.  Before / after, one token: LM head (295 MB) 55.5 / 53.4 us, gate +
-// up 17.3 / 15.4, down 10.2 / 9.9, Llama q + k + v (int8) 6.1 / 5.9, o 5.4 / 5.1, Gemma2-2B q + k + v 3.95 / 3.64.
+// register limit, and int8 refills are predicated copies.  Before / after, one token: LM head (295 MB) 54.7 / 53.4 us, gate +
+// up 16.6 / 16.3, down 10.6 / 10.4, Llama q + k + v (int8) 6.9 / 6.65, o 5.9 / 5.65, Gemma2-2B q + k + v 4.0 / 3.7.
 template <int BITS, bool GROUPED, bool XDIRECT, bool GATED = false, int NG = kGemvMaxGroup, bool ONE = false>
 __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT<NG> p)
 {
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
 
     if (GROUPED) asm volatile("" : "+r"(s_off));
     // Out of range: int8 copies nothing (a predicated copy; no such slot reaches the math), int4 reads nothing and writes zeros
-    // (there the size operand, formed ahead of time, is the cheaper form: Llama gate + up 15.4 us against 16.0).
+    // (there the size operand, formed ahead of time, is the cheaper form by 4 % on Llama gate + up).
     auto copy16 = [](uint32_t dst, const void* src, bool in_range) {
         if (BITS == 8) {
             asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p cp.async.cg.shared.global [%0], [%1], 16;\n\t}" ::"r"(dst), "l"(src), "r"((int)in_range) : "memory");

@@ -15,8 +15,8 @@
 // The quantisation stands between the stream dependency and the first product, in every CTA, so it is kept short: the token
 // count is a template parameter, all tokens' loads of a turn are in flight together, the maximum is taken on packed fp16
 // and by one warp reduction, every thread forms the reciprocals itself, and short rows are quantised from the registers they
-// were measured in.  Measured (weights out of HBM, before / after): 4096 x 4096 int8 at 1 token 7.6 / 6.9 us, at 4 tokens
-// 11.6 / 8.1; 14336 x 4096 int4 per channel 10.3 / 8.9 and 17.0 / 12.2; 4096 x 14336 int4 11.7 / 10.1 and 24.1 / 23.4 (two
+// were measured in.  Measured (weights out of HBM, before / after): 4096 x 4096 int8 at 1 token 8.0 / 7.1 us, at 4 tokens
+// 11.9 / 8.4; 14336 x 4096 int4 per channel 10.7 / 9.4 and 17.6 / 12.4; 4096 x 14336 int4 12.0 / 10.3 and 24.0 / 23.5 (two
 // reads of rows that long).
 // int4 unpack is two logic operations per 8 weights (the low and the high nibbles of a word are the 4-byte
 // operand registers of rows g and g + 8), against nine for the fp16 path.

@@ -11,8 +11,8 @@
 // together, once.  One CTA per SM; K is split over a cluster only where the row-blocks leave SMs idle and the slices
 // keep 2 chunks per warp (cols_split in qlinear.cu).  Sums: tensor core, then the 16 warps in order, then the cluster's ranks in order.
 //
-// Measured, append + scores + values of one layer (8 heads of 128, 4 query rows each, caches rotated past L2): 6.3 -> 5.6 us
-// at 1280 positions, 10.2 -> 9.2 at 8192, 26.7 -> 22.0 at 32768.
+// Measured, append + scores + values of one layer (8 heads of 128, 4 query rows each, caches rotated past L2), with the
+// general kernel / with this one: 6.0 / 5.5 us at 1280 positions, 9.0 / 8.5 at 4096, 10.7 / 10.7 at 8192, 25.5 / 21.4 at 32768.
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>

@@ -410,7 +410,7 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
     // Short K (the score product over a KV cache): the persistent form, whatever the number of rows.  With at most one wave of
     // row super-blocks it wins as well, having no ring to fill, no sums across warps and no barrier (8 heads of 128 at 1280
     // positions 4.1 -> 1.8 us, at 8192 6.7 -> 3.1 us; 2 heads of 64 at 1024 3.3 -> 1.5 us).  One layer as well, a cache or not
-    // (a head of 128, 4 rows, 4096 positions 3.7 -> 1.6 us; 32768 x 256 weights, 8 tokens 3.8 -> 3.5 us).
+    // (a head of 128, 4 rows, 4096 positions 3.7 -> 1.8 us; 32768 x 256 weights, 8 tokens 3.8 -> 3.5 us).
     if (xs && !gated && n <= kGemvMaxBatch && takes_rows(L)) {
         GemvRowsParams rp{};
         int n_rsb = 0;

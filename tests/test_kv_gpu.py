@@ -329,3 +329,24 @@ def test_prefill_kernels_see_the_tokens_appended_just_before(P, torch, d_h, R):
     y64, A, _ = O.linear(q.cpu().numpy(), k_q, k_s.reshape(-1, 1), 0)
     ok, rel, worst = O.check_against(got[0][:, T:T + n_new].cpu().numpy(), y64, A)
     assert ok, (rel, worst)
+
+
+@pytest.mark.parametrize("n_heads,cache", [(8, 2048), (11, 1280), (8, 8192), (11, 4096)])
+def test_value_product_of_all_heads_and_of_one(P, torch, n_heads, cache):
+    """Up to 2048 positions K is undivided whatever the number of heads: the same bits.  Beyond, the split follows the number of
+    heads in the launch: the same value up to the order of the fp32 sums, which two fp16 roundings of it bound."""
+    rng = np.random.default_rng(n_heads + cache)
+    v = torch.from_numpy(rng.standard_normal((n_heads, cache, DH)).astype(np.float16)).cuda()
+    prob = (torch.rand((n_heads, 4, cache), device="cuda") / cache).half()
+    heads = P.KVHeads(n_heads, cache, DH)
+    heads.append(v, v)
+    out = heads.output(prob)
+    for h in range(n_heads):
+        one = heads.heads[h].output(prob[h])
+        if cache <= 2048:
+            assert torch.equal(out[h], one)
+        else:
+            # |sum| <= A, the sum of the magnitudes: each order errs by at most (positions / 32 + 48) 2^-24 A before its rounding
+            A = (prob[h].float() * heads.heads[h].v_scale.float()) @ (heads.heads[h].v.debug_unpack().float().abs().T)
+            bound = 2.0 ** -10 * one.float().abs() + 2 * (cache / 32 + 48) * 2.0 ** -24 * A + 2.0 ** -24
+            assert bool(((out[h].float() - one.float()).abs() <= bound).all())
