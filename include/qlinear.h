@@ -156,8 +156,8 @@ typedef enum { QL_ACT_IDENTITY = 0, QL_ACT_SILU = 1, QL_ACT_GELU_TANH = 2 } ql_a
  *     y[m,n] = fp16( act(gate[m,n]) * up[m,n] ),   gate = x . W_gate^T,  up = x . W_up^T   (both in fp32)
  * with act = identity, SiLU g / (1 + exp(-g)) (the Llama family) or the tanh form of GELU (the Gemma family);
  * the paper names no activation.  Neither projection is written to memory: for M <= 8 one decode launch
- * holds both branches of every output channel in the same CTA, and so does one launch of the batch kernel for the token counts and
- * weights (of both layers) stated at qlinear_forward; for M > 128 (and layers of a multiple of 256
+ * holds both branches of every output channel in the same CTA, and so does one launch of the batch kernel for up to 32 tokens, and for up to
+ * 64 where the two layers have at most 48 million weights; for M > 128 (and layers of a multiple of 256
  * channels after padding to 128) the CTA-pair prefill kernel keeps the two projections of a tile in its two
  * tensor-memory accumulators and the epilogue writes only their product, which halves the write-back.
  * Shapes outside those cases (up to 128 tokens of more weights than the batch kernel takes, other channel counts at more tokens, K not a
@@ -373,7 +373,7 @@ uint32_t qlinear_version(void);
  * this process (1 after the first call, for good).  qlinear_debug_plan_kv_output does for the (first) launch of
  * qlinear_kv_output_heads over n_heads caches like h_v what qlinear_debug_plan does for the other decode launches: {CTAs per
  * cluster, chunks per warp, clusters of the launch, clusters that run at once}.  qlinear_debug_takes_batch_kernel returns 1 if a
- * forward call (n = 1), a group or a gated pair (n = 2) of these layers on M tokens runs on the kernel for a batch of tokens. */
+ * forward call (n = 1) or a group of these layers on M tokens runs on the kernel for a batch of tokens. */
 int32_t qlinear_debug_plan(qlinear_t h, int32_t M, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_plan_kv_output(qlinear_t h_v, int32_t n_heads, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_takes_batch_kernel(const qlinear_t* hs, int32_t n, int32_t M);

@@ -471,7 +471,7 @@ cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pd
 }
 
 // Which launches take this kernel: up to 32 tokens all of them, up to 48 those with at most 48 million weights, up to 64 those with at most
-// 30 million (int8: 24).  Beyond, its MMAs take longer than the prefill kernel, whose tiles of these widths cost the same dequantisation
+// 30 million (int8: 24) or, gated, 48 million (the other route is a group launch into the shared scratch and a pass over it).  Beyond, its MMAs take longer than the prefill kernel, whose tiles of these widths cost the same dequantisation
 // whatever M is.  Measured, us this kernel / the prefill kernel, int4 in groups (int8: 3 to 12 % less in its favour):
 //   weights                     32 tokens    48           64
 //     9 M (Gemma2-2B q + k + v)  6.8 / 11.4   8.7 / 13.8  11.1 / 15.6
@@ -482,13 +482,13 @@ cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pd
 //    59 M (Llama down)          18.8 / 23.1  24.3 / 25.8  30.0 / 27.9     (14336 x 4096: 20.2 / 21.8, 26.3 / 22.1, 32.2 / 22.2)
 //   117 M (Llama gate + up)     36.9 / 42.1  47.7 / 43.1  59.0 / 43.8
 // QLINEAR_MID_MAX_M lowers the number of tokens up to which this holds (0: never).
-bool takes_mid(const qlinear_s* const* hs, int n, int M)
+bool takes_mid(const qlinear_s* const* hs, int n, int M, bool gated = false)
 {
     if (M > 64 || M > config().mid_max_m) return false;
     if (M <= 32) return true;
     int64_t weights = 0;
     for (int i = 0; i < n; ++i) weights += (int64_t)hs[i]->L.N * hs[i]->L.K;
-    return weights <= (M <= 48 ? 48000000 : hs[0]->L.bits == 4 ? 30000000 : 24000000);
+    return weights <= (M <= 48 || gated ? 48000000 : hs[0]->L.bits == 4 ? 30000000 : 24000000);
 }
 
 template <int BITS, bool GROUPED, bool GATED, bool KSCALE = false>
@@ -913,7 +913,7 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
         void* ys[2] = {y, y};
         const ql_status s = forward_gemv(hs, 2, x, ys, M, st, act);
         if (s != QL_ERR_UNSUPPORTED) return s;
-    } else if (M > hg->gemv_max_m && takes_mid(hs, 2, M)) {
+    } else if (M > hg->gemv_max_m && takes_mid(hs, 2, M, true)) {
         const void* xs[2] = {x, x};
         return forward_mid(hs, 2, xs, &y, M, st, act);
     } else if (M > hg->gemv_max_m && gemm_pair_applicable(a, M)) {       // prefill: both accumulators of the CTA-pair kernel

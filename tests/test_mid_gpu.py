@@ -147,3 +147,25 @@ def test_lines_between_the_batch_kernel_and_the_prefill_kernel(P, torch, N, K, b
     y64, A, _ = O.linear(x, q[rows], s[rows], group)
     ok, rel, worst = O.check_against(y.cpu().numpy()[:, rows], y64, A)
     assert ok, (rel, worst)
+
+
+def test_gated_pair_between_the_lines_needs_no_scratch(P, torch):
+    """64 tokens, 38 million weights: a forward call of that size is the prefill kernel's, the gated pair stays one launch of the
+    batch kernel: gated calls on two streams that are not ordered against each other, which may not share the device scratch."""
+    layer = spec(8192, 2304, 4, 32)
+    w = [C.layer_weights(6700 + i, layer) for i in range(2)]
+    gate, up = (P.QLinear.from_weights(q, s, 4, 32, device="cuda:0") for q, s in w)
+    xs = [torch.from_numpy(C.layer_activations(6700 + i, layer, 64)).cuda() for i in range(2)]
+    first = [P.qlinear_forward_gated(gate, up, x, "silu") for x in xs]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs = [torch.empty_like(f) for f in first]
+    torch.cuda.synchronize()
+    for _ in range(50):
+        for x, o, st in zip(xs, outs, streams):
+            P.qlinear_forward_gated(gate, up, x, "silu", out=o, stream=st)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(first, outs)) and gate.device_status() == (0, 0)
+    rows = np.r_[0:64, 8128:8192]
+    g64, bound, _ = O.gated_linear(xs[0].cpu().numpy(), w[0][0][rows], w[0][1][rows], w[1][0][rows], w[1][1][rows], 32, "silu")
+    ok, rel, worst = O.check_gated(first[0].cpu().numpy()[:, rows], g64, bound)
+    assert ok, (rel, worst)
