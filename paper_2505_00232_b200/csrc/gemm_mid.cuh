@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kMidThreads, 2) gemm_mid_kernel(const MidParam
     using S = MidSmem<BITS, GROUPED, NT>;
     constexpr int NS = S::kStages, CHUNK_K = BITS == 4 ? 64 : 32, BB = kWeightBlockBytes + (GROUPED ? kScaleBlockBytes : 0);
     constexpr int UNITS = S::kKStep / 8;                                 // 16-byte pieces of a token's stage
-    extern __shared__ __align__(128) unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, c = lane & 3;
 

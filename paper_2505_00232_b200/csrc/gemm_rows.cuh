@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256, 2) gemm_rows_kernel(const GemmRowsParams 
     using S = GemmRowsSmem<NKC, NT>;
     constexpr int UNITS = NKC * 4;                                       // 16-byte pieces of a token
     constexpr int K = 32 * NKC;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(smem_raw), out0 = smem0 + 2 * S::kXBytes;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, c = lane & 3;
     const int i0 = (int)((int64_t)blockIdx.x * p.n_tiles / gridDim.x), i1 = (int)((int64_t)(blockIdx.x + 1) * p.n_tiles / gridDim.x);

@@ -119,7 +119,6 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_kernel(const GemvParamsT
     static_assert(kGemvRing == 8, "one scale copy per lane covers exactly 8 chunks");
     constexpr int WARP_SMEM = kGemvRing * 512 + (GROUPED ? 2 * 512 : 0);
     unsigned char* ring = smem_raw + p.x_bytes + warp * WARP_SMEM;
-    unsigned char* sbuf = ring + kGemvRing * 512;
     uint32_t ring_u32 = (uint32_t)__cvta_generic_to_shared(ring) + lane * 16;
     if (BITS == 4) asm volatile("" : "+r"(ring_u32));
     const uint32_t sbuf_u32 = ring_u32 + kGemvRing * 512;
