@@ -111,10 +111,11 @@ ql_status qlinear_create(const qlinear_desc* desc, const void* packed_dev, int d
  *   x_dev  device, fp16 [M, K] row-major contiguous, 16-byte aligned, read-only during the call.
  *   y_dev  device, fp16 [M, N] row-major contiguous, 16-byte aligned, must not overlap x_dev.
  * Asynchronous: returns after the launch; allocates nothing; never synchronises.  M <= 8 runs the
- * decode kernel, larger M a matrix-multiply kernel (Section 3.7; qlinear_path_for): the kernel for a batch of tokens up to
- * 32 tokens, up to 48 for layers (or groups) of at most 48 million weights and up to 64 for at most 30 million (int8: 24), the
- * prefill kernel beyond.  The environment variable QLINEAR_MID_MAX_M lowers the token count up to which the batch kernel is used (0:
- * never).  int8 layers of K = 64, 128 or 256 have kernels of their own, for M <= 8 and for any larger M.
+ * decode kernel, larger M a matrix-multiply kernel (Section 3.7; qlinear_path_for): up to 64 tokens, and on layers too small to
+ * fill the prefill kernel's tiles beyond, a kernel for a batch of tokens (one with warp-level MMAs for few weights, one with the
+ * weights in tensor memory for more), else the prefill kernel.  The environment variable QLINEAR_MID_MAX_M lowers the token count from
+ * which calls of up to 64 tokens go to the prefill kernel (0: all of them).  int8 layers of K = 64, 128 or 256 have kernels of
+ * their own, for M <= 8 and for any larger M.
  * Errors: QL_ERR_INVALID_ARG (null / misaligned pointers, M < 1, M*K or M*N beyond 2^31-1 elements),
  * QL_ERR_CUDA (launch failure, reported synchronously), QL_ERR_DEVICE_TIMEOUT (an earlier kernel of this
  * library on the handle's DEVICE gave up a bounded wait: its output is invalid; nothing is launched, and every
@@ -130,7 +131,7 @@ ql_status qlinear_forward(qlinear_t h, const void* x_dev, void* y_dev, int32_t M
  * the same reason: launch overhead and memory-bound work).  Every output is bit-identical to what
  * qlinear_forward gives for that layer only if the K split chosen for the group equals the layer's own;
  * it always meets the same tolerance, and is run-to-run deterministic.  For larger M the layers share
- * one launch of the batch kernel (sizes: qlinear_forward), or one launch of the prefill kernel when every layer qualifies for its
+ * one launch of a batch kernel (sizes: qlinear_forward), or one launch of the prefill kernel when every layer qualifies for its
  * CTA-pair form (a multiple of 256 output channels after padding to 128); the tiles of all layers then
  * fill the persistent grid together.  Otherwise they run one after the other.
  *   hs      host array of n handles; ys_dev host array of n device pointers (fp16 [M, N_i], 16-byte
@@ -156,11 +157,11 @@ typedef enum { QL_ACT_IDENTITY = 0, QL_ACT_SILU = 1, QL_ACT_GELU_TANH = 2 } ql_a
  *     y[m,n] = fp16( act(gate[m,n]) * up[m,n] ),   gate = x . W_gate^T,  up = x . W_up^T   (both in fp32)
  * with act = identity, SiLU g / (1 + exp(-g)) (the Llama family) or the tanh form of GELU (the Gemma family);
  * the paper names no activation.  Neither projection is written to memory: for M <= 8 one decode launch
- * holds both branches of every output channel in the same CTA, and so does one launch of the batch kernel for up to 32 tokens, and for up to
- * 64 where the two layers have at most 48 million weights; for M > 128 (and layers of a multiple of 256
+ * holds both branches of every output channel in the same CTA, and so does one launch of a batch kernel for up to 64 tokens, and beyond on
+ * layers too small to fill the prefill kernel's tiles; for larger M (and layers of a multiple of 256
  * channels after padding to 128) the CTA-pair prefill kernel keeps the two projections of a tile in its two
  * tensor-memory accumulators and the epilogue writes only their product, which halves the write-back.
- * Shapes outside those cases (up to 128 tokens of more weights than the batch kernel takes, other channel counts at more tokens, K not a
+ * Shapes outside those cases (65 to 128 tokens of many weights, other channel counts at more tokens, K not a
  * multiple of the decode chunk at M <= 8) run the two projections into the device's shared scratch and a small element-wise kernel after them: same
  * result, no saving; such calls must be ordered against K-split prefill calls like those among themselves.
  *   h_gate, h_up  two layers on one device with the same N, K, bits and group
@@ -373,7 +374,8 @@ uint32_t qlinear_version(void);
  * this process (1 after the first call, for good).  qlinear_debug_plan_kv_output does for the (first) launch of
  * qlinear_kv_output_heads over n_heads caches like h_v what qlinear_debug_plan does for the other decode launches: {CTAs per
  * cluster, chunks per warp, clusters of the launch, clusters that run at once}.  qlinear_debug_takes_batch_kernel returns 1 if a
- * forward call (n = 1) or a group of these layers on M tokens runs on the kernel for a batch of tokens. */
+ * forward call (n = 1) or a group of these layers on M tokens belongs to the batch stage by its size (calls beyond it belong to the
+ * prefill stage, whose choice of kernel includes the batch kernel with the weights in tensor memory). */
 int32_t qlinear_debug_plan(qlinear_t h, int32_t M, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_plan_kv_output(qlinear_t h_v, int32_t n_heads, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_takes_batch_kernel(const qlinear_t* hs, int32_t n, int32_t M);

@@ -87,14 +87,13 @@ struct TaMaps {
 };
 
 // The packed body of a layer as a 2-D tensor of 64-byte rows; box = the block(s) of one 64-k step.
-// i8: the integer form's box (128 k: two int4 blocks or four int8 blocks; per-channel schemes only).
-inline bool w_tensor_map(const Layout& L, const uint8_t* blob, CUtensorMap* out, bool i8 = false)
+// wide: the box of a 128-k step (two int4 blocks or four int8 blocks): the integer form and gemm_narrow.cuh.
+inline bool w_tensor_map(const Layout& L, const uint8_t* blob, CUtensorMap* out, bool wide = false)
 {
     EncodeTiledFn enc = get_encode_tiled();
     if (!enc) return false;
-    if (i8 && L.grouped) return false;
     const int64_t rows = (int64_t)L.n_rsb * L.n_kc * (L.block_bytes / 64);
-    const int box_rows = (i8 ? 2 : 1) * (L.bits == 4 ? L.block_bytes / 64 : 2 * (kWeightBlockBytes / 64));
+    const int box_rows = (wide ? 2 : 1) * (L.bits == 4 ? L.block_bytes / 64 : 2 * (kWeightBlockBytes / 64));
     if (rows < box_rows || rows > 0x7FFFFFFFll) return false;
     const cuuint64_t gdim[2] = {64, (cuuint64_t)rows};
     const cuuint64_t gstr[1] = {64};

@@ -35,6 +35,7 @@ __device__ unsigned int* g_status_host;
 #include "gemm_rows.cuh"
 #include "gemm_pair.cuh"
 #include "gemm_pair_ta.cuh"
+#include "gemm_narrow.cuh"
 #include "norm.cuh"
 #include "rope.cuh"
 
@@ -55,7 +56,7 @@ struct Config {
     int warps_per_sm;        // QLINEAR_GEMV_WARPS_PER_SM: residency target of the cluster decode kernel
     bool oversubscribe;      // QLINEAR_GEMV_OVERSUBSCRIBE=0: the group-scaled int4 decode kernel never takes more CTAs than fit at once
     int force_ks;            // QLINEAR_GEMV_KS: forced K split of the cluster decode kernel (0 = planned)
-    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M of a forward call that the kernel for a batch of tokens may serve (0: none; at most 64); see takes_mid
+    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M up to 64 that the kernels for a batch of tokens may serve (0: none); see takes_mid, narrow_is_faster
     bool xdirect;            // QLINEAR_GEMV_XDIRECT: x fragments straight from global memory
     int kernel;              // QLINEAR_GEMV_KERNEL: 0 / 1 cluster kernel (default), 2 streaming kernel
     int stream_ctas_per_sm, stream_stages;
@@ -140,8 +141,8 @@ struct qlinear_s {
     bool use_stream;
     int stream_P, stream_stages;
     CUtensorMap wmap;          // the packed body as rows of 64 bytes (prefill kernel with the weights in tensor memory)
-    CUtensorMap wmap_i8;       // the same with the integer form's box (128 k per step)
-    bool wmap_ok, wmap_i8_ok;
+    CUtensorMap wmap_wide;     // the same with a box of 128 k per step (the integer form, gemm_narrow.cuh)
+    bool wmap_ok, wmap_wide_ok;
     DeviceState* dev;
     // Set by the first append: the blob is a KV cache, and the kernel before a reader in the stream may be writing it.  Its readers
     // then touch it only after griddepcontrol.wait (`late` in their parameters), or are launched without the programmatic edge
@@ -447,6 +448,144 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
+template <int BITS, bool GROUPED, bool GATED, int G>
+cudaError_t launch_narrow_g(const qlinear_s* h, const NarrowMaps& maps, const NarrowParams& prm, int grid, cudaStream_t st)
+{
+    static std::atomic<bool> attr_set[kMaxDevices];
+    auto kern = gemm_narrow_kernel<BITS, GROUPED, GATED, G>;
+    cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, kNarrowSmem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(narrow_threads(G));
+    cfg.dynamicSmemBytes = kNarrowSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attrs[2];
+    int na = 0;
+    if (prm.cl > 1) {
+        attrs[na].id = cudaLaunchAttributeClusterDimension;
+        attrs[na].val.clusterDim.x = prm.cl;
+        attrs[na].val.clusterDim.y = attrs[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    if (h->pdl) {
+        attrs[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attrs[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
+    cfg.attrs = attrs;
+    cfg.numAttrs = na;
+    return cudaLaunchKernelEx(&cfg, kern, maps, prm);
+}
+
+template <int BITS, bool GROUPED, bool GATED>
+cudaError_t launch_narrow(const qlinear_s* h, const NarrowMaps& maps, const NarrowParams& prm, int grid, cudaStream_t st)
+{
+    // three groups where the accumulators leave tensor memory for their slots; int8 unpacks faster and has 16 KB stages: two
+    if constexpr (BITS == 4)
+        if (prm.bn <= 32) return launch_narrow_g<BITS, GROUPED, GATED, 3>(h, maps, prm, grid, st);
+    return launch_narrow_g<BITS, GROUPED, GATED, 2>(h, maps, prm, grid, st);
+}
+
+// Token blocks and K parts of a launch of gemm_narrow.cuh over `rows` row super-blocks, and the microseconds of its busiest SM.  A CTA
+// alone on its SM takes 0.5 per weight tile of 128 k, two take 0.62 each; clusters of 4 and 8 lie inside a GPC, so fewer fit than the
+// SMs alone would hold; ramps as measured (within 10 % over the shapes named in gemm_narrow.cuh, 9 to 512 tokens).
+struct NarrowPlan { int n_tb, bn, cl; double us; };
+NarrowPlan plan_narrow(const Layout& L, int rows, bool gated, int M, int num_sms)
+{
+    NarrowPlan pl{};
+    pl.n_tb = (M + 63) / 64;
+    pl.bn = ((M + pl.n_tb - 1) / pl.n_tb + 15) / 16 * 16;
+    const int64_t tiles = (int64_t)rows * pl.n_tb;
+    const int n_steps = (L.K + kNarrowKStep - 1) / kNarrowKStep;
+    pl.us = 1e30;
+    for (int i = 0; i < 4 && (1 << i) <= n_steps; ++i) {
+        static const double ramp[4] = {3.5, 3.8, 4.0, 4.3}, fit1[4] = {1.0, 1.0, 0.89, 0.81}, fit2[4] = {1.0, 1.0, 0.92, 0.87};
+        const int cl = 1 << i, n = (n_steps * (gated ? 2 : 1) + cl - 1) / cl;
+        const double alone = fit1[i] * num_sms / cl, pair = 2 * fit2[i] * num_sms / cl;
+        const double us = tiles <= alone ? ramp[i] + 0.5 * n : std::ceil(tiles / pair) * (ramp[i] + 1.3 + 0.62 * n);
+        if (us < pl.us) { pl.us = us; pl.cl = cl; }
+    }
+    return pl;
+}
+
+// n layers that share x, K and scheme; act >= 0: the gated form (n == 2, equal shapes, ys[0] the output).
+ql_status forward_narrow(const qlinear_s* const* hs, int n, const void* x, void* const* ys, int M, cudaStream_t st, int act = -1)
+{
+    const qlinear_s* h = hs[0];
+    const Layout& L = h->L;
+    const bool gated = act >= 0;
+    NarrowMaps maps;
+    NarrowParams prm{};
+    int units = 0;
+    for (int i = 0; i < kGemmMaxGroup; ++i) maps.w[i] = hs[i < n ? i : 0]->wmap_wide;
+    for (int i = 0; i < n; ++i) {
+        const Layout& Li = hs[i]->L;
+        prm.chan_scales[i] = Li.grouped ? nullptr : reinterpret_cast<const __half*>(hs[i]->blob + Li.chan_scale_offset);
+        prm.y[i] = static_cast<__half*>(ys[gated ? 0 : i]);
+        prm.N[i] = Li.N;
+        units += Li.n_rsb;
+        prm.unit_end[i] = units;
+    }
+    if (gated) units = L.n_rsb;
+    const NarrowPlan pl = plan_narrow(L, units, gated, M, h->num_sms);
+    prm.n_tb = pl.n_tb; prm.bn = pl.bn; prm.cl = pl.cl;
+    prm.n_layers = n; prm.M = M; prm.K = L.K; prm.n_kc = L.n_kc; prm.w_rows = L.block_bytes / 64; prm.act = gated ? act : 0;
+    prm.n_steps = (L.K + kNarrowKStep - 1) / kNarrowKStep;
+    prm.late = any_cache(hs, n);
+    // Ring lengths: weight stages a multiple of the groups; x stages even where every stage feeds one issuer (see the kernel).
+    prm.nw = L.bits == 4 && prm.bn <= 48 ? 6 : 4;
+    prm.nx = std::min(kNarrowMaxX, (kNarrowRing - prm.nw * (L.bits == 4 ? 2 : 4) * L.block_bytes) / (prm.bn * 256));
+    if (!gated) prm.nx &= ~1;
+    prm.a_col = (2 * prm.bn + 31) / 32 * 32;
+    if (!x_tensor_map(x, L.K, M, prm.bn, &maps.x)) return QL_ERR_CUDA;
+    const int grid = units * prm.n_tb * prm.cl;
+    cudaError_t e;
+    if (gated) e = L.bits == 8 ? launch_narrow<8, false, true>(h, maps, prm, grid, st) : L.grouped ? launch_narrow<4, true, true>(h, maps, prm, grid, st) : launch_narrow<4, false, true>(h, maps, prm, grid, st);
+    else e = L.bits == 8 ? launch_narrow<8, false, false>(h, maps, prm, grid, st) : L.grouped ? launch_narrow<4, true, false>(h, maps, prm, grid, st) : launch_narrow<4, false, false>(h, maps, prm, grid, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
+// Microseconds of the prefill kernels on n layers in one launch (one launch each where a layer's row super-blocks are odd), within 15 % of
+// what was measured at 65 to 512 tokens: 0.30 to 0.36 per 64-k step and tile of up to 256 tokens, 3 per tile, 10 for a K split that meets in
+// the scratch; the single-CTA kernel 0.6 per step; the gated form on the shared-memory kernel 0.55 per step.
+double prefill_us(const qlinear_s* const* hs, int n, int M, bool gated, int num_sms)
+{
+    const Layout& L = hs[0]->L;
+    const int mblk = (M + 255) / 256, steps = (L.K + 63) / 64, clusters = num_sms / 2;
+    const double bn = (double)M / mblk;
+    int rsb = 0;
+    bool even = true;
+    for (int i = 0; i < n; ++i) { rsb += hs[i]->L.n_rsb; even = even && hs[i]->L.n_rsb % 2 == 0; }
+    if (!even) {
+        double us = 0.0;
+        for (int i = 0; i < n; ++i) us += std::ceil((double)hs[i]->L.n_rsb * mblk / num_sms) * (0.6 * steps + 3.0);
+        return us + (gated ? 3.0 : 0.0);
+    }
+    const int tiles = rsb / 2 * mblk, split = gemm_pair_ta_split(tiles, steps, num_sms, true);
+    const double rounds = std::max(1.0, std::min(std::ceil((double)tiles * split / clusters), (double)tiles * split / clusters + 0.3));
+    const double us = rounds * (steps * (0.3 + 0.00025 * bn) / split + 3.0) + (split > 1 ? 10.0 : 0.0);
+    if (!gated) return us;
+    const int positions = rsb / 4 * mblk;
+    if (M > 128 && positions < clusters) return std::ceil((double)positions / clusters) * (1.1 * steps + 3.0);
+    return us + (M > 128 ? 0.0 : 3.0);
+}
+
+// Whether a call of the prefill stage (or, up to 64 tokens, one that takes_mid leaves to it) runs on gemm_narrow.cuh: by the estimates of
+// both, which lie within 15 % of the times in gemm_narrow.cuh's header; hence 10 % in favour of the prefill kernels.
+// (QLINEAR_MID_MAX_M < M <= 64: the prefill kernels, whatever the estimate.)
+bool narrow_is_faster(const qlinear_s* const* hs, int n, int M, bool gated = false)
+{
+    if (M <= 64 && M > config().mid_max_m) return false;
+    int rows = 0;
+    for (int i = 0; i < n; ++i) {
+        if (!hs[i]->wmap_wide_ok) return false;
+        rows += hs[i]->L.n_rsb;
+    }
+    return plan_narrow(hs[0]->L, gated ? hs[0]->L.n_rsb : rows, gated, M, hs[0]->num_sms).us < 0.9 * prefill_us(hs, n, M, gated, hs[0]->num_sms);
+}
+
 template <int BITS, bool GROUPED, int NT, bool GATED, bool KSCALE>
 cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pdl, cudaStream_t st)
 {
@@ -470,17 +609,11 @@ cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pd
     return launch(kern, prm, dim3((unsigned)(tiles * prm.cl)), dim3(kMidThreads), S::kTotal, st, prm.cl, pdl);
 }
 
-// Which launches take this kernel: up to 32 tokens all of them, up to 48 those with at most 48 million weights, up to 64 those with at most
-// 30 million (int8: 24) or, gated, 48 million (the other route is a group launch into the shared scratch and a pass over it).  Beyond, its MMAs take longer than the prefill kernel, whose tiles of these widths cost the same dequantisation
-// whatever M is.  Measured, us this kernel / the prefill kernel, int4 in groups (int8: 3 to 12 % less in its favour):
-//   weights                     32 tokens    48           64
-//     9 M (Gemma2-2B q + k + v)  6.8 / 11.4   8.7 / 13.8  11.1 / 15.6
-//    21 M (its down)            12.7 / 16.7  16.7 / 19.3  20.9 / 21.4
-//    25 M (Llama q + k + v)     11.9 / 15.5  15.4 / 17.4  18.3 / 18.7     (int8 12.4 / 15.2, 16.8 / 16.9, 19.8 / 18.2)
-//    34 M (32768 x 1024)        11.1 / 15.4  14.5 / 15.8  17.5 / 15.9
-//    42 M (its gate + up)       13.1 / 18.7  16.5 / 19.0  19.6 / 19.6
-//    59 M (Llama down)          18.8 / 23.1  24.3 / 25.8  30.0 / 27.9     (14336 x 4096: 20.2 / 21.8, 26.3 / 22.1, 32.2 / 22.2)
-//   117 M (Llama gate + up)     36.9 / 42.1  47.7 / 43.1  59.0 / 43.8
+// Which launches are the batch stage's: up to 32 tokens all of them, up to 48 those with at most 48 million weights, up to 64 those with at
+// most 30 million (int8: 24) or, gated, 48 million.  The stage has two kernels (batch_takes_narrow); a launch beyond the line goes to the
+// prefill stage, where narrow_is_faster compares gemm_narrow.cuh with the prefill kernels.  At 64 tokens that is the same kernel on
+// both sides of the line (Llama gate + up 26 us there, 44 on the prefill kernel); the line itself is where gemm_mid.cuh and the prefill
+// kernel are even (21 M weights at 64 tokens 20.9 / 21.4, 34 M 17.5 / 15.9, 59 M at 48 tokens 24.3 / 25.8, 14336 x 4096 26.3 / 22.1).
 // QLINEAR_MID_MAX_M lowers the number of tokens up to which this holds (0: never).
 bool takes_mid(const qlinear_s* const* hs, int n, int M, bool gated = false)
 {
@@ -503,13 +636,38 @@ cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, bool pdl, 
     return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
 }
 
-// n layers that share K and scheme, layer i on xs[i]; act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
+// Calls of the batch stage that run on gemm_narrow.cuh: from a number of weights on (of the whole launch) that falls with the number of
+// tokens, because the warp-level MMAs of gemm_mid.cuh cost in proportion to the tokens and the other kernel has the longer ramp.  Measured,
+// us gemm_mid.cuh / gemm_narrow.cuh:
+//   weights                        16 tokens     24           32           48           64
+//     0.3 M (512 x 512)             2.8 /  3.7   3.0 /  3.8   3.3 /  4.0   3.8 /  4.2   4.1 /  4.5
+//     1 M (1024 x 1024, int8)       3.2 /  4.3   3.5 /  4.5   4.0 /  4.6   4.6 /  5.0   5.2 /  5.3
+//     5 M (gated 2688 x 1024)       4.1 /  5.1   4.7 /  5.5   5.5 /  5.8   7.1 /  6.8   8.5 /  7.6
+//     9 M (Gemma2-2B q + k + v)     5.0 /  5.8   5.8 /  6.3   6.9 /  6.4   8.9 /  7.3  10.5 /  7.9
+//    21 M (its down)                8.9 /  8.9  11.2 /  9.3  12.8 /  9.6  16.7 / 10.2  20.9 / 11.5
+//    25 M (Llama q + k + v)         8.8 /  9.1  10.8 /  9.4  12.3 /  9.6  16.7 / 11.4
+//    42 M (Gemma2-2B gate + up)     9.4 / 12.4  11.6 / 12.7  13.2 / 13.6  16.6 / 14.6  19.7 / 14.8
+//    59 M (Llama down)             13.8 / 13.5  16.6 / 14.0  18.9 / 14.3
+//   117 M (Llama gate + up)        26.0 / 22.7  31.9 / 23.2  37.0 / 23.6
+bool batch_takes_narrow(const qlinear_s* const* hs, int n, int M, bool gated)
+{
+    int64_t weights = 0;
+    for (int i = 0; i < n; ++i) {
+        if (!hs[i]->wmap_wide_ok) return false;
+        weights += (int64_t)hs[i]->L.N * hs[i]->L.K;
+    }
+    return weights >= (M <= 16 ? 50000000 : M <= 24 ? (gated ? 50000000 : 20000000) : M <= 32 ? (gated ? 50000000 : 8000000) : M <= 48 ? 4000000 : 1500000);
+}
+
+// n layers that share K and scheme, layer i on xs[i] (one x for all of them on gemm_narrow.cuh, as in every call but the value product);
+// act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
 // kscales != nullptr (int8 layers): layer i's input is multiplied by kscales[i][0 .. K).
 ql_status forward_mid(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st, int act = -1,
                       const void* const* kscales = nullptr)
 {
     const qlinear_s* h = hs[0];
     const Layout& L = h->L;
+    if (!kscales && batch_takes_narrow(hs, n, M, act >= 0)) return forward_narrow(hs, n, xs[0], ys, M, st, act);
     MidParams prm{};
     int units = 0;
     for (int i = 0; i < n; ++i) {
@@ -761,7 +919,7 @@ extern "C" ql_status qlinear_create(const qlinear_desc* d, const void* packed_de
     h->pdl = cfg.pdl;
     h->n_rb = (L.N + kRbRows - 1) / kRbRows;
     h->wmap_ok = w_tensor_map(L, h->blob, &h->wmap);
-    h->wmap_i8_ok = !L.grouped && (L.K % 128) == 0 && w_tensor_map(L, h->blob, &h->wmap_i8, true);
+    h->wmap_wide_ok = w_tensor_map(L, h->blob, &h->wmap_wide, true);
     for (int M = 1; M <= 8; ++M) {
         h->gemv[M] = plan_gemv(L, h->n_rb, M, sms);
         if (h->gemv[M].grid <= 0 && M <= h->gemv_max_m) { delete h; return QL_ERR_UNSUPPORTED; }   // no decode plan fits this shape
@@ -809,6 +967,7 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
     }
     if (takes_rows(h->L)) return forward_gemm_rows(&h, 1, &x, &y, M, st);
     if (takes_mid(&h, 1, M)) return forward_mid(&h, 1, &x, &y, M, st);
+    if (narrow_is_faster(&h, 1, M)) return forward_narrow(&h, 1, x, &y, M, st);
     {
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_ok ? &h->wmap : nullptr;
@@ -842,6 +1001,11 @@ extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const
         const void* xs[kGemvMaxGroup];
         for (int i = 0; i < n; ++i) xs[i] = x;
         return forward_mid(const_cast<const qlinear_s* const*>(hs), n, xs, ys, M, static_cast<cudaStream_t>(stream));
+    }
+    if (n > 1 && M > hs[0]->gemv_max_m && narrow_is_faster(hs, n, M)) {
+        DeviceGuard guard(hs[0]->device);
+        if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
+        return forward_narrow(const_cast<const qlinear_s* const*>(hs), n, x, ys, M, static_cast<cudaStream_t>(stream));
     }
     if (n > 1 && M > hs[0]->gemv_max_m) {                                // prefill: one launch of the CTA-pair kernel
         bool pair_ok = true;
@@ -909,6 +1073,9 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
     if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     qlinear_s* hs[2] = {hg, hu};
+    // the unfused route's product of this size fits the scratch (where it does not, only the fused kernels of the prefill stage serve the call)
+    const int64_t n = (int64_t)M * a.N;
+    const bool fits = (size_t)n * 2 * sizeof(__half) <= gemm_pair_scratch_bytes(hg->num_sms);
     if (M <= hg->gemv_max_m && !hg->use_stream) {                        // decode: both branches in one launch
         void* ys[2] = {y, y};
         const ql_status s = forward_gemv(hs, 2, x, ys, M, st, act);
@@ -916,6 +1083,9 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
     } else if (M > hg->gemv_max_m && takes_mid(hs, 2, M, true)) {
         const void* xs[2] = {x, x};
         return forward_mid(hs, 2, xs, &y, M, st, act);
+    } else if (M > hg->gemv_max_m && (fits || gemm_pair_applicable(a, M)) && narrow_is_faster(hs, 2, M, true)) {
+        void* ys[2] = {y, y};
+        return forward_narrow(hs, 2, x, ys, M, st, act);
     } else if (M > hg->gemv_max_m && gemm_pair_applicable(a, M)) {       // prefill: both accumulators of the CTA-pair kernel
         GemmPairLayers set{};
         set.n = 2;
@@ -926,8 +1096,7 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
         return gemm_pair_forward_gated(set, x, M, act, st, hg->device, hg->pdl, hg->num_sms);
     }
     // Unfused: the two projections into the device's shared scratch, then the element-wise product.
-    const int64_t n = (int64_t)M * a.N;
-    if ((size_t)n * 2 * sizeof(__half) > gemm_pair_scratch_bytes(hg->num_sms)) return QL_ERR_UNSUPPORTED;
+    if (!fits) return QL_ERR_UNSUPPORTED;
     __half* g = reinterpret_cast<__half*>(hg->dev->gemm_scratch);
     __half* u = g + ((n + 7) & ~(int64_t)7);
     void* ys[2] = {g, u};
@@ -982,7 +1151,7 @@ extern "C" ql_status qlinear_forward_a8(qlinear_t h, const void* x, void* y, int
         quantize_activations_kernel<<<M, 256, 0, st>>>(static_cast<const __half*>(x), xq, sx, rs, M, L.K);
         if (cudaGetLastError() != cudaSuccess) return QL_ERR_CUDA;
         GemmPairLayers set{};
-        set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_i8_ok ? &h->wmap_i8 : nullptr;
+        set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_wide_ok ? &h->wmap_wide : nullptr;
         if (gemm_pair_ta_i8_applicable(set, M, h->num_sms)) return gemm_pair_ta_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms);
         return gemm_pair_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms);
     }
