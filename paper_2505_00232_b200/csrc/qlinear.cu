@@ -1354,10 +1354,10 @@ extern "C" ql_status qlinear_embed(qlinear_t h, const int32_t* ids, int32_t n, v
     prm.y = static_cast<__half*>(y);
     prm.n = n; prm.N = L.N; prm.K = L.K; prm.n_kc = L.n_kc; prm.block_bytes = L.block_bytes;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (L.bits == 8) embed_kernel<8, false><<<n, 128, 0, st>>>(prm);
-    else if (L.grouped) embed_kernel<4, true><<<n, 128, 0, st>>>(prm);
-    else embed_kernel<4, false><<<n, 128, 0, st>>>(prm);
-    return cudaGetLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+    auto kern = L.bits == 8 ? embed_kernel<8, false> : L.grouped ? embed_kernel<4, true> : embed_kernel<4, false>;
+    const cudaError_t e = launch(kern, prm, dim3(n), dim3(128), 0, st, 1, h->pdl);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
 extern "C" ql_status qlinear_residual_rmsnorm(const void* x, const void* residual, const void* gamma, float eps, float gamma_offset,
