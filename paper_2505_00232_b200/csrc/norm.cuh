@@ -53,7 +53,6 @@ template <int VPT>
 __global__ void __launch_bounds__(kNormThreads) residual_rmsnorm_kernel(const NormParams p)
 {
     __shared__ float warp_sum[kNormThreads / 32];
-    __shared__ float rstd_s;
     const int m = blockIdx.x;
     const int64_t row = (int64_t)m * p.K;
     const int n_vec = p.K >> 3;
@@ -106,12 +105,9 @@ __global__ void __launch_bounds__(kNormThreads) residual_rmsnorm_kernel(const No
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
     if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = ss;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const float t = ((warp_sum[0] + warp_sum[1]) + (warp_sum[2] + warp_sum[3])) + ((warp_sum[4] + warp_sum[5]) + (warp_sum[6] + warp_sum[7]));
-        rstd_s = 1.0f / sqrtf(t / (float)p.K + p.eps);                   // IEEE division and square root
-    }
-    __syncthreads();
-    const float rstd = rstd_s;
+    // (every thread: cheaper than a second barrier)
+    const float t = ((warp_sum[0] + warp_sum[1]) + (warp_sum[2] + warp_sum[3])) + ((warp_sum[4] + warp_sum[5]) + (warp_sum[6] + warp_sum[7]));
+    const float rstd = 1.0f / sqrtf(t / (float)p.K + p.eps);             // IEEE division and square root
 
     auto finish = [&](int v, float a[8], const uint4* gv) {
         float g[8];

@@ -1418,7 +1418,7 @@ extern "C" ql_status qlinear_rope_qkv(const void* q, const void* k, const void* 
     const int items = (h_q + h_kv) * (d_h / 16) + h_kv * (d_h / 8);
     const int passes = (items + kRopeThreads - 1) / kRopeThreads;
     const int threads = std::min(kRopeThreads, (((items + passes - 1) / passes) + 31) / 32 * 32);
-    const cudaError_t e = launch(rope_qkv_kernel, prm, dim3(B * S), dim3(threads), 0, static_cast<cudaStream_t>(stream), 1, config().pdl);
+    const cudaError_t e = launch(rope_qkv_kernel, prm, dim3(B * S, B * S <= 64 ? passes : 1), dim3(threads), 0, static_cast<cudaStream_t>(stream), 1, config().pdl);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
