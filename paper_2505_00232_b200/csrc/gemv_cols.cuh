@@ -38,7 +38,7 @@ struct GemvColsParams {
     const __half* xscale[kGemvMaxBatch];         // [K]
     __half* y[kGemvMaxBatch];                    // [M, N]
     int32_t n_layers, M, N, K, n_rb, n_kc, cl, cps;   // layers of equal shape: n_rb row-blocks each
-    int32_t late;                                // as in GemvParamsT
+    int32_t hold0, hold1;                        // chunks that the kernel before this one may be writing (a KV cache): read after griddepcontrol.wait only
 };
 
 __global__ void __launch_bounds__(kColsThreads, 1) gemv_cols_kernel(const GemvColsParams p)
@@ -70,11 +70,15 @@ __global__ void __launch_bounds__(kColsThreads, 1) gemv_cols_kernel(const GemvCo
         }
         asm volatile("cp.async.commit_group;" ::: "memory");             // (an empty group keeps the count in step)
     };
-    if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int i = 0; i < kColsRing; ++i) copy_w(kc0 + i);
+    auto held = [&](int kc) { return kc >= p.hold0 && kc < p.hold1; };
+    for (int i = 0; i < kColsRing; ++i)
+        if (!held(kc0 + i)) copy_w(kc0 + i);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int i = 0; i < kColsRing; ++i) copy_x(kc0 + i);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int i = 0; i < kColsRing; ++i) {
+        if (held(kc0 + i)) copy_w(kc0 + i);
+        copy_x(kc0 + i);                                                 // (commits the chunk's group; what was requested earlier is part of the first)
+    }
 
     auto lds128 = [](uint32_t addr) {
         uint4 v;

@@ -29,7 +29,7 @@ struct GemvRowsParams {
     int32_t N[kGemvMaxBatch];
     int32_t rsb_end[kGemvMaxBatch];              // row super-blocks of layers 0..i
     int32_t n_layers, M, K, n_rsb, block_bytes;
-    int32_t late;                                // as in GemvParamsT
+    int32_t hold0, hold1;                        // rows that the kernel before this one may be writing (a KV cache): read after griddepcontrol.wait only
 };
 
 // NKC: chunks of 32 along K (K = 32 * NKC).
@@ -63,10 +63,16 @@ __global__ void __launch_bounds__(kGemvThreads, NKC <= 4 ? 4 : 3) gemv_rows_kern
     };
 
     int sb = blockIdx.x, stage = 0;
-    if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
-    issue(sb, 0);                                                       // weights do not depend on the previous kernel
+    bool held = false;                                                  // the first super-block holds rows that may still be written
+    if (sb < p.n_rsb) {
+        int ly, sb_local;
+        place(sb, ly, sb_local);
+        held = sb_local * kRsbRows < p.hold1 && (sb_local + 1) * kRsbRows > p.hold0;
+    }
+    if (!held) issue(sb, 0);                                            // everything else does not depend on the previous kernel
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (held) issue(sb, 0);
 
     for (; sb < p.n_rsb; sb += gridDim.x, stage ^= 1) {
         issue(sb + gridDim.x, stage ^ 1);

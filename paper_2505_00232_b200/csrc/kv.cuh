@@ -43,46 +43,51 @@ struct KvAppendParams {
     int32_t k_n_kc, v_n_kc;
 };
 
-// One CTA (128 threads) per new token and head; d_h <= 1024.
-__global__ void __launch_bounds__(128) kv_append_kernel(const KvAppendParams p)
+// One CTA of two warps per new token and head, one for the key and one for the value vector; d_h <= 1024, a multiple of 32.  Bound: the
+// chain of latencies (previous kernel -> vector -> amax -> scale -> bytes), so a warp keeps its vector in registers and there is no
+// barrier and no shared memory.  The dependents are released only after the wait: whoever runs beside this kernel then knows
+// that every kernel before it is complete, and that only the bytes of these tokens may still change.
+__global__ void __launch_bounds__(64) kv_append_kernel(const KvAppendParams p)
 {
-    __shared__ float wmax[2][4];
-    __shared__ float sc[2];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int i = blockIdx.x, t = p.pos + i, hd = blockIdx.y;
-    const int64_t src = hd * p.head_stride + i * p.token_stride;
-    const __half* kv[2] = {p.k_new + src, p.v_new + src};
-    float am[2] = {0.f, 0.f};
-    for (int j = threadIdx.x; j < p.d_h; j += 128) {
-        am[0] = fmaxf(am[0], fabsf(__half2float(kv[0][j])));
-        am[1] = fmaxf(am[1], fabsf(__half2float(kv[1][j])));
-    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int i = blockIdx.x, t = p.pos + i, hd = blockIdx.y, lane = threadIdx.x & 31;
+    const bool value = threadIdx.x >= 32;
+    const __half* src = (value ? p.v_new : p.k_new) + hd * p.head_stride + i * p.token_stride;
+    constexpr int NV = 8;                                                // 4-value vectors per lane: a head of 128 keeps every lane busy
+    const int n_vec = p.d_h >> 2;
+    uint2 u[NV];
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
+    for (int j = 0; j < NV; ++j) u[j] = lane + 32 * j < n_vec ? *reinterpret_cast<const uint2*>(src + 4 * (lane + 32 * j)) : make_uint2(0, 0);
+    __half2 mx = __float2half2_rn(0.f);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) am[s] = fmaxf(am[s], __shfl_xor_sync(0xffffffffu, am[s], o));
-        if ((threadIdx.x & 31) == 0) wmax[s][threadIdx.x >> 5] = am[s];
+    for (int j = 0; j < NV; ++j) {
+        const __half2* h = reinterpret_cast<const __half2*>(&u[j]);
+        mx = __hmax2(mx, __hmax2(__habs2(h[0]), __habs2(h[1])));
     }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        const int s = threadIdx.x;
-        const float a = fmaxf(fmaxf(wmax[s][0], wmax[s][1]), fmaxf(wmax[s][2], wmax[s][3]));
-        const __half h0 = __float2half_rn(__fdiv_rn(a, 127.f));
-        const bool dead = __half2float(h0) == 0.f;                       // a zero vector, or a scale below fp16's range
-        sc[s] = dead ? 0.f : __half2float(h0);                           // 0 marks "store zeros"
-        const __half h = dead ? __float2half_rn(1.f) : h0;
-        if (s == 0) p.k_scales[hd][t] = h; else p.v_scale[hd][t] = h;
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < p.d_h; j += 128) {
+    const float2 m = __half22float2(mx);
+    // (bits of a non-negative float: ordered like unsigned integers)
+    const float amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(m.x, m.y))));
+    const __half h0 = __float2half_rn(__fdiv_rn(amax, 127.f));
+    const bool dead = __half2float(h0) == 0.f;                           // a zero vector, or a scale below fp16's range: zeros, scale 1
+    const float sc = dead ? 1.f : __half2float(h0);
+    if (lane == 0) (value ? p.v_scale[hd] : p.k_scales[hd])[t] = __float2half_rn(sc);
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            int q = 0;
-            if (sc[s] != 0.f) q = max(-127, min(127, __float2int_rn(__fdiv_rn(__half2float(kv[s][j]), sc[s]))));
-            const uint8_t stored = (uint8_t)(q + 128);
-            if (s == 0) p.k_body[hd][int8_weight_offset(t, j, p.k_n_kc)] = stored;  // K: row = token, k = dimension
-            else p.v_body[hd][int8_weight_offset(j, t, p.v_n_kc)] = stored;         // V: row = dimension, k = token
+    for (int j = 0; j < NV; ++j) {
+        const int v = lane + 32 * j;
+        if (v >= n_vec) break;
+        const __half* h = reinterpret_cast<const __half*>(&u[j]);
+        uint32_t q[4];                                                   // as stored: q + 128
+#pragma unroll
+        for (int e = 0; e < 4; ++e) q[e] = dead ? 128u : (uint32_t)(max(-127, min(127, __float2int_rn(__fdiv_rn(__half2float(h[e]), sc)))) + 128);
+        if (value) {                                                     // V: row = dimension, k = token: rows g and g + 1 lie 64 bytes apart
+            uint8_t* dst = p.v_body[hd] + int8_weight_offset(4 * v, t, p.v_n_kc);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dst[64 * e] = (uint8_t)q[e];
+        } else {                                                         // K: row = token, k = dimension: pairs of k in each of a lane's words
+            uint8_t* dst = p.k_body[hd] + int8_weight_offset(t, 4 * v, p.k_n_kc);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) *reinterpret_cast<uint16_t*>(dst + 4 * e) = (uint16_t)(q[2 * e] | q[2 * e + 1] << 8);
         }
     }
 }

@@ -145,9 +145,13 @@ struct qlinear_s {
     bool wmap_ok, wmap_wide_ok;
     DeviceState* dev;
     // Set by the first append: the blob is a KV cache, and the kernel before a reader in the stream may be writing it.  Its readers
-    // then touch it only after griddepcontrol.wait (`late` in their parameters), or are launched without the programmatic edge
-    // (early(): int8 activations, the streaming kernel).  (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
+    // then touch it only after griddepcontrol.wait (`late` in their parameters; the decode readers of a cache: only the tokens of the last
+    // append, `hold`), or are launched without the programmatic edge (early(): int8 activations, the streaming kernel).  (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
     std::atomic<bool> cache{false};
+    // Tokens [first, end) of the last append, end in the high half.  While a reader runs ahead of its griddepcontrol.wait nothing else of
+    // the cache can be in flight: an append releases its dependents only past its own wait, when every kernel before it is complete.
+    // (A reader captured in a graph keeps the range of its capture; an append outside the graph is complete before the graph starts.)
+    std::atomic<uint64_t> appended{0};
     bool early() const { return pdl && !cache.load(std::memory_order_relaxed); }
 };
 
@@ -158,6 +162,19 @@ bool any_cache(const qlinear_s* const* hs, int n)
     for (int i = 0; i < n; ++i)
         if (hs[i]->cache.load(std::memory_order_relaxed)) return true;
     return false;
+}
+
+// The tokens that appends in flight may be writing in the caches of a launch: [first, end), empty if there are none.
+void held_tokens(const qlinear_s* const* hs, int n, int32_t* first, int32_t* end)
+{
+    *first = *end = 0;
+    for (int i = 0; i < n; ++i) {
+        const uint64_t a = hs[i]->appended.load(std::memory_order_relaxed);
+        const int32_t a0 = (int32_t)(a & 0xffffffffu), a1 = (int32_t)(a >> 32);
+        if (a1 <= a0) continue;
+        *first = *end == 0 ? a0 : std::min(*first, a0);
+        *end = std::max(*end, a1);
+    }
 }
 
 constexpr int kGemvMaxSmem = 96 * 1024;
@@ -379,7 +396,9 @@ ql_status forward_gemv_cols(qlinear_s* const* hs, int n, const void* const* xs, 
         p.y[i] = static_cast<__half*>(ys[i]);
     }
     p.n_layers = n; p.M = M; p.N = L.N; p.K = L.K; p.n_rb = h->n_rb; p.n_kc = L.n_kc;
-    p.late = any_cache(hs, n);
+    held_tokens(hs, n, &p.hold0, &p.hold1);
+    p.hold0 /= 32;
+    p.hold1 = (p.hold1 + 31) / 32;
     static std::atomic<bool> attr_set[kMaxDevices];
     cudaError_t e = ensure_smem_attr(gemv_cols_kernel, attr_set, h->device, kColsSmem);
     if (e != cudaSuccess) { cudaGetLastError(); return QL_ERR_CUDA; }
@@ -425,7 +444,7 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
             n_rsb += Li.n_rsb;
             rp.rsb_end[i] = n_rsb;
         }
-        rp.late = any_cache(hs, n);
+        held_tokens(hs, n, &rp.hold0, &rp.hold1);
         rp.n_layers = n; rp.M = M; rp.K = L.K; rp.n_rsb = n_rsb; rp.block_bytes = L.block_bytes;
         const cudaError_t e = L.n_kc == 2 ? launch_gemv_rows<2>(h, rp, st) : L.n_kc == 4 ? launch_gemv_rows<4>(h, rp, st) : launch_gemv_rows<8>(h, rp, st);
         return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
@@ -1218,15 +1237,18 @@ extern "C" ql_status qlinear_kv_append_heads(const qlinear_t* hk, const qlinear_
         prm.k_scales[i] = reinterpret_cast<__half*>(kb + K.chan_scale_offset);
         prm.v_body[i] = vb + V.body_offset;
         prm.v_scale[i] = static_cast<__half*>(v_scales[i]);
-        hk[i]->cache.store(true, std::memory_order_relaxed);
-        hv[i]->cache.store(true, std::memory_order_relaxed);
+        const uint64_t range = (uint64_t)(uint32_t)(pos + n_new) << 32 | (uint32_t)pos;
+        for (qlinear_s* h : {hk[i], hv[i]}) {
+            h->cache.store(true, std::memory_order_relaxed);
+            h->appended.store(range, std::memory_order_relaxed);
+        }
     }
     prm.k_new = static_cast<const __half*>(k_new);
     prm.v_new = static_cast<const __half*>(v_new);
     prm.head_stride = head_stride; prm.token_stride = token_stride;
     prm.d_h = K.K; prm.cache_size = K.N; prm.pos = pos; prm.n_new = n_new;
     prm.k_n_kc = K.n_kc; prm.v_n_kc = V.n_kc;
-    const cudaError_t e = launch(kv_append_kernel, prm, dim3(n_new, n_heads), dim3(128), 0, static_cast<cudaStream_t>(stream), 1, hk[0]->pdl);
+    const cudaError_t e = launch(kv_append_kernel, prm, dim3(n_new, n_heads), dim3(64), 0, static_cast<cudaStream_t>(stream), 1, hk[0]->pdl);
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
@@ -1414,7 +1436,8 @@ extern "C" ql_status qlinear_rope_qkv(const void* q, const void* k, const void* 
     prm.pos = pos; prm.cos_t = cos_t; prm.sin_t = sin_t;
     prm.q_out = static_cast<__half*>(q_out); prm.k_out = static_cast<__half*>(k_out); prm.v_out = static_cast<__half*>(v_out);
     prm.B = B; prm.S = S; prm.h_q = h_q; prm.h_kv = h_kv; prm.d_h = d_h; prm.n_pos = n_pos;
-    // threads: the work items of a token (8-element vectors of half a head) spread evenly over the fewest passes
+    // threads: the work items of a token (8-element vectors of half a head) spread evenly over the fewest passes, which are CTAs
+    // of their own where the tokens leave SMs idle
     const int items = (h_q + h_kv) * (d_h / 16) + h_kv * (d_h / 8);
     const int passes = (items + kRopeThreads - 1) / kRopeThreads;
     const int threads = std::min(kRopeThreads, (((items + passes - 1) / passes) + 31) / 32 * 32);
