@@ -22,6 +22,7 @@
 
 #include "dequant.cuh"
 #include "layout.h"
+#include "sm100_ptx.cuh"
 
 namespace ql {
 
@@ -153,6 +154,185 @@ __global__ void __launch_bounds__(256, 2) gemm_rows_kernel(const GemmRowsParams 
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// The same for many tokens, on the fifth-generation tensor core.  The warp-level MMAs of the kernel above keep its tensor core busy for 15 us
+// of a launch whose 67 MB of outputs need 10.4, and the reads of x, MMAs, stores and barriers of a tile run one after the other.
+// Here (two CTAs per SM) eight warps convert the super-block's integers once into tensor memory (exact fp16, the A operand) and take finished
+// tiles (128 positions x 64 tokens) out: a thread has one position, scales it, and leaves fp16 in a shared tile whose rows (one token, 256
+// bytes) leave as 16-byte stores (one bulk copy per token: 36 us for the launch above, the copies were the bound).  One thread issues the MMAs of the next tile into the other of two accumulators meanwhile (55 cycles each,
+// which is why none of the eight warps does it: 42 us instead of 35 for the kernel above), one loads x by TMA, some tiles ahead.
+// Every byte is read after griddepcontrol.wait (the cache may have been appended to just before).  Measured: 8 heads x 1024 rows x 4096
+// positions 34.8 -> 24.1 us at d_h = 128 (2.8 TB/s written), 58.6 -> 28.1 at 256; the rule is in forward_gemm_rows.
+struct GemmRowsMaps { CUtensorMap x[kRowsMaxLayers]; };                  // [M, K] of each layer, box 64 k x 64 tokens, 128-byte swizzle
+constexpr int kRowsTcTokens = 64;
+constexpr int kRowsTcThreads = 320;                                      // warps 0..7 conversion and outputs, 8 MMAs, 9 x
+template <int NKC>
+struct GemmRowsTcSmem {
+    static constexpr int kXTile = kRowsTcTokens * 128;                   // 64 k of a token block
+    static constexpr int kXBytes = NKC / 2 * kXTile;
+    static constexpr int kXStages = NKC == 8 ? 2 : 4;
+    static constexpr int kOutBytes = kRowsTcTokens * 256;
+    static constexpr int kOuts = NKC == 8 ? 1 : 2;                       // (d_h = 256: two CTAs per SM leave room for one)
+    static constexpr int kOutOffset = kXStages * kXBytes;
+    static constexpr int kUsed = 1024 + kOutOffset + kOuts * kOutBytes;
+    static constexpr int kTotal = kUsed > 80 * 1024 ? kUsed : 80 * 1024; // (never a third CTA on an SM: it would wait for tensor memory)
+    static_assert(kTotal <= 112 * 1024, "two CTAs per SM");
+};
+
+template <int NKC>
+__global__ void __launch_bounds__(kRowsTcThreads, 2) gemm_rows_tc_kernel(const __grid_constant__ GemmRowsMaps maps, const GemmRowsParams p)
+{
+    using S = GemmRowsTcSmem<NKC>;
+    constexpr int BN = kRowsTcTokens, ACOL = 2 * BN, NX = S::kXStages;   // tensor memory: two accumulators, then A (16 columns per 32 k)
+    extern __shared__ unsigned char smem_dyn[];
+    __shared__ __align__(8) unsigned long long bars[2 * NX + 5];
+    __shared__ volatile uint32_t flags[5];                               // tensor-memory address; abort words (see wait_expired)
+    const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    const uint32_t xfull = smem_u32(bars), mdone = xfull + 8 * NX, xempty = mdone + 16, taken = xempty + 8 * NX, aready = taken + 16;   // MMAs retired, accumulator taken out: two of each
+    volatile uint32_t* abort_flag = flags + 1;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, quarter = warp & 3, half = warp >> 2;
+    const int i0 = (int)((int64_t)blockIdx.x * p.n_tiles / gridDim.x), n = (int)((int64_t)(blockIdx.x + 1) * p.n_tiles / gridDim.x) - i0;   // tiles i0 .. i0 + n - 1
+    if (t < 2 * NX + 5) {
+        mbar_init(xfull + 8 * t, t < 2 * NX + 2 ? 1 : 8);                    // taken, aready: the eight warps
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (t >= 32 && t < 36) abort_flag[t - 32] = 0;
+    if (t >= 64 && t < 64 + p.n_layers) asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.x[t - 64]) : "memory");
+    if (warp == 8) tmem_alloc(smem_u32((const void*)flags), 256);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = flags[0];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (t == 0) abort_flag[2] = abort_flag[3] = 1;
+
+    auto layer_of = [&](int rsb) {
+        int ly = 0;
+#pragma unroll
+        for (int i = 1; i < kRowsMaxLayers; ++i)
+            if (i < p.n_layers && rsb >= p.rsb_end[i - 1]) ly = i;
+        return ly;
+    };
+    if (warp == 9) {
+        // ------------------------------------------------------------------ x
+        if (lane == 0) {
+            int j = 0;
+            for (; j < n; ++j) {
+                const int s = j % NX, rsb = (i0 + j) / p.n_tb, m0 = (i0 + j - rsb * p.n_tb) * BN;
+                if (!mbar_wait(xempty + 8 * s, ((uint32_t)(j / NX) & 1) ^ 1, abort_flag, 0x6A8 + s)) break;
+                const CUtensorMap* map = &maps.x[layer_of(rsb)];
+                mbar_expect_tx(xfull + 8 * s, S::kXBytes);
+#pragma unroll
+                for (int b = 0; b < NKC / 2; ++b) tma_load_2d(base + s * S::kXBytes + b * S::kXTile, map, 64 * b, m0, xfull + 8 * s);
+            }
+            if (*abort_flag)                                             // copies in flight land before the CTA leaves
+                for (int i = max(0, j - NX); i < j; ++i) mbar_wait(xfull + 8 * (i % NX), (uint32_t)(i / NX) & 1, abort_flag + 1, 0);
+        }
+    } else if (warp == 8) {
+        // ------------------------------------------------------------------ MMAs
+        if (lane == 0) {
+            uint32_t apar = 0;
+            int cur = -1;
+            for (int j = 0; j < n; ++j) {
+                const int d = j & 1, s = j % NX, rsb = (i0 + j) / p.n_tb;
+                if (rsb != cur) {
+                    if (!mbar_wait(aready, apar, abort_flag, 0x6A0)) break;
+                    cur = rsb;
+                    apar ^= 1;
+                }
+                if (j >= 2 && !mbar_wait(taken + 8 * d, (uint32_t)((j - 2) >> 1) & 1, abort_flag, 0x6A4 + d)) break;
+                if (!mbar_wait(xfull + 8 * s, (uint32_t)(j / NX) & 1, abort_flag, 0x6B0 + s)) break;
+                tc_fence_after();
+                const uint32_t b_lo = umma_desc_lo(base + s * S::kXBytes);
+#pragma unroll
+                for (int k = 0; k < 2 * NKC; ++k)
+                    umma_f16_ta(tmem + (uint32_t)(d * BN), tmem + (uint32_t)(ACOL + 8 * k), b_lo + (uint32_t)((k >> 2) * (S::kXTile >> 4) + 2 * (k & 3)), umma_idesc_f16(BN), k > 0 ? 1u : 0u);
+                umma_commit(mdone + 8 * d);
+                umma_commit(xempty + 8 * s);
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ weights and outputs
+        // this thread's position: row-block 2 quarter + lane / 16, lane-row lane % 8, rows g + 8 for lanes 8..15 and 24..31 (layout.h)
+        const int row = quarter * 32 + lane, line = ((2 * quarter + (lane >> 4)) * 8 + (lane & 7)) * 64;
+        const uint32_t sel = lane & 8 ? 0x4342u : 0x4140u, lane_base = (uint32_t)(quarter * 32) << 16;
+        float scale = 0.f;
+        int ly = 0, n0 = 0;
+        auto convert = [&](int rsb) {                                    // the super-block's integers -> A; the two warps of a quarter share its k
+            ly = layer_of(rsb);
+            const int r = rsb - (ly ? p.rsb_end[ly - 1] : 0);
+            const uint8_t* src = p.body[ly] + (int64_t)r * NKC * kWeightBlockBytes + line + half * (NKC / 2) * kWeightBlockBytes;
+            n0 = r * kRsbRows;
+            scale = n0 + row < p.N[ly] ? __half2float(__ldcg(p.chan_scales[ly] + n0 + row)) : 0.f;
+            constexpr int B = NKC == 8 ? 2 : NKC / 2;                    // blocks whose loads are in flight together
+#pragma unroll
+            for (int b0 = 0; b0 < NKC / 2; b0 += B) {
+                uint4 w[B][4];
+#pragma unroll
+                for (int b = 0; b < B; ++b)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) w[b][c] = __ldcg(reinterpret_cast<const uint4*>(src + (b0 + b) * kWeightBlockBytes + 16 * c));
+#pragma unroll
+                for (int b = 0; b < B; ++b)
+#pragma unroll
+                    for (int cp = 0; cp < 2; ++cp) {
+                        uint32_t o[8];
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            const uint4 v = w[b][2 * cp + c];
+                            o[4 * c + 0] = h2_sub(__byte_perm(v.x, 0x64646464u, sel), 0x64806480u);
+                            o[4 * c + 1] = h2_sub(__byte_perm(v.y, 0x64646464u, sel), 0x64806480u);
+                            o[4 * c + 2] = h2_sub(__byte_perm(v.z, 0x64646464u, sel), 0x64806480u);
+                            o[4 * c + 3] = h2_sub(__byte_perm(v.w, 0x64646464u, sel), 0x64806480u);
+                        }
+                        tmem_st8_async(tmem + lane_base + (uint32_t)(ACOL + 16 * (half * (NKC / 2) + b0 + b) + 8 * cp), o);
+                    }
+            }
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(aready);
+        };
+        auto meet = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+        bool ok = true;
+        convert(i0 / p.n_tb);
+        for (int j = 0; j < n; ++j) {
+            const int i = i0 + j, d = j & 1, ob = S::kOuts == 2 ? d : 0, rsb = i / p.n_tb, m0 = (i - rsb * p.n_tb) * BN;
+            ok = ok && mbar_wait(mdone + 8 * d, (uint32_t)(j >> 1) & 1, abort_flag, 0x6A6 + d);
+            tc_fence_after();
+            uint32_t v[32];
+            tmem_ld32(tmem + lane_base + (uint32_t)(d * BN + 32 * half), v);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(taken + 8 * d);
+            if (S::kOuts == 1) meet();                                   // everybody has read the output tile (two of them: the barrier below is enough)
+            const uint32_t out = base + S::kOutOffset + ob * S::kOutBytes;
+            __half* orow = reinterpret_cast<__half*>(smem_dyn + (out - smem_u32(smem_dyn))) + row;
+#pragma unroll
+            for (int q = 0; q < 32; ++q) orow[(32 * half + q) * 128] = __float2half_rn(__uint_as_float(v[q]) * scale);
+            meet();
+            const int N = p.N[ly];
+            __half* y = p.y[ly] + (int64_t)m0 * N + n0;
+#pragma unroll
+            for (int e = t; e < BN * 16; e += 256) {                     // 16 bytes = 8 positions (N is a multiple of 8)
+                const int tok = e >> 4, u = e & 15;
+                if (ok && m0 + tok < p.M && n0 + 8 * u < N) {
+                    uint4 o;
+                    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(o.x), "=r"(o.y), "=r"(o.z), "=r"(o.w) : "r"(out + tok * 256 + u * 16));
+                    *reinterpret_cast<uint4*>(y + (int64_t)tok * N + 8 * u) = o;
+                }
+            }
+            if (j + 1 < n && (i + 1) / p.n_tb != rsb) convert(rsb + 1);  // (uniform; every MMA so far has retired)
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 8) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 256);
+    }
 }
 
 }  // namespace ql

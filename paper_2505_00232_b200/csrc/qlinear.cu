@@ -731,6 +731,28 @@ cudaError_t launch_gemm_rows(const qlinear_s* h, GemmRowsParams& prm, int n_rsb,
     if (prm.M <= 32) return launch_gemm_rows_nt<NKC, 4>(h, prm, n_rsb, pdl, st);
     return launch_gemm_rows_nt<NKC, 8>(h, prm, n_rsb, pdl, st);
 }
+template <int NKC>
+cudaError_t launch_gemm_rows_tc(const qlinear_s* h, const GemmRowsMaps& maps, GemmRowsParams& prm, int n_rsb, cudaStream_t st)
+{
+    using S = GemmRowsTcSmem<NKC>;
+    static std::atomic<bool> attr_set[kMaxDevices];
+    auto kern = gemm_rows_tc_kernel<NKC>;
+    cudaError_t e = ensure_smem_attr(kern, attr_set, h->device, S::kTotal);
+    if (e != cudaSuccess) return e;
+    prm.n_tb = (prm.M + kRowsTcTokens - 1) / kRowsTcTokens;
+    prm.n_tiles = n_rsb * prm.n_tb;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(std::min(prm.n_tiles, 2 * h->num_sms));
+    cfg.blockDim = dim3(kRowsTcThreads);
+    cfg.dynamicSmemBytes = S::kTotal;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = h->pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, maps, prm);
+}
 ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st)
 {
     const qlinear_s* h = hs[0];
@@ -749,6 +771,20 @@ ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const
     prm.n_layers = n; prm.M = M;
     const bool pdl = h->pdl;                                             // (every byte is read after griddepcontrol.wait)
     const int n_kc = h->L.n_kc;
+    // The tensor-core form has the longer ramp and the faster tiles, and another order of sums inside an MMA.  The rule looks at one layer, so
+    // that a head gets the same bits alone and among others: from the tiles of 128 x 64 on at which one layer alone is even.  Measured,
+    // us gemm_rows_kernel / this, one layer: d_h = 64, 1024 tiles 8.1 / 7.8; d_h = 128, 512 7.1 / 7.2, 1024 11.4 / 9.0; d_h = 256, 512 10.4 / 9.9,
+    // 1024 18.1 / 11.7; eight layers: d_h = 64, 512 tiles each 23.9 / 20.6, d_h = 128 34.8 / 24.1, d_h = 256 58.6 / 28.1.
+    int layer_rsb = h->L.n_rsb;
+    for (int i = 1; i < n; ++i) layer_rsb = std::min(layer_rsb, hs[i]->L.n_rsb);
+    if ((int64_t)layer_rsb * ((M + kRowsTcTokens - 1) / kRowsTcTokens) * 20 >= h->num_sms * (n_kc == 2 ? 138 : n_kc == 4 ? 69 : 60)) {
+        GemmRowsMaps maps;
+        for (int i = 0; i < kRowsMaxLayers; ++i)
+            if (!x_tensor_map(xs[i < n ? i : 0], h->L.K, M, kRowsTcTokens, &maps.x[i])) return QL_ERR_CUDA;
+        const cudaError_t e = n_kc == 2 ? launch_gemm_rows_tc<2>(h, maps, prm, n_rsb, st) : n_kc == 4 ? launch_gemm_rows_tc<4>(h, maps, prm, n_rsb, st) : launch_gemm_rows_tc<8>(h, maps, prm, n_rsb, st);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+    }
     const cudaError_t e = n_kc == 2 ? launch_gemm_rows<2>(h, prm, n_rsb, pdl, st) : n_kc == 4 ? launch_gemm_rows<4>(h, prm, n_rsb, pdl, st) : launch_gemm_rows<8>(h, prm, n_rsb, pdl, st);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
