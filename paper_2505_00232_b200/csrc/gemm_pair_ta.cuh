@@ -505,8 +505,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             const uint32_t gpar = (uint32_t)(GATED ? j >> 1 : j) & 1;   // phase of the group barriers: once per output tile
             bool live = true;
             if (!GATED || gl == 0) {
-                // the bulk copies of the previous output tile have read their rows of the shared tile
-                if (grp_thread < 64) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                // the four warps have read their rows of the previous output tile
                 __syncwarp();
                 if (lane == 0) mbar_arrive(grp_bar(wi, 0));
                 live = mbar_wait(grp_bar(wi, 0), gpar, abort_flag, 0xC00 + wi);
@@ -562,7 +561,6 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                         else store32([](float v, int) { return v; });
                     }
                 }
-                fence_async_smem();
             }
             if (GATED && gl == 0) {                                      // the product is sent when the up tile is done
                 if (!live) ok = false;
@@ -571,12 +569,17 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             __syncwarp();
             if (lane == 0) mbar_arrive(grp_bar(wi, 1));
             live = mbar_wait(grp_bar(wi, 1), gpar, abort_flag, 0xC10 + wi) && live;
-            if (live && grp_thread < n_cols && m0 + grp_thread < p.M) {
-                const int n0 = rsb * kRsbRows;
-                const uint32_t bytes = (uint32_t)min(kRsbRows, N - n0) * 2;
-                bulk_copy_s2g(p.ly[ly] + (int64_t)(m0 + grp_thread) * N + n0, out_addr + (uint32_t)(64 * wi + grp_thread) * 256, bytes);
+            if (live) {
+                // 16-byte stores, a row of 256 bytes per half warp (N is a multiple of 8).  (One bulk copy per token occupied the TMA unit,
+                // which the loads of the next tile need.)
+                const int n0 = rsb * kRsbRows, u = grp_thread & 15, tok0 = grp_thread >> 4, left = min(n_cols, p.M - m0);
+                if (n0 + 8 * u < N) {
+                    __half* dst = p.ly[ly] + (int64_t)(m0 + tok0) * N + n0 + 8 * u;
+                    const uint32_t src = out_addr + (uint32_t)(64 * wi + tok0) * 256 + 16 * u;
+#pragma unroll 2
+                    for (int tok = 0; tok0 + tok < left; tok += 8) *reinterpret_cast<uint4*>(dst + (int64_t)tok * N) = lds_u128(src + tok * 256);
+                }
             }
-            if (grp_thread < 64) asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             if (!live) ok = false;
         };
         auto tile_complete = [&](int j) {                                // non-blocking: has the j-th tile's last MMA retired?
@@ -662,7 +665,6 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             }
         }
         while (epi_warp && ok && next_epi < n_units) { epilogue(next_epi); ++next_epi; }
-        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // y written before the kernel ends
     }
 
     tc_fence_before();
