@@ -56,34 +56,39 @@ extern "C" ql_status qlinear_pack(const qlinear_desc* d, const int8_t* q, const 
     for (int rsb = 0; rsb < L.n_rsb; ++rsb)
         for (int kc = 0; kc < L.n_kc; ++kc) {
             uint8_t* blk = out + block_offset(L, rsb, kc);
-            for (int rb = 0; rb < 8; ++rb)
-                for (int lane = 0; lane < 32; ++lane) {
-                    const int g = lane >> 2, c = lane & 3;
-                    const int row0 = rsb * kRsbRows + rb * kRbRows + g;
-                    uint32_t words[4];
-                    if (L.bits == 4) {
-                        for (int i = 0; i < 4; ++i) {
-                            uint32_t w = 0;
-                            for (int p = 0; p < 8; ++p) {
-                                int row = row0 + 8 * int4_nibble_rowsel(p);
-                                int k = kc * 64 + int4_k_in_chunk(c, i, int4_nibble_slot(p));
-                                w |= (uint32_t)((qv(row, k) + 8) & 0xF) << (4 * p);
+            // get(row, k): the integer there; blocks inside the matrix are read without bounds checks
+            auto fill = [&](auto get) {
+                for (int rb = 0; rb < 8; ++rb)
+                    for (int lane = 0; lane < 32; ++lane) {
+                        const int g = lane >> 2, c = lane & 3;
+                        const int row0 = rsb * kRsbRows + rb * kRbRows + g;
+                        uint32_t words[4];
+                        if (L.bits == 4) {
+                            for (int i = 0; i < 4; ++i) {
+                                uint32_t w = 0;
+                                for (int p = 0; p < 8; ++p) {
+                                    int row = row0 + 8 * int4_nibble_rowsel(p);
+                                    int k = kc * 64 + int4_k_in_chunk(c, i, int4_nibble_slot(p));
+                                    w |= (uint32_t)((get(row, k) + 8) & 0xF) << (4 * p);
+                                }
+                                words[i] = w;
                             }
-                            words[i] = w;
-                        }
-                    } else {
-                        for (int wi = 0; wi < 4; ++wi) {
-                            uint32_t w = 0;
-                            for (int b = 0; b < 4; ++b) {
-                                int row = row0 + 8 * int8_byte_rowsel(b);
-                                int k = kc * 32 + int8_k_in_chunk(c, wi, b);
-                                w |= (uint32_t)((qv(row, k) + 128) & 0xFF) << (8 * b);
+                        } else {
+                            for (int wi = 0; wi < 4; ++wi) {
+                                uint32_t w = 0;
+                                for (int b = 0; b < 4; ++b) {
+                                    int row = row0 + 8 * int8_byte_rowsel(b);
+                                    int k = kc * 32 + int8_k_in_chunk(c, wi, b);
+                                    w |= (uint32_t)((get(row, k) + 128) & 0xFF) << (8 * b);
+                                }
+                                words[wi] = w;
                             }
-                            words[wi] = w;
                         }
+                        std::memcpy(blk + rb * 512 + lane * 16, words, 16);
                     }
-                    std::memcpy(blk + rb * 512 + lane * 16, words, 16);
-                }
+            };
+            if ((rsb + 1) * kRsbRows <= N && (kc + 1) * L.chunk_k <= K) fill([&](int row, int k) -> int { return q[(int64_t)row * K + k]; });
+            else fill(qv);
             if (L.grouped) {
                 uint16_t* sc = reinterpret_cast<uint16_t*>(blk + kWeightBlockBytes);
                 for (int rb = 0; rb < 8; ++rb)
