@@ -11,7 +11,7 @@
 //   * tensor memory (512 columns): one 256-column fp32 accumulator + 8 A slots of 32 columns (64 k of fp16); there
 //     is no room for a second accumulator, so the epilogue is not hidden under the next tile.  It is kept short
 //     instead: 16 warps take the accumulator out together (64 columns each) as soon as they see the tile complete,
-//     free it, and leave fp16 values in a shared output tile that bulk copies drain under the next main loop;
+//     free it, and leave fp16 values in a shared output tile, from which the four warps of 64 tokens store whole rows;
 //     meanwhile up to 6 A slots of the next tile are already filled, so the MMA restarts at once;
 //   * a thread of a dequantise warp owns ONE tile row (its TMEM lane): it needs 32 consecutive k of that row, which
 //     the packed block keeps in four 16-byte pieces (lane columns c = 0..3 of its row-block line), 64 bytes apart
@@ -434,7 +434,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         // The epilogue of the j-th tile of this cluster: this warp takes columns (tokens) 64 wi .. + 63 of its lane
         // quarter (32 channels) out of the accumulator, frees the accumulator, and leaves fp16 values in the
         // shared output tile [token][channel]; the four warps that share the 64 tokens then meet at a barrier
-        // and send each token's 256 bytes to y with one bulk copy, which drains under the next tile's main loop.
+        // and store the tokens' rows of 256 bytes to y, 16 bytes per thread.
         const uint32_t out_addr = base + S::kOutOffset;
         unsigned char* out_ptr = base_ptr + S::kOutOffset;
         const int grp_thread = quarter * 32 + lane;                      // 0..127 inside the group of four warps
