@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(kMidThreads, 2) gemm_mid_kernel(const MidParam
     const int N = p.N[GATED ? 0 : ly];
     uint2 cs[2] = {make_uint2(0x3C003C00u, 0x3C003C00u), make_uint2(0x3C003C00u, 0x3C003C00u)};
     if (!GROUPED && row0 < N) {
-        cs[0] = __ldcg(reinterpret_cast<const uint2*>(p.chan_scales[GATED ? 0 : ly] + row0));
-        if (GATED) cs[1] = __ldcg(reinterpret_cast<const uint2*>(p.chan_scales[1] + row0));
+        cs[0] = ld_cg_u64(p.chan_scales[GATED ? 0 : ly] + row0);
+        if (GATED) cs[1] = ld_cg_u64(p.chan_scales[1] + row0);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll

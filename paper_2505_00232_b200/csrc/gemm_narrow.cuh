@@ -283,12 +283,18 @@ __global__ void __launch_bounds__(narrow_threads(G), 2) gemm_narrow_kernel(const
         // ------------------------------------------------------------------ epilogue: a thread has one channel, the groups take turns at 8 tokens
         const int n = rsb * kRsbRows + quarter * 32 + lane, N = p.N[GATED ? 0 : ly];
         float sc0 = 1.f, sc1 = 1.f;
-        if (!GROUPED && p.cl == 1 && n < N) {
-            sc0 = __half2float(__ldcg(p.chan_scales[GATED ? 0 : ly] + n));
-            if (GATED) sc1 = __half2float(__ldcg(p.chan_scales[1] + n));
-        }
+        auto load_scales = [&] {
+            if (!GROUPED && p.cl == 1 && n < N) {
+                sc0 = __half2float(ld_cg_half(p.chan_scales[GATED ? 0 : ly] + n));
+                if (GATED) sc1 = __half2float(ld_cg_half(p.chan_scales[1] + n));
+            }
+        };
+        // Early, unless the kernel before this one may still be writing them: a group without a step of its own has waited for nothing
+        // so far.  (The accumulators are complete only past the x producer's griddepcontrol.wait.)
+        if (!p.late) load_scales();
         ok = ok && mbar_wait(tfull_bar, 0, abort_flag, 0x680);
         if (ok) {
+            if (p.late) load_scales();
             tc_fence_after();
             float* part = reinterpret_cast<float*>(base_ptr) + quarter * 32 + lane;   // [layer of the pair][token][channel]
             __half* yc = p.y[GATED ? 0 : ly] + (int64_t)m0 * N + n;
@@ -331,7 +337,7 @@ __global__ void __launch_bounds__(narrow_threads(G), 2) gemm_narrow_kernel(const
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) sc[r][i] = !GROUPED && row0 < N ? __half2float(__ldcg(p.chan_scales[GATED ? r : ly] + row0 + i)) : 1.f;
+                for (int i = 0; i < 4; ++i) sc[r][i] = !GROUPED && row0 < N ? __half2float(ld_cg_half(p.chan_scales[GATED ? r : ly] + row0 + i)) : 1.f;
             for (int tok = crank + (t >> 5) * p.cl; tok < bn && m0 + tok < p.M; tok += 4 * G * p.cl) {
                 float v[R][4];
 #pragma unroll

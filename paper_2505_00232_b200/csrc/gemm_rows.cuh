@@ -100,11 +100,11 @@ __global__ void __launch_bounds__(256, 2) gemm_rows_kernel(const GemmRowsParams 
             const int r = rsb - (ly ? p.rsb_end[ly - 1] : 0);
             const uint8_t* src = p.body[ly] + (int64_t)r * NKC * kWeightBlockBytes + t * 16;
 #pragma unroll
-            for (int kc = 0; kc < NKC; ++kc) w[kc] = __ldcg(reinterpret_cast<const uint4*>(src + kc * kWeightBlockBytes));
+            for (int kc = 0; kc < NKC; ++kc) w[kc] = ld_cg_u128(src + kc * kWeightBlockBytes);
             row_base = r * kRsbRows;
             const int row = row_base + warp * 16 + g;
-            s0 = row < p.N[ly] ? __half2float(__ldcg(p.chan_scales[ly] + row)) : 0.f;
-            s1 = row + 8 < p.N[ly] ? __half2float(__ldcg(p.chan_scales[ly] + row + 8)) : 0.f;
+            s0 = row < p.N[ly] ? __half2float(ld_cg_half(p.chan_scales[ly] + row)) : 0.f;
+            s1 = row + 8 < p.N[ly] ? __half2float(ld_cg_half(p.chan_scales[ly] + row + 8)) : 0.f;
         }
         asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncthreads();                                                 // this tile's x has landed; the output tile has been sent
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kRowsTcThreads, 2) gemm_rows_tc_kernel(const _
             const int r = rsb - (ly ? p.rsb_end[ly - 1] : 0);
             const uint8_t* src = p.body[ly] + (int64_t)r * NKC * kWeightBlockBytes + line + half * (NKC / 2) * kWeightBlockBytes;
             n0 = r * kRsbRows;
-            scale = n0 + row < p.N[ly] ? __half2float(__ldcg(p.chan_scales[ly] + n0 + row)) : 0.f;
+            scale = n0 + row < p.N[ly] ? __half2float(ld_cg_half(p.chan_scales[ly] + n0 + row)) : 0.f;
             constexpr int B = NKC == 8 ? 2 : NKC / 2;                    // blocks whose loads are in flight together
 #pragma unroll
             for (int b0 = 0; b0 < NKC / 2; b0 += B) {
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(kRowsTcThreads, 2) gemm_rows_tc_kernel(const _
 #pragma unroll
                 for (int b = 0; b < B; ++b)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) w[b][c] = __ldcg(reinterpret_cast<const uint4*>(src + (b0 + b) * kWeightBlockBytes + 16 * c));
+                    for (int c = 0; c < 4; ++c) w[b][c] = ld_cg_u128(src + (b0 + b) * kWeightBlockBytes + 16 * c);
 #pragma unroll
                 for (int b = 0; b < B; ++b)
 #pragma unroll

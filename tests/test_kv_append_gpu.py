@@ -67,3 +67,40 @@ def test_products_of_tokens_appended_just_before(P, torch, n_heads, d_h, cache, 
         y64, A, _ = O.linear(q[h].cpu().numpy(), k_q, k_s.reshape(-1, 1), 0)
         ok, rel, worst = O.check_against(got[1][h, :, :T].cpu().numpy(), y64, A)
         assert ok, (h, rel, worst)
+
+
+@pytest.mark.parametrize("n_heads,d_h,cache,R", [(4, 96, 16384, 64), (2, 96, 15680, 49), (1, 96, 41728, 33), (2, 32, 46880, 64), (2, 160, 16384, 64)])
+def test_scores_of_a_batch_of_rows_see_the_scales_appended_just_before(P, torch, n_heads, d_h, cache, R):
+    """Head dimensions that the row kernels do not take, so many positions that the batch kernel with the weights in tensor memory serves the
+    scores in one K part, and (up to 128 of K) a step for one of its two groups of warps only: the other one waits for nothing before
+    its outputs.  Append and scores captured and replayed on new tokens, against the same calls with the host waiting in between."""
+    T, n_new = cache - 100, 64
+    start = torch.randn((n_heads, T, d_h), device="cuda").half()
+    pair = [P.KVHeads(n_heads, cache, d_h) for _ in range(2)]
+    for kv in pair:
+        kv.append(start, start)
+    q = torch.randn((n_heads, R, d_h), device="cuda").half()
+    kn = torch.zeros((n_heads, n_new, d_h), dtype=torch.float16, device="cuda")
+
+    def step(kv, wait):
+        kv.length = T
+        kv.append(kn, kn)
+        wait()
+        return kv.scores(q)
+    step(pair[0], lambda: None)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = step(pair[0], lambda: None)
+    for i in range(20):
+        kn.copy_(torch.randn_like(kn) * (0.1 if i & 1 else 10.0))
+        graph.replay()
+        torch.cuda.synchronize()
+        want = step(pair[1], torch.cuda.synchronize)
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
+    assert pair[0].heads[0].k.device_status() == (0, 0)
+    k_q, k_s = O.kv_quantize_rows(kn[0].cpu().numpy())
+    y64, A, _ = O.linear(q[0].cpu().numpy(), k_q, k_s.reshape(-1, 1), 0)
+    ok, rel, worst = O.check_against(got[0, :, T:T + n_new].cpu().numpy(), y64, A)
+    assert ok, (rel, worst)
