@@ -375,10 +375,14 @@ uint32_t qlinear_version(void);
  * qlinear_kv_output_heads over n_heads caches like h_v what qlinear_debug_plan does for the other decode launches: {CTAs per
  * cluster, chunks per warp, clusters of the launch, clusters that run at once}.  qlinear_debug_takes_batch_kernel returns 1 if a
  * forward call (n = 1) or a group of these layers on M tokens belongs to the batch stage by its size (calls beyond it belong to the
- * prefill stage, whose choice of kernel includes the batch kernel with the weights in tensor memory). */
+ * prefill stage, whose choice of kernel includes the batch kernel with the weights in tensor memory).
+ * qlinear_debug_kv_hold gives the tokens [*first, *end) of n caches that a decode reader of theirs on this stream would leave until the
+ * kernel before it is complete: those of the last append if that was enqueued on the same stream and in the same capture, all of
+ * them (an *end beyond any cache) if it was enqueued elsewhere, none for layers that nothing was appended to. */
 int32_t qlinear_debug_plan(qlinear_t h, int32_t M, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_plan_kv_output(qlinear_t h_v, int32_t n_heads, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_takes_batch_kernel(const qlinear_t* hs, int32_t n, int32_t M);
+ql_status qlinear_debug_kv_hold(const qlinear_t* hs, int32_t n, void* stream, int32_t* first, int32_t* end);
 uint32_t qlinear_debug_config_reads(void);
 
 #ifdef __cplusplus

@@ -145,13 +145,16 @@ struct qlinear_s {
     bool wmap_ok, wmap_wide_ok;
     DeviceState* dev;
     // Set by the first append: the blob is a KV cache, and the kernel before a reader in the stream may be writing it.  Its readers
-    // then touch it only after griddepcontrol.wait (`late` in their parameters; the decode readers of a cache: only the tokens of the last
-    // append, `hold`), or are launched without the programmatic edge (early(): int8 activations, the streaming kernel).  (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
+    // then touch it only after griddepcontrol.wait (`late` in their parameters; the decode readers of a cache: only the tokens that held_tokens
+    // names), or are launched without the programmatic edge (early(): int8 activations, the streaming kernel).  (Written under no lock: a caller that enqueues a reader behind an append has ordered the two calls.)
     std::atomic<bool> cache{false};
-    // Tokens [first, end) of the last append, end in the high half.  While a reader runs ahead of its griddepcontrol.wait nothing else of
-    // the cache can be in flight: an append releases its dependents only past its own wait, when every kernel before it is complete.
-    // (A reader captured in a graph keeps the range of its capture; an append outside the graph is complete before the graph starts.)
-    std::atomic<uint64_t> appended{0};
+    // The last append that was launched: its tokens [first, end) and where it was enqueued.  Guarded by g_append_mutex[device].
+    struct Append {
+        int32_t first = 0, end = 0;
+        cudaStream_t stream = nullptr;
+        unsigned long long capture = 0;      // id of the stream capture that recorded it, 0: none
+        bool alone = false;                  // every append to this cache in that capture was enqueued on this stream
+    } append;
     bool early() const { return pdl && !cache.load(std::memory_order_relaxed); }
 };
 
@@ -164,16 +167,41 @@ bool any_cache(const qlinear_s* const* hs, int n)
     return false;
 }
 
-// The tokens that appends in flight may be writing in the caches of a launch: [first, end), empty if there are none.
-void held_tokens(const qlinear_s* const* hs, int n, int32_t* first, int32_t* end)
+// Held while an append is launched and recorded, so that appends to one cache are recorded in the order in which they were enqueued.
+std::mutex g_append_mutex[kMaxDevices];
+
+// The capture that a launch on `st` would be recorded in (0: none); false where that cannot be told, or where the handle does not name one
+// stream (cudaStreamPerThread).
+bool capture_of(cudaStream_t st, unsigned long long* id)
+{
+    *id = 0;
+    if (st == cudaStreamPerThread) return false;
+    cudaStreamCaptureStatus status;
+    if (cudaStreamGetCaptureInfo(st, &status, id) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (status == cudaStreamCaptureStatusNone) *id = 0;
+    return status != cudaStreamCaptureStatusInvalidated;
+}
+
+// The tokens [first, end) that appends may still be writing in the caches of a decode launch on `st` while it runs ahead of its
+// griddepcontrol.wait; empty for layers that are no cache.  Those of the last append, where that append was enqueued on the same stream and
+// in the same capture: an append releases its dependents only past its own wait, when every kernel before it in the stream is
+// complete, and what other streams hold is behind an event, a full dependency.  Everything where the last append was enqueued elsewhere (an
+// append before it may then be the one in flight: a capture between append and reader, a second stream), and where a capture
+// has appends on several streams (the edges that join them may all be programmatic).
+constexpr int32_t kHoldAll = 0x7fffffe0;                                 // (a multiple of 32)
+void held_tokens(const qlinear_s* const* hs, int n, cudaStream_t st, int32_t* first, int32_t* end)
 {
     *first = *end = 0;
+    if (!any_cache(hs, n)) return;
+    unsigned long long capture;
+    const bool known = capture_of(st, &capture);
+    std::lock_guard<std::mutex> lock(g_append_mutex[hs[0]->device]);
     for (int i = 0; i < n; ++i) {
-        const uint64_t a = hs[i]->appended.load(std::memory_order_relaxed);
-        const int32_t a0 = (int32_t)(a & 0xffffffffu), a1 = (int32_t)(a >> 32);
-        if (a1 <= a0) continue;
-        *first = *end == 0 ? a0 : std::min(*first, a0);
-        *end = std::max(*end, a1);
+        if (!hs[i]->cache.load(std::memory_order_relaxed)) continue;
+        const qlinear_s::Append& a = hs[i]->append;
+        if (!known || !a.alone || a.stream != st || a.capture != capture) { *first = 0; *end = kHoldAll; return; }
+        *first = *end == 0 ? a.first : std::min(*first, a.first);
+        *end = std::max(*end, a.end);
     }
 }
 
@@ -396,7 +424,7 @@ ql_status forward_gemv_cols(qlinear_s* const* hs, int n, const void* const* xs, 
         p.y[i] = static_cast<__half*>(ys[i]);
     }
     p.n_layers = n; p.M = M; p.N = L.N; p.K = L.K; p.n_rb = h->n_rb; p.n_kc = L.n_kc;
-    held_tokens(hs, n, &p.hold0, &p.hold1);
+    held_tokens(hs, n, st, &p.hold0, &p.hold1);
     p.hold0 /= 32;
     p.hold1 = (p.hold1 + 31) / 32;
     static std::atomic<bool> attr_set[kMaxDevices];
@@ -444,7 +472,7 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
             n_rsb += Li.n_rsb;
             rp.rsb_end[i] = n_rsb;
         }
-        held_tokens(hs, n, &rp.hold0, &rp.hold1);
+        held_tokens(hs, n, st, &rp.hold0, &rp.hold1);
         rp.n_layers = n; rp.M = M; rp.K = L.K; rp.n_rsb = n_rsb; rp.block_bytes = L.block_bytes;
         const cudaError_t e = L.n_kc == 2 ? launch_gemv_rows<2>(h, rp, st) : L.n_kc == 4 ? launch_gemv_rows<4>(h, rp, st) : launch_gemv_rows<8>(h, rp, st);
         return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
@@ -1273,19 +1301,27 @@ extern "C" ql_status qlinear_kv_append_heads(const qlinear_t* hk, const qlinear_
         prm.k_scales[i] = reinterpret_cast<__half*>(kb + K.chan_scale_offset);
         prm.v_body[i] = vb + V.body_offset;
         prm.v_scale[i] = static_cast<__half*>(v_scales[i]);
-        const uint64_t range = (uint64_t)(uint32_t)(pos + n_new) << 32 | (uint32_t)pos;
-        for (qlinear_s* h : {hk[i], hv[i]}) {
-            h->cache.store(true, std::memory_order_relaxed);
-            h->appended.store(range, std::memory_order_relaxed);
-        }
     }
     prm.k_new = static_cast<const __half*>(k_new);
     prm.v_new = static_cast<const __half*>(v_new);
     prm.head_stride = head_stride; prm.token_stride = token_stride;
     prm.d_h = K.K; prm.cache_size = K.N; prm.pos = pos; prm.n_new = n_new;
     prm.k_n_kc = K.n_kc; prm.v_n_kc = V.n_kc;
-    const cudaError_t e = launch(kv_append_kernel, prm, dim3(n_new, n_heads), dim3(64), 0, static_cast<cudaStream_t>(stream), 1, hk[0]->pdl);
-    return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    unsigned long long capture;
+    const bool known = capture_of(st, &capture);
+    std::lock_guard<std::mutex> lock(g_append_mutex[hk[0]->device]);
+    if (launch(kv_append_kernel, prm, dim3(n_new, n_heads), dim3(64), 0, st, 1, hk[0]->pdl) != cudaSuccess) {
+        cudaGetLastError();                                              // nothing is in flight: the append before it stays the last one
+        return QL_ERR_CUDA;
+    }
+    for (int i = 0; i < n_heads; ++i)
+        for (qlinear_s* h : {hk[i], hv[i]}) {
+            const bool joined = capture && h->append.capture == capture && (h->append.stream != st || !h->append.alone);
+            h->append = {pos, pos + n_new, st, capture, known && !joined};
+            h->cache.store(true, std::memory_order_relaxed);
+        }
+    return QL_OK;
 }
 
 extern "C" ql_status qlinear_kv_append(qlinear_t hk, qlinear_t hv, const void* k_new, const void* v_new, void* v_scale,
@@ -1688,6 +1724,17 @@ extern "C" int32_t qlinear_debug_plan_kv_output(qlinear_t h, int32_t n_heads, in
     const int n = n_out < 4 ? n_out : 4;
     for (int i = 0; i < n; ++i) out[i] = v[i];
     return n;
+}
+
+extern "C" ql_status qlinear_debug_kv_hold(const qlinear_t* hs, int32_t n, void* stream, int32_t* first, int32_t* end)
+{
+    if (!hs || !first || !end || n < 1 || n > kGemvMaxBatch) return QL_ERR_INVALID_ARG;
+    for (int i = 0; i < n; ++i)
+        if (!hs[i] || hs[i]->device != hs[0]->device) return QL_ERR_INVALID_ARG;
+    DeviceGuard guard(hs[0]->device);
+    if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
+    held_tokens(hs, n, static_cast<cudaStream_t>(stream), first, end);
+    return QL_OK;
 }
 
 extern "C" int32_t qlinear_debug_takes_batch_kernel(const qlinear_t* hs, int32_t n, int32_t M)
