@@ -114,7 +114,8 @@ ql_status qlinear_create(const qlinear_desc* desc, const void* packed_dev, int d
  * decode kernel, larger M a matrix-multiply kernel (Section 3.7; qlinear_path_for): up to 64 tokens, and on layers too small to
  * fill the prefill kernel's tiles beyond, a kernel for a batch of tokens (one with warp-level MMAs for few weights, one with the
  * weights in tensor memory for more), else the prefill kernel.  The environment variable QLINEAR_MID_MAX_M lowers the token count from
- * which calls of up to 64 tokens go to the prefill kernel (0: all of them).  int8 layers of K = 64, 128 or 256 have kernels of
+ * which calls of up to 64 tokens go to the prefill kernel (0: all of them); QLINEAR_GEMM_NARROW=0 leaves the kernel with the
+ * weights in tensor memory out at every token count, 2 takes it wherever it can serve the call (1, the default: where it is faster).  int8 layers of K = 64, 128 or 256 have kernels of
  * their own, for M <= 8 and for any larger M.
  * Errors: QL_ERR_INVALID_ARG (null / misaligned pointers, M < 1, M*K or M*N beyond 2^31-1 elements),
  * QL_ERR_CUDA (launch failure, reported synchronously), QL_ERR_DEVICE_TIMEOUT (an earlier kernel of this
@@ -376,12 +377,27 @@ uint32_t qlinear_version(void);
  * cluster, chunks per warp, clusters of the launch, clusters that run at once}.  qlinear_debug_takes_batch_kernel returns 1 if a
  * forward call (n = 1) or a group of these layers on M tokens belongs to the batch stage by its size (calls beyond it belong to the
  * prefill stage, whose choice of kernel includes the batch kernel with the weights in tensor memory).
+ * qlinear_debug_route evaluates, without a device, the dispatch of a call beyond the decode stage on layers like these (n = 1: forward, more:
+ * a group, gated: a pair) on a GPU of num_sms SMs; up to n_out of {the kernel (ql_kernel); its tokens per tile and K parts (NARROW, PAIR_TA, SINGLE;
+ * else 0 and 1); the estimates behind the choice in ns: NARROW, the prefill kernels}; returns how many it wrote (0 on bad arguments).
  * qlinear_debug_kv_hold gives the tokens [*first, *end) of n caches that a decode reader of theirs on this stream would leave until the
  * kernel before it is complete: those of the last append if that was enqueued on the same stream and in the same capture, all of
  * them (an *end beyond any cache) if it was enqueued elsewhere, none for layers that nothing was appended to. */
 int32_t qlinear_debug_plan(qlinear_t h, int32_t M, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_plan_kv_output(qlinear_t h_v, int32_t n_heads, int32_t* out, int32_t n_out);
 int32_t qlinear_debug_takes_batch_kernel(const qlinear_t* hs, int32_t n, int32_t M);
+typedef enum {
+    QL_KERNEL_DECODE = 1,    /* M <= 8 */
+    QL_KERNEL_ROWS = 2,      /* int8, K = 64, 128 or 256 */
+    QL_KERNEL_ROWS_TC = 3,   /*   the same, the tensor-core form for many rows */
+    QL_KERNEL_MID = 4,       /* batch of tokens, warp-level MMAs */
+    QL_KERNEL_NARROW = 5,    /* batch of tokens and small layers, weights in tensor memory */
+    QL_KERNEL_PAIR_TA = 6,   /* prefill, CTA pairs, weights in tensor memory */
+    QL_KERNEL_PAIR = 7,      /* prefill, CTA pairs, weights through shared memory */
+    QL_KERNEL_SINGLE = 8,    /* prefill, single CTA */
+    QL_KERNEL_SEPARATE = 9   /* a group: one call per layer; a gated pair: two projections and an element-wise product */
+} ql_kernel;
+int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_t M, int32_t gated, int32_t num_sms, int32_t* out, int32_t n_out);
 ql_status qlinear_debug_kv_hold(const qlinear_t* hs, int32_t n, void* stream, int32_t* first, int32_t* end);
 uint32_t qlinear_debug_config_reads(void);
 

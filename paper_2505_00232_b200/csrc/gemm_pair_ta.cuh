@@ -88,13 +88,15 @@ struct TaMaps {
 
 // The packed body of a layer as a 2-D tensor of 64-byte rows; box = the block(s) of one 64-k step.
 // wide: the box of a 128-k step (two int4 blocks or four int8 blocks): the integer form and gemm_narrow.cuh.
+inline int w_map_box_rows(const Layout& L, bool wide) { return (wide ? 2 : 1) * (L.bits == 4 ? L.block_bytes / 64 : 2 * (kWeightBlockBytes / 64)); }
+inline int64_t w_map_rows(const Layout& L) { return (int64_t)L.n_rsb * L.n_kc * (L.block_bytes / 64); }
+inline bool w_map_fits(const Layout& L, bool wide) { return w_map_rows(L) >= w_map_box_rows(L, wide) && w_map_rows(L) <= 0x7FFFFFFFll; }
 inline bool w_tensor_map(const Layout& L, const uint8_t* blob, CUtensorMap* out, bool wide = false)
 {
     EncodeTiledFn enc = get_encode_tiled();
-    if (!enc) return false;
-    const int64_t rows = (int64_t)L.n_rsb * L.n_kc * (L.block_bytes / 64);
-    const int box_rows = (wide ? 2 : 1) * (L.bits == 4 ? L.block_bytes / 64 : 2 * (kWeightBlockBytes / 64));
-    if (rows < box_rows || rows > 0x7FFFFFFFll) return false;
+    if (!enc || !w_map_fits(L, wide)) return false;
+    const int64_t rows = w_map_rows(L);
+    const int box_rows = w_map_box_rows(L, wide);
     const cuuint64_t gdim[2] = {64, (cuuint64_t)rows};
     const cuuint64_t gstr[1] = {64};
     const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
@@ -691,6 +693,15 @@ inline int gemm_pair_ta_split(int tiles, int n_ksteps, int num_sms, bool have_sc
     return split;
 }
 
+// Tokens per tile: M in as few blocks of at most 256 as it takes, all of the same width (the MMA's N, a multiple of 32).  A
+// narrower tile costs the same dequantisation and less tensor-core time, x traffic and epilogue
+// (a Llama block at 100 tokens 145.9 -> 136.9 us, at 300 224.9 -> 211.1).
+inline int gemm_pair_ta_width(int M)
+{
+    const int n_mblk = (M + 255) / 256;
+    return ((M + n_mblk - 1) / n_mblk + 31) / 32 * 32;
+}
+
 // act < 0: the plain form.  act >= 0: the gated form, set = {gate, up} of equal shape, y[0] the output.
 // scratch / counters: the device's shared fp32 scratch and arrival counters for the K-split case (null: no split).
 // a8_scale != nullptr: the integer form; x is then the int8 activations, a8_scale / a8_rowsum their per-token arrays, and
@@ -703,11 +714,8 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const void* x, int M, c
     using S = GemmTaSmem<BITS, I8>;
     const Layout& L = *set.L[0];
     TaMaps maps;
-    // Tokens per tile: M in as few blocks of at most 256 as it takes, all of the same width (the MMA's N, a multiple of 32).  A
-    // narrower tile costs the same dequantisation and less tensor-core time, x traffic and epilogue
-    // (a Llama block at 100 tokens 145.9 -> 136.9 us, at 300 224.9 -> 211.1).
-    // The integer form keeps 256: it gains nothing at 300 tokens, and its epilogue is short of registers.
-    const int n_mblk = (M + 255) / 256, bn = I8 ? 256 : ((M + n_mblk - 1) / n_mblk + 31) / 32 * 32;
+    // The integer form keeps 256 tokens: a narrower tile gains nothing at 300 tokens, and its epilogue is short of registers.
+    const int n_mblk = (M + 255) / 256, bn = I8 ? 256 : gemm_pair_ta_width(M);
     if (!x_tensor_map(x, L.K, M, bn / 2, &maps.x, I8 ? 1 : 2)) return QL_ERR_CUDA;
     for (int i = 0; i < kGemmMaxGroup; ++i) maps.w[i] = *set.wmap[i < set.n ? i : 0];
     auto kern = gemm_pair_ta_kernel<BITS, GROUPED, GATED, I8>;
@@ -819,16 +827,6 @@ inline ql_status gemm_pair_ta_forward_i8(const GemmPairLayers& set, const void* 
     const Layout& L = *set.L[0];
     if (L.bits == 8) return gemm_pair_ta_launch<8, false, false, true>(set, xq, M, st, device, pdl, num_sms, -1, nullptr, nullptr, scale, rowsum);
     return gemm_pair_ta_launch<4, false, false, true>(set, xq, M, st, device, pdl, num_sms, -1, nullptr, nullptr, scale, rowsum);
-}
-
-// The CTA-pair prefill call: the tensor-memory form where it applies, else the shared-memory form.
-inline ql_status gemm_pair_forward_auto(const GemmPairLayers& set, const void* x, int M, cudaStream_t st,
-                                        int device, bool pdl, int num_sms, float* scratch, unsigned int* counters)
-{
-    if (gemm_pair_ta_applicable(set, M, num_sms)) return gemm_pair_ta_forward(set, x, M, st, device, pdl, num_sms, scratch, counters);
-    for (int i = 0; i < set.n; ++i)
-        if (!gemm_pair_applicable(*set.L[i], M)) return QL_ERR_UNSUPPORTED;
-    return gemm_pair_forward(set, x, M, st, device, pdl, num_sms, scratch, counters);
 }
 
 }  // namespace ql

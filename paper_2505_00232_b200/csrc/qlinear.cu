@@ -57,6 +57,7 @@ struct Config {
     bool oversubscribe;      // QLINEAR_GEMV_OVERSUBSCRIBE=0: the group-scaled int4 decode kernel never takes more CTAs than fit at once
     int force_ks;            // QLINEAR_GEMV_KS: forced K split of the cluster decode kernel (0 = planned)
     int mid_max_m;           // QLINEAR_MID_MAX_M: largest M up to 64 that the kernels for a batch of tokens may serve (0: none); see takes_mid, narrow_is_faster
+    int narrow;              // QLINEAR_GEMM_NARROW: 0 gemm_narrow.cuh serves no call, 1 by the rules (default), 2 every call that it can serve
     bool xdirect;            // QLINEAR_GEMV_XDIRECT: x fragments straight from global memory
     int kernel;              // QLINEAR_GEMV_KERNEL: 0 / 1 cluster kernel (default), 2 streaming kernel
     int stream_ctas_per_sm, stream_stages;
@@ -76,6 +77,7 @@ void load_config()
     c.oversubscribe = env_int("QLINEAR_GEMV_OVERSUBSCRIBE", 1) != 0;
     c.force_ks = env_int("QLINEAR_GEMV_KS", 0);
     c.mid_max_m = env_int("QLINEAR_MID_MAX_M", 64);
+    c.narrow = env_int("QLINEAR_GEMM_NARROW", 1);
     c.xdirect = env_int("QLINEAR_GEMV_XDIRECT", 1) != 0;
     const char* kc = std::getenv("QLINEAR_GEMV_KERNEL");
     c.kernel = !kc ? 0 : !std::strcmp(kc, "cluster") ? 1 : !std::strcmp(kc, "stream") ? 2 : 0;
@@ -624,12 +626,13 @@ double prefill_us(const qlinear_s* const* hs, int n, int M, bool gated, int num_
 // (QLINEAR_MID_MAX_M < M <= 64: the prefill kernels, whatever the estimate.)
 bool narrow_is_faster(const qlinear_s* const* hs, int n, int M, bool gated = false)
 {
-    if (M <= 64 && M > config().mid_max_m) return false;
+    if ((M <= 64 && M > config().mid_max_m) || config().narrow == 0) return false;
     int rows = 0;
     for (int i = 0; i < n; ++i) {
         if (!hs[i]->wmap_wide_ok) return false;
         rows += hs[i]->L.n_rsb;
     }
+    if (config().narrow == 2) return true;
     return plan_narrow(hs[0]->L, gated ? hs[0]->L.n_rsb : rows, gated, M, hs[0]->num_sms).us < 0.9 * prefill_us(hs, n, M, gated, hs[0]->num_sms);
 }
 
@@ -698,23 +701,23 @@ cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, bool pdl, 
 //   117 M (Llama gate + up)        26.0 / 22.7  31.9 / 23.2  37.0 / 23.6
 bool batch_takes_narrow(const qlinear_s* const* hs, int n, int M, bool gated)
 {
+    if (config().narrow == 0) return false;
     int64_t weights = 0;
     for (int i = 0; i < n; ++i) {
         if (!hs[i]->wmap_wide_ok) return false;
         weights += (int64_t)hs[i]->L.N * hs[i]->L.K;
     }
+    if (config().narrow == 2) return true;
     return weights >= (M <= 16 ? 50000000 : M <= 24 ? (gated ? 50000000 : 20000000) : M <= 32 ? (gated ? 50000000 : 8000000) : M <= 48 ? 4000000 : 1500000);
 }
 
-// n layers that share K and scheme, layer i on xs[i] (one x for all of them on gemm_narrow.cuh, as in every call but the value product);
-// act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
+// n layers that share K and scheme, layer i on xs[i]; act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
 // kscales != nullptr (int8 layers): layer i's input is multiplied by kscales[i][0 .. K).
 ql_status forward_mid(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st, int act = -1,
                       const void* const* kscales = nullptr)
 {
     const qlinear_s* h = hs[0];
     const Layout& L = h->L;
-    if (!kscales && batch_takes_narrow(hs, n, M, act >= 0)) return forward_narrow(hs, n, xs[0], ys, M, st, act);
     MidParams prm{};
     int units = 0;
     for (int i = 0; i < n; ++i) {
@@ -781,6 +784,17 @@ cudaError_t launch_gemm_rows_tc(const qlinear_s* h, const GemmRowsMaps& maps, Ge
     cfg.numAttrs = h->pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, maps, prm);
 }
+
+// Which of the two kernels for short K a layer takes, the smallest of those in one launch: the tensor-core form has the longer ramp and the
+// faster tiles, and another order of sums inside an MMA.  The rule looks at one layer, so that a head gets the same bits alone and among
+// others: from the tiles of 128 x 64 on at which one layer alone is even.  Measured, us gemm_rows_kernel / gemm_rows_tc_kernel, one layer:
+// d_h = 64, 1024 tiles 8.1 / 7.8; d_h = 128, 512 7.1 / 7.2, 1024 11.4 / 9.0; d_h = 256, 512 10.4 / 9.9, 1024 18.1 / 11.7; eight layers: d_h = 64,
+// 512 tiles each 23.9 / 20.6, d_h = 128 34.8 / 24.1, d_h = 256 58.6 / 28.1.
+bool rows_take_tc(int layer_rsb, int n_kc, int M, int num_sms)
+{
+    return (int64_t)layer_rsb * ((M + kRowsTcTokens - 1) / kRowsTcTokens) * 20 >= num_sms * (n_kc == 2 ? 138 : n_kc == 4 ? 69 : 60);
+}
+
 ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st)
 {
     const qlinear_s* h = hs[0];
@@ -799,13 +813,9 @@ ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const
     prm.n_layers = n; prm.M = M;
     const bool pdl = h->pdl;                                             // (every byte is read after griddepcontrol.wait)
     const int n_kc = h->L.n_kc;
-    // The tensor-core form has the longer ramp and the faster tiles, and another order of sums inside an MMA.  The rule looks at one layer, so
-    // that a head gets the same bits alone and among others: from the tiles of 128 x 64 on at which one layer alone is even.  Measured,
-    // us gemm_rows_kernel / this, one layer: d_h = 64, 1024 tiles 8.1 / 7.8; d_h = 128, 512 7.1 / 7.2, 1024 11.4 / 9.0; d_h = 256, 512 10.4 / 9.9,
-    // 1024 18.1 / 11.7; eight layers: d_h = 64, 512 tiles each 23.9 / 20.6, d_h = 128 34.8 / 24.1, d_h = 256 58.6 / 28.1.
     int layer_rsb = h->L.n_rsb;
     for (int i = 1; i < n; ++i) layer_rsb = std::min(layer_rsb, hs[i]->L.n_rsb);
-    if ((int64_t)layer_rsb * ((M + kRowsTcTokens - 1) / kRowsTcTokens) * 20 >= h->num_sms * (n_kc == 2 ? 138 : n_kc == 4 ? 69 : 60)) {
+    if (rows_take_tc(layer_rsb, n_kc, M, h->num_sms)) {
         GemmRowsMaps maps;
         for (int i = 0; i < kRowsMaxLayers; ++i)
             if (!x_tensor_map(xs[i < n ? i : 0], h->L.K, M, kRowsTcTokens, &maps.x[i])) return QL_ERR_CUDA;
@@ -816,6 +826,38 @@ ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const
     const cudaError_t e = n_kc == 2 ? launch_gemm_rows<2>(h, prm, n_rsb, pdl, st) : n_kc == 4 ? launch_gemm_rows<4>(h, prm, n_rsb, pdl, st) : launch_gemm_rows<8>(h, prm, n_rsb, pdl, st);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
+GemmPairLayers pair_layers(const qlinear_s* const* hs, int n, void* const* ys)
+{
+    GemmPairLayers set{};
+    set.n = n;
+    set.late = any_cache(hs, n);
+    for (int i = 0; i < n; ++i) {
+        set.L[i] = &hs[i]->L; set.blob[i] = hs[i]->blob; set.y[i] = ys ? ys[i] : nullptr;
+        set.wmap[i] = hs[i]->wmap_ok ? &hs[i]->wmap : nullptr;
+    }
+    return set;
+}
+
+// The unfused gating route's two projections fit the device's scratch.
+bool gate_fits_scratch(int N, int M, int num_sms) { return (size_t)M * N * 2 * sizeof(__half) <= gemm_pair_scratch_bytes(num_sms); }
+
+// The kernel of a call beyond the decode stage: one layer, n > 1 layers that share x, or (gated) a pair.
+ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
+{
+    const Layout& L = hs[0]->L;
+    const int sms = hs[0]->num_sms;
+    if (n == 1 && takes_rows(L)) return rows_take_tc(L.n_rsb, L.n_kc, M, sms) ? QL_KERNEL_ROWS_TC : QL_KERNEL_ROWS;
+    if (takes_mid(hs, n, M, gated)) return batch_takes_narrow(hs, n, M, gated) ? QL_KERNEL_NARROW : QL_KERNEL_MID;
+    // (a pair whose unfused product does not fit the scratch has only ever been served by the fused kernels of the prefill stage)
+    if ((!gated || gate_fits_scratch(L.N, M, sms) || gemm_pair_applicable(L, M)) && narrow_is_faster(hs, n, M, gated)) return QL_KERNEL_NARROW;
+    const GemmPairLayers set = pair_layers(hs, n, nullptr);
+    if (gated && !gemm_pair_applicable(L, M)) return QL_KERNEL_SEPARATE;
+    if (gemm_pair_ta_applicable(set, M, sms, gated)) return QL_KERNEL_PAIR_TA;
+    for (int i = 0; i < n; ++i)
+        if (!gemm_pair_applicable(hs[i]->L, M)) return n > 1 ? QL_KERNEL_SEPARATE : QL_KERNEL_SINGLE;
+    return QL_KERNEL_PAIR;
 }
 
 // y = act(g) * u, element-wise (the unfused form of the gating, for shapes the fused kernels do not take).
@@ -867,6 +909,17 @@ ql_status forward_gemv_stream(const qlinear_s* h, const void* x, void* y, int M,
     else if (L.grouped) e = launch_stream<4, true>(h, prm, st);
     else e = launch_stream<4, false>(h, prm, st);
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
+// The CTA-pair prefill kernels: `kernel` says which (QL_KERNEL_PAIR_TA, QL_KERNEL_PAIR); act >= 0: both accumulators for a gated pair.
+ql_status forward_pair(const qlinear_s* const* hs, int n, ql_kernel kernel, const void* x, void* const* ys, int M, cudaStream_t st, int act = -1)
+{
+    const qlinear_s* h = hs[0];
+    const GemmPairLayers set = pair_layers(hs, n, ys);
+    if (act >= 0) return kernel == QL_KERNEL_PAIR_TA ? gemm_pair_ta_forward_gated(set, x, M, act, st, h->device, h->pdl, h->num_sms)
+                                                     : gemm_pair_forward_gated(set, x, M, act, st, h->device, h->pdl, h->num_sms);
+    return kernel == QL_KERNEL_PAIR_TA ? gemm_pair_ta_forward(set, x, M, st, h->device, h->pdl, h->num_sms, h->dev->gemm_scratch, h->dev->gemm_counters)
+                                       : gemm_pair_forward(set, x, M, st, h->device, h->pdl, h->num_sms, h->dev->gemm_scratch, h->dev->gemm_counters);
 }
 
 // ---- debug: the integers as the device unpack routines see them
@@ -1048,17 +1101,16 @@ extern "C" ql_status qlinear_forward(qlinear_t h, const void* x, void* y, int32_
         if (h->use_stream) return forward_gemv_stream(h, x, y, M, st);
         return forward_gemv(&h, 1, x, &y, M, st, -1, takes_rows(h->L) ? &x : nullptr);   // (short K: the persistent form, see there)
     }
-    if (takes_rows(h->L)) return forward_gemm_rows(&h, 1, &x, &y, M, st);
-    if (takes_mid(&h, 1, M)) return forward_mid(&h, 1, &x, &y, M, st);
-    if (narrow_is_faster(&h, 1, M)) return forward_narrow(&h, 1, x, &y, M, st);
-    {
-        GemmPairLayers set{};
-        set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_ok ? &h->wmap : nullptr;
-        set.late = any_cache(&h, 1);
-        const ql_status s = gemm_pair_forward_auto(set, x, M, st, h->device, h->pdl, h->num_sms, h->dev->gemm_scratch, h->dev->gemm_counters);
-        if (s != QL_ERR_UNSUPPORTED) return s;                           // (an odd number of row super-blocks: the single-CTA kernel)
+    const ql_kernel kernel = gemm_route(&h, 1, M, false);
+    switch (kernel) {
+        case QL_KERNEL_ROWS:
+        case QL_KERNEL_ROWS_TC: return forward_gemm_rows(&h, 1, &x, &y, M, st);
+        case QL_KERNEL_MID: return forward_mid(&h, 1, &x, &y, M, st);
+        case QL_KERNEL_NARROW: return forward_narrow(&h, 1, x, &y, M, st);
+        case QL_KERNEL_PAIR_TA:
+        case QL_KERNEL_PAIR: return forward_pair(&h, 1, kernel, x, &y, M, st);
+        default: return gemm_forward(h->L, h->blob, x, y, M, st, h->device, h->pdl, h->num_sms, any_cache(&h, 1));
     }
-    return gemm_forward(h->L, h->blob, x, y, M, st, h->device, h->pdl, h->num_sms, any_cache(&h, 1));
 }
 
 extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const void* x, void* const* ys, int32_t M, void* stream)
@@ -1078,34 +1130,16 @@ extern "C" ql_status qlinear_forward_group(const qlinear_t* hs, int32_t n, const
         if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
         return forward_gemv(const_cast<qlinear_s* const*>(hs), n, x, ys, M, static_cast<cudaStream_t>(stream));
     }
-    if (n > 1 && M > hs[0]->gemv_max_m && takes_mid(hs, n, M)) {
-        DeviceGuard guard(hs[0]->device);
-        if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
-        const void* xs[kGemvMaxGroup];
-        for (int i = 0; i < n; ++i) xs[i] = x;
-        return forward_mid(const_cast<const qlinear_s* const*>(hs), n, xs, ys, M, static_cast<cudaStream_t>(stream));
-    }
-    if (n > 1 && M > hs[0]->gemv_max_m && narrow_is_faster(hs, n, M)) {
-        DeviceGuard guard(hs[0]->device);
-        if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
-        return forward_narrow(const_cast<const qlinear_s* const*>(hs), n, x, ys, M, static_cast<cudaStream_t>(stream));
-    }
-    if (n > 1 && M > hs[0]->gemv_max_m) {                                // prefill: one launch of the CTA-pair kernel
-        bool pair_ok = true;
-        for (int i = 0; i < n; ++i) pair_ok = pair_ok && (hs[i]->L.n_rsb % 2) == 0 && (gemm_pair_applicable(hs[i]->L, M) || (hs[i]->wmap_ok && gemm_config().ta));
-        if (pair_ok) {
+    if (n > 1 && M > hs[0]->gemv_max_m) {
+        const ql_kernel kernel = gemm_route(hs, n, M, false);
+        if (kernel != QL_KERNEL_SEPARATE) {
             DeviceGuard guard(hs[0]->device);
             if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
-            GemmPairLayers set{};
-            set.n = n;
-            set.late = any_cache(hs, n);
-            for (int i = 0; i < n; ++i) {
-                set.L[i] = &hs[i]->L; set.blob[i] = hs[i]->blob; set.y[i] = ys[i];
-                set.wmap[i] = hs[i]->wmap_ok ? &hs[i]->wmap : nullptr;
-            }
-            const ql_status s = gemm_pair_forward_auto(set, x, M, static_cast<cudaStream_t>(stream), hs[0]->device, hs[0]->pdl, hs[0]->num_sms,
-                                                       hs[0]->dev->gemm_scratch, hs[0]->dev->gemm_counters);
-            if (s != QL_ERR_UNSUPPORTED) return s;
+            const void* xs[kGemvMaxGroup];
+            for (int i = 0; i < n; ++i) xs[i] = x;
+            if (kernel == QL_KERNEL_MID) return forward_mid(hs, n, xs, ys, M, static_cast<cudaStream_t>(stream));
+            if (kernel == QL_KERNEL_NARROW) return forward_narrow(hs, n, x, ys, M, static_cast<cudaStream_t>(stream));
+            return forward_pair(hs, n, kernel, x, ys, M, static_cast<cudaStream_t>(stream));
         }
     }
     for (int i = 0; i < n; ++i) {
@@ -1156,30 +1190,21 @@ extern "C" ql_status qlinear_forward_gated(qlinear_t hg, qlinear_t hu, const voi
     if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     qlinear_s* hs[2] = {hg, hu};
-    // the unfused route's product of this size fits the scratch (where it does not, only the fused kernels of the prefill stage serve the call)
-    const int64_t n = (int64_t)M * a.N;
-    const bool fits = (size_t)n * 2 * sizeof(__half) <= gemm_pair_scratch_bytes(hg->num_sms);
     if (M <= hg->gemv_max_m && !hg->use_stream) {                        // decode: both branches in one launch
         void* ys[2] = {y, y};
         const ql_status s = forward_gemv(hs, 2, x, ys, M, st, act);
         if (s != QL_ERR_UNSUPPORTED) return s;
-    } else if (M > hg->gemv_max_m && takes_mid(hs, 2, M, true)) {
+    } else if (M > hg->gemv_max_m) {
+        const ql_kernel kernel = gemm_route(hs, 2, M, true);
         const void* xs[2] = {x, x};
-        return forward_mid(hs, 2, xs, &y, M, st, act);
-    } else if (M > hg->gemv_max_m && (fits || gemm_pair_applicable(a, M)) && narrow_is_faster(hs, 2, M, true)) {
         void* ys[2] = {y, y};
-        return forward_narrow(hs, 2, x, ys, M, st, act);
-    } else if (M > hg->gemv_max_m && gemm_pair_applicable(a, M)) {       // prefill: both accumulators of the CTA-pair kernel
-        GemmPairLayers set{};
-        set.n = 2;
-        set.late = any_cache(hs, 2);
-        set.L[0] = &hg->L; set.blob[0] = hg->blob; set.y[0] = y; set.wmap[0] = hg->wmap_ok ? &hg->wmap : nullptr;
-        set.L[1] = &hu->L; set.blob[1] = hu->blob; set.y[1] = y; set.wmap[1] = hu->wmap_ok ? &hu->wmap : nullptr;
-        if (gemm_pair_ta_applicable(set, M, hg->num_sms, true)) return gemm_pair_ta_forward_gated(set, x, M, act, st, hg->device, hg->pdl, hg->num_sms);
-        return gemm_pair_forward_gated(set, x, M, act, st, hg->device, hg->pdl, hg->num_sms);
+        if (kernel == QL_KERNEL_MID) return forward_mid(hs, 2, xs, &y, M, st, act);
+        if (kernel == QL_KERNEL_NARROW) return forward_narrow(hs, 2, x, ys, M, st, act);
+        if (kernel != QL_KERNEL_SEPARATE) return forward_pair(hs, 2, kernel, x, ys, M, st, act);
     }
     // Unfused: the two projections into the device's shared scratch, then the element-wise product.
-    if (!fits) return QL_ERR_UNSUPPORTED;
+    if (!gate_fits_scratch(a.N, M, hg->num_sms)) return QL_ERR_UNSUPPORTED;
+    const int64_t n = (int64_t)M * a.N;
     __half* g = reinterpret_cast<__half*>(hg->dev->gemm_scratch);
     __half* u = g + ((n + 7) & ~(int64_t)7);
     void* ys[2] = {g, u};
@@ -1724,6 +1749,39 @@ extern "C" int32_t qlinear_debug_plan_kv_output(qlinear_t h, int32_t n_heads, in
     const int n = n_out < 4 ? n_out : 4;
     for (int i = 0; i < n; ++i) out[i] = v[i];
     return n;
+}
+
+extern "C" int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_t M, int32_t gated, int32_t num_sms, int32_t* out, int32_t n_out)
+{
+    if (!ds || n < 1 || n > kGemvMaxGroup || M < 1 || num_sms < 2 || !out || (gated && n != 2)) return 0;
+    qlinear_s layers[kGemvMaxGroup];                                     // (host state only; nothing reads their device pointers)
+    const qlinear_s* hs[kGemvMaxGroup];
+    int rows = 0;
+    for (int i = 0; i < n; ++i) {
+        qlinear_s& h = layers[i];
+        if (!make_layout(ds[i].N, ds[i].K, ds[i].bits, ds[i].group, &h.L)) return 0;
+        if (h.L.K != layers[0].L.K || h.L.bits != layers[0].L.bits || h.L.group != layers[0].L.group || (gated && h.L.N != layers[0].L.N)) return 0;
+        h.num_sms = num_sms;
+        h.wmap_ok = w_map_fits(h.L, false);
+        h.wmap_wide_ok = w_map_fits(h.L, true);
+        hs[i] = &h;
+        rows += h.L.n_rsb;
+    }
+    if (M <= config().gemv_max_m) { out[0] = QL_KERNEL_DECODE; return 1; }
+    const Layout& L = layers[0].L;
+    const NarrowPlan pl = plan_narrow(L, gated ? L.n_rsb : rows, gated, M, num_sms);
+    const ql_kernel kernel = gemm_route(hs, n, M, gated);
+    int32_t width = 0, parts = 1;
+    if (kernel == QL_KERNEL_NARROW) { width = pl.bn; parts = pl.cl; }
+    if (kernel == QL_KERNEL_SINGLE) width = gemm_pick_bn(L, M, num_sms);
+    if (kernel == QL_KERNEL_PAIR_TA) {
+        width = gemm_pair_ta_width(M);
+        if (!gated) parts = gemm_pair_ta_split(rows / 2 * ((M + 255) / 256), (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, true);
+    }
+    const int32_t v[5] = {kernel, width, parts, (int32_t)(1000 * pl.us), (int32_t)(1000 * prefill_us(hs, n, M, gated, num_sms))};
+    const int k = n_out < 5 ? n_out : 5;
+    for (int i = 0; i < k; ++i) out[i] = v[i];
+    return k;
 }
 
 extern "C" ql_status qlinear_debug_kv_hold(const qlinear_t* hs, int32_t n, void* stream, int32_t* first, int32_t* end)

@@ -53,13 +53,14 @@ def assert_gated(y, x, gate_w, up_w, group, act, rows=2048):
 
 
 CASES = [
-    # (M, N, K, bits, group, act): decode (fused in one launch), a batch of tokens (fused), prefill (fused in the CTA-pair kernel:
-    # M > 128 and a multiple of 256 channels after padding), and shapes that take the unfused route
+    # (M, N, K, bits, group, act): decode (fused in one launch), a batch of tokens (fused), prefill, and shapes that take the unfused route.
+    # All above 64 tokens are small enough for the batch kernel; test_routes_gpu.py leaves it out: then four of them run in the CTA-pair
+    # kernel (M > 128 and a multiple of 256 channels after padding) and two are unfused
     (1, 2048, 4096, 4, 32, "silu"), (4, 1160, 2304, 4, 32, "gelu_tanh"), (8, 520, 1024, 8, 0, "silu"), (3, 264, 512, 4, 0, "identity"),
     (2, 200, 352, 4, 32, "silu"),                                        # K not a whole number of int4 chunks: unfused
     (300, 512, 1024, 4, 32, "silu"), (1024, 256, 2304, 4, 32, "gelu_tanh"), (257, 1000, 512, 8, 0, "silu"), (700, 768, 384, 4, 0, "identity"),
     (24, 264, 256, 4, 32, "silu"),                                       # a batch of tokens
-    (128, 384, 512, 8, 0, "gelu_tanh"), (200, 384, 512, 4, 32, "silu"),   # unfused: more tokens than a batch and M <= 128, odd tile count
+    (128, 384, 512, 8, 0, "gelu_tanh"), (200, 384, 512, 4, 32, "silu"),   # (unfused there: M <= 128, odd tile count)
 ]
 
 

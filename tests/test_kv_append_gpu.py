@@ -69,7 +69,10 @@ def test_products_of_tokens_appended_just_before(P, torch, n_heads, d_h, cache, 
         assert ok, (h, rel, worst)
 
 
-@pytest.mark.parametrize("n_heads,d_h,cache,R", [(4, 96, 16384, 64), (2, 96, 15680, 49), (1, 96, 41728, 33), (2, 32, 46880, 64), (2, 160, 16384, 64)])
+BATCH = [(4, 96, 16384, 64), (2, 96, 15680, 49), (1, 96, 41728, 33), (2, 32, 46880, 64), (2, 160, 16384, 64)]
+
+
+@pytest.mark.parametrize("n_heads,d_h,cache,R", BATCH)
 def test_scores_of_a_batch_of_rows_see_the_scales_appended_just_before(P, torch, n_heads, d_h, cache, R):
     """Head dimensions that the row kernels do not take, so many positions that the batch kernel with the weights in tensor memory serves the
     scores in one K part, and (up to 128 of K) a step for one of its two groups of warps only: the other one waits for nothing before

@@ -54,16 +54,19 @@ def check(P, torch, N, K, bits, group, M, rows, act="silu"):
         assert torch.equal(gated, again) and torch.equal(one, lins[0].forward(xd))
 
 
-@pytest.mark.parametrize("bits,group", [(4, 32), (4, 0), (8, 0)])
-@pytest.mark.parametrize("M", [65, 96, 97, 128, 129, 300])
-@pytest.mark.parametrize("N,K", [(8, 160), (136, 352), (264, 1024), (640, 1152)])
-def test_small_layers(P, torch, M, N, K, bits, group):
+SMALL = [(N, K, bits, group, M) for N, K in ((8, 160), (136, 352), (264, 1024), (640, 1152)) for M in (65, 96, 97, 128, 129, 300)
+         for bits, group in ((4, 32), (4, 0), (8, 0))]
+LARGE = [(2304, 3776, 4, 32, 25), (2304, 4032, 4, 0, 32), (2312, 3712, 8, 0, 31), (2304, 9216, 4, 32, 17), (4096, 12544, 4, 32, 9),
+         (4104, 12576, 8, 0, 16), (1024, 4096, 4, 32, 33), (1032, 4000, 8, 0, 48), (1032, 1664, 4, 128, 49), (1032, 1568, 8, 0, 64), (14336, 1024, 4, 32, 64)]
+
+
+@pytest.mark.parametrize("N,K,bits,group,M", SMALL)
+def test_small_layers(P, torch, N, K, bits, group, M):
     """Several token blocks; K with a last half step (352 and 1152 are odd in 64 k), with 32 k of it (160, 352), a K split."""
     check(P, torch, N, K, bits, group, M, np.arange(N), "gelu_tanh" if M == 97 else "silu")
 
 
-@pytest.mark.parametrize("N,K,bits,group,M", [(2304, 3776, 4, 32, 25), (2304, 4032, 4, 0, 32), (2312, 3712, 8, 0, 31), (2304, 9216, 4, 32, 17), (4096, 12544, 4, 32, 9),
-                                              (4104, 12576, 8, 0, 16), (1024, 4096, 4, 32, 33), (1032, 4000, 8, 0, 48), (1032, 1664, 4, 128, 49), (1032, 1568, 8, 0, 64), (14336, 1024, 4, 32, 64)])
+@pytest.mark.parametrize("N,K,bits,group,M", LARGE)
 def test_large_layers_of_the_batch_stage(P, torch, N, K, bits, group, M):
     """Up to 64 tokens, where the number of weights calls for this kernel; int4 in groups up to 32 tokens: three groups."""
     check(P, torch, N, K, bits, group, M, np.r_[0:64, N - 72:N])

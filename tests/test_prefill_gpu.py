@@ -70,12 +70,15 @@ def rand_case(seed, M, N, K, bits, group):
 
 
 SMALL = [
-    # (M, N, K, bits, group): ragged M / N / K tails, every scheme.  Up to 64 tokens these run on the kernel for a batch of tokens;
-    # test_narrow_tiles runs them on the single-CTA kernel's tiles of 32 and 64 tokens.
+    # (M, N, K, bits, group): ragged M / N / K tails, every scheme.  Up to 64 tokens these run on the kernels for a batch of tokens;
+    # test_narrow_tiles runs them on the single-CTA kernel's tiles of 32 and 64 tokens.  Most of the others are small enough for the batch
+    # kernel with the weights in tensor memory; test_routes_gpu.py runs them all with that kernel left out, test_routes_cpu.py says what runs then.
     (9, 8, 32, 8, 0), (16, 128, 64, 4, 32), (17, 136, 160, 8, 0), (33, 200, 352, 4, 32), (64, 256, 512, 4, 0),
     (127, 264, 2304, 4, 32), (128, 128, 1056, 8, 0), (129, 384, 1024, 4, 32), (300, 520, 1056, 8, 0),
     (256, 40, 256, 4, 64), (257, 16, 384, 4, 128), (512, 1000, 96, 8, 0), (1024, 256, 2304, 4, 32),
     (700, 384, 4096, 8, 0), (2048, 128, 14336, 4, 32),
+    # enough tiles for 256 tokens each on the single-CTA kernel (an odd number of row super-blocks)
+    (1671, 11816, 64, 4, 32), (600, 4872, 160, 8, 0),
     # few tiles: the CTA-pair kernel splits K across clusters and adds the parts through scratch
     (600, 512, 2048, 8, 0), (300, 256, 4096, 4, 32), (1024, 1024, 1024, 4, 0),
 ]

@@ -89,8 +89,9 @@ def test_bit_identical_to_the_shared_memory_form(P, torch, tmp_path):
         assert np.array_equal(y.view(np.uint16), ref[str(i)].view(np.uint16)), f"case {c}"
 
 
-# Tiles of 32, 64, 96 and 128 tokens (one block of at most 128): whole along K, in two and in four parts.  A child process leaves the kernel
-# for a batch of tokens out, which takes most launches of up to 64 tokens before this one sees them.
+# Tiles of 32, 64, 96 and 128 tokens (one block of at most 128): whole along K, in two and in four parts.  A child process leaves the batch
+# stage out, which takes most launches of up to 64 tokens before this kernel sees them.  (By the rules these layers are the batch
+# kernel's, which test_routes_gpu.py switches off: the wider tiles, the small case of STRESS and the fallback below run there.)
 WIDTHS = [(M, N, K, bits, group) for M in (20, 33, 40, 64, 65, 96, 100, 128)
           for N, K, bits, group in ((512, 448, 4, 32), (504, 1024, 8, 0), (248, 2304, 4, 0), (768, 2304, 4, 32), (256, 4096, 8, 0))]
 WIDTHS_CHILD = """
@@ -119,7 +120,7 @@ def test_tile_widths_up_to_128_tokens(P, torch, tmp_path):
         y64, A, _ = O.linear(x, q, s, group)
         ok, rel, worst = O.check_against(got[str(i)], y64, A)
         assert ok, (c, rel, worst)
-        if M > 64:                                       # the same kernel without the switch
+        if M > 64:                                       # the same kernel without that switch
             assert np.array_equal(run(P, torch, *c, 7700 + M + N)[3].view(np.uint16), got[str(i)].view(np.uint16)), c
     for M in (20, 40, 96, 128):
         w = [case(7800 + i, M, 512, 2304, 4, 32) for i in range(2)]
@@ -130,7 +131,7 @@ def test_tile_widths_up_to_128_tokens(P, torch, tmp_path):
 
 
 def test_guard_band_around_y(P, torch):
-    """The output tile leaves through bulk copies of whole 256-byte rows: nothing outside [M, N] may be written."""
+    """The output tile leaves as 16-byte stores of whole 256-byte rows: nothing outside [M, N] may be written."""
     M, N, K, bits, group = 300, 19448, 128, 4, 32                        # ragged last row super-block (120 channels)
     q, s, x = case(11, M, N, K, bits, group)
     desc = P.Desc(N, K, bits, group)

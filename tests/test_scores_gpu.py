@@ -8,7 +8,10 @@ from oracle import qlinear_oracle as O
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n_heads,d_h,cache,T,R", [(2, 64, 8160, 8000, 1000), (3, 128, 4064, 3000, 1001), (9, 128, 2080, 2080, 2017), (2, 256, 992, 900, 4000), (1, 128, 160, 160, 20001)])
+CASES = [(2, 64, 8160, 8000, 1000), (3, 128, 4064, 3000, 1001), (9, 128, 2080, 2080, 2017), (2, 256, 992, 900, 4000), (1, 128, 160, 160, 20001)]
+
+
+@pytest.mark.parametrize("n_heads,d_h,cache,T,R", CASES)
 def test_scores_of_very_many_rows(_built_library, n_heads, d_h, cache, T, R):
     import torch
     import paper_2505_00232_b200 as P
