@@ -379,7 +379,7 @@ uint32_t qlinear_version(void);
  * prefill stage, whose choice of kernel includes the batch kernel with the weights in tensor memory).
  * qlinear_debug_route evaluates, without a device, the dispatch of a call beyond the decode stage on layers like these (n = 1: forward, more:
  * a group, gated: a pair) on a GPU of num_sms SMs; up to n_out of {the kernel (ql_kernel); its tokens per tile and K parts (NARROW, PAIR_TA, SINGLE;
- * else 0 and 1); the estimates behind the choice in ns: NARROW, the prefill kernels}; returns how many it wrote (0 on bad arguments).
+ * else 0 and 1); the estimates behind the choice in ns: NARROW, the kernel that takes the call otherwise}; returns how many it wrote (0 on bad arguments).
  * qlinear_debug_kv_hold gives the tokens [*first, *end) of n caches that a decode reader of theirs on this stream would leave until the
  * kernel before it is complete: those of the last append if that was enqueued on the same stream and in the same capture, all of
  * them (an *end beyond any cache) if it was enqueued elsewhere, none for layers that nothing was appended to. */

@@ -1,4 +1,4 @@
-// Kernel for a batch of 9 to 64 tokens on few weights (gemm_narrow.cuh takes more: batch_takes_narrow in qlinear.cu), and for products with few output channels and any number of tokens (the
+// Kernel for a batch of 9 to 64 tokens on few weights (gemm_narrow.cuh takes more: gemm_route in qlinear.cu), and for products with few output channels and any number of tokens (the
 // value product of an attention over a KV cache held as weights: N = d_h).  Between the two stages of paper Section 3.7:
 // too many tokens for the 8 MMA columns of the decode kernel, too few to fill the 256-token tiles of the prefill kernel,
 // which then multiplies padding and, with few tiles, leaves most SMs without work.
@@ -18,7 +18,7 @@
 //
 // Measured, weights out of HBM, against the 256-token-tile kernel that served these sizes: Llama gate + up 25.9 us at 16 tokens (47.3 before),
 // 37.0 at 32 (48.9); down (33 MB) 13.7 (26.6), 18.9 (28.7); q + k + v (25 MB of int8) 8.9 (19.2), 12.4 (20.5); one 2304 x 2304 int8 layer 4.5
-// (11.7), 6.0 (13.7).  Against gemm_narrow.cuh: see batch_takes_narrow in qlinear.cu.  Value product of 1024 rows over 4096 positions,
+// (11.7), 6.0 (13.7).  Against gemm_narrow.cuh: see gemm_route in qlinear.cu.  Value product of 1024 rows over 4096 positions,
 // d_h = 128: a pass over the probabilities for the scales and a single-CTA matmul on 8 CTAs 38.5 us, now 9.8.
 #pragma once
 #include <cooperative_groups.h>

@@ -22,7 +22,7 @@
 // Measured, us, weights out of HBM, the route before (gemm_mid.cuh to about 64 tokens, then the prefill kernels) / this one, int4 in groups
 // (qkv, o int8): Llama gate + up at 32 tokens 37.0 / 23.5, at 64 43.8 / 26.0; down 18.8 / 14.0, 27.9 / 15.8, at 128 29.3 / 22.7; q + k + v 12.3 /
 // 9.6, 18.1 / 11.9, 19.4 / 16.3; o at 128 tokens 19.1 / 12.2; Gemma2-2B down 12.8 / 9.6, 20.8 / 11.5, at 256 27.6 / 23.3; 1024 x 1024 at 128
-// tokens 12.4 / 5.4, at 512 16.0 / 7.3; a gated pair of 2688 x 1024 at 128 28.8 / 9.6.  The rule that picks it: narrow_is_faster in qlinear.cu.
+// tokens 12.4 / 5.4, at 512 16.0 / 7.3; a gated pair of 2688 x 1024 at 128 28.8 / 9.6.  The rule that picks it: gemm_route in qlinear.cu.
 #pragma once
 #include "gemm_pair_ta.cuh"
 

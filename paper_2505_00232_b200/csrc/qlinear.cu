@@ -56,7 +56,7 @@ struct Config {
     int warps_per_sm;        // QLINEAR_GEMV_WARPS_PER_SM: residency target of the cluster decode kernel
     bool oversubscribe;      // QLINEAR_GEMV_OVERSUBSCRIBE=0: the group-scaled int4 decode kernel never takes more CTAs than fit at once
     int force_ks;            // QLINEAR_GEMV_KS: forced K split of the cluster decode kernel (0 = planned)
-    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M up to 64 that the kernels for a batch of tokens may serve (0: none); see takes_mid, narrow_is_faster
+    int mid_max_m;           // QLINEAR_MID_MAX_M: largest M up to 64 that the kernels for a batch of tokens may serve (0: none); see takes_mid, narrow_can
     int narrow;              // QLINEAR_GEMM_NARROW: 0 gemm_narrow.cuh serves no call, 1 by the rules (default), 2 every call that it can serve
     bool xdirect;            // QLINEAR_GEMV_XDIRECT: x fragments straight from global memory
     int kernel;              // QLINEAR_GEMV_KERNEL: 0 / 1 cluster kernel (default), 2 streaming kernel
@@ -536,10 +536,14 @@ cudaError_t launch_narrow(const qlinear_s* h, const NarrowMaps& maps, const Narr
     return launch_narrow_g<BITS, GROUPED, GATED, 2>(h, maps, prm, grid, st);
 }
 
-// Token blocks and K parts of a launch of gemm_narrow.cuh over `rows` row super-blocks, and the microseconds of its busiest SM.  A CTA
-// alone on its SM takes 0.5 per weight tile of 128 k, two take 0.62 each; clusters of 4 and 8 lie inside a GPC, so fewer fit than the
-// SMs alone would hold; ramps as measured (within 10 % over the shapes named in gemm_narrow.cuh, 9 to 512 tokens).
-struct NarrowPlan { int n_tb, bn, cl; double us; };
+// (The rules below run on every call: whole-number arithmetic in place of calls into the mathematics library, whose code is cold then.)
+inline double round_up(double x) { const int64_t i = (int64_t)x; return (double)(i + ((double)i < x)); }       // x >= 0
+inline int log2_of(int parts) { return parts == 8 ? 3 : parts >> 1; }                                           // 1, 2, 4 or 8
+
+// Token blocks and K parts of a launch of gemm_narrow.cuh over `rows` row super-blocks: the parts by the cost of the busiest SM.  (Costs for
+// comparing the parts with each other only; narrow_us estimates a launch.)  A CTA alone on its SM takes 0.5 per weight tile of 128 k, two
+// take 0.62 each; clusters of 4 and 8 lie inside a GPC, so fewer fit than the SMs alone would hold.
+struct NarrowPlan { int n_tb, bn, cl; };
 NarrowPlan plan_narrow(const Layout& L, int rows, bool gated, int M, int num_sms)
 {
     NarrowPlan pl{};
@@ -547,13 +551,13 @@ NarrowPlan plan_narrow(const Layout& L, int rows, bool gated, int M, int num_sms
     pl.bn = ((M + pl.n_tb - 1) / pl.n_tb + 15) / 16 * 16;
     const int64_t tiles = (int64_t)rows * pl.n_tb;
     const int n_steps = (L.K + kNarrowKStep - 1) / kNarrowKStep;
-    pl.us = 1e30;
+    double best = 1e30;
     for (int i = 0; i < 4 && (1 << i) <= n_steps; ++i) {
         static const double ramp[4] = {3.5, 3.8, 4.0, 4.3}, fit1[4] = {1.0, 1.0, 0.89, 0.81}, fit2[4] = {1.0, 1.0, 0.92, 0.87};
         const int cl = 1 << i, n = (n_steps * (gated ? 2 : 1) + cl - 1) / cl;
         const double alone = fit1[i] * num_sms / cl, pair = 2 * fit2[i] * num_sms / cl;
-        const double us = tiles <= alone ? ramp[i] + 0.5 * n : std::ceil(tiles / pair) * (ramp[i] + 1.3 + 0.62 * n);
-        if (us < pl.us) { pl.us = us; pl.cl = cl; }
+        const double us = tiles <= alone ? ramp[i] + 0.5 * n : round_up(tiles / pair) * (ramp[i] + 1.3 + 0.62 * n);
+        if (us < best) { best = us; pl.cl = cl; }
     }
     return pl;
 }
@@ -596,44 +600,19 @@ ql_status forward_narrow(const qlinear_s* const* hs, int n, const void* x, void*
     return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
-// Microseconds of the prefill kernels on n layers in one launch (one launch each where a layer's row super-blocks are odd), within 15 % of
-// what was measured at 65 to 512 tokens: 0.30 to 0.36 per 64-k step and tile of up to 256 tokens, 3 per tile, 10 for a K split that meets in
-// the scratch; the single-CTA kernel 0.6 per step; the gated form on the shared-memory kernel 0.55 per step.
-double prefill_us(const qlinear_s* const* hs, int n, int M, bool gated, int num_sms)
+// K parts per tile of gemm_mid.cuh: what the busiest SM has to do, in stages (two CTAs per SM at once, and about 4 stages' time for the
+// ramp at the start of a CTA and the sums at its end).  Powers of two: clusters of 3, 5, 6 or 7 CTAs do not fill a GPC, so
+// fewer run at once than the slots counted here (Llama q + k + v at 16 tokens, 48 tiles: 12.1 us as 6 parts, 8.3 as 4).
+int mid_parts(int tiles, int n_steps, int num_sms)
 {
-    const Layout& L = hs[0]->L;
-    const int mblk = (M + 255) / 256, steps = (L.K + 63) / 64, clusters = num_sms / 2;
-    const double bn = (double)M / mblk;
-    int rsb = 0;
-    bool even = true;
-    for (int i = 0; i < n; ++i) { rsb += hs[i]->L.n_rsb; even = even && hs[i]->L.n_rsb % 2 == 0; }
-    if (!even) {
-        double us = 0.0;
-        for (int i = 0; i < n; ++i) us += std::ceil((double)hs[i]->L.n_rsb * mblk / num_sms) * (0.6 * steps + 3.0);
-        return us + (gated ? 3.0 : 0.0);
+    const int slots = 2 * num_sms;
+    double best = 1e30;
+    int parts = 1;
+    for (int cl = 1; cl <= 8 && cl <= n_steps; cl *= 2) {
+        const double cost = (double)((tiles * cl + slots - 1) / slots) * ((double)n_steps / cl + 4.0 + (cl > 1 ? 1.0 : 0.0));
+        if (cost < best) { best = cost; parts = cl; }
     }
-    const int tiles = rsb / 2 * mblk, split = gemm_pair_ta_split(tiles, steps, num_sms, true);
-    const double rounds = std::max(1.0, std::min(std::ceil((double)tiles * split / clusters), (double)tiles * split / clusters + 0.3));
-    const double us = rounds * (steps * (0.3 + 0.00025 * bn) / split + 3.0) + (split > 1 ? 10.0 : 0.0);
-    if (!gated) return us;
-    const int positions = rsb / 4 * mblk;
-    if (M > 128 && positions < clusters) return std::ceil((double)positions / clusters) * (1.1 * steps + 3.0);
-    return us + (M > 128 ? 0.0 : 3.0);
-}
-
-// Whether a call of the prefill stage (or, up to 64 tokens, one that takes_mid leaves to it) runs on gemm_narrow.cuh: by the estimates of
-// both, which lie within 15 % of the times in gemm_narrow.cuh's header; hence 10 % in favour of the prefill kernels.
-// (QLINEAR_MID_MAX_M < M <= 64: the prefill kernels, whatever the estimate.)
-bool narrow_is_faster(const qlinear_s* const* hs, int n, int M, bool gated = false)
-{
-    if ((M <= 64 && M > config().mid_max_m) || config().narrow == 0) return false;
-    int rows = 0;
-    for (int i = 0; i < n; ++i) {
-        if (!hs[i]->wmap_wide_ok) return false;
-        rows += hs[i]->L.n_rsb;
-    }
-    if (config().narrow == 2) return true;
-    return plan_narrow(hs[0]->L, gated ? hs[0]->L.n_rsb : rows, gated, M, hs[0]->num_sms).us < 0.9 * prefill_us(hs, n, M, gated, hs[0]->num_sms);
+    return parts;
 }
 
 template <int BITS, bool GROUPED, int NT, bool GATED, bool KSCALE>
@@ -646,24 +625,14 @@ cudaError_t launch_mid_nt(const qlinear_s* h, MidParams& prm, int units, bool pd
     if (e != cudaSuccess) return e;
     prm.n_tb = (prm.M + S::kTokens - 1) / S::kTokens;
     prm.n_steps = (prm.n_kc + 1) / 2;
-    // K parts per tile: what the busiest SM has to do, in stages (two CTAs per SM at once, and about 4 stages' time for the
-    // ramp at the start of a CTA and the sums at its end).  Powers of two: clusters of 3, 5, 6 or 7 CTAs do not fill a GPC, so
-    // fewer run at once than the slots counted here (Llama q + k + v at 16 tokens, 48 tiles: 12.1 us as 6 parts, 8.3 as 4).
-    const int tiles = units * prm.n_tb, slots = 2 * h->num_sms;
-    double best = 1e30;
-    prm.cl = 1;
-    for (int cl = 1; cl <= 8 && cl <= prm.n_steps; cl *= 2) {
-        const double cost = std::ceil((double)tiles * cl / slots) * ((double)prm.n_steps / cl + 4.0 + (cl > 1 ? 1.0 : 0.0));
-        if (cost < best) { best = cost; prm.cl = cl; }
-    }
+    const int tiles = units * prm.n_tb;
+    prm.cl = mid_parts(tiles, prm.n_steps, h->num_sms);
     return launch(kern, prm, dim3((unsigned)(tiles * prm.cl)), dim3(kMidThreads), S::kTotal, st, prm.cl, pdl);
 }
 
 // Which launches are the batch stage's: up to 32 tokens all of them, up to 48 those with at most 48 million weights, up to 64 those with at
-// most 30 million (int8: 24) or, gated, 48 million.  The stage has two kernels (batch_takes_narrow); a launch beyond the line goes to the
-// prefill stage, where narrow_is_faster compares gemm_narrow.cuh with the prefill kernels.  At 64 tokens that is the same kernel on
-// both sides of the line (Llama gate + up 26 us there, 44 on the prefill kernel); the line itself is where gemm_mid.cuh and the prefill
-// kernel are even (21 M weights at 64 tokens 20.9 / 21.4, 34 M 17.5 / 15.9, 59 M at 48 tokens 24.3 / 25.8, 14336 x 4096 26.3 / 22.1).
+// most 30 million (int8: 24) or, gated, 48 million; the others are the prefill stage's.  gemm_narrow.cuh takes calls of both stages
+// (gemm_route); the line is where gemm_mid.cuh and the prefill kernel are even (21 M weights at 64 tokens 20.9 / 21.4, 34 M 17.5 / 15.9, 59 M at 48 tokens 24.3 / 25.8, 14336 x 4096 26.3 / 22.1).
 // QLINEAR_MID_MAX_M lowers the number of tokens up to which this holds (0: never).
 bool takes_mid(const qlinear_s* const* hs, int n, int M, bool gated = false)
 {
@@ -684,31 +653,6 @@ cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, bool pdl, 
     if (prm.M > 64 && units * ((prm.M + 63) / 64) * 8 <= 2 * h->num_sms) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
     if (prm.M <= 48) return launch_mid_nt<BITS, GROUPED, 6, GATED, KSCALE>(h, prm, units, pdl, st);
     return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
-}
-
-// Calls of the batch stage that run on gemm_narrow.cuh: from a number of weights on (of the whole launch) that falls with the number of
-// tokens, because the warp-level MMAs of gemm_mid.cuh cost in proportion to the tokens and the other kernel has the longer ramp.  Measured,
-// us gemm_mid.cuh / gemm_narrow.cuh:
-//   weights                        16 tokens     24           32           48           64
-//     0.3 M (512 x 512)             2.8 /  3.7   3.0 /  3.8   3.3 /  4.0   3.8 /  4.2   4.1 /  4.5
-//     1 M (1024 x 1024, int8)       3.2 /  4.3   3.5 /  4.5   4.0 /  4.6   4.6 /  5.0   5.2 /  5.3
-//     5 M (gated 2688 x 1024)       4.1 /  5.1   4.7 /  5.5   5.5 /  5.8   7.1 /  6.8   8.5 /  7.6
-//     9 M (Gemma2-2B q + k + v)     5.0 /  5.8   5.8 /  6.3   6.9 /  6.4   8.9 /  7.3  10.5 /  7.9
-//    21 M (its down)                8.9 /  8.9  11.2 /  9.3  12.8 /  9.6  16.7 / 10.2  20.9 / 11.5
-//    25 M (Llama q + k + v)         8.8 /  9.1  10.8 /  9.4  12.3 /  9.6  16.7 / 11.4
-//    42 M (Gemma2-2B gate + up)     9.4 / 12.4  11.6 / 12.7  13.2 / 13.6  16.6 / 14.6  19.7 / 14.8
-//    59 M (Llama down)             13.8 / 13.5  16.6 / 14.0  18.9 / 14.3
-//   117 M (Llama gate + up)        26.0 / 22.7  31.9 / 23.2  37.0 / 23.6
-bool batch_takes_narrow(const qlinear_s* const* hs, int n, int M, bool gated)
-{
-    if (config().narrow == 0) return false;
-    int64_t weights = 0;
-    for (int i = 0; i < n; ++i) {
-        if (!hs[i]->wmap_wide_ok) return false;
-        weights += (int64_t)hs[i]->L.N * hs[i]->L.K;
-    }
-    if (config().narrow == 2) return true;
-    return weights >= (M <= 16 ? 50000000 : M <= 24 ? (gated ? 50000000 : 20000000) : M <= 32 ? (gated ? 50000000 : 8000000) : M <= 48 ? 4000000 : 1500000);
 }
 
 // n layers that share K and scheme, layer i on xs[i]; act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
@@ -843,21 +787,127 @@ GemmPairLayers pair_layers(const qlinear_s* const* hs, int n, void* const* ys)
 // The unfused gating route's two projections fit the device's scratch.
 bool gate_fits_scratch(int N, int M, int num_sms) { return (size_t)M * N * 2 * sizeof(__half) <= gemm_pair_scratch_bytes(num_sms); }
 
-// The kernel of a call beyond the decode stage: one layer, n > 1 layers that share x, or (gated) a pair.
-ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
+// Estimates of a launch, us, as consecutive launches with the weights out of HBM take it: what lies between gemm_narrow.cuh and the kernels
+// that served its calls before.  Fitted to 4636 calls of random shapes (8 to 32768 channels, K 32 to 16384, at most 80 million weights, 9 to 2048
+// tokens, plain and gated, the three schemes), each on both routes.  Measured / estimate on 4609 other calls, 5th and 95th percentile (1st
+// and 99th): narrow_us 0.87 and 1.10 (0.75, 1.18), mid_us 0.90 and 1.13 (0.87, 1.21), prefill_us on the CTA-pair kernel 0.83 and 1.40 (0.80, 1.69: gated
+// pairs of K up to 128, far from the line), on the single-CTA kernel 0.85 and 1.07 (0.79, 1.16), on the shared-memory gated form 0.90 and
+// 1.12 (0.89, 1.19), unfused 0.85 and 1.09 (0.81, 1.16).
+// What a CTA's time is multiplied by for the others on its SM, `ctas` of them in clusters of cl, two to an SM: each SM's share slows the CTA by
+// `share`; beyond two per SM further rounds, of which the last one costs `last` at least.  (Clusters of 4 and 8 lie inside a GPC: fewer fit.)
+double sm_load(double ctas, int cl, int num_sms, double share, double last)
+{
+    const double u = ctas / (num_sms * (cl == 8 ? 0.87 : cl == 4 ? 0.97 : 1.0));
+    return u <= 2.0 ? 1.0 + share * u : (1.0 + 2.0 * share) * std::min(round_up(u / 2.0), u / 2.0 + last);
+}
+
+int total_rsb(const qlinear_s* const* hs, int n) { int t = 0; for (int i = 0; i < n; ++i) t += hs[i]->L.n_rsb; return t; }
+double out_mb(const qlinear_s* const* hs, int n, int M) { double t = 0; for (int i = 0; i < n; ++i) t += 2e-6 * M * hs[i]->L.N; return t; }
+
+double narrow_us(const qlinear_s* const* hs, int n, int M, bool gated)
+{
+    const Layout& L = hs[0]->L;
+    const int rows = gated ? L.n_rsb : total_rsb(hs, n);
+    const NarrowPlan pl = plan_narrow(L, rows, gated, M, hs[0]->num_sms);
+    const int steps = ((L.K + kNarrowKStep - 1) / kNarrowKStep + pl.cl - 1) / pl.cl * (gated ? 2 : 1);
+    const double cta = steps * (L.bits == 4 ? 0.381 : 0.413) + 1.08 + pl.bn * (0.0244 + (pl.cl == 1 ? 0.0 : gated ? 0.0196 : 0.0054));
+    return 0.72 + 0.098 * log2_of(pl.cl) + sm_load((double)rows * pl.n_tb * pl.cl, pl.cl, hs[0]->num_sms, 0.41, 0.31) * cta;
+}
+
+double mid_us(const qlinear_s* const* hs, int n, int M, bool gated)      // up to 64 tokens
+{
+    const Layout& L = hs[0]->L;
+    const int nt = M <= 16 ? 2 : M <= 24 ? 3 : M <= 32 ? 4 : M <= 48 ? 6 : 8, units = gated ? (L.N + 63) / 64 : total_rsb(hs, n);
+    const int n_steps = (L.n_kc + 1) / 2, cl = mid_parts(units, n_steps, hs[0]->num_sms);
+    const double step = L.bits == 8 ? 0.121 + 0.0507 * nt : 0.185 + 0.0877 * nt;
+    const double cta = (n_steps + cl - 1) / cl * step + 0.425 + nt * (0.144 + (cl > 1 ? 0.044 : 0.0));
+    return 0.77 + 0.118 * log2_of(cl) + sm_load((double)units * cl, cl, hs[0]->num_sms, 0.576, 0.25) * cta;
+}
+
+double pair_ta_us(const Layout& L, int pairs, int M, int layers, bool split, double mb, int num_sms)
+{
+    const int mblk = (M + 255) / 256, bn = gemm_pair_ta_width(M), steps = (L.K + kGemmKStep - 1) / kGemmKStep;
+    const int parts = split ? gemm_pair_ta_split(pairs * mblk, steps, num_sms, true) : 1;
+    const double rounds = round_up((double)pairs * mblk * parts / (num_sms / 2));
+    return 2.5 + 0.0061 * bn + rounds * (layers * ((steps + parts - 1) / parts) * (0.199 + 0.0004 * bn)) + (parts > 1 ? 7.1 + 0.0125 * bn : 0.0) + 0.37 * mb;
+}
+
+double single_us(const Layout& L, int M, double mb, int num_sms)
+{
+    const int bn = gemm_pick_bn(L, M, num_sms), steps = (L.K + kGemmKStep - 1) / kGemmKStep;
+    const double w = (double)L.n_rsb * ((M + bn - 1) / bn) / num_sms;
+    return 4.5 + 0.0038 * bn + std::max(1.0, std::min(round_up(w), w + 0.76)) * (0.0175 * bn + steps * (0.203 + 0.0011 * bn)) + 0.28 * mb;
+}
+
+// `kernel`: what prefill_kernel says of the call.
+double prefill_us(ql_kernel kernel, const qlinear_s* const* hs, int n, int M, bool gated)
+{
+    const Layout& L = hs[0]->L;
+    const int sms = hs[0]->num_sms, steps = (L.K + kGemmKStep - 1) / kGemmKStep;
+    const double mb = out_mb(hs, gated ? 1 : n, M);
+    if (kernel == QL_KERNEL_SINGLE) return single_us(L, M, mb, sms);
+    if (kernel == QL_KERNEL_SEPARATE) {
+        if (gated && L.n_rsb % 2 == 0) return 4.2 + pair_ta_us(L, L.n_rsb, M, 1, false, 2 * mb, sms) + 0.92 * mb;
+        double us = gated ? 1.7 + 0.92 * mb : 0.0;
+        for (int i = 0; i < n; ++i) {
+            const Layout& Li = hs[i]->L;
+            const double m = out_mb(hs + i, 1, M);
+            us += Li.n_rsb % 2 ? single_us(Li, M, m, sms) : pair_ta_us(Li, Li.n_rsb / 2, M, 1, true, m, sms);
+        }
+        return us;
+    }
+    if (gated && kernel == QL_KERNEL_PAIR)
+        return 5.5 + 0.044 * std::min(M, 256) + round_up((double)(L.n_rsb / 2) * ((M + 255) / 256) / (sms / 2)) * 0.84 * steps + 0.3 * mb;
+    return gated ? pair_ta_us(L, L.n_rsb / 2, M, 2, false, mb, sms) : pair_ta_us(L, total_rsb(hs, n) / 2, M, 1, true, mb, sms);
+}
+
+ql_kernel prefill_kernel(const qlinear_s* const* hs, int n, int M, bool gated)
 {
     const Layout& L = hs[0]->L;
     const int sms = hs[0]->num_sms;
-    if (n == 1 && takes_rows(L)) return rows_take_tc(L.n_rsb, L.n_kc, M, sms) ? QL_KERNEL_ROWS_TC : QL_KERNEL_ROWS;
-    if (takes_mid(hs, n, M, gated)) return batch_takes_narrow(hs, n, M, gated) ? QL_KERNEL_NARROW : QL_KERNEL_MID;
-    // (a pair whose unfused product does not fit the scratch has only ever been served by the fused kernels of the prefill stage)
-    if ((!gated || gate_fits_scratch(L.N, M, sms) || gemm_pair_applicable(L, M)) && narrow_is_faster(hs, n, M, gated)) return QL_KERNEL_NARROW;
     const GemmPairLayers set = pair_layers(hs, n, nullptr);
     if (gated && !gemm_pair_applicable(L, M)) return QL_KERNEL_SEPARATE;
     if (gemm_pair_ta_applicable(set, M, sms, gated)) return QL_KERNEL_PAIR_TA;
     for (int i = 0; i < n; ++i)
         if (!gemm_pair_applicable(hs[i]->L, M)) return n > 1 ? QL_KERNEL_SEPARATE : QL_KERNEL_SINGLE;
     return QL_KERNEL_PAIR;
+}
+
+// Whether gemm_narrow.cuh can serve the call at all.  (QLINEAR_MID_MAX_M < M <= 64: the prefill kernels, whatever the estimate.  A pair whose
+// unfused product does not fit the scratch has only ever been served by the fused kernels of the prefill stage.)
+bool narrow_can(const qlinear_s* const* hs, int n, int M, bool gated, bool batch)
+{
+    if (config().narrow == 0 || (M <= 64 && M > config().mid_max_m)) return false;
+    for (int i = 0; i < n; ++i)
+        if (!hs[i]->wmap_wide_ok) return false;
+    return batch || !gated || gate_fits_scratch(hs[0]->L.N, M, hs[0]->num_sms) || gemm_pair_applicable(hs[0]->L, M);
+}
+
+// The kernel of a call beyond the decode stage: one layer, n > 1 layers that share x, or (gated) a pair.  gemm_narrow.cuh where its
+// estimate is 3 % below that of gemm_mid.cuh, 5 % below that of the CTA-pair kernel, and up to 5 % above those of the three other forms (single
+// CTA, shared-memory gating, unfused gating).  No line is always right with these errors.  Of the 4636 calls that the estimates were fitted to and
+// 4609 others, 30 run more than 3 % slower this way than on the other route: 23 of 3613 against gemm_mid.cuh (by 24 % at most), 2 of 1429 against the
+// CTA-pair kernel (11 %), 5 of 4203 against the other forms (9 %).  Measured, us, the route otherwise / gemm_narrow.cuh:
+//   weights                        16 tokens     24           32           48           64
+//     0.3 M (512 x 512)             2.8 /  3.7   3.0 /  3.8   3.3 /  4.0   3.8 /  4.2   4.1 /  4.5
+//     1 M (1024 x 1024, int8)       3.2 /  4.3   3.5 /  4.5   4.0 /  4.6   4.6 /  5.0   5.2 /  5.3
+//     5 M (gated 2688 x 1024)       4.1 /  5.1   4.7 /  5.5   5.5 /  5.8   7.1 /  6.8   8.5 /  7.6
+//     9 M (Gemma2-2B q + k + v)     5.0 /  5.8   5.8 /  6.3   6.9 /  6.4   8.9 /  7.3  10.5 /  7.9
+//    21 M (its down)                8.9 /  8.9  11.2 /  9.3  12.8 /  9.6  16.7 / 10.2  20.9 / 11.5
+//    25 M (Llama q + k + v)         8.8 /  9.1  10.8 /  9.4  12.3 /  9.6  16.7 / 11.4
+//    42 M (Gemma2-2B gate + up)     9.4 / 12.4  11.6 / 12.7  13.2 / 13.6  16.6 / 14.6  19.7 / 14.8
+//    59 M (Llama down)             13.8 / 13.5  16.6 / 14.0  18.9 / 14.3               27.9 / 15.8
+//   117 M (Llama gate + up)        26.0 / 22.7  31.9 / 23.2  37.0 / 23.6               43.8 / 26.0
+ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
+{
+    const Layout& L = hs[0]->L;
+    if (n == 1 && takes_rows(L)) return rows_take_tc(L.n_rsb, L.n_kc, M, hs[0]->num_sms) ? QL_KERNEL_ROWS_TC : QL_KERNEL_ROWS;
+    const bool batch = takes_mid(hs, n, M, gated);
+    const ql_kernel other = batch ? QL_KERNEL_MID : prefill_kernel(hs, n, M, gated);
+    if (!narrow_can(hs, n, M, gated, batch)) return other;
+    if (config().narrow == 2) return QL_KERNEL_NARROW;
+    const double limit = batch ? 0.97 * mid_us(hs, n, M, gated) : (other == QL_KERNEL_PAIR_TA ? 0.95 : 1.05) * prefill_us(other, hs, n, M, gated);
+    return narrow_us(hs, n, M, gated) < limit ? QL_KERNEL_NARROW : other;
 }
 
 // y = act(g) * u, element-wise (the unfused form of the gating, for shapes the fused kernels do not take).
@@ -1778,7 +1828,8 @@ extern "C" int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_
         width = gemm_pair_ta_width(M);
         if (!gated) parts = gemm_pair_ta_split(rows / 2 * ((M + 255) / 256), (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, true);
     }
-    const int32_t v[5] = {kernel, width, parts, (int32_t)(1000 * pl.us), (int32_t)(1000 * prefill_us(hs, n, M, gated, num_sms))};
+    const double other = takes_mid(hs, n, M, gated) ? mid_us(hs, n, M, gated) : prefill_us(prefill_kernel(hs, n, M, gated), hs, n, M, gated);
+    const int32_t v[5] = {kernel, width, parts, (int32_t)(1000 * narrow_us(hs, n, M, gated)), (int32_t)(1000 * other)};
     const int k = n_out < 5 ? n_out : 5;
     for (int i = 0; i < k; ++i) out[i] = v[i];
     return k;

@@ -74,9 +74,9 @@ BATCH = [(4, 96, 16384, 64), (2, 96, 15680, 49), (1, 96, 41728, 33), (2, 32, 468
 
 @pytest.mark.parametrize("n_heads,d_h,cache,R", BATCH)
 def test_scores_of_a_batch_of_rows_see_the_scales_appended_just_before(P, torch, n_heads, d_h, cache, R):
-    """Head dimensions that the row kernels do not take, so many positions that the batch kernel with the weights in tensor memory serves the
-    scores in one K part, and (up to 128 of K) a step for one of its two groups of warps only: the other one waits for nothing before
-    its outputs.  Append and scores captured and replayed on new tokens, against the same calls with the host waiting in between."""
+    """Head dimensions that the row kernels do not take and many positions: the batch kernels.  On the one with the weights in tensor
+    memory (test_routes_gpu.py has it serve them) these are launches of one K part, and (up to 128 of K) of a step for one of its two groups of
+    warps only: the other one waits for nothing before its outputs.  Append and scores captured and replayed on new tokens, against the same calls with the host waiting in between."""
     T, n_new = cache - 100, 64
     start = torch.randn((n_heads, T, d_h), device="cuda").half()
     pair = [P.KVHeads(n_heads, cache, d_h) for _ in range(2)]

@@ -1,6 +1,7 @@
 """The tensor-core kernel for a batch of tokens and for prompts on small layers, against the CPU oracle, on a B200: edges of its
 token blocks (16 to 64 wide, one or several), of the 128-channel super-blocks and of its 128-k steps, with and without a K split,
-with two and with three groups of unpacking warps."""
+with two and with three groups of unpacking warps.  Some of the calls are near a line of the dispatch; test_routes_gpu.py runs all of them on
+this kernel."""
 import numpy as np
 import pytest
 
@@ -68,7 +69,7 @@ def test_small_layers(P, torch, N, K, bits, group, M):
 
 @pytest.mark.parametrize("N,K,bits,group,M", LARGE)
 def test_large_layers_of_the_batch_stage(P, torch, N, K, bits, group, M):
-    """Up to 64 tokens, where the number of weights calls for this kernel; int4 in groups up to 32 tokens: three groups."""
+    """Up to 64 tokens, layers large enough for this kernel or nearly so; int4 up to 32 tokens: three groups."""
     check(P, torch, N, K, bits, group, M, np.r_[0:64, N - 72:N])
 
 

@@ -11,6 +11,16 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SMS = 148                                               # of a B200
 DECODE, ROWS, ROWS_TC, MID, NARROW, PAIR_TA, PAIR, SINGLE, SEPARATE = range(1, 10)
 
+# (channels of the layers, K, bits, group, tokens, gated, kernel)
+CLEAR = [([14336] * 2, 4096, 4, 32, 32, 1, NARROW), ([4096], 14336, 4, 32, 32, 0, NARROW), ([4096, 1024, 1024], 4096, 8, 0, 32, 0, NARROW),
+         ([2304], 9216, 4, 32, 48, 0, NARROW), ([1024], 1024, 8, 0, 128, 0, NARROW), ([1024], 1024, 4, 32, 512, 0, NARROW),
+         ([2688] * 2, 1024, 4, 32, 128, 1, NARROW), ([2680], 64, 4, 32, 411, 0, NARROW), ([512], 512, 4, 32, 16, 0, MID),
+         ([1024], 1024, 8, 0, 24, 0, MID), ([9216] * 2, 2304, 4, 32, 16, 1, MID), ([11816] * 2, 64, 4, 0, 48, 1, MID), ([512] * 2, 2048, 4, 0, 32, 1, MID),
+         ([4096], 14336, 4, 32, 2048, 0, PAIR_TA), ([14336] * 2, 4096, 4, 32, 777, 1, PAIR_TA), ([4096, 1024, 1024], 4096, 8, 0, 1024, 0, PAIR_TA),
+         # what the smoke run has for the prefill kernels
+         ([4096], 512, 4, 32, 1024, 0, PAIR_TA), ([128], 96, 8, 0, 300, 0, SINGLE), ([3072] * 2, 4096, 4, 32, 1500, 1, PAIR),
+         ([6936], 10144, 4, 32, 1500, 0, SINGLE)]
+
 CHILD = """
 import ctypes, json, sys
 sys.path.insert(0, {root!r})
@@ -35,6 +45,7 @@ print(json.dumps({{
     "late_batch": [route([c], d, 8, 0, R) for _, d, c, R in test_kv_append_gpu.BATCH],
     "narrow_small": [[route([N], K, b, g, M), route([N, N + 136], K, b, g, M), route([N, N], K, b, g, M, 1)] for N, K, b, g, M in test_narrow_gpu.SMALL],
     "narrow_large": [route([N], K, b, g, M) for N, K, b, g, M in test_narrow_gpu.LARGE],
+    "clear": [route(*c[:6]) for c in {clear!r}],
     "lines": [route([N], K, b, g, M) for N, K, b, g, M, _ in test_mid_gpu.LINES],
     "scores": [route([c], d, 8, 0, R) for _, d, c, _, R in test_scores_gpu.CASES]}}))
 """
@@ -42,7 +53,7 @@ print(json.dumps({{
 
 def routes(**env):
     env = {**{k: v for k, v in os.environ.items() if not k.startswith("QLINEAR_")}, **env}
-    r = subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, sms=SMS)], check=True, env=env, cwd=ROOT, timeout=600, stdout=subprocess.PIPE)
+    r = subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, sms=SMS, clear=CLEAR)], check=True, env=env, cwd=ROOT, timeout=600, stdout=subprocess.PIPE)
     return json.loads(r.stdout)
 
 
@@ -65,13 +76,17 @@ def kernels(rs):
     return [r[0] for r in rs]
 
 
-def test_the_kernel_for_a_batch_serves_its_tests(by_rule, always_narrow):
-    """Under the switch all of them, with both forms of the K split and every number of groups of warps; by the rule the large layers."""
+def test_the_kernel_for_a_batch_serves_its_tests(always_narrow):
+    """Under the switch all of them, with and without a K split, at the narrowest and the widest token block."""
     flat = [r for three in always_narrow["narrow_small"] for r in three] + always_narrow["narrow_large"]
     assert set(kernels(flat)) == {NARROW}
     assert {r[2] for r in flat} >= {1, 2, 4, 8} and min(r[1] for r in flat) == 16 and max(r[1] for r in flat) == 64
-    assert kernels(by_rule["narrow_large"]) == [NARROW] * len(by_rule["narrow_large"])
-    assert kernels(by_rule["late_batch"]) == [NARROW] * len(by_rule["late_batch"]) and {r[2] for r in by_rule["late_batch"]} == {1}
+    assert kernels(always_narrow["late_batch"]) == [NARROW] * 5 and {r[2] for r in always_narrow["late_batch"]} == {1}
+
+
+def test_calls_far_from_the_lines_go_to_the_faster_kernel(by_rule):
+    """Both sides measured at twice the other's time or nearly so, except where the comment in gemm_route gives the figures."""
+    assert kernels(by_rule["clear"]) == [c[-1] for c in CLEAR]
 
 
 def test_the_score_kernel_of_many_rows_serves_its_tests(by_rule):

@@ -18,7 +18,7 @@ WITHOUT = {
     "test_kv_append_gpu.py": "batch_of_rows_see",
     "test_mid_gpu.py": "oracle or lines or outside",
 }
-ALWAYS = {"test_narrow_gpu.py": "", "test_gated_gpu.py": "gated_parity", "test_kv_gpu.py": "prefill_kernels_see", "test_prefill_gpu.py": "one_hot or zero_input"}
+ALWAYS = {"test_narrow_gpu.py": "", "test_kv_append_gpu.py": "batch_of_rows_see", "test_gated_gpu.py": "gated_parity", "test_kv_gpu.py": "prefill_kernels_see", "test_prefill_gpu.py": "one_hot or zero_input"}
 
 
 def child(setting, name, chosen):
