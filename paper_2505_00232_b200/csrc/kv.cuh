@@ -43,27 +43,43 @@ struct KvAppendParams {
     int32_t k_n_kc, v_n_kc;
 };
 
-// One CTA of two warps per new token and head, one for the key and one for the value vector; d_h <= 1024, a multiple of 32.  Bound: the
-// chain of latencies (previous kernel -> vector -> amax -> scale -> bytes), so a warp keeps its vector in registers and there is no
-// barrier and no shared memory.  The dependents are released only after the wait: whoever runs beside this kernel then knows
-// that every kernel before it is complete, and that only the bytes of these tokens may still change.
-__global__ void __launch_bounds__(64) kv_append_kernel(const KvAppendParams p)
+// One CTA per new token and head, d_h <= 1024, a multiple of 32; warps in pairs, one for the key and one for the value vector, each pair
+// for the 32 E dimensions of its slice.  Bound: the chain of latencies (previous kernel -> vector -> amax -> scale -> bytes); with many
+// tokens and wide heads the stores, a sector of its own for every byte of V.  Every warp takes the amax of the whole vector itself (it is
+// in L1 for all but the first), so there is no barrier and no shared memory.  The dependents are released only after the wait: whoever
+// runs beside this kernel then knows that every kernel before it is complete, and that only the bytes of these tokens may still change.
+// Measured, us, 128 threads striding over both vectors with two barriers / a warp per vector, four dimensions in a row per lane / this: one
+// token of 8 heads of 128 1.81 / 1.62 / 1.62, of 1024 3.67 / 3.54 / 2.32; 256 tokens of 8 heads of 128 3.67 / 4.07 / 3.40, of 256 5.20 / 6.57 / 4.38, of
+// 1024 12.0 / 19.6 / 11.4; 2048 tokens of 8 heads of 128 18.5 / 17.7 / 17.5, of 1024 60.6 / 85.3 / 71.3 (every warp reads the whole vector).
+template <int E, bool SPREAD>
+__global__ void __launch_bounds__(E == 2 ? 1024 : 512) kv_append_kernel(const KvAppendParams p)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int i = blockIdx.x, t = p.pos + i, hd = blockIdx.y, lane = threadIdx.x & 31;
-    const bool value = threadIdx.x >= 32;
+    const int i = blockIdx.x, t = p.pos + i, hd = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool value = warp & 1;
     const __half* src = (value ? p.v_new : p.k_new) + hd * p.head_stride + i * p.token_stride;
-    constexpr int NV = 8;                                                // 4-value vectors per lane: a head of 128 keeps every lane busy
-    const int n_vec = p.d_h >> 2;
-    uint2 u[NV];
+    // This lane's dimensions: E in a row for K (their bytes lie in a word or two).  For V 32 apart (SPREAD), so that the lanes of a store are
+    // consecutive rows, 8 lines of 128 bytes (with 4 in a row per lane 16 lines: 2048 vectors of 1024 14.8 us instead of 11.4), or, for few
+    // vectors, in a row too: one load instead of E.
+    const bool apart = SPREAD && value;
+    const int own = (warp >> 1) * 32 * E + (apart ? lane : lane * E), step = apart ? 32 : 1;
+    __align__(2 * E) __half h[E];
+    if (apart) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) u[j] = lane + 32 * j < n_vec ? *reinterpret_cast<const uint2*>(src + 4 * (lane + 32 * j)) : make_uint2(0, 0);
+        for (int e = 0; e < E; ++e) h[e] = own + 32 * e < p.d_h ? src[own + 32 * e] : __float2half_rn(0.f);
+    } else if (own < p.d_h) {
+        if constexpr (E == 4) *reinterpret_cast<uint2*>(h) = *reinterpret_cast<const uint2*>(src + own);
+        else *reinterpret_cast<uint32_t*>(h) = *reinterpret_cast<const uint32_t*>(src + own);
+    }
     __half2 mx = __float2half2_rn(0.f);
+    uint4 u[4];                                                          // the whole vector, 8 values per lane and piece
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const __half2* h = reinterpret_cast<const __half2*>(&u[j]);
-        mx = __hmax2(mx, __hmax2(__habs2(h[0]), __habs2(h[1])));
+    for (int j = 0; j < 4; ++j) u[j] = (lane + 32 * j) * 8 < p.d_h ? *reinterpret_cast<const uint4*>(src + (lane + 32 * j) * 8) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const __half2* v = reinterpret_cast<const __half2*>(&u[j]);
+        mx = __hmax2(mx, __hmax2(__hmax2(__habs2(v[0]), __habs2(v[1])), __hmax2(__habs2(v[2]), __habs2(v[3]))));
     }
     const float2 m = __half22float2(mx);
     // (bits of a non-negative float: ordered like unsigned integers)
@@ -71,24 +87,18 @@ __global__ void __launch_bounds__(64) kv_append_kernel(const KvAppendParams p)
     const __half h0 = __float2half_rn(__fdiv_rn(amax, 127.f));
     const bool dead = __half2float(h0) == 0.f;                           // a zero vector, or a scale below fp16's range: zeros, scale 1
     const float sc = dead ? 1.f : __half2float(h0);
-    if (lane == 0) (value ? p.v_scale[hd] : p.k_scales[hd])[t] = __float2half_rn(sc);
+    if (threadIdx.x < 64 && lane == 0) (value ? p.v_scale[hd] : p.k_scales[hd])[t] = __float2half_rn(sc);
+    uint32_t q[E];                                                       // as stored: q + 128
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const int v = lane + 32 * j;
-        if (v >= n_vec) break;
-        const __half* h = reinterpret_cast<const __half*>(&u[j]);
-        uint32_t q[4];                                                   // as stored: q + 128
+    for (int e = 0; e < E; ++e) q[e] = dead ? 128u : (uint32_t)(max(-127, min(127, __float2int_rn(__fdiv_rn(__half2float(h[e]), sc)))) + 128);
+    if (value) {                                                         // V: row = dimension, k = token
 #pragma unroll
-        for (int e = 0; e < 4; ++e) q[e] = dead ? 128u : (uint32_t)(max(-127, min(127, __float2int_rn(__fdiv_rn(__half2float(h[e]), sc)))) + 128);
-        if (value) {                                                     // V: row = dimension, k = token: rows g and g + 1 lie 64 bytes apart
-            uint8_t* dst = p.v_body[hd] + int8_weight_offset(4 * v, t, p.v_n_kc);
+        for (int e = 0; e < E; ++e)                                      // (next row: 64 bytes; 32 rows: two row-blocks of 512; a slice lies in one super-block)
+            if (own + step * e < p.d_h) p.v_body[hd][int8_weight_offset(own, t, p.v_n_kc) + (SPREAD ? 1024 : 64) * e] = (uint8_t)q[e];
+    } else if (own < p.d_h) {                                            // K: row = token, k = dimension: pairs of k in each of a lane's words
+        uint8_t* dst = p.k_body[hd] + int8_weight_offset(t, own, p.k_n_kc);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) dst[64 * e] = (uint8_t)q[e];
-        } else {                                                         // K: row = token, k = dimension: pairs of k in each of a lane's words
-            uint8_t* dst = p.k_body[hd] + int8_weight_offset(t, 4 * v, p.k_n_kc);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) *reinterpret_cast<uint16_t*>(dst + 4 * e) = (uint16_t)(q[2 * e] | q[2 * e + 1] << 8);
-        }
+        for (int e = 0; e < E / 2; ++e) *reinterpret_cast<uint16_t*>(dst + 4 * e) = (uint16_t)(q[2 * e] | q[2 * e + 1] << 8);
     }
 }
 

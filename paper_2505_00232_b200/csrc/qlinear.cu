@@ -1386,7 +1386,15 @@ extern "C" ql_status qlinear_kv_append_heads(const qlinear_t* hk, const qlinear_
     unsigned long long capture;
     const bool known = capture_of(st, &capture);
     std::lock_guard<std::mutex> lock(g_append_mutex[hk[0]->device]);
-    if (launch(kv_append_kernel, prm, dim3(n_new, n_heads), dim3(64), 0, st, 1, hk[0]->pdl) != cudaSuccess) {
+    // Two dimensions per lane where the chain of latencies is the bound, four where the stores of many wide vectors are (half the warps then
+    // read each vector).  Measured, us 2 / 4 per lane: one token of 8 heads of 128 1.62 / 1.78, of 1024 2.32 / 2.38; 512 vectors of 256 2.50 / 2.66,
+    // 2048 4.62 / 4.38; 512 of 512 3.36 / 3.32, 2048 7.84 / 6.73; 128 of 1024 2.73 / 2.65, 2048 17.5 / 11.4.  The value bytes spread from 32768 values on:
+    // in a row / spread, one token of a head of 32 1.38 / 1.85, of 128 1.36 / 1.46; 128 vectors of 128 1.79 / 1.78, 512 2.47 / 2.13, 2048 3.84 / 3.40.
+    const int64_t values = (int64_t)n_new * n_heads * K.K;
+    const bool wide = K.K > 128 && values * K.K >= (int64_t)1 << 27;
+    const auto kern = wide ? kv_append_kernel<4, true> : values >= 32768 ? kv_append_kernel<2, true> : kv_append_kernel<2, false>;
+    const int per_warp = wide ? 128 : 64;
+    if (launch(kern, prm, dim3(n_new, n_heads), dim3(64 * ((K.K + per_warp - 1) / per_warp)), 0, st, 1, hk[0]->pdl) != cudaSuccess) {
         cudaGetLastError();                                              // nothing is in flight: the append before it stays the last one
         return QL_ERR_CUDA;
     }

@@ -254,3 +254,26 @@ def test_a_reader_behind_an_append_that_is_not_the_last_recorded(P, torch, case,
         torch.cuda.synchronize()
         assert all(torch.equal(x, y) for x, y in zip(got, want))
     assert kv.heads[0].k.device_status() == (0, 0)
+
+
+# heads, d_h, new tokens: both sides of the line between two and four dimensions per lane, d_h not a multiple of a warp's slice
+@pytest.mark.parametrize("n_heads,d_h,n_new", [(1, 32, 3), (3, 96, 40), (16, 128, 300), (8, 160, 40), (8, 160, 660), (2, 256, 5), (16, 256, 130), (2, 992, 3), (2, 992, 70), (1, 1024, 127), (4, 1024, 33)])
+def test_appended_integers_and_scales_of_any_width(P, torch, n_heads, d_h, n_new):
+    cache, pos = (n_new + 31) // 32 * 32 + 64, 37
+    rng = np.random.default_rng(d_h + n_new)
+    k, v = ((rng.standard_normal((n_heads, n_new, d_h)) * rng.uniform(0.1, 9.0, size=(n_heads, n_new, 1))).astype(np.float16) for _ in range(2))
+    v[0, 1], k[n_heads - 1, 2] = 0, 2.0 ** -20                # a zero vector; a scale below fp16's range
+    kv = P.KVHeads(n_heads, cache, d_h)
+    kv.length = pos
+    kv.append(torch.from_numpy(k).cuda(), torch.from_numpy(v).cuda())
+    torch.cuda.synchronize()
+    where = slice(pos, pos + n_new)
+    for h, c in enumerate(kv.heads):
+        k_q, k_s = O.kv_quantize_rows(k[h])
+        v_q, v_s = O.kv_quantize_rows(v[h])
+        got_k, got_v = c.k.debug_unpack().cpu().numpy(), c.v.debug_unpack().cpu().numpy()
+        assert (got_k[where] == k_q).all() and (got_v[:, where] == v_q.T).all()
+        assert (np.delete(got_k, np.r_[where], 0) == 0).all() and (np.delete(got_v, np.r_[where], 1) == 0).all()
+        _, ks = P.qlinear_unpack(c.k.desc, c.k.packed.cpu().numpy())
+        assert (ks.reshape(-1)[where].view(np.uint16) == k_s.view(np.uint16)).all()
+        assert (c.v_scale.cpu().numpy()[where].view(np.uint16) == v_s.view(np.uint16)).all()
