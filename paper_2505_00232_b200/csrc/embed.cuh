@@ -2,12 +2,13 @@
 // table is stored with int4 weights, like the feed-forward layers): y[t, :] = fp16(s * q[ids[t], :]).
 //
 // The table is an ordinary packed layer (N = vocabulary, K = hidden size), so the LM head and the
-// embedding can share one blob.  A CTA serves one token: its threads walk the 16-byte pieces of the
+// embedding can share one blob.  A CTA serves one token (short rows: several): its threads walk the 16-byte pieces of the
 // token's row (one piece = the row's weights of one lane column in one K chunk), unpack them with the
 // same routine the decode and prefill kernels use, and multiply by the scale: one fp16 multiplication of
 // an exact integer is the correctly rounded product.  A piece holds runs of 8 consecutive k, which leave
 // as 16-byte stores.  Bound: HBM (2048 rows of 4096 from a table of 128256: 21.5 MB, 3.3 us at the measured
-// copy rate).
+// copy rate); with short rows the CTAs themselves, each with its wait for the kernel before
+// (8192 rows of 32 9.1 us with a CTA per token, 5.9 without the programmatic launch, 2.1 with 8 tokens to a CTA; 8192 rows of 512 9.1, 7.6, 3.4).
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -24,19 +25,24 @@ struct EmbedParams {
     const int32_t* ids;                  // [n] row numbers; rows outside [0, N) give zeros
     __half* y;                           // [n, K]
     int32_t n, N, K, n_kc, block_bytes;
+    int32_t log2_tokens;                 // 1 << log2_tokens tokens per CTA, 128 >> log2_tokens threads each
 };
 
-template <int BITS, bool GROUPED>
+// SEVERAL: tokens per CTA (else one)
+template <int BITS, bool GROUPED, bool SEVERAL>
 __global__ void __launch_bounds__(128) embed_kernel(const EmbedParams p)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");                  // ids and the output buffer may be the previous kernel's
-    const int t = blockIdx.x;
+    // (unsigned: with a signed stride the compiler unrolls the loop below, 0.2 us more at two pieces per thread)
+    const unsigned lanes = SEVERAL ? 128u >> p.log2_tokens : blockDim.x, first = SEVERAL ? threadIdx.x & (lanes - 1) : threadIdx.x;
+    const int t = SEVERAL ? (blockIdx.x << p.log2_tokens) + (threadIdx.x >> (7 - p.log2_tokens)) : blockIdx.x;
+    if (SEVERAL && t >= p.n) return;
     const int row = p.ids[t];
     __half* yrow = p.y + (int64_t)t * p.K;
     constexpr int CHUNK_K = BITS == 4 ? 64 : 32;
     if (row < 0 || row >= p.N) {
-        for (int k = threadIdx.x * 8; k < p.K; k += blockDim.x * 8) *reinterpret_cast<uint4*>(yrow + k) = make_uint4(0, 0, 0, 0);
+        for (int k = (int)first * 8; k < p.K; k += lanes * 8) *reinterpret_cast<uint4*>(yrow + k) = make_uint4(0, 0, 0, 0);
         return;
     }
     const int rsb = row / kRsbRows, rb = (row % kRsbRows) / kRbRows;
@@ -44,7 +50,7 @@ __global__ void __launch_bounds__(128) embed_kernel(const EmbedParams p)
     const uint8_t* base = p.body + (int64_t)rsb * p.n_kc * p.block_bytes + rb * 512 + g * 64;
     uint32_t s2[2];                                                     // scales of the chunk's two groups, in both halves
     s2[0] = s2[1] = GROUPED ? 0u : 0x10001u * (uint32_t)__half_as_ushort(p.chan_scales[row]);
-    for (int piece = threadIdx.x; piece < p.n_kc * 4; piece += blockDim.x) {
+    for (int piece = (int)first; piece < p.n_kc * 4; piece += lanes) {
         const int kc = piece >> 2, c = piece & 3;
         const uint8_t* blk = base + (int64_t)kc * p.block_bytes;
         const uint4 w = *reinterpret_cast<const uint4*>(blk + c * 16);

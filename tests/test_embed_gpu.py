@@ -67,3 +67,24 @@ def test_embed_table_is_also_an_lm_head(P, torch):
     y = lin.forward(torch.from_numpy(x).cuda()).cpu().numpy()
     y64, A, _ = O.linear(x, q, s, 32)
     assert O.check_against(y, y64, A)[0]
+
+
+@pytest.mark.parametrize("bits,group", [(8, 0), (4, 0), (4, 32)])
+@pytest.mark.parametrize("K", [32, 96, 160, 512, 1024])
+@pytest.mark.parametrize("n", [1184, 1191, 20000])
+def test_many_short_rows(P, torch, K, bits, group, n):
+    """Several tokens to a CTA: a last CTA that is not full, rows whose pieces do not fill their threads, ids outside the table."""
+    N = 1000
+    rng = np.random.default_rng(n + K)
+    q = rng.integers(*((-8, 8) if bits == 4 else (-128, 128)), size=(N, K)).astype(np.int8)
+    s = (rng.uniform(1e-3, 1e-2, size=(N, K // group if group else 1))).astype(np.float16)
+    lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
+    ids = rng.integers(0, N, size=n).astype(np.int32)
+    ids[[0, n // 2, n - 1]] = -1, N, N - 1
+    buf = torch.full((n + 2, K), 7.0, dtype=torch.float16, device="cuda")
+    lin.embed(torch.from_numpy(ids).cuda(), out=buf[1:-1])
+    torch.cuda.synchronize()
+    inside = (ids >= 0) & (ids < N)
+    full = np.repeat(s.astype(np.float64), group, axis=1) if group else s.astype(np.float64)
+    want = np.where(inside[:, None], (full * q)[np.where(inside, ids, 0)], 0.0).astype(np.float16)
+    assert (buf[1:-1].cpu().numpy() == want).all() and (buf[0] == 7).all() and (buf[-1] == 7).all()
