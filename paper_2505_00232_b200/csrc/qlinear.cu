@@ -730,13 +730,17 @@ cudaError_t launch_gemm_rows_tc(const qlinear_s* h, const GemmRowsMaps& maps, Ge
 }
 
 // Which of the two kernels for short K a layer takes, the smallest of those in one launch: the tensor-core form has the longer ramp and the
-// faster tiles, and another order of sums inside an MMA.  The rule looks at one layer, so that a head gets the same bits alone and among
-// others: from the tiles of 128 x 64 on at which one layer alone is even.  Measured, us gemm_rows_kernel / gemm_rows_tc_kernel, one layer:
-// d_h = 64, 1024 tiles 8.1 / 7.8; d_h = 128, 512 7.1 / 7.2, 1024 11.4 / 9.0; d_h = 256, 512 10.4 / 9.9, 1024 18.1 / 11.7; eight layers: d_h = 64,
-// 512 tiles each 23.9 / 20.6, d_h = 128 34.8 / 24.1, d_h = 256 58.6 / 28.1.
+// faster tiles, converts each super-block's weights once for all of its token blocks, and has another order of sums inside an MMA.  The rule
+// looks at one layer, so that a head gets the same bits alone and among others: from the tiles of 128 x 64 on at which one layer alone is about
+// even, and at d_h = 128 from 3 token blocks on.  Measured, time of gemm_rows_tc_kernel / gemm_rows_kernel, of one layer and of eight:
+//   d_h = 64, 1024 tiles (cache 32768, 8192, 2048) 0.99, 0.98, 0.94 and 0.91, 0.85, 0.84; 768 tiles 1.05, 1.04, 1.02 and 0.93, 0.87, 0.85
+//   d_h = 128, 512 tiles (16384, 8192, 4096) 1.06, 1.04, 1.00 and 0.89, 0.76, 0.68; 1024 0.86, 0.85, 0.78 and 0.78, 0.69, 0.64
+//   d_h = 128, 2 token blocks of 32768 positions 1.06 and 1.07 (40.4 / 43.2 us), 3 0.95 and 0.96
+//   d_h = 256, 512 tiles (32768, 16384, 8192, 4096) 0.99, 1.16, 0.97, 0.94 and 0.77, 0.63, 0.53, 0.48
 bool rows_take_tc(int layer_rsb, int n_kc, int M, int num_sms)
 {
-    return (int64_t)layer_rsb * ((M + kRowsTcTokens - 1) / kRowsTcTokens) * 20 >= num_sms * (n_kc == 2 ? 138 : n_kc == 4 ? 69 : 60);
+    const int n_tb = (M + kRowsTcTokens - 1) / kRowsTcTokens;
+    return (int64_t)layer_rsb * n_tb * 20 >= num_sms * (n_kc == 2 ? 138 : n_kc == 4 ? 69 : 60) && (n_kc != 4 || n_tb >= 3);
 }
 
 ql_status forward_gemm_rows(const qlinear_s* const* hs, int n, const void* const* xs, void* const* ys, int M, cudaStream_t st)

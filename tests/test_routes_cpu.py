@@ -21,6 +21,10 @@ CLEAR = [([14336] * 2, 4096, 4, 32, 32, 1, NARROW), ([4096], 14336, 4, 32, 32, 0
          ([4096], 512, 4, 32, 1024, 0, PAIR_TA), ([128], 96, 8, 0, 300, 0, SINGLE), ([3072] * 2, 4096, 4, 32, 1500, 1, PAIR),
          ([6936], 10144, 4, 32, 1500, 0, SINGLE)]
 
+# (d_h, cache, rows, kernel): both sides of the lines for scores of many rows
+SCORE_LINES = [(64, 8192, 1024, ROWS_TC), (64, 8192, 896, ROWS), (128, 32768, 128, ROWS), (128, 32768, 129, ROWS_TC), (128, 8192, 512, ROWS_TC), (128, 8192, 448, ROWS),
+               (256, 32768, 128, ROWS_TC), (256, 4096, 896, ROWS_TC), (256, 4096, 832, ROWS)]
+
 CHILD = """
 import ctypes, json, sys
 sys.path.insert(0, {root!r})
@@ -46,6 +50,7 @@ print(json.dumps({{
     "narrow_small": [[route([N], K, b, g, M), route([N, N + 136], K, b, g, M), route([N, N], K, b, g, M, 1)] for N, K, b, g, M in test_narrow_gpu.SMALL],
     "narrow_large": [route([N], K, b, g, M) for N, K, b, g, M in test_narrow_gpu.LARGE],
     "clear": [route(*c[:6]) for c in {clear!r}],
+    "score_lines": [route([c], d, 8, 0, R) for d, c, R, _ in {score_lines!r}],
     "lines": [route([N], K, b, g, M) for N, K, b, g, M, _ in test_mid_gpu.LINES],
     "scores": [route([c], d, 8, 0, R) for _, d, c, _, R in test_scores_gpu.CASES]}}))
 """
@@ -53,7 +58,7 @@ print(json.dumps({{
 
 def routes(**env):
     env = {**{k: v for k, v in os.environ.items() if not k.startswith("QLINEAR_")}, **env}
-    r = subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, sms=SMS, clear=CLEAR)], check=True, env=env, cwd=ROOT, timeout=600, stdout=subprocess.PIPE)
+    r = subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, sms=SMS, clear=CLEAR, score_lines=SCORE_LINES)], check=True, env=env, cwd=ROOT, timeout=600, stdout=subprocess.PIPE)
     return json.loads(r.stdout)
 
 
@@ -91,6 +96,7 @@ def test_calls_far_from_the_lines_go_to_the_faster_kernel(by_rule):
 
 def test_the_score_kernel_of_many_rows_serves_its_tests(by_rule):
     assert kernels(by_rule["scores"]) == [ROWS_TC] * len(by_rule["scores"])
+    assert kernels(by_rule["score_lines"]) == [c[-1] for c in SCORE_LINES]
 
 
 def test_the_prefill_kernels_serve_their_tests(without_narrow):
