@@ -55,17 +55,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
-// Non-blocking: has the phase completed?  Asked ahead of the point where the answer is needed, its latency is hidden.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-
 // Bounded hot wait: polls without a suspend hint or back-off, for the single threads on the critical path of a
 // pipeline (the MMA issuer, the TMA producer), whose wake-up latency is paid on every step.
 __device__ __forceinline__ bool mbar_wait_hot(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t code)
@@ -123,11 +112,6 @@ __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uin
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-// Shared -> global bulk copy (16-byte aligned addresses, size a multiple of 16), tracked by the thread's bulk async-group.
-__device__ __forceinline__ void bulk_copy_s2g(void* dst, uint32_t src, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
 }
 // Loads through L2 of bytes that the kernel before this one may have written (the scales and integers of a KV cache): volatile and with a
 // memory clobber, neither of which __ldcg has, so that the compiler keeps them behind the wait that the source has in front of them.
