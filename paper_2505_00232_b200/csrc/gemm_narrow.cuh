@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(narrow_threads(G), 2) gemm_narrow_kernel(const
             umma_commit(tfull_bar);
         }
     } else if (warp >= kNarrowFirstWorker) {
-        // ------------------------------------------------------------------ dequantise: two groups of four warps take turns
+        // ------------------------------------------------------------------ dequantise: the groups of four warps take turns
         const int quarter = warp & 3, wg = (warp - kNarrowFirstWorker) >> 2;
         const DequantRow64 dq(quarter, lane);
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;

@@ -2,8 +2,8 @@
 // queries over a KV cache (paper Section 3.8: the K cache is a layer with O = cache positions and I = d_h), for up to 8 KV
 // heads of a layer in one launch.
 //
-// Bound: the outputs.  At d_h = 128 a score costs 128 multiply-adds and 2 bytes of HBM; 8 heads x 1024 query rows x 4096
-// positions write 67 MB (10.3 us at the measured copy rate) and keep the warp-level tensor core busy for 15 us (8.05 cycles per
+// Bound: the outputs.  At d_h = 128 a score costs 128 multiply-adds and 2 bytes of HBM; 8 heads x 256 query rows x 4096
+// positions write 17 MB (2.6 us at the measured copy rate) and keep the warp-level tensor core busy for 3.8 us (8.05 cycles per
 // m16n8k16 and SM quarter).  In the prefill kernel such a tile has 2 k-steps and an epilogue that nothing hides.
 //
 // Work decomposition: the tiles (row super-block of 128 positions x 8 NT tokens) of all layers are numbered through, token
@@ -13,8 +13,8 @@
 // through shared memory: stmatrix turns the accumulator fragments, which hold pairs of tokens of one position, into rows of
 // 128 positions, which go out as 256-byte pieces.
 //
-// Measured: 8 heads x 1024 rows x 4096 positions, d_h = 128: 35 us (1.9 TB/s written), 72 us as eight launches of the prefill
-// kernel; 8 heads x 64 rows 4.4 us against 42; 8 heads of 256 x 256 rows 18.6 us against 50.
+// Measured, d_h = 128, 8 heads: 256 rows x 4096 positions 11.6 us (1.4 TB/s written), 128 rows 7.1, 256 rows x 2048 positions 7.1, 64 rows 4.0; 8
+// heads of 256, 128 rows x 4096 positions 10.6.  (As eight launches of the prefill kernel 42 us for 64 rows x 4096 positions, 4.4 here.)
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -156,14 +156,14 @@ __global__ void __launch_bounds__(256, 2) gemm_rows_kernel(const GemmRowsParams 
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// The same for many tokens, on the fifth-generation tensor core.  The warp-level MMAs of the kernel above keep its tensor core busy for 15 us
-// of a launch whose 67 MB of outputs need 10.4, and the reads of x, MMAs, stores and barriers of a tile run one after the other.
+// The same for many tokens, on the fifth-generation tensor core.  At 8 heads x 1024 rows x 4096 positions the warp-level MMAs of the kernel
+// above keep its tensor core busy for 15 us of a launch whose 67 MB of outputs need 10.4, and the reads of x, MMAs, stores and barriers of a tile run one after the other.
 // Here (two CTAs per SM) eight warps convert the super-block's integers once into tensor memory (exact fp16, the A operand) and take finished
 // tiles (128 positions x 64 tokens) out: a thread has one position, scales it, and leaves fp16 in a shared tile whose rows (one token, 256
 // bytes) leave as 16-byte stores (one bulk copy per token: 36 us for the launch above, the copies were the bound).  One thread issues the MMAs of the next tile into the other of two accumulators meanwhile (55 cycles each,
 // which is why none of the eight warps does it: 42 us instead of 35 for the kernel above), one loads x by TMA, some tiles ahead.
 // Every byte is read after griddepcontrol.wait (the cache may have been appended to just before).  Measured: 8 heads x 1024 rows x 4096
-// positions 34.8 -> 24.1 us at d_h = 128 (2.8 TB/s written), 58.6 -> 28.1 at 256; the rule is in forward_gemm_rows.
+// positions 34.8 -> 24.1 us at d_h = 128 (2.8 TB/s written), 58.6 -> 28.1 at 256; the rule is rows_take_tc in qlinear.cu.
 struct GemmRowsMaps { CUtensorMap x[kRowsMaxLayers]; };                  // [M, K] of each layer, box 64 k x 64 tokens, 128-byte swizzle
 constexpr int kRowsTcTokens = 64;
 constexpr int kRowsTcThreads = 320;                                      // warps 0..7 conversion and outputs, 8 MMAs, 9 x
