@@ -792,17 +792,19 @@ GemmPairLayers pair_layers(const qlinear_s* const* hs, int n, void* const* ys)
 bool gate_fits_scratch(int N, int M, int num_sms) { return (size_t)M * N * 2 * sizeof(__half) <= gemm_pair_scratch_bytes(num_sms); }
 
 // Estimates of a launch, us, as consecutive launches with the weights out of HBM take it: what lies between gemm_narrow.cuh and the kernels
-// that served its calls before.  Fitted to 4636 calls of random shapes (8 to 32768 channels, K 32 to 16384, at most 80 million weights, 9 to 2048
-// tokens, plain and gated, the three schemes), each on both routes.  Measured / estimate on 4609 other calls, 5th and 95th percentile (1st
-// and 99th): narrow_us 0.87 and 1.10 (0.75, 1.18), mid_us 0.90 and 1.13 (0.87, 1.21), prefill_us on the CTA-pair kernel 0.83 and 1.40 (0.80, 1.69: gated
-// pairs of K up to 128, far from the line), on the single-CTA kernel 0.85 and 1.07 (0.79, 1.16), on the shared-memory gated form 0.90 and
-// 1.12 (0.89, 1.19), unfused 0.85 and 1.09 (0.81, 1.16).
-// What a CTA's time is multiplied by for the others on its SM, `ctas` of them in clusters of cl, two to an SM: each SM's share slows the CTA by
-// `share`; beyond two per SM further rounds, of which the last one costs `last` at least.  (Clusters of 4 and 8 lie inside a GPC: fewer fit.)
-double sm_load(double ctas, int cl, int num_sms, double share, double last)
+// that served its calls before.  Fitted to 9217 calls of random shapes (8 to 32768 channels, K 32 to 16384, at most 80 million weights, 9 to 2048
+// tokens, plain and gated, the three schemes), each on both routes; long calls and the shapes of the two models weigh more.  Measured /
+// estimate, 5th and 95th percentile (1st and 99th): narrow_us 0.90 and 1.11 (0.84, 1.17), mid_us 0.90 and 1.11 (0.85, 1.16), prefill_us on the
+// CTA-pair kernel 0.83 and 1.19 (0.81, 1.70: gated pairs of K up to 128, far from the line), on the single-CTA kernel 0.86 and 1.07 (0.79, 1.17), on
+// the shared-memory gated form 0.89 and 1.14 (0.88, 1.19), unfused 0.86 and 1.05 (0.81, 1.13).
+// What a CTA's time is multiplied by for the others of the launch, `ctas` in all in clusters of cl, two to an SM: up to one per SM they slow it
+// down by `first`, the second ones by `second` more; beyond two per SM further rounds, of which the last one costs `last` at least.
+// (Clusters of 4 and 8 lie inside a GPC: fewer fit.)
+double sm_load(double ctas, int cl, int num_sms, double first, double second, double last)
 {
     const double u = ctas / (num_sms * (cl == 8 ? 0.87 : cl == 4 ? 0.97 : 1.0));
-    return u <= 2.0 ? 1.0 + share * u : (1.0 + 2.0 * share) * std::min(round_up(u / 2.0), u / 2.0 + last);
+    if (u <= 2.0) return 1.0 + first * std::min(u, 1.0) + second * std::max(u - 1.0, 0.0);
+    return (1.0 + first + second) * std::min(round_up(u / 2.0), u / 2.0 + last);
 }
 
 int total_rsb(const qlinear_s* const* hs, int n) { int t = 0; for (int i = 0; i < n; ++i) t += hs[i]->L.n_rsb; return t; }
@@ -814,8 +816,8 @@ double narrow_us(const qlinear_s* const* hs, int n, int M, bool gated)
     const int rows = gated ? L.n_rsb : total_rsb(hs, n);
     const NarrowPlan pl = plan_narrow(L, rows, gated, M, hs[0]->num_sms);
     const int steps = ((L.K + kNarrowKStep - 1) / kNarrowKStep + pl.cl - 1) / pl.cl * (gated ? 2 : 1);
-    const double cta = steps * (L.bits == 4 ? 0.381 : 0.413) + 1.08 + pl.bn * (0.0244 + (pl.cl == 1 ? 0.0 : gated ? 0.0196 : 0.0054));
-    return 0.72 + 0.098 * log2_of(pl.cl) + sm_load((double)rows * pl.n_tb * pl.cl, pl.cl, hs[0]->num_sms, 0.41, 0.31) * cta;
+    const double cta = steps * (L.bits == 4 ? 0.350 : 0.391) + 1.44 + pl.bn * (0.0204 + (pl.cl == 1 ? 0.0 : gated ? 0.0197 : 0.0067));
+    return 0.47 + 0.087 * log2_of(pl.cl) + sm_load((double)rows * pl.n_tb * pl.cl, pl.cl, hs[0]->num_sms, 0.489, 0.259, 0.37) * cta;
 }
 
 double mid_us(const qlinear_s* const* hs, int n, int M, bool gated)      // up to 64 tokens
@@ -823,9 +825,9 @@ double mid_us(const qlinear_s* const* hs, int n, int M, bool gated)      // up t
     const Layout& L = hs[0]->L;
     const int nt = M <= 16 ? 2 : M <= 24 ? 3 : M <= 32 ? 4 : M <= 48 ? 6 : 8, units = gated ? (L.N + 63) / 64 : total_rsb(hs, n);
     const int n_steps = (L.n_kc + 1) / 2, cl = mid_parts(units, n_steps, hs[0]->num_sms);
-    const double step = L.bits == 8 ? 0.121 + 0.0507 * nt : 0.185 + 0.0877 * nt;
-    const double cta = (n_steps + cl - 1) / cl * step + 0.425 + nt * (0.144 + (cl > 1 ? 0.044 : 0.0));
-    return 0.77 + 0.118 * log2_of(cl) + sm_load((double)units * cl, cl, hs[0]->num_sms, 0.576, 0.25) * cta;
+    const double step = L.bits == 8 ? 0.113 + 0.0511 * nt : 0.174 + 0.0886 * nt;
+    const double cta = (n_steps + cl - 1) / cl * step + 0.313 + nt * (0.127 + (cl > 1 ? 0.054 : 0.0));
+    return 0.96 + 0.093 * log2_of(cl) + sm_load((double)units * cl, cl, hs[0]->num_sms, 0.772, 0.252, 0.46) * cta;
 }
 
 double pair_ta_us(const Layout& L, int pairs, int M, int layers, bool split, double mb, int num_sms)
@@ -833,7 +835,7 @@ double pair_ta_us(const Layout& L, int pairs, int M, int layers, bool split, dou
     const int mblk = (M + 255) / 256, bn = gemm_pair_ta_width(M), steps = (L.K + kGemmKStep - 1) / kGemmKStep;
     const int parts = split ? gemm_pair_ta_split(pairs * mblk, steps, num_sms, true) : 1;
     const double rounds = round_up((double)pairs * mblk * parts / (num_sms / 2));
-    return 2.5 + 0.0061 * bn + rounds * (layers * ((steps + parts - 1) / parts) * (0.199 + 0.0004 * bn)) + (parts > 1 ? 7.1 + 0.0125 * bn : 0.0) + 0.37 * mb;
+    return 2.66 + 0.0058 * bn + rounds * (layers * ((steps + parts - 1) / parts) * (0.236 + 0.0003 * bn)) + (parts > 1 ? 6.2 + 0.0162 * bn : 0.0) + 0.34 * mb;
 }
 
 double single_us(const Layout& L, int M, double mb, int num_sms)
@@ -888,10 +890,10 @@ bool narrow_can(const qlinear_s* const* hs, int n, int M, bool gated, bool batch
 }
 
 // The kernel of a call beyond the decode stage: one layer, n > 1 layers that share x, or (gated) a pair.  gemm_narrow.cuh where its
-// estimate is 3 % below that of gemm_mid.cuh, 5 % below that of the CTA-pair kernel, and up to 5 % above those of the three other forms (single
-// CTA, shared-memory gating, unfused gating).  No line is always right with these errors.  Of the 4636 calls that the estimates were fitted to and
-// 4609 others, 30 run more than 3 % slower this way than on the other route: 23 of 3613 against gemm_mid.cuh (by 24 % at most), 2 of 1429 against the
-// CTA-pair kernel (11 %), 5 of 4203 against the other forms (9 %).  Measured, us, the route otherwise / gemm_narrow.cuh:
+// estimate is below that of gemm_mid.cuh, 7 % below that of the CTA-pair kernel, or below those of the three other forms (single CTA,
+// shared-memory gating, unfused gating).  No line is always right with these errors.  Of the calls above and 3110 others, 80 run more than 3 %
+// slower this way than on the other route: 54 of 4821 against gemm_mid.cuh (two of them by 46 and 26 %, the others by 24 % at most), 17 of 2018
+// against the CTA-pair kernel (19 %), 9 of 5488 against the other forms (9 %); all together take 0.8 % more than on the faster route each.  Measured, us, the route otherwise / gemm_narrow.cuh:
 //   weights                        16 tokens     24           32           48           64
 //     0.3 M (512 x 512)             2.8 /  3.7   3.0 /  3.8   3.3 /  4.0   3.8 /  4.2   4.1 /  4.5
 //     1 M (1024 x 1024, int8)       3.2 /  4.3   3.5 /  4.5   4.0 /  4.6   4.6 /  5.0   5.2 /  5.3
@@ -910,7 +912,7 @@ ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
     const ql_kernel other = batch ? QL_KERNEL_MID : prefill_kernel(hs, n, M, gated);
     if (!narrow_can(hs, n, M, gated, batch)) return other;
     if (config().narrow == 2) return QL_KERNEL_NARROW;
-    const double limit = batch ? 0.97 * mid_us(hs, n, M, gated) : (other == QL_KERNEL_PAIR_TA ? 0.95 : 1.05) * prefill_us(other, hs, n, M, gated);
+    const double limit = batch ? mid_us(hs, n, M, gated) : (other == QL_KERNEL_PAIR_TA ? 0.93 : 1.0) * prefill_us(other, hs, n, M, gated);
     return narrow_us(hs, n, M, gated) < limit ? QL_KERNEL_NARROW : other;
 }
 
