@@ -39,6 +39,7 @@ struct GemvColsParams {
     __half* y[kGemvMaxBatch];                    // [M, N]
     int32_t n_layers, M, N, K, n_rb, n_kc, cl, cps;   // layers of equal shape: n_rb row-blocks each
     int32_t hold0, hold1;                        // chunks that the kernel before this one may be writing (a KV cache): read after griddepcontrol.wait only
+    int32_t late;                                // all of them (see GemvRowsParams)
 };
 
 __global__ void __launch_bounds__(kColsThreads, 1) gemv_cols_kernel(const GemvColsParams p)
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(kColsThreads, 1) gemv_cols_kernel(const GemvCo
         asm volatile("cp.async.commit_group;" ::: "memory");             // (an empty group keeps the count in step)
     };
     auto held = [&](int kc) { return kc >= p.hold0 && kc < p.hold1; };
+    if (p.late) asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int i = 0; i < kColsRing; ++i)
         if (!held(kc0 + i)) copy_w(kc0 + i);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

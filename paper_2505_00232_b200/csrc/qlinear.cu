@@ -207,6 +207,15 @@ void held_tokens(const qlinear_s* const* hs, int n, cudaStream_t st, int32_t* fi
     }
 }
 
+// The same for a launch over caches of up to `tokens`: true, and an empty range, where all of them are held.
+bool hold_range(const qlinear_s* const* hs, int n, cudaStream_t st, int32_t tokens, int32_t* first, int32_t* end)
+{
+    held_tokens(hs, n, st, first, end);
+    const bool all = *first == 0 && *end >= tokens;
+    if (all) *end = 0;
+    return all;
+}
+
 constexpr int kGemvMaxSmem = 96 * 1024;
 
 // n_rb: row-blocks of the launch (one layer, or all layers of a group that shares x).
@@ -426,7 +435,7 @@ ql_status forward_gemv_cols(qlinear_s* const* hs, int n, const void* const* xs, 
         p.y[i] = static_cast<__half*>(ys[i]);
     }
     p.n_layers = n; p.M = M; p.N = L.N; p.K = L.K; p.n_rb = h->n_rb; p.n_kc = L.n_kc;
-    held_tokens(hs, n, st, &p.hold0, &p.hold1);
+    p.late = hold_range(hs, n, st, L.K, &p.hold0, &p.hold1);
     p.hold0 /= 32;
     p.hold1 = (p.hold1 + 31) / 32;
     static std::atomic<bool> attr_set[kMaxDevices];
@@ -474,7 +483,9 @@ ql_status forward_gemv(qlinear_s* const* hs, int n, const void* x, void* const* 
             n_rsb += Li.n_rsb;
             rp.rsb_end[i] = n_rsb;
         }
-        held_tokens(hs, n, st, &rp.hold0, &rp.hold1);
+        int32_t longest = 0;
+        for (int i = 0; i < n; ++i) longest = std::max(longest, hs[i]->L.N);
+        rp.late = hold_range(hs, n, st, longest, &rp.hold0, &rp.hold1);
         rp.n_layers = n; rp.M = M; rp.K = L.K; rp.n_rsb = n_rsb; rp.block_bytes = L.block_bytes;
         const cudaError_t e = L.n_kc == 2 ? launch_gemv_rows<2>(h, rp, st) : L.n_kc == 4 ? launch_gemv_rows<4>(h, rp, st) : launch_gemv_rows<8>(h, rp, st);
         return e == cudaSuccess ? QL_OK : QL_ERR_CUDA;
