@@ -67,6 +67,7 @@ struct GemmParams {
     // quantised row (device arrays, padded to whole token tiles)
     const float* a8_scale;
     const int32_t* a8_rowsum;
+    int32_t a8_last;                         // tensor-memory form: the last group of four of them
 };
 constexpr int kGemmMaxGroup = 4;
 

@@ -44,6 +44,8 @@
 // Protocol between the two CTAs: own loads only; the leader issues; commits are multicast to both CTAs; the peer relays
 // "slot ready" (see the relay below).
 #pragma once
+#include <type_traits>
+
 #include "gemm_pair.cuh"
 
 namespace ql {
@@ -227,14 +229,17 @@ struct DequantRowTa {
 // I8 (per-channel schemes, not gated): maps.x describes int8 activations; the stored weight integers go to the A slots
 // unconverted, the MMAs are kind::i8 with an s32 accumulator, and the epilogue removes the storage offset (offset x the
 // sum of the token's quantised row) and applies both scales (paper Section 3.7, prefill stage).
-template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false>
+// PARTS: the launch has K parts (p.split is 2 or 4).  An instantiation of its own: the registers of one epilogue are the kernel's limit
+// (Gemma2-2B q + k + v at 777 tokens, which has no parts, 16.8 us with both in one kernel, 16.5 without).
+template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false, bool PARTS = false>
 __global__ void __launch_bounds__(kPairThreads, 1)
 gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
 {
     static_assert(!I8 || (!GATED && !GROUPED), "the integer form: per-channel scales, plain output");
+    static_assert(!GATED || !PARTS, "a gated tile has no parts");
     using S = GemmTaSmem<BITS, I8>;
     constexpr int NX = S::kXStages, NW = S::kWStages, NA = S::kASlots;
-    const int bn = I8 ? 256 : p.bn;                                                 // tokens per tile: a multiple of 32, at most 256
+    const int bn = p.bn;                                                 // tokens per tile: a multiple of 32, at most 256
     constexpr int W_BOX_BYTES = I8 ? S::kWBytes : BITS == 4 ? (GROUPED ? kWeightBlockBytes + kScaleBlockBytes : kWeightBlockBytes) : 2 * kWeightBlockBytes;
     extern __shared__ unsigned char smem_dyn[];
     uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -263,7 +268,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     const int first_tile = blockIdx.x >> 1, tile_stride = gridDim.x >> 1;   // tile = (rsb pair, token block)
     // K split (p.split = 2 or 4 parts per tile; launches with so few tiles that every cluster then has ONE unit of work):
     // work unit v = tile * split + part, this cluster's part covers k-steps [it_base, it_base + n_steps) of its tile
-    const int P = GATED ? 1 : p.split;
+    const int P = PARTS ? p.split : 1;
     const int part = P > 1 ? first_tile % P : 0;
     const int it_base = part * p.n_ksteps / P;
     const int n_steps = (part + 1) * p.n_ksteps / P - it_base;          // k-steps per unit of work of this cluster
@@ -440,58 +445,109 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         const uint32_t out_addr = base + S::kOutOffset;
         unsigned char* out_ptr = base_ptr + S::kOutOffset;
         const int grp_thread = quarter * 32 + lane;                      // 0..127 inside the group of four warps
-        const int n_cols = I8 ? 64 : max(0, min(64, bn - 64 * wi));                // columns (tokens) of this warp: 0, 32 or 64
-        // K-split tile: every part parks its fp32 accumulator in the device's scratch ([token][channel], a warp writes
-        // 128 contiguous bytes per token), frees the accumulator and counts itself in; the part that arrives last adds all
-        // parts in part order (fixed order, no float atomics, nobody waits) and stores y.
-        auto split_epilogue = [&](int j, int tile) {
+        const int n_cols = max(0, min(64, bn - 64 * wi));                // columns (tokens) of this warp: 0, 32 or 64
+        // K-split tile: every part parks its accumulator (fp32; integer form: s32) in the device's scratch ([4 tokens][channel][token], 16
+        // bytes per thread, 512 per warp) and counts itself in; the part that arrives last adds all parts in part order (fixed
+        // order, no float atomics, nobody waits) and stores y.  A cluster has one unit of work here: its own part is still in
+        // tensor memory, and the stages are free, so a thread copies what it needs of the other parts there, all its tokens (P = 4:
+        // 32 at a time) in flight.  Instructions count here, too: 64 outputs per thread, 16 warps.  (Loaded into registers 8 tokens at a time, a
+        // Gemma2-2B down projection of 777 tokens in 2 parts took 33.7 us, now 30.4; with part numbers known at run time only, 38.7.)
+        auto split_epilogue = [&](int j, int tile, auto parts) {
+            constexpr int NP = decltype(parts)::value;
             int rsb = 2 * (tile / n_mblk) + (int)rank;
             const int ly = pair_layer(p, rsb);
             const int N = p.lN[ly];
             const int m0 = (tile % n_mblk) * bn + 64 * wi;
-            float* slab0 = p.scratch + ((int64_t)((tile * P) * 2 + (int)rank) * bn + 64 * wi) * 128 + grp_thread;   // part 0
+            float* slab0 = p.scratch + ((int64_t)((tile * NP) * 2 + (int)rank) * bn + 64 * wi) * 128 + grp_thread * 4;   // part 0
             const int64_t part_stride = (int64_t)2 * bn * 128;
             unsigned int* cnt = p.counters + ((tile * 2 + (int)rank) * 4 + wi) * 4 + quarter;
             if (!mbar_wait(tfull_bar, (uint32_t)(j & 1), abort_flag, 0x500)) { ok = false; return; }
             tc_fence_after();
             const uint32_t taddr = tmem_base + lane_base + (uint32_t)(64 * wi);
+            const int m_left = min(n_cols, p.M - m0);                    // (tokens beyond M are nobody's)
             float* mine = slab0 + part * part_stride;
 #pragma unroll 1
-            for (int cc = 0; cc < n_cols; cc += 16) {
+            for (int cc = 0; cc < m_left; cc += 16) {
                 uint32_t r[16];
                 tmem_ld16(taddr + (uint32_t)cc, r);
 #pragma unroll
-                for (int q = 0; q < 16; ++q) __stcg(mine + (cc + q) * 128, __uint_as_float(r[q]));
+                for (int q = 0; q < 4; ++q)
+                    __stcg(reinterpret_cast<uint4*>(mine + (cc + 4 * q) * 128), make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]));
             }
-            tc_fence_before();
             __threadfence();
             __syncwarp();
             unsigned int old = 0;
-            if (lane == 0) { mbar_arrive_remote_relaxed(tempty_bar, 0); old = atomicAdd(cnt, 1u); }
+            if (lane == 0) old = atomicAdd(cnt, 1u);
             old = __shfl_sync(0xffffffffu, old, 0);
-            if ((int)old != P - 1) return;
+            if ((int)old != NP - 1) return;
             __threadfence();
             const int n = rsb * kRsbRows + quarter * 32 + lane;
             float scale = 1.f;
             if (!GROUPED && n < N) scale = __half2float(p.lscales[ly][n]);
-            __half* yrow = p.ly[ly] + (int64_t)m0 * N + n;
-            const int m_left = min(n_cols, p.M - m0);
+            __half* yp = p.ly[ly] + (int64_t)m0 * N + n;
+            constexpr int kBatch = NP == 2 ? 64 : 32;                    // tokens
+            constexpr int kPartBytes = kBatch * 128, kWarpBytes = (NP - 1) * kPartBytes + (I8 ? 512 : 0);   // of a warp
+            static_assert(kTaEpilogueWarps * kWarpBytes <= S::kBarOffset, "the stages and the output tile hold the parts");
+            const uint32_t warp_stage = base + (uint32_t)((warp - kTaFirstDequantWarp) * kWarpBytes), stage = warp_stage + lane * 16;
+            if constexpr (I8) {                                          // the 64 tokens' scales and row sums, behind the parts
+                const int m = min(m0 + 4 * (lane & 15), p.a8_last);
+                const void* src = lane < 16 ? static_cast<const void*>(p.a8_scale + m) : p.a8_rowsum + m;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage + (NP - 1) * kPartBytes), "l"(src) : "memory");
+            }
 #pragma unroll 1
-            for (int cc = 0; cc < m_left; cc += 8) {
-                float acc[8];
+            for (int c0 = 0; c0 < m_left; c0 += kBatch) {
+                const int left = min(kBatch, m_left - c0);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) acc[q] = __ldcg(slab0 + (cc + q) * 128);
-                for (int pp = 1; pp < P; ++pp) {
-                    float v[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) v[q] = __ldcg(slab0 + pp * part_stride + (cc + q) * 128);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) acc[q] += v[q];
+                for (int o = 0; o < NP - 1; ++o) {                       // the others, in part order
+                    const float* src = slab0 + (o + (o >= part ? 1 : 0)) * part_stride + c0 * 128;
+#pragma unroll 4
+                    for (int tok = 0; tok < left; tok += 4)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage + o * kPartBytes + tok * 128), "l"(src + tok * 128) : "memory");
                 }
-                if (n < N) {
+                asm volatile("cp.async.wait_all;" ::: "memory");         // (a thread reads the parts that it copied itself)
+                if constexpr (I8) __syncwarp();
+#pragma unroll 1
+                for (int cc = 0; cc < left; cc += 16) {
+                    uint32_t own[16];
+                    tmem_ld16(taddr + (uint32_t)(c0 + cc), own);
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (cc + q < m_left) yrow[(int64_t)(cc + q) * N] = __float2half_rn(acc[q] * scale);
+                    for (int q4 = 0; q4 < 4; ++q4) {
+                        if (cc + 4 * q4 >= left) break;
+                        uint32_t v[NP][4];
+                        [[maybe_unused]] uint4 sx, rs;
+                        if constexpr (I8) {
+                            const uint32_t a = warp_stage + (NP - 1) * kPartBytes + (c0 + cc + 4 * q4) * 4;
+                            sx = lds_u128(a);
+                            rs = lds_u128(a + 256);
+                        }
+#pragma unroll
+                        for (int o = 0; o < NP - 1; ++o) {
+                            const uint4 w = lds_u128(stage + o * kPartBytes + (cc + 4 * q4) * 128);
+                            v[o][0] = w.x; v[o][1] = w.y; v[o][2] = w.z; v[o][3] = w.w;
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            // part order: the own part goes in at its place (two parts: a sum of two has no order)
+                            const uint32_t mine_i = own[4 * q4 + i];
+                            auto add = [](uint32_t x, uint32_t y) { return I8 ? x + y : __float_as_uint(__uint_as_float(x) + __uint_as_float(y)); };
+                            uint32_t sum;
+                            if (NP == 2) sum = add(v[0][i], mine_i);
+                            else {
+                                sum = add(part == 0 ? mine_i : v[0][i], part == 0 ? v[0][i] : part == 1 ? mine_i : v[1][i]);
+                                sum = add(sum, part <= 1 ? v[1][i] : part == 2 ? mine_i : v[2][i]);
+                                sum = add(sum, part <= 2 ? v[2][i] : mine_i);
+                            }
+                            const int tok = c0 + cc + 4 * q4 + i;
+                            float o = __uint_as_float(sum) * scale;
+                            if constexpr (I8) {
+                                constexpr int OFF = BITS == 4 ? 8 : 128; // as in the epilogue without parts
+                                const uint32_t f = i == 0 ? sx.x : i == 1 ? sx.y : i == 2 ? sx.z : sx.w, r = i == 0 ? rs.x : i == 1 ? rs.y : i == 2 ? rs.z : rs.w;
+                                o = __uint_as_float(f) * (scale * (float)((int)sum - OFF * (int)r));
+                            }
+                            if (n < N && tok < m_left) *yp = __float2half_rn(o);
+                            yp += N;
+                        }
+                    }
                 }
             }
             if (lane == 0) *cnt = 0;                                     // ready for the next launch
@@ -499,7 +555,11 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         auto epilogue = [&](int j) {
             int tile, gl;
             unit(j, tile, gl);
-            if (P > 1) { split_epilogue(j, tile); return; }
+            if constexpr (PARTS) {
+                if (P == 2) split_epilogue(j, tile, std::integral_constant<int, 2>{});
+                else split_epilogue(j, tile, std::integral_constant<int, 4>{});
+                return;
+            }
             int rsb = 2 * (tile / n_mblk) + (int)rank;
             const int ly = GATED ? 0 : pair_layer(p, rsb);
             const int N = p.lN[ly];
@@ -530,26 +590,34 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                     if (lane == 0) mbar_arrive_remote_relaxed(tempty_bar, 0);
                 };
                 if (n_cols == 0) release();
+                if constexpr (I8) {
+                    // acc = sum (q + off) * xq: remove off * (sum of the token's quantised row), then both scales; the tokens' scales and row
+                    // sums come as whole lines (the arrays are padded to whole tiles).  16 tokens at a time: with 32 the loads of all of
+                    // them were scheduled ahead of the arithmetic, at the price of 124 bytes of spills.
+                    constexpr int OFF = BITS == 4 ? 8 : 128;
+#pragma unroll 1
+                    for (int cc = 0; cc < n_cols; cc += 16) {
+                        uint32_t r[16];
+                        tmem_ld16(taddr + (uint32_t)cc, r);
+                        if (cc + 16 >= n_cols) release();
 #pragma unroll
-                for (int cc = 0; cc < 64; cc += 32) {
-                    if (cc >= n_cols) break;
-                    uint32_t r[32];
-                    tmem_ld32(taddr + (uint32_t)cc, r);
-                    if (cc + 32 >= n_cols) release();
-                    if (I8) {
-                        // acc = sum (q + off) * xq: remove off * (sum of the token's quantised row), then both scales; the 32
-                        // tokens' scales and row sums come as whole lines (the arrays are padded to whole tiles)
-                        constexpr int OFF = BITS == 4 ? 8 : 128;
-#pragma unroll
-                        for (int v4 = 0; v4 < 8; ++v4) {
-                            const float4 f = __ldg(reinterpret_cast<const float4*>(p.a8_scale + m0 + cc) + v4);
-                            const int4 i = __ldg(reinterpret_cast<const int4*>(p.a8_rowsum + m0 + cc) + v4);
+                        for (int v4 = 0; v4 < 4; ++v4) {
+                            const int m = min(m0 + cc + 4 * v4, p.a8_last);
+                            const float4 f = __ldcg(reinterpret_cast<const float4*>(p.a8_scale + m));
+                            const int4 i = __ldcg(reinterpret_cast<const int4*>(p.a8_rowsum + m));
                             orow[(cc + 4 * v4 + 0) * 128] = __float2half_rn(f.x * (scale * (float)((int)r[4 * v4 + 0] - OFF * i.x)));
                             orow[(cc + 4 * v4 + 1) * 128] = __float2half_rn(f.y * (scale * (float)((int)r[4 * v4 + 1] - OFF * i.y)));
                             orow[(cc + 4 * v4 + 2) * 128] = __float2half_rn(f.z * (scale * (float)((int)r[4 * v4 + 2] - OFF * i.z)));
                             orow[(cc + 4 * v4 + 3) * 128] = __float2half_rn(f.w * (scale * (float)((int)r[4 * v4 + 3] - OFF * i.w)));
                         }
-                    } else {
+                    }
+                } else {
+#pragma unroll
+                    for (int cc = 0; cc < 64; cc += 32) {
+                        if (cc >= n_cols) break;
+                        uint32_t r[32];
+                        tmem_ld32(taddr + (uint32_t)cc, r);
+                        if (cc + 32 >= n_cols) release();
                         // (the kind of activation is chosen outside the element loop: inside it, the compiler evaluates
                         // every kind and selects)
                         auto store32 = [&](auto f) {
@@ -678,47 +746,42 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     }
 }
 
-// The tensor-memory form: tiles of up to 256 tokens, whole tiles dealt out round-robin, or (fewer tiles than half the CTA pairs)
-// 2 or 4 K parts per tile that meet in the device's scratch.
-// K parts per tile for a launch of `tiles` tiles: 1 unless the tiles would leave half of the CTA pairs (or more) idle.
-inline int gemm_pair_ta_split(int tiles, int n_ksteps, int num_sms, bool have_scratch)
-{
-    const int clusters = num_sms / 2;
-    int split = 1;
-    if (!have_scratch || tiles >= clusters) return 1;
-    if (gemm_config().force_split > 0) split = gemm_config().force_split >= 4 ? 4 : gemm_config().force_split >= 2 ? 2 : 1;
-    else if (tiles * 4 <= clusters) split = 4;
-    else if (tiles * 2 <= clusters) split = 2;
-    while (split > 1 && (n_ksteps / split < 8 || tiles * split > clusters)) split >>= 1;
-    return split;
-}
-
-// Tokens per tile: M in as few blocks of at most 256 as it takes, all of the same width (the MMA's N, a multiple of 32).  A
+// Token blocks: M in as few blocks of at most 256 as it takes, all of the same width (the MMA's N, a multiple of 32).  A
 // narrower tile costs the same dequantisation and less tensor-core time, x traffic and epilogue
 // (a Llama block at 100 tokens 145.9 -> 136.9 us, at 300 224.9 -> 211.1).
-inline int gemm_pair_ta_width(int M)
+// K parts per tile: 1 unless the tiles would leave half of the CTA pairs (or more) idle.
+struct TaPlan { int n_mblk, bn, split; };
+inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int num_sms, bool may_split)
 {
-    const int n_mblk = (M + 255) / 256;
-    return ((M + n_mblk - 1) / n_mblk + 31) / 32 * 32;
+    const int clusters = num_sms / 2;
+    TaPlan pl;
+    pl.n_mblk = (M + 255) / 256;
+    pl.bn = ((M + pl.n_mblk - 1) / pl.n_mblk + 31) / 32 * 32;
+    pl.split = 1;
+    const int tiles = pairs * pl.n_mblk;
+    if (!may_split || tiles >= clusters) return pl;
+    if (gemm_config().force_split > 0) pl.split = gemm_config().force_split >= 4 ? 4 : gemm_config().force_split >= 2 ? 2 : 1;
+    else if (tiles * 4 <= clusters) pl.split = 4;
+    else if (tiles * 2 <= clusters) pl.split = 2;
+    while (pl.split > 1 && (n_ksteps / pl.split < 8 || tiles * pl.split > clusters)) pl.split >>= 1;
+    return pl;
 }
 
 // act < 0: the plain form.  act >= 0: the gated form, set = {gate, up} of equal shape, y[0] the output.
 // scratch / counters: the device's shared fp32 scratch and arrival counters for the K-split case (null: no split).
 // a8_scale != nullptr: the integer form; x is then the int8 activations, a8_scale / a8_rowsum their per-token arrays, and
 // set.wmap the integer form's weight maps (boxes of 128 k).
-template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false>
-ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const void* x, int M, cudaStream_t st, int device, bool pdl, int num_sms, int act = -1,
+template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false, bool PARTS = false>
+ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const TaPlan& pl, const void* x, int M, cudaStream_t st, int device, bool pdl, int num_sms, int act = -1,
                               float* scratch = nullptr, unsigned int* counters = nullptr,
                               const float* a8_scale = nullptr, const int32_t* a8_rowsum = nullptr)
 {
     using S = GemmTaSmem<BITS, I8>;
     const Layout& L = *set.L[0];
     TaMaps maps;
-    // The integer form keeps 256 tokens: a narrower tile gains nothing at 300 tokens, and its epilogue is short of registers.
-    const int n_mblk = (M + 255) / 256, bn = I8 ? 256 : gemm_pair_ta_width(M);
-    if (!x_tensor_map(x, L.K, M, bn / 2, &maps.x, I8 ? 1 : 2)) return QL_ERR_CUDA;
+    if (!x_tensor_map(x, L.K, M, pl.bn / 2, &maps.x, I8 ? 1 : 2)) return QL_ERR_CUDA;
     for (int i = 0; i < kGemmMaxGroup; ++i) maps.w[i] = *set.wmap[i < set.n ? i : 0];
-    auto kern = gemm_pair_ta_kernel<BITS, GROUPED, GATED, I8>;
+    auto kern = gemm_pair_ta_kernel<BITS, GROUPED, GATED, I8, PARTS>;
     static std::atomic<bool> attr_set[64];
     if (device >= 0 && device < 64 && !attr_set[device]) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal) != cudaSuccess) {
@@ -745,10 +808,11 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const void* x, int M, c
     prm.n_ksteps = (L.K + S::kKStep - 1) / S::kKStep;
     prm.a8_scale = a8_scale; prm.a8_rowsum = a8_rowsum;
     prm.n_rsb = n_rsb;
-    prm.bn = bn;
+    prm.bn = pl.bn;
+    prm.a8_last = (M + 255) / 256 * 256 - 4;
     prm.late = set.late;
-    prm.n_tiles = (n_rsb / 2) * n_mblk;
-    prm.split = (GATED || I8) ? 1 : gemm_pair_ta_split(prm.n_tiles, prm.n_ksteps, num_sms, scratch && counters);
+    prm.n_tiles = (n_rsb / 2) * pl.n_mblk;
+    prm.split = PARTS ? pl.split : 1;
     prm.scratch = scratch;
     prm.counters = counters;
     prm.n_whole = prm.n_tiles;
@@ -799,34 +863,43 @@ inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, 
         const unsigned char* y = static_cast<const unsigned char*>(set.y[i]);
         if (y >= s0 && y < s0 + gemm_pair_scratch_bytes(num_sms)) scratch = nullptr;
     }
-    if (L.bits == 8) return gemm_pair_ta_launch<8, false>(set, x, M, st, device, pdl, num_sms, -1, scratch, counters);
-    if (L.grouped) return gemm_pair_ta_launch<4, true>(set, x, M, st, device, pdl, num_sms, -1, scratch, counters);
-    return gemm_pair_ta_launch<4, false>(set, x, M, st, device, pdl, num_sms, -1, scratch, counters);
+    const TaPlan pl = gemm_pair_ta_plan(set.n_rsb() / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, scratch && counters);
+    if (pl.split > 1) {
+        if (L.bits == 8) return gemm_pair_ta_launch<8, false, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, -1, scratch, counters);
+        if (L.grouped) return gemm_pair_ta_launch<4, true, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, -1, scratch, counters);
+        return gemm_pair_ta_launch<4, false, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, -1, scratch, counters);
+    }
+    if (L.bits == 8) return gemm_pair_ta_launch<8, false>(set, pl, x, M, st, device, pdl, num_sms);
+    if (L.grouped) return gemm_pair_ta_launch<4, true>(set, pl, x, M, st, device, pdl, num_sms);
+    return gemm_pair_ta_launch<4, false>(set, pl, x, M, st, device, pdl, num_sms);
 }
 
 // Gated form: set = {gate, up}, both pair-applicable and of equal shape; y[0] receives act(gate) * up.
 inline ql_status gemm_pair_ta_forward_gated(const GemmPairLayers& set, const void* x, int M, int act, cudaStream_t st, int device, bool pdl, int num_sms)
 {
     const Layout& L = *set.L[0];
-    if (L.bits == 8) return gemm_pair_ta_launch<8, false, true>(set, x, M, st, device, pdl, num_sms, act);
-    if (L.grouped) return gemm_pair_ta_launch<4, true, true>(set, x, M, st, device, pdl, num_sms, act);
-    return gemm_pair_ta_launch<4, false, true>(set, x, M, st, device, pdl, num_sms, act);
+    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, false);
+    if (L.bits == 8) return gemm_pair_ta_launch<8, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
+    if (L.grouped) return gemm_pair_ta_launch<4, true, true>(set, pl, x, M, st, device, pdl, num_sms, act);
+    return gemm_pair_ta_launch<4, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
 }
 
 // Integer form (per-channel schemes, K a multiple of 128): xq int8 [M, K] with per-token scale and row sum; set.wmap
-// holds the integer form's weight maps.  No K split: launches with fewer tiles than half the CTA pairs stay on the
-// shared-memory kernel.
-inline bool gemm_pair_ta_i8_applicable(const GemmPairLayers& set, int M, int num_sms)
+// holds the integer form's weight maps.  scratch / counters: for K parts (null: none).
+inline bool gemm_pair_ta_i8_applicable(const GemmPairLayers& set, int M)
 {
-    if (!gemm_config().ta || M <= 128 || !set.wmap[0]) return false;
-    return set.L[0]->n_rsb / 2 * ((M + 255) / 256) * 2 > num_sms / 2;
+    return gemm_config().ta && M > 128 && set.wmap[0];
 }
 inline ql_status gemm_pair_ta_forward_i8(const GemmPairLayers& set, const void* xq, const float* scale, const int32_t* rowsum, int M,
-                                         cudaStream_t st, int device, bool pdl, int num_sms)
+                                         cudaStream_t st, int device, bool pdl, int num_sms, float* scratch, unsigned int* counters)
 {
     const Layout& L = *set.L[0];
-    if (L.bits == 8) return gemm_pair_ta_launch<8, false, false, true>(set, xq, M, st, device, pdl, num_sms, -1, nullptr, nullptr, scale, rowsum);
-    return gemm_pair_ta_launch<4, false, false, true>(set, xq, M, st, device, pdl, num_sms, -1, nullptr, nullptr, scale, rowsum);
+    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + 127) / 128, num_sms, scratch && counters);
+    if (pl.split > 1)
+        return L.bits == 8 ? gemm_pair_ta_launch<8, false, false, true, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, scratch, counters, scale, rowsum)
+                           : gemm_pair_ta_launch<4, false, false, true, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, scratch, counters, scale, rowsum);
+    if (L.bits == 8) return gemm_pair_ta_launch<8, false, false, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, nullptr, nullptr, scale, rowsum);
+    return gemm_pair_ta_launch<4, false, false, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, nullptr, nullptr, scale, rowsum);
 }
 
 }  // namespace ql

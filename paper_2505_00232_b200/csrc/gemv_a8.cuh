@@ -361,7 +361,9 @@ __global__ void __launch_bounds__(256) quantize_activations_kernel(const __half*
     __shared__ float wmax[8];
     __shared__ int wsum[8];
     __shared__ float recip;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the matmul behind it may set up and request its weights; it reads what is written here, in scratch that the matmul before may still be
+    // reading, past its own wait (its epilogue with loads that pass L1 by)
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
     const int m = blockIdx.x;
     const uint4* row = reinterpret_cast<const uint4*>(x + (int64_t)m * K);
     float am = 0.f;

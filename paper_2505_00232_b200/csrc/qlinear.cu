@@ -843,10 +843,10 @@ double mid_us(const qlinear_s* const* hs, int n, int M, bool gated)      // up t
 
 double pair_ta_us(const Layout& L, int pairs, int M, int layers, bool split, double mb, int num_sms)
 {
-    const int mblk = (M + 255) / 256, bn = gemm_pair_ta_width(M), steps = (L.K + kGemmKStep - 1) / kGemmKStep;
-    const int parts = split ? gemm_pair_ta_split(pairs * mblk, steps, num_sms, true) : 1;
-    const double rounds = round_up((double)pairs * mblk * parts / (num_sms / 2));
-    return 2.66 + 0.0058 * bn + rounds * (layers * ((steps + parts - 1) / parts) * (0.236 + 0.0003 * bn)) + (parts > 1 ? 6.2 + 0.0162 * bn : 0.0) + 0.34 * mb;
+    const int steps = (L.K + kGemmKStep - 1) / kGemmKStep;
+    const TaPlan pl = gemm_pair_ta_plan(pairs, M, steps, num_sms, split);
+    const double rounds = round_up((double)pairs * pl.n_mblk * pl.split / (num_sms / 2));
+    return 2.66 + 0.0058 * pl.bn + rounds * (layers * ((steps + pl.split - 1) / pl.split) * (0.236 + 0.0003 * pl.bn)) + (pl.split > 1 ? 6.2 + 0.0162 * pl.bn : 0.0) + 0.34 * mb;
 }
 
 double single_us(const Layout& L, int M, double mb, int num_sms)
@@ -1302,6 +1302,22 @@ cudaError_t launch_a8(const qlinear_s* h, const GemvA8Params& prm, const GemvPla
 }
 }  // namespace
 
+namespace {
+cudaError_t launch_quantize(const __half* x, signed char* xq, float* scale, int32_t* rowsum, int M, int K, cudaStream_t st, bool pdl)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(M);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, quantize_activations_kernel, x, xq, scale, rowsum, M, K);
+}
+}  // namespace
+
 extern "C" ql_status qlinear_forward_a8(qlinear_t h, const void* x, void* y, int32_t M, void* stream)
 {
     if (!h || !x || !y || M < 1) return QL_ERR_INVALID_ARG;
@@ -1323,11 +1339,15 @@ extern "C" ql_status qlinear_forward_a8(qlinear_t h, const void* x, void* y, int
         signed char* xq = reinterpret_cast<signed char*>(base);
         float* sx = reinterpret_cast<float*>(base + xq_bytes);
         int32_t* rs = reinterpret_cast<int32_t*>(base + xq_bytes + arr);
-        quantize_activations_kernel<<<M, 256, 0, st>>>(static_cast<const __half*>(x), xq, sx, rs, M, L.K);
-        if (cudaGetLastError() != cudaSuccess) return QL_ERR_CUDA;
+        if (launch_quantize(static_cast<const __half*>(x), xq, sx, rs, M, L.K, st, h->pdl) != cudaSuccess) { cudaGetLastError(); return QL_ERR_CUDA; }
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_wide_ok ? &h->wmap_wide : nullptr;
-        if (gemm_pair_ta_i8_applicable(set, M, h->num_sms)) return gemm_pair_ta_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms);
+        if (gemm_pair_ta_i8_applicable(set, M)) {
+            // the K parts of few tiles meet behind the activations, where the scratch holds both
+            const size_t used = xq_bytes + 2 * arr, parts = (size_t)(h->num_sms / 2) * 2 * 256 * 128 * sizeof(float);
+            float* scratch = used + parts <= gemm_pair_scratch_bytes(h->num_sms) ? reinterpret_cast<float*>(base + used) : nullptr;
+            return gemm_pair_ta_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms, scratch, h->dev->gemm_counters);
+        }
         return gemm_pair_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms);
     }
     const GemvPlan pl = plan_gemv(L, h->n_rb, M, h->num_sms, false, true);
@@ -1853,8 +1873,9 @@ extern "C" int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_
     if (kernel == QL_KERNEL_NARROW) { width = pl.bn; parts = pl.cl; }
     if (kernel == QL_KERNEL_SINGLE) width = gemm_pick_bn(L, M, num_sms);
     if (kernel == QL_KERNEL_PAIR_TA) {
-        width = gemm_pair_ta_width(M);
-        if (!gated) parts = gemm_pair_ta_split(rows / 2 * ((M + 255) / 256), (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, true);
+        const TaPlan pl = gemm_pair_ta_plan((gated ? L.n_rsb : rows) / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, !gated);
+        width = pl.bn;
+        parts = pl.split;
     }
     const double other = takes_mid(hs, n, M, gated) ? mid_us(hs, n, M, gated) : prefill_us(prefill_kernel(hs, n, M, gated), hs, n, M, gated);
     const int32_t v[5] = {kernel, width, parts, (int32_t)(1000 * narrow_us(hs, n, M, gated)), (int32_t)(1000 * other)};
