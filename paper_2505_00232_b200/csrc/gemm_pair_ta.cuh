@@ -746,25 +746,49 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     }
 }
 
-// Token blocks: M in as few blocks of at most 256 as it takes, all of the same width (the MMA's N, a multiple of 32).  A
-// narrower tile costs the same dequantisation and less tensor-core time, x traffic and epilogue
-// (a Llama block at 100 tokens 145.9 -> 136.9 us, at 300 224.9 -> 211.1).
-// K parts per tile: 1 unless the tiles would leave half of the CTA pairs (or more) idle.
+// Estimate of a launch, us, as consecutive launches with the weights out of HBM take it, without the store of y (integer form: and the
+// quantisation before it): `layers` tiles (gated: 2) of n_ksteps steps in each of pairs * n_mblk positions of bn tokens, K in `split` parts.  A launch on
+// at most half of the CTA pairs leaves the others to the next one's start.  Fitted to 240 (integer form: 240) combinations of layer and
+// tokens (256 x 1024 to 14336 x 4096, 129 to 1400 tokens) with up to 15 plans each.
+inline double gemm_pair_ta_us(int pairs, int n_mblk, int bn, int split, int n_ksteps, int layers, bool i8, int num_sms)
+{
+    const int units = pairs * n_mblk * split, clusters = num_sms / 2, rounds = (units + clusters - 1) / clusters, steps = (n_ksteps + split - 1) / split;
+    const double more = units * 2 > clusters ? 1.0 : 0.0;
+    if (i8) return 5.94 + 0.00896 * bn + rounds * steps * (0.2494 + 0.00006 * bn) + (split == 4 ? 2.09 + 0.0273 * bn : split == 2 ? 1.58 + 0.0116 * bn : 0.0) + 0.8 * more + 1.83 * (rounds - 1);
+    if (layers == 2) return 5.48 + rounds * (0.0206 * bn - 1.35 + steps * (0.4395 + 0.00083 * bn));   // (the store included)
+    return 3.01 + 0.0003 * bn + rounds * steps * (0.1966 + 0.00038 * bn) + (split == 4 ? 2.77 + 0.023 * bn : split == 2 ? 2.13 + 0.013 * bn : 0.0) + 1.22 * more - 0.51 * (rounds - 1);
+}
+
+// Token blocks, all of one width (the MMA's N, a multiple of 32 up to 256), and K parts per tile: what the estimate says is fastest.  Few wide
+// tiles read the weights least often; narrow ones spread a small layer over the GPU, and unlike K parts, whose sums meet in the scratch, they
+// cost little else.  Of the 480 combinations above the plan taken is 0.6 % (integer form: 2.0 %) slower than the fastest of the
+// plans measured (worst 9 and 15 %), and against blocks of at most 256 tokens with K parts wherever half of the CTA pairs had no tile, us before / now:
+// 2048 x 2304 at 512 tokens 19.9 / 12.2, 2304 x 2048 at 777 18.8 / 12.7, 4096 x 4096 at 512 24.9 / 21.2, 2304 x 9216 at 300 25.1 / 20.7, 4096 x 14336
+// at 1400 144 / 133; integer form (which had no parts, and few tiles in shared memory) 1024 x 4096 at 1024 39.3 / 18.2, 2304 x 9216 at 777 66.0 / 31.4.
+// Calls that gemm_narrow.cuh takes by a wide margin (up to 128 tokens, two pairs of row super-blocks or 1024 k) keep the plan with the fewest
+// blocks here: gemm_route compares the two, and what is left of them has large K parts.
 struct TaPlan { int n_mblk, bn, split; };
-inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int num_sms, bool may_split)
+inline bool gemm_pair_ta_searches(int pairs, int M, int n_ksteps, bool i8) { return i8 || (M > 128 && pairs > 2 && n_ksteps > 16); }
+inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int layers, bool i8, int num_sms, bool may_split)
 {
     const int clusters = num_sms / 2;
-    TaPlan pl;
-    pl.n_mblk = (M + 255) / 256;
-    pl.bn = ((M + pl.n_mblk - 1) / pl.n_mblk + 31) / 32 * 32;
-    pl.split = 1;
-    const int tiles = pairs * pl.n_mblk;
-    if (!may_split || tiles >= clusters) return pl;
-    if (gemm_config().force_split > 0) pl.split = gemm_config().force_split >= 4 ? 4 : gemm_config().force_split >= 2 ? 2 : 1;
-    else if (tiles * 4 <= clusters) pl.split = 4;
-    else if (tiles * 2 <= clusters) pl.split = 2;
-    while (pl.split > 1 && (n_ksteps / pl.split < 8 || tiles * pl.split > clusters)) pl.split >>= 1;
-    return pl;
+    const int forced = gemm_config().force_split >= 4 ? 4 : gemm_config().force_split >= 2 ? 2 : gemm_config().force_split;
+    const bool search = gemm_pair_ta_searches(pairs, M, n_ksteps, i8);
+    TaPlan best{};
+    double best_us = 1e30;
+    for (int bn = 256; bn >= 32; bn -= 32) {
+        const int n_mblk = (M + bn - 1) / bn, tiles = pairs * n_mblk;
+        if (((M + n_mblk - 1) / n_mblk + 31) / 32 * 32 != bn) continue;  // (as many blocks, and narrower: comes later)
+        for (int split = 1; split <= 4; split *= 2) {
+            // one unit per CTA pair, which bounds the scratch
+            if (split > 1 && (!may_split || tiles * split > clusters || n_ksteps / split < (search ? 2 : 8))) break;
+            double us = search ? gemm_pair_ta_us(pairs, n_mblk, bn, split, n_ksteps, layers, i8, num_sms) : 1.0 / split;
+            if (forced && split != forced) us += 1e6 / split;            // (the parts asked for, or the most that the launch can have)
+            if (us < best_us) { best_us = us; best = TaPlan{n_mblk, bn, split}; }
+        }
+        if (!search) break;
+    }
+    return best;
 }
 
 // act < 0: the plain form.  act >= 0: the gated form, set = {gate, up} of equal shape, y[0] the output.
@@ -848,9 +872,12 @@ inline bool gemm_pair_ta_applicable(const GemmPairLayers& set, int M, int num_sm
     if (!gemm_config().ta || !gemm_config().pair) return false;
     for (int i = 0; i < set.n; ++i)
         if (!set.wmap[i] || (set.L[i]->n_rsb % 2)) return false;
-    // the gated form needs a whole number of positions per round of the grid's clusters to be worth it; the plain form
-    // takes every launch (few tiles: fewer clusters, or a K split through the device scratch)
-    return !gated || (M > 128 && (set.L[0]->n_rsb / 2) * ((M + 255) / 256) >= num_sms / 2);
+    // The plain form takes every launch.  The gated one where a position is left for every CTA pair in blocks of 256 tokens, and from 3073
+    // channels on with as many blocks as the plan finds (us, shared-memory form or gemm_narrow.cuh / this one: 9216 x 2304 at 300 tokens
+    // 47 / 28, at 512 47 / 33; 14336 x 4096 at 200 72 / 45; 6144 x 1792 at 512 37 / 24).  (Time alone would draw that line lower, 3072 x 4096 at 1500
+    // tokens 68 / 54: there the shared-memory form keeps calls that reach it by rule, in the tests and in smoke().)
+    const int pairs = set.L[0]->n_rsb / 2;
+    return !gated || (M > 128 && (pairs > 12 || pairs * ((M + 255) / 256) >= num_sms / 2));
 }
 
 inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, int M, cudaStream_t st, int device, bool pdl, int num_sms,
@@ -863,7 +890,7 @@ inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, 
         const unsigned char* y = static_cast<const unsigned char*>(set.y[i]);
         if (y >= s0 && y < s0 + gemm_pair_scratch_bytes(num_sms)) scratch = nullptr;
     }
-    const TaPlan pl = gemm_pair_ta_plan(set.n_rsb() / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, scratch && counters);
+    const TaPlan pl = gemm_pair_ta_plan(set.n_rsb() / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, 1, false, num_sms, scratch && counters);
     if (pl.split > 1) {
         if (L.bits == 8) return gemm_pair_ta_launch<8, false, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, -1, scratch, counters);
         if (L.grouped) return gemm_pair_ta_launch<4, true, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, -1, scratch, counters);
@@ -878,7 +905,7 @@ inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, 
 inline ql_status gemm_pair_ta_forward_gated(const GemmPairLayers& set, const void* x, int M, int act, cudaStream_t st, int device, bool pdl, int num_sms)
 {
     const Layout& L = *set.L[0];
-    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, false);
+    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, 2, false, num_sms, false);
     if (L.bits == 8) return gemm_pair_ta_launch<8, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
     if (L.grouped) return gemm_pair_ta_launch<4, true, true>(set, pl, x, M, st, device, pdl, num_sms, act);
     return gemm_pair_ta_launch<4, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
@@ -894,7 +921,7 @@ inline ql_status gemm_pair_ta_forward_i8(const GemmPairLayers& set, const void* 
                                          cudaStream_t st, int device, bool pdl, int num_sms, float* scratch, unsigned int* counters)
 {
     const Layout& L = *set.L[0];
-    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + 127) / 128, num_sms, scratch && counters);
+    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + 127) / 128, 1, true, num_sms, scratch && counters);
     if (pl.split > 1)
         return L.bits == 8 ? gemm_pair_ta_launch<8, false, false, true, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, scratch, counters, scale, rowsum)
                            : gemm_pair_ta_launch<4, false, false, true, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, scratch, counters, scale, rowsum);

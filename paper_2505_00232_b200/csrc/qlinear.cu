@@ -806,7 +806,8 @@ bool gate_fits_scratch(int N, int M, int num_sms) { return (size_t)M * N * 2 * s
 // that served its calls before.  Fitted to 9217 calls of random shapes (8 to 32768 channels, K 32 to 16384, at most 80 million weights, 9 to 2048
 // tokens, plain and gated, the three schemes), each on both routes; long calls and the shapes of the two models weigh more.  Measured /
 // estimate, 5th and 95th percentile (1st and 99th): narrow_us 0.90 and 1.11 (0.84, 1.17), mid_us 0.90 and 1.11 (0.85, 1.16), prefill_us on the
-// CTA-pair kernel 0.83 and 1.19 (0.81, 1.70: gated pairs of K up to 128, far from the line), on the single-CTA kernel 0.86 and 1.07 (0.79, 1.17), on
+// CTA-pair kernel's plans of the fewest blocks 0.83 and 1.19 (0.81, 1.70: gated pairs of K up to 128, far from the line; those it searches, of 700 later
+// calls: 0.88 and 1.12), on the single-CTA kernel 0.86 and 1.07 (0.79, 1.17), on
 // the shared-memory gated form 0.89 and 1.14 (0.88, 1.19), unfused 0.86 and 1.05 (0.81, 1.13).
 // What a CTA's time is multiplied by for the others of the launch, `ctas` in all in clusters of cl, two to an SM: up to one per SM they slow it
 // down by `first`, the second ones by `second` more; beyond two per SM further rounds, of which the last one costs `last` at least.
@@ -844,7 +845,8 @@ double mid_us(const qlinear_s* const* hs, int n, int M, bool gated)      // up t
 double pair_ta_us(const Layout& L, int pairs, int M, int layers, bool split, double mb, int num_sms)
 {
     const int steps = (L.K + kGemmKStep - 1) / kGemmKStep;
-    const TaPlan pl = gemm_pair_ta_plan(pairs, M, steps, num_sms, split);
+    const TaPlan pl = gemm_pair_ta_plan(pairs, M, steps, layers, false, num_sms, split);
+    if (gemm_pair_ta_searches(pairs, M, steps, false)) return gemm_pair_ta_us(pairs, pl.n_mblk, pl.bn, pl.split, steps, layers, false, num_sms) + (layers == 2 ? 0.0 : 0.286 * mb);
     const double rounds = round_up((double)pairs * pl.n_mblk * pl.split / (num_sms / 2));
     return 2.66 + 0.0058 * pl.bn + rounds * (layers * ((steps + pl.split - 1) / pl.split) * (0.236 + 0.0003 * pl.bn)) + (pl.split > 1 ? 6.2 + 0.0162 * pl.bn : 0.0) + 0.34 * mb;
 }
@@ -901,10 +903,10 @@ bool narrow_can(const qlinear_s* const* hs, int n, int M, bool gated, bool batch
 }
 
 // The kernel of a call beyond the decode stage: one layer, n > 1 layers that share x, or (gated) a pair.  gemm_narrow.cuh where its
-// estimate is below that of gemm_mid.cuh, 7 % below that of the CTA-pair kernel, or below those of the three other forms (single CTA,
-// shared-memory gating, unfused gating).  No line is always right with these errors.  Of the calls above and 3110 others, 80 run more than 3 %
-// slower this way than on the other route: 54 of 4821 against gemm_mid.cuh (two of them by 46 and 26 %, the others by 24 % at most), 17 of 2018
-// against the CTA-pair kernel (19 %), 9 of 5488 against the other forms (9 %); all together take 0.8 % more than on the faster route each.  Measured, us, the route otherwise / gemm_narrow.cuh:
+// estimate is below that of gemm_mid.cuh, the CTA-pair kernel or the three other forms (single CTA, shared-memory gating, unfused gating).  No line is always right with these errors.  Of the calls above and 3110 others, 80 run more than 3 %
+// slower this way than on the other route: 54 of 4821 against gemm_mid.cuh (two of them by 46 and 26 %, the others by 24 % at most), 9
+// of 5488 against the other forms (9 %).  Against the CTA-pair kernel with its plans searched, 700 calls take 0.3 % more than on the faster route each,
+// the worst 21 %.  Measured, us, the route otherwise / gemm_narrow.cuh:
 //   weights                        16 tokens     24           32           48           64
 //     0.3 M (512 x 512)             2.8 /  3.7   3.0 /  3.8   3.3 /  4.0   3.8 /  4.2   4.1 /  4.5
 //     1 M (1024 x 1024, int8)       3.2 /  4.3   3.5 /  4.5   4.0 /  4.6   4.6 /  5.0   5.2 /  5.3
@@ -923,7 +925,7 @@ ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
     const ql_kernel other = batch ? QL_KERNEL_MID : prefill_kernel(hs, n, M, gated);
     if (!narrow_can(hs, n, M, gated, batch)) return other;
     if (config().narrow == 2) return QL_KERNEL_NARROW;
-    const double limit = batch ? mid_us(hs, n, M, gated) : (other == QL_KERNEL_PAIR_TA ? 0.93 : 1.0) * prefill_us(other, hs, n, M, gated);
+    const double limit = batch ? mid_us(hs, n, M, gated) : prefill_us(other, hs, n, M, gated);
     return narrow_us(hs, n, M, gated) < limit ? QL_KERNEL_NARROW : other;
 }
 
@@ -1873,7 +1875,7 @@ extern "C" int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_
     if (kernel == QL_KERNEL_NARROW) { width = pl.bn; parts = pl.cl; }
     if (kernel == QL_KERNEL_SINGLE) width = gemm_pick_bn(L, M, num_sms);
     if (kernel == QL_KERNEL_PAIR_TA) {
-        const TaPlan pl = gemm_pair_ta_plan((gated ? L.n_rsb : rows) / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, num_sms, !gated);
+        const TaPlan pl = gemm_pair_ta_plan((gated ? L.n_rsb : rows) / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, gated ? 2 : 1, false, num_sms, !gated);
         width = pl.bn;
         parts = pl.split;
     }

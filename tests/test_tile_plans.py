@@ -1,0 +1,87 @@
+"""Plans of the CTA-pair prefill kernel that divide a launch more finely than blocks of 256 tokens: narrower blocks, K parts, and gated pairs
+with fewer positions of 256 tokens than CTA pairs.  Which plan a call gets is checked without a device."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from oracle import qlinear_oracle as O
+from workloads import configs as C
+
+SMS = 148
+PAIR_TA = 6
+# (tokens, channels, K, bits, group, width, parts): remainders in tokens, channels, k; the last block nearly empty
+PLAIN = [(300, 2304, 9216, 4, 32, 160, 4), (257, 2800, 8224, 8, 0, 96, 2), (641, 4096, 2176, 4, 0, 192, 1), (1409, 2560, 1152, 4, 128, 224, 1), (1030, 4864, 1152, 8, 0, 160, 1)]
+GATED = [(330, 6144, 1120, 8, 0, 128), (130, 9216, 1120, 8, 0, 96), (259, 13312, 1088, 4, 0, 160)]
+# integer form (its plan is not asked for): one pair of row super-blocks to many, one k-step to many, parts and narrow blocks
+A8 = [(129, 256, 128, 4), (130, 200, 8192, 8), (200, 1024, 4096, 4), (333, 2296, 9216, 8), (700, 1024, 2304, 4), (1030, 4096, 1152, 8), (641, 9216, 256, 4)]
+
+
+@pytest.fixture(scope="module")
+def P(_built_library):
+    import paper_2505_00232_b200 as P
+    return P
+
+
+def spec(N, K, bits, group):
+    return C.LayerSpec("t", N, K, bits, group, *((-8, 7) if bits == 4 else (-128, 127)))
+
+
+def route(P, Ns, K, bits, group, M, gated):
+    ds = (type(P.Desc(8, 32, 8, 0).c()) * len(Ns))(*[P.Desc(N, K, bits, group).c() for N in Ns])
+    out = (ctypes.c_int32 * 5)()
+    assert P.lib.qlinear_debug_route(ds, len(Ns), M, gated, SMS, out, 5) >= 3
+    return list(out)
+
+
+def test_the_calls_below_get_these_plans(P):
+    assert [route(P, [N], K, b, g, M, 0)[:3] for M, N, K, b, g, _, _ in PLAIN] == [[PAIR_TA, w, p] for *_, w, p in PLAIN]
+    assert [route(P, [N, N], K, b, g, M, 1)[:3] for M, N, K, b, g, _ in GATED] == [[PAIR_TA, w, 1] for *_, w in GATED]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,bits,group", [c[:5] for c in PLAIN])
+def test_plain(P, M, N, K, bits, group):
+    import torch
+    q, s = C.layer_weights(8100 + M, spec(N, K, bits, group))
+    x = C.layer_activations(8100 + M, spec(N, K, bits, group), M)
+    lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
+    xd = torch.from_numpy(x).cuda()
+    guard = torch.full((M + 2, N), -7.0, dtype=torch.float16, device="cuda")
+    y = lin.forward(xd, out=guard[1:-1])
+    assert torch.equal(y, lin.forward(xd)) and (guard[0] == -7.0).all() and (guard[-1] == -7.0).all()
+    assert lin.device_status() == (0, 0)
+    y64, A, _ = O.linear(x, q, s, group)
+    d = np.abs(y.cpu().numpy().astype(np.float64) - y64)
+    assert (d <= O.ELEM_TOL * A).all() and np.linalg.norm(d) <= O.REL_L2_TOL * np.linalg.norm(y64)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,bits,group", [c[:5] for c in GATED])
+def test_gated(P, M, N, K, bits, group):
+    import torch
+    from tests.test_gated_gpu import assert_gated
+    gw, uw = (C.layer_weights(8200 + M + i, spec(N, K, bits, group)) for i in range(2))
+    x = C.layer_activations(8200 + M, spec(N, K, bits, group), M)
+    lg, lu = (P.QLinear.from_weights(q, s, bits, group, device="cuda:0") for q, s in (gw, uw))
+    xd = torch.from_numpy(x).cuda()
+    y = P.qlinear_forward_gated(lg, lu, xd, "silu")
+    assert torch.equal(y, P.qlinear_forward_gated(lg, lu, xd, "silu")) and lg.device_status() == (0, 0)
+    rows = np.r_[0:300, N - 300:N]
+    assert_gated(y.cpu().numpy()[:, rows], x, (gw[0][rows], gw[1][rows]), (uw[0][rows], uw[1][rows]), group, "silu")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,bits", A8)
+def test_integer_form(P, M, N, K, bits):
+    import torch
+    from tests.test_a8_gpu import assert_a8
+    q, s = C.layer_weights(8300 + M, spec(N, K, bits, 0))
+    x = C.layer_activations(8300 + M, spec(N, K, bits, 0), M)
+    lin = P.QLinear.from_weights(q, s, bits, 0, device="cuda:0")
+    xd = torch.from_numpy(x).cuda()
+    y = lin.forward_a8(xd)
+    again = [lin.forward_a8(xd) for _ in range(10)]
+    assert all(torch.equal(y, a) for a in again) and lin.device_status() == (0, 0)
+    rows = np.r_[0:128, N - 128:N] if N > 2304 else np.r_[0:N]
+    assert_a8(y.cpu().numpy()[:, rows], x, q[rows], s[rows], 0)
