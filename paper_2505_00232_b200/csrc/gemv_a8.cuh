@@ -17,7 +17,9 @@
 // and by one warp reduction, every thread forms the reciprocals itself, and short rows are quantised from the registers they
 // were measured in.  Measured (weights out of HBM, before / after): 4096 x 4096 int8 at 1 token 8.0 / 7.1 us, at 4 tokens
 // 11.9 / 8.4; 14336 x 4096 int4 per channel 10.7 / 9.4 and 17.6 / 12.4; 4096 x 14336 int4 12.0 / 10.3 and 24.0 / 23.5 (two
-// reads of rows that long).
+// reads of rows that long).  Since then the chunks go in pairs and a warp adds the offset terms of its groups across its lanes (one after the
+// other they were a chain of shared-memory loads at the end): 7.1 / 6.5, 9.3 / 8.2 and 10.3 / 9.4 at 1 token.  Tried and not better: the
+// maxima of a cluster's K ranges through distributed shared memory, rounding by an addition instead of a conversion.
 // int4 unpack is two logic operations per 8 weights (the low and the high nibbles of a word are the 4-byte
 // operand registers of rows g and g + 8), against nine for the fp16 path.
 #pragma once
@@ -118,12 +120,25 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_a8_kernel(const GemvA8Pa
     // Weights do not depend on the previous kernel: fill the ring before waiting for it.
     if (GROUPED) copy16(sbuf_u32, wsrc + s_off, kc0 + (lane >> 2) < kc1);
 #pragma unroll
-    for (int d = 0; d < kGemvRing; ++d) {
+    for (int d = 0; d < kGemvRing; ++d) {                                // one commit group per pair of chunks
         copy16(ring_u32 + d * 512, wsrc, kc0 + d < kc1);
-        commit();
+        if (d & 1) commit();
         wsrc += p.block_bytes;
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // One token: the per-channel scales of the (at most 4) outputs that this thread will store, which are weights too, are requested now, so that
+    // their latency does not sit at the very end (4096 x 4096 int8 7.0 -> 6.5 us; with more tokens their registers are worth more, 8 tokens 12.0 -> 12.4).
+    constexpr bool EARLY_SCALES = T == 1 && !GROUPED;
+    const int t = threadIdx.x;
+    [[maybe_unused]] unsigned short pre_scale[4];
+    if (EARLY_SCALES) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int idx = t + k * kGemvThreads;
+            const int row = (rb_group * rb_per_cta + (idx >> 7)) * kRbRows + ((idx & 127) >> 4) + 8 * ((idx >> 1) & 1);
+            pre_scale[k] = idx < (p.cl > 1 ? 128 : rb_per_cta * 128) && row < p.N ? __half_as_ushort(p.chan_scales[row]) : 0;
+        }
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // ---- step 1a: amax of every token over its WHOLE row (every CTA needs it, whatever its K range)
@@ -241,69 +256,81 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_a8_kernel(const GemvA8Pa
     const signed char* xrow = xq + min(g, p.M - 1) * p.xq_stride + 8 * c;   // columns g >= M copy the last token, never stored
     [[maybe_unused]] const uint32_t sc_u32 = sbuf_u32 - lane * 16 + g * 8;   // (read by the grouped form only)
     int sflip = 0;
+    auto chunk_math = [&](const uint4& w, const uint2& sc, int kl) {     // kl: first k of the chunk inside the CTA's range
+        if (BITS == 4) {
+            const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {                                // the chunk's two 32-k groups
+                uint32_t a[4];
+                a[0] = ww[2 * h] & 0x0F0F0F0Fu;                          // row g:     k 8c + {0, 2, 1, 3}
+                a[1] = (ww[2 * h] >> 4) & 0x0F0F0F0Fu;                   // row g + 8
+                a[2] = ww[2 * h + 1] & 0x0F0F0F0Fu;                      // row g:     k 8c + 4 + {0, 2, 1, 3}
+                a[3] = (ww[2 * h + 1] >> 4) & 0x0F0F0F0Fu;
+                const uint2 xb = *reinterpret_cast<const uint2*>(xrow + kl + 32 * h);
+                if (GROUPED) {
+                    const int2 off = *reinterpret_cast<const int2*>(sg + ((kl >> 5) + h) * 8 + 2 * c);
+                    const int cin[4] = {off.x, off.y, off.x, off.y};
+                    int acc[4];
+                    imma_16832(acc, a, xb.x, xb.y, cin);
+                    const __half2 s_lo = *reinterpret_cast<const __half2*>(&sc.x);      // row g:   G0, G1
+                    const __half2 s_hi = *reinterpret_cast<const __half2*>(&sc.y);      // row g+8: G0, G1
+                    const float s0 = h == 0 ? __low2float(s_lo) : __high2float(s_lo);
+                    const float s8 = h == 0 ? __low2float(s_hi) : __high2float(s_hi);
+                    ftotal[0] = fmaf(s0, (float)acc[0], ftotal[0]);
+                    ftotal[1] = fmaf(s0, (float)acc[1], ftotal[1]);
+                    ftotal[2] = fmaf(s8, (float)acc[2], ftotal[2]);
+                    ftotal[3] = fmaf(s8, (float)acc[3], ftotal[3]);
+                } else {
+                    imma_16832(itotal, a, xb.x, xb.y, itotal);
+                }
+            }
+        } else {
+            uint32_t a[4];
+            a[0] = __byte_perm(w.x, w.y, 0x5410);                        // row g:     k 8c + 0..3
+            a[1] = __byte_perm(w.x, w.y, 0x7632);                        // row g + 8
+            a[2] = __byte_perm(w.z, w.w, 0x5410);                        // row g:     k 8c + 4..7
+            a[3] = __byte_perm(w.z, w.w, 0x7632);
+            const uint2 xb = *reinterpret_cast<const uint2*>(xrow + kl);
+            imma_16832(itotal, a, xb.x, xb.y, itotal);
+        }
+    };
     for (int kc = kc0; kc < kc1; kc += kGemvRing) {
 #pragma unroll
-        for (int d = 0; d < kGemvRing; ++d) {
+        for (int d = 0; d < kGemvRing; d += 2) {                         // two chunks read and their slots refilled before the math
             if (kc + d >= kc1) break;
-            asm volatile("cp.async.wait_group %0;" ::"n"(kGemvRing - 1) : "memory");
+            asm volatile("cp.async.wait_group %0;" ::"n"(kGemvRing / 2 - 1) : "memory");
             if (GROUPED && d == 0) {
                 __syncwarp();                                            // scales of this pass visible; last pass's reads done
                 copy16(sbuf_u32 + (sflip ^ 1) * 512, wsrc + s_off, kc + kGemvRing + (lane >> 2) < kc1);
             }
-            const uint4 w = *reinterpret_cast<const uint4*>(ring + d * 512 + lane * 16);
-            uint2 sc = make_uint2(0, 0);
-            if (GROUPED) sc = *reinterpret_cast<const uint2*>(sbuf + sflip * 512 + d * 64 + g * 8);
-            copy16(ring_u32 + d * 512, wsrc, kc + d + kGemvRing < kc1);
-            commit();
-            wsrc += p.block_bytes;
-            const int kl = (kc + d - kc_cta0) * CHUNK_K;                 // first k of the chunk inside the CTA's range
-            if (BITS == 4) {
-                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {                            // the chunk's two 32-k groups
-                    uint32_t a[4];
-                    a[0] = ww[2 * h] & 0x0F0F0F0Fu;                      // row g:     k 8c + {0, 2, 1, 3}
-                    a[1] = (ww[2 * h] >> 4) & 0x0F0F0F0Fu;               // row g + 8
-                    a[2] = ww[2 * h + 1] & 0x0F0F0F0Fu;                  // row g:     k 8c + 4 + {0, 2, 1, 3}
-                    a[3] = (ww[2 * h + 1] >> 4) & 0x0F0F0F0Fu;
-                    const uint2 xb = *reinterpret_cast<const uint2*>(xrow + kl + 32 * h);
-                    if (GROUPED) {
-                        const int2 off = *reinterpret_cast<const int2*>(sg + ((kl >> 5) + h) * 8 + 2 * c);
-                        const int cin[4] = {off.x, off.y, off.x, off.y};
-                        int acc[4];
-                        imma_16832(acc, a, xb.x, xb.y, cin);
-                        const __half2 s_lo = *reinterpret_cast<const __half2*>(&sc.x);      // row g:   G0, G1
-                        const __half2 s_hi = *reinterpret_cast<const __half2*>(&sc.y);      // row g+8: G0, G1
-                        const float s0 = h == 0 ? __low2float(s_lo) : __high2float(s_lo);
-                        const float s8 = h == 0 ? __low2float(s_hi) : __high2float(s_hi);
-                        ftotal[0] = fmaf(s0, (float)acc[0], ftotal[0]);
-                        ftotal[1] = fmaf(s0, (float)acc[1], ftotal[1]);
-                        ftotal[2] = fmaf(s8, (float)acc[2], ftotal[2]);
-                        ftotal[3] = fmaf(s8, (float)acc[3], ftotal[3]);
-                    } else {
-                        imma_16832(itotal, a, xb.x, xb.y, itotal);
-                    }
-                }
-            } else {
-                uint32_t a[4];
-                a[0] = __byte_perm(w.x, w.y, 0x5410);                    // row g:     k 8c + 0..3
-                a[1] = __byte_perm(w.x, w.y, 0x7632);                    // row g + 8
-                a[2] = __byte_perm(w.z, w.w, 0x5410);                    // row g:     k 8c + 4..7
-                a[3] = __byte_perm(w.z, w.w, 0x7632);
-                const uint2 xb = *reinterpret_cast<const uint2*>(xrow + kl);
-                imma_16832(itotal, a, xb.x, xb.y, itotal);
+            const uint4 w0 = *reinterpret_cast<const uint4*>(ring + d * 512 + lane * 16);
+            const uint4 w1 = *reinterpret_cast<const uint4*>(ring + (d + 1) * 512 + lane * 16);
+            uint2 sc0 = make_uint2(0, 0), sc1 = make_uint2(0, 0);
+            if (GROUPED) {
+                sc0 = *reinterpret_cast<const uint2*>(sbuf + sflip * 512 + d * 64 + g * 8);
+                sc1 = *reinterpret_cast<const uint2*>(sbuf + sflip * 512 + (d + 1) * 64 + g * 8);
             }
+            copy16(ring_u32 + d * 512, wsrc, kc + d + kGemvRing < kc1);
+            copy16(ring_u32 + (d + 1) * 512, wsrc + p.block_bytes, kc + d + 1 + kGemvRing < kc1);
+            commit();
+            wsrc += 2 * (int64_t)p.block_bytes;
+            const int kl = (kc + d - kc_cta0) * CHUNK_K;
+            chunk_math(w0, sc0, kl);
+            if (kc + d + 1 < kc1) chunk_math(w1, sc1, kl + CHUNK_K);
         }
         sflip ^= 1;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (!GROUPED) {                                                      // the offset term of this warp's K slice, per token column
-        int o0 = 0, o1 = 0;
+        // (lane (g, c) takes every eighth group of its two columns)
         const int g0 = ((kc0 - kc_cta0) * CHUNK_K) >> 5, g1 = ((kc1 - kc_cta0) * CHUNK_K) >> 5;
-        for (int gi = g0; gi < g1; ++gi) {
+        int o0 = 0, o1 = 0;
+        for (int gi = g0 + g; gi < g1; gi += 8) {
             const int2 off = *reinterpret_cast<const int2*>(sg + gi * 8 + 2 * c);
             o0 += off.x; o1 += off.y;
         }
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) { o0 += __shfl_xor_sync(0xffffffffu, o0, o); o1 += __shfl_xor_sync(0xffffffffu, o1, o); }
         itotal[0] += o0; itotal[1] += o1; itotal[2] += o0; itotal[3] += o1;
     }
 
@@ -313,13 +340,13 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_a8_kernel(const GemvA8Pa
     __syncthreads();
 
     // element e of a row-block's 128 results: lane e / 4, register e % 4
-    auto store_out = [&](int rbl, int e, float fsum, int isum) {
+    auto store_out = [&](int rbl, int e, float fsum, int isum, float early) {
         const int out_rb = rb_group * rb_per_cta + rbl;
         const int el = e >> 2, i = e & 3;
         const int row = out_rb * kRbRows + (el >> 2) + 8 * (i >> 1);
         const int tok = 2 * (el & 3) + (i & 1);
         if (row < p.N && tok < p.M) {
-            const float v = GROUPED ? fsum : __half2float(p.chan_scales[row]) * (float)isum;
+            const float v = GROUPED ? fsum : (EARLY_SCALES ? early : __half2float(p.chan_scales[row])) * (float)isum;
             p.y[(int64_t)tok * p.N + row] = __float2half_rn(scale_x[tok] * v);
         }
     };
@@ -327,7 +354,6 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_a8_kernel(const GemvA8Pa
         if (GROUPED) f += __int_as_float(bits); else i += bits;
     };
 
-    const int t = threadIdx.x;
     if (p.cl > 1) {                                                      // ks_cta == 8: one row-block per CTA
         cg::cluster_group cluster = cg::this_cluster();
         if (t < 128) {
@@ -339,16 +365,24 @@ __global__ void __launch_bounds__(kGemvThreads, 4) gemv_a8_kernel(const GemvA8Pa
         if (crank == 0 && t < 128) {
             float f = 0.f; int i = 0;
             for (int r = 0; r < p.cl; ++r) add(f, i, *cluster.map_shared_rank(&part[t], r));
-            store_out(0, t, f, i);
+            store_out(0, t, f, i, EARLY_SCALES ? __half2float(__ushort_as_half(pre_scale[0])) : 0.f);
         }
         // peers keep `part` alive until it has been read: a rendezvous only (relaxed arrive, plain wait)
         asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
     } else {
-        for (int idx = t; idx < rb_per_cta * 128; idx += kGemvThreads) {
+        // (rb_per_cta <= 8: at most 4 elements per thread)
+        auto finish = [&](int idx, unsigned short early) {
             const int rbl = idx >> 7, e = idx & 127;
             float f = 0.f; int i = 0;
             for (int s = 0; s < p.ks_cta; ++s) add(f, i, red[rbl * p.ks_cta + s][e]);
-            store_out(rbl, e, f, i);
+            store_out(rbl, e, f, i, EARLY_SCALES ? __half2float(__ushort_as_half(early)) : 0.f);
+        };
+        if constexpr (EARLY_SCALES) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (t + k * kGemvThreads < rb_per_cta * 128) finish(t + k * kGemvThreads, pre_scale[k]);
+        } else {
+            for (int idx = t; idx < rb_per_cta * 128; idx += kGemvThreads) finish(idx, 0);
         }
     }
 }
