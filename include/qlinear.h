@@ -233,6 +233,8 @@ ql_status qlinear_kv_append(qlinear_t h_k, qlinear_t h_v, const void* k_new_dev,
 ql_status qlinear_kv_scores(qlinear_t h_k, const void* q_rows_dev, void* scores_dev, int32_t R, void* cuda_stream);
 ql_status qlinear_kv_output(qlinear_t h_v, const void* prob_dev, const void* v_scale_dev, void* tmp_dev, void* out_dev,
                             int32_t R, void* cuda_stream);
+/* Whether that call would write to tmp_dev (1) or not (0: any aligned pointer will do, for instance out_dev). */
+int32_t qlinear_kv_output_uses_tmp(qlinear_t h_v, const void* prob_dev, const void* v_scale_dev, int32_t R);
 
 /* The same three steps for ALL KV heads of an attention layer at once (n_heads <= 16 cache pairs of equal shape, arrays
  * of handles h_k[i], h_v[i] and of their scale arrays v_scale_dev[i], all host arrays of device pointers): one launch per

@@ -1,4 +1,4 @@
-"""Thin ctypes binding over libqlinear.so (see include/qlinear.h): argument marshalling only.
+"""Thin binding over libqlinear.so (see include/qlinear.h): argument marshalling only, by ctypes and, for the calls on tensors, csrc/native.cpp.
 
 Every arithmetic step runs inside the library's CUDA kernels (or, for pack/unpack, its host
 packer).  torch is used for device memory and streams.  There is no CPU fallback: if the shared
@@ -22,7 +22,7 @@ QL_ACT_IDENTITY, QL_ACT_SILU, QL_ACT_GELU_TANH = 0, 1, 2
 ACTIVATIONS = {"identity": QL_ACT_IDENTITY, "silu": QL_ACT_SILU, "gelu_tanh": QL_ACT_GELU_TANH}
 
 EXPORTS = (
-    "qlinear_packed_size", "qlinear_pack", "qlinear_unpack", "qlinear_create", "qlinear_forward", "qlinear_forward_group", "qlinear_forward_batch", "qlinear_forward_gated", "qlinear_forward_a8", "qlinear_quantize_activations", "qlinear_kv_append", "qlinear_kv_scores", "qlinear_kv_output", "qlinear_kv_append_heads", "qlinear_kv_scores_heads", "qlinear_kv_output_heads", "qlinear_embed", "qlinear_residual_rmsnorm", "qlinear_rope_qkv",
+    "qlinear_packed_size", "qlinear_pack", "qlinear_unpack", "qlinear_create", "qlinear_forward", "qlinear_forward_group", "qlinear_forward_batch", "qlinear_forward_gated", "qlinear_forward_a8", "qlinear_quantize_activations", "qlinear_kv_append", "qlinear_kv_scores", "qlinear_kv_output", "qlinear_kv_output_uses_tmp", "qlinear_kv_append_heads", "qlinear_kv_scores_heads", "qlinear_kv_output_heads", "qlinear_embed", "qlinear_residual_rmsnorm", "qlinear_rope_qkv",
     "qlinear_path_for", "qlinear_debug_unpack_device", "qlinear_debug_expire_wait", "qlinear_debug_null_launch", "qlinear_device_status", "qlinear_decode_static", "qlinear_destroy",
     "qlinear_status_string", "qlinear_version", "qlinear_debug_plan", "qlinear_debug_plan_kv_output", "qlinear_debug_takes_batch_kernel", "qlinear_debug_kv_hold", "qlinear_debug_route", "qlinear_debug_config_reads",
 )
@@ -76,6 +76,8 @@ def _load() -> ctypes.CDLL:
     lib.qlinear_kv_scores.restype = ctypes.c_int
     lib.qlinear_kv_output.argtypes = [vp, vp, vp, vp, vp, i32, vp]
     lib.qlinear_kv_output.restype = ctypes.c_int
+    lib.qlinear_kv_output_uses_tmp.argtypes = [vp, vp, vp, i32]
+    lib.qlinear_kv_output_uses_tmp.restype = i32
     lib.qlinear_embed.argtypes = [vp, vp, ctypes.c_int32, vp, vp]
     lib.qlinear_embed.restype = ctypes.c_int
     lib.qlinear_residual_rmsnorm.argtypes = [vp, vp, vp, ctypes.c_float, ctypes.c_float, vp, vp, i32, i32, ctypes.c_int, vp]
@@ -177,20 +179,33 @@ def qlinear_unpack(desc: Desc, packed: np.ndarray):
 
 
 # ---------------------------------------------------------------------------- device calls
-# A small layer takes the GPU a few microseconds, less than these calls took the host: so the raw handle of the current
-# stream is asked for without building a Stream object, pointers go to ctypes as plain integers (the argument types are
-# declared), and a tensor's properties are checked in one expression.  Measured: QLinear.forward at one token 11.6 -> 6.7 us.
-_half = _raw_stream = _device = None
+# A small layer takes the GPU a few microseconds, less than these calls took the host.  So every call on tensors first goes to the module built
+# from csrc/native.cpp, which checks the arguments, allocates the outputs and calls the library; it returns None for everything
+# that is not the common form of the call (subclasses, tracing, wrong shapes, ...), and the Python below it then does the call, or raises.
+# Measured, us per call of the host: QLinear.forward at one token 6.7 -> 3.9, qlinear_forward_group of three layers 14.0 -> 6.1,
+# qlinear_residual_rmsnorm 11.1 -> 4.7, qlinear_rope_qkv 15.5 -> 5.2, KVCache.output 11.0 -> 5.4.
+_half = _raw_stream = _device = _native = None
+_NATIVE_API = ("qlinear_forward", "qlinear_forward_a8", "qlinear_forward_group", "qlinear_forward_gated", "qlinear_residual_rmsnorm", "qlinear_rope_qkv", "qlinear_embed",
+               "qlinear_kv_append_heads", "qlinear_kv_scores_heads", "qlinear_kv_output_heads", "qlinear_kv_output", "qlinear_kv_output_uses_tmp")
 
 
-def _bind_torch() -> None:
-    """torch is imported with the first device object, not with the package (packing needs none of it)."""
-    global _half, _raw_stream, _device
+def _bind_torch():
+    """torch is imported with the first device object, not with the package (packing needs none of it).  Returns the native module."""
+    global _half, _raw_stream, _device, _native
     import torch
+    if _native is None:
+        from . import _native as native                                  # (no fallback: the build makes it beside libqlinear.so)
+        native.init(_check, *(ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in _NATIVE_API))
+        _native = native
     # (a torch without CUDA has neither entry point: its own error comes from the calls that need a device)
     _device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
     _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", lambda device: torch.cuda.current_stream(device).cuda_stream)
     _half = torch.float16
+    return _native
+
+
+def _raw(stream):
+    return None if stream is None else stream.cuda_stream
 
 
 def _stream_ptr(stream) -> int:
@@ -275,6 +290,10 @@ def kv_scores_batch(caches, q_rows, stream=None):
 
 def qlinear_forward_group(lins, x, outs=None, stream=None):
     """x: fp16 CUDA tensor [M, K] -> list of fp16 [M, N_i], one per layer (one launch for M <= 8)."""
+    if outs is None:
+        y = (_native or _bind_torch()).forward_group(lins, x, _raw(stream))
+        if y is not None:
+            return y
     K = lins[0].desc.K
     if not _is_x(x, K):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_group (x must be contiguous fp16 CUDA [M, K])")
@@ -295,6 +314,10 @@ def qlinear_forward_gated_raw(gate, up, x_ptr: int, y_ptr: int, M: int, act: str
 
 def qlinear_forward_gated(gate, up, x, act: str = "silu", out=None, stream=None):
     """y = act(x . W_gate^T) * (x . W_up^T) as fp16 [M, N], from one fused launch where the shape allows."""
+    if act in ACTIVATIONS:
+        y = (_native or _bind_torch()).forward_gated(gate._native, up._native, x, ACTIVATIONS[act], out, _raw(stream))
+        if y is not None:
+            return y
     K, N = gate.desc.K, gate.desc.N
     if not _is_x(x, K):
         raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_gated (x must be contiguous fp16 CUDA [M, K])")
@@ -325,8 +348,9 @@ def qlinear_quantize_activations(x, stream=None):
 def qlinear_residual_rmsnorm(x, residual, gamma, eps: float, gamma_offset: float = 0.0, h_out=None, y_out=None, want_h=True, stream=None):
     """x, residual (or None) fp16 CUDA [M, K], gamma fp16 [K] -> (h, y): h = x + residual, y = rmsnorm(h) * (gamma_offset + gamma).
     h_out / y_out may be given (h_out may be x or residual: in place); want_h=False skips the h output (h is then None)."""
-    if _half is None:
-        _bind_torch()
+    hy = (_native or _bind_torch()).residual_rmsnorm(x, residual, gamma, eps, gamma_offset, h_out, y_out, want_h, _raw(stream))
+    if hy is not None:
+        return hy
     dev = x.get_device()
     def ok(t, shape):
         return t.dtype == _half and t.get_device() == dev and t.is_cuda and t.is_contiguous() and tuple(t.shape) == shape
@@ -351,6 +375,9 @@ def qlinear_residual_rmsnorm(x, residual, gamma, eps: float, gamma_offset: float
 def qlinear_rope_qkv(q, k, v, pos, cos, sin, B: int, S: int, h_q: int, h_kv: int, d_h: int, stream=None):
     """q fp16 CUDA [B*S, h_q*d_h], k, v [B*S, h_kv*d_h], pos int32 [B*S], cos / sin fp32 [n_pos, d_h/2]
     -> (q_out [B*h_kv, S*h_q/h_kv, d_h], k_out [B*h_kv, S, d_h], v_out [B*h_kv, S, d_h]): rotary embedding + layout change."""
+    qkv = (_native or _bind_torch()).rope_qkv(q, k, v, pos, cos, sin, B, S, h_q, h_kv, d_h, _raw(stream))
+    if qkv is not None:
+        return qkv
     import torch
     T = B * S
     dev = q.get_device()
@@ -390,6 +417,7 @@ class QLinear:
         _check(lib.qlinear_create(ctypes.byref(desc.c()), packed.data_ptr(),
                                   self.device.index or 0, ctypes.byref(h)), "qlinear_create")
         self._h = h
+        self._native = (h.value, desc.K, desc.N)
 
     @classmethod
     def from_weights(cls, q: np.ndarray, s: np.ndarray, bits: int, group: int = 0, device=None) -> "QLinear":
@@ -398,6 +426,9 @@ class QLinear:
 
     def forward(self, x, out=None, stream=None):
         """x: fp16 CUDA tensor [M, K] -> y fp16 [M, N] (qlinear_forward on the current stream)."""
+        y = _native.forward(self._native, x, out, _raw(stream))
+        if y is not None:
+            return y
         if not _is_x(x, self.desc.K):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward (x must be contiguous fp16 CUDA [M, K])")
         M = x.shape[0]
@@ -410,6 +441,9 @@ class QLinear:
 
     def forward_a8(self, x, out=None, stream=None):
         """The decode call with int8 activations quantised inside the kernel (qlinear_forward_a8), M <= 8."""
+        y = _native.forward_a8(self._native, x, out, _raw(stream))
+        if y is not None:
+            return y
         if not _is_x(x, self.desc.K):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_forward_a8 (x must be contiguous fp16 CUDA [M, K])")
         M = x.shape[0]
@@ -430,6 +464,9 @@ class QLinear:
 
     def embed(self, ids, out=None, stream=None):
         """ids: int32 CUDA tensor [n] -> fp16 [n, K], the dequantised rows ids of the table (qlinear_embed)."""
+        y = _native.embed(self._native, ids, out, _raw(stream))
+        if y is not None:
+            return y
         import torch
         if ids.dim() != 1 or ids.dtype != torch.int32 or not ids.is_cuda or not ids.is_contiguous():
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_embed (ids must be a contiguous int32 CUDA vector)")
@@ -468,7 +505,7 @@ class QLinear:
     def close(self) -> None:
         if getattr(self, "_h", None):
             lib.qlinear_destroy(self._h)
-            self._h = None
+            self._h = self._native = None
 
     def __del__(self):
         try:
@@ -488,6 +525,7 @@ class KVCache:
         self.k = QLinear(kd, qlinear_pack(kd, np.zeros((cache_size, d_h), np.int8), np.zeros((cache_size, 1), np.float16)), device)
         self.v = QLinear(vd, qlinear_pack(vd, np.zeros((d_h, cache_size), np.int8), np.ones((d_h, 1), np.float16)), device)
         self.v_scale = torch.zeros((cache_size,), dtype=torch.float16, device=device)
+        self._v_scale_ptr = self.v_scale.data_ptr()
 
     def append(self, k_new, v_new, stream=None):
         """k_new, v_new: fp16 CUDA [n_new, d_h], written to positions length .. length + n_new - 1."""
@@ -504,6 +542,9 @@ class KVCache:
 
     def scores(self, q_rows, stream=None):
         """q_rows fp16 [R, d_h] -> fp16 [R, cache_size] (positions beyond `length` score 0)."""
+        y = _native.kv_scores_one(self.k._native, q_rows, None, _raw(stream))
+        if y is not None:
+            return y
         if not _is_x(q_rows, self.d_h):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_scores (q_rows must be contiguous fp16 CUDA [R, d_h])")
         out = q_rows.new_empty((q_rows.shape[0], self.cache_size))
@@ -513,6 +554,9 @@ class KVCache:
 
     def output(self, prob, stream=None):
         """prob fp16 [R, cache_size] -> fp16 [R, d_h]."""
+        y = _native.kv_output(self.v._native, self._v_scale_ptr, prob, _raw(stream))
+        if y is not None:
+            return y
         if not _is_x(prob, self.cache_size):
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_output (prob must be contiguous fp16 CUDA [R, cache_size])")
         tmp = prob.new_empty(prob.shape)
@@ -534,16 +578,23 @@ class KVHeads:
         self._hk = arr(*[c.k._h for c in self.heads])
         self._hv = arr(*[c.v._h for c in self.heads])
         self._vs = arr(*[c.v_scale.data_ptr() for c in self.heads])
+        self._native = (n_heads, cache_size, d_h, ctypes.addressof(self._hk), ctypes.addressof(self._hv), ctypes.addressof(self._vs))
 
     def append_raw(self, k_ptr: int, v_ptr: int, head_stride: int, token_stride: int, n_new: int, stream=None) -> None:
         _check(lib.qlinear_kv_append_heads(self._hk, self._hv, self.n, k_ptr, v_ptr, head_stride, token_stride,
                                            self._vs, self.length, n_new, _stream_ptr(stream)), "qlinear_kv_append_heads")
+        self._appended(n_new)
+
+    def _appended(self, n_new: int) -> None:
         self.length += n_new
         for c in self.heads:
             c.length = self.length
 
     def append(self, k_new, v_new, stream=None):
         """k_new, v_new: fp16 CUDA [n_heads, n_new, d_h] (the k_out / v_out of qlinear_rope_qkv)."""
+        n_new = _native.kv_append(self._native, self.length, k_new, v_new, _raw(stream))
+        if n_new is not None:
+            return self._appended(n_new)
         import torch
         for t in (k_new, v_new):
             if t.dim() != 3 or t.shape[0] != self.n or t.shape[2] != self.d_h or t.dtype != torch.float16 or not t.is_cuda or not t.is_contiguous():
@@ -559,6 +610,9 @@ class KVHeads:
 
     def scores(self, q_rows, stream=None):
         """q_rows fp16 [n_heads, R, d_h] -> fp16 [n_heads, R, cache_size]."""
+        y = _native.kv_scores(self._native, q_rows, _raw(stream))
+        if y is not None:
+            return y
         import torch
         if q_rows.dim() != 3 or q_rows.shape[0] != self.n or q_rows.shape[2] != self.d_h or q_rows.dtype != torch.float16 or not q_rows.is_cuda or not q_rows.is_contiguous():
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_scores_heads (q_rows must be contiguous fp16 CUDA [n_heads, R, d_h])")
@@ -572,6 +626,9 @@ class KVHeads:
 
     def output(self, prob, stream=None):
         """prob fp16 [n_heads, R, cache_size] -> fp16 [n_heads, R, d_h]."""
+        y = _native.kv_output_heads(self._native, prob, _raw(stream))
+        if y is not None:
+            return y
         import torch
         if prob.dim() != 3 or prob.shape[0] != self.n or prob.shape[2] != self.cache_size or prob.dtype != torch.float16 or not prob.is_cuda or not prob.is_contiguous():
             raise QLinearError(QL_ERR_INVALID_ARG, "qlinear_kv_output_heads (prob must be contiguous fp16 CUDA [n_heads, R, cache_size])")

@@ -1522,6 +1522,12 @@ bool value_product_is_large(const Layout& V, int R)
 }
 }  // namespace
 
+extern "C" int32_t qlinear_kv_output_uses_tmp(qlinear_t hv, const void* prob, const void* v_scale, int32_t R)
+{
+    if (!hv || ((reinterpret_cast<uintptr_t>(prob) | reinterpret_cast<uintptr_t>(v_scale)) & 15)) return 1;
+    return R <= hv->gemv_max_m ? hv->use_stream : value_product_is_large(hv->L, R);
+}
+
 extern "C" ql_status qlinear_kv_output(qlinear_t hv, const void* prob, const void* v_scale, void* tmp, void* out, int32_t R, void* stream)
 {
     if (!hv || !prob || !v_scale || !tmp || !out || R < 1 || hv->L.bits != 8) return QL_ERR_INVALID_ARG;
@@ -1529,18 +1535,15 @@ extern "C" ql_status qlinear_kv_output(qlinear_t hv, const void* prob, const voi
     const int T = hv->L.K;
     if ((int64_t)R * T > INT32_MAX) return QL_ERR_INVALID_ARG;
     // decode-sized products whose cache length is a whole number of chunks: the scales are applied inside the kernel
-    if (!((reinterpret_cast<uintptr_t>(prob) | reinterpret_cast<uintptr_t>(v_scale)) & 15)) {
-        const ql_status s = qlinear_kv_output_heads(&hv, 1, prob, &v_scale, out, R, stream);
-        if (s != QL_ERR_UNSUPPORTED) return s;
+    if (!qlinear_kv_output_uses_tmp(hv, prob, v_scale, R)) {
+        if (R <= hv->gemv_max_m) return qlinear_kv_output_heads(&hv, 1, prob, &v_scale, out, R, stream);
         // more rows: the kernel that takes any number of tokens against few channels, with the scales folded in on the way
-        if (R > hv->gemv_max_m && !value_product_is_large(hv->L, R)) {
-            if ((int64_t)R * hv->L.N > INT32_MAX) return QL_ERR_INVALID_ARG;   // (the limit of qlinear_forward)
-            if (device_timed_out(hv)) return QL_ERR_DEVICE_TIMEOUT;
-            DeviceGuard guard(hv->device);
-            if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
-            const qlinear_s* h = hv;
-            return forward_mid(&h, 1, &prob, &out, R, static_cast<cudaStream_t>(stream), -1, &v_scale);
-        }
+        if ((int64_t)R * hv->L.N > INT32_MAX) return QL_ERR_INVALID_ARG;   // (the limit of qlinear_forward)
+        if (device_timed_out(hv)) return QL_ERR_DEVICE_TIMEOUT;
+        DeviceGuard guard(hv->device);
+        if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
+        const qlinear_s* h = hv;
+        return forward_mid(&h, 1, &prob, &out, R, static_cast<cudaStream_t>(stream), -1, &v_scale);
     }
     {
         DeviceGuard guard(hv->device);

@@ -1,0 +1,86 @@
+"""The native half of the binding: what it does not take goes to the Python half, and what it takes gives the same results."""
+import numpy as np
+import pytest
+
+from workloads import configs as C
+
+
+@pytest.fixture(scope="module")
+def P(_built_library):
+    import paper_2505_00232_b200 as P
+    return P
+
+
+def test_anything_but_plain_cuda_tensors_is_left_to_python(P):
+    import torch
+    native = P.binding._bind_torch()
+    x, ids = torch.zeros((2, 64), dtype=torch.float16), torch.zeros((3,), dtype=torch.int32)
+
+    class Sub(torch.Tensor):
+        pass
+    layer, heads = (1, 64, 8), (2, 32, 64, 1, 1, 1)
+    for a in (x, x.as_subclass(Sub), x.numpy(), None, 3):
+        assert native.forward(layer, a, None, None) is None and native.forward_a8(layer, a, None, None) is None
+        assert native.forward_gated(layer, layer, a, 1, None, None) is None and native.embed(layer, a, None, None) is None
+        assert native.residual_rmsnorm(a, None, a, 1e-5, 0.0, None, None, True, None) is None
+        assert native.rope_qkv(a, a, a, ids, x, x, 1, 2, 1, 1, 64, None) is None
+        assert native.kv_append(heads, 0, a, a, None) is None and native.kv_scores(heads, a, None) is None and native.kv_output_heads(heads, a, None) is None
+        assert native.kv_output(layer, 1, a, None) is None and native.kv_scores_one(layer, a, None, None) is None
+        assert native.forward_group([], a, None) is None and native.forward_group([object()], a, None) is None
+    assert native.forward(None, x, None, None) is None                   # (a closed layer)
+    with pytest.raises(P.QLinearError):
+        P.qlinear_residual_rmsnorm(x, None, x[0], 1e-5)
+
+
+@pytest.mark.gpu
+def test_both_halves_agree(P, monkeypatch):
+    import torch
+    native = P.binding._bind_torch()
+
+    class Python:                                                        # leaves every call to the Python half
+        def __getattr__(self, name):
+            return lambda *a: None
+    rng = np.random.default_rng(5)
+    f16 = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float16)).cuda()
+    mk = lambda N, K, bits, group: P.QLinear.from_weights(*C.layer_weights(5, C.LayerSpec("t", N, K, bits, group, *((-8, 7) if bits == 4 else (-128, 127)))), bits, group, device="cuda:0")
+    lins, gate, up, table = [mk(N, 512, 8, 0) for N in (256, 64, 64)], mk(256, 512, 4, 32), mk(256, 512, 4, 32), mk(1000, 128, 4, 32)
+    pos, ang = torch.arange(6, device="cuda", dtype=torch.int32), torch.rand((16, 32), device="cuda")
+
+    def calls():
+        out, kv = [], P.KVHeads(2, 1280, 64)
+        for M in (1, 5, 40, 300):
+            x = inputs[M]
+            out += [lins[0].forward(x), *P.qlinear_forward_group(lins, x), P.qlinear_forward_gated(gate, up, x, "silu"), *P.qlinear_residual_rmsnorm(x, x, x[0].contiguous(), 1e-5)]
+            o = torch.empty((M, 256), device="cuda", dtype=torch.float16)
+            assert lins[0].forward(x, out=o, stream=torch.cuda.current_stream()) is o and P.qlinear_forward_gated(gate, up, x, "gelu_tanh", out=o) is o
+            h, y = P.qlinear_residual_rmsnorm(x, None, x[0].contiguous(), 1e-5, 1, y_out=o2(M), want_h=False)
+            assert h is None
+            out += [o, y]
+            if M <= 8 or M > 128:
+                out.append(lins[0].forward_a8(x))
+        q, k, v = P.qlinear_rope_qkv(inputs["q"], inputs["k"], inputs["v"], pos, ang, ang, 1, 6, 4, 2, 64)
+        kv.append(k, v)
+        kv.append(k, v)
+        assert kv.length == 12 == kv.heads[1].length
+        for R in (4, 64):
+            prob = inputs["prob"][:, :R].contiguous()
+            out += [kv.scores(inputs["rows"][:, :R].contiguous()), kv.heads[1].scores(inputs["rows"][1, :R]), kv.heads[0].output(prob[0])] + ([kv.output(prob)] if R <= 8 else [])
+        return out + [q, k, v, table.embed(inputs["ids"])]
+
+    o2 = lambda M: torch.empty((M, 512), device="cuda", dtype=torch.float16)
+    inputs = {M: f16(M, 512) for M in (1, 5, 40, 300)}
+    inputs.update(q=f16(6, 256), k=f16(6, 128), v=f16(6, 128), rows=f16(2, 64, 64), prob=f16(2, 64, 1280), ids=torch.tensor([3, 999, -1, 1000], device="cuda", dtype=torch.int32))
+    fast = calls()
+    monkeypatch.setattr(P.binding, "_native", Python())
+    slow = calls()
+    monkeypatch.setattr(P.binding, "_native", native)
+    assert len(fast) == len(slow) and all(a.dtype == b.dtype and a.shape == b.shape and torch.equal(a, b) for a, b in zip(fast, slow))
+    for bad in (f16(3, 511), f16(3, 512).t(), f16(3, 512).float()):
+        with pytest.raises(P.QLinearError) as e:
+            lins[0].forward(bad)
+        assert e.value.status == P.QL_ERR_INVALID_ARG
+    with pytest.raises(P.QLinearError):
+        lins[0].forward(inputs[1], out=torch.empty((2, 256), device="cuda", dtype=torch.float16))
+    gate.close()
+    with pytest.raises(P.QLinearError):
+        gate.forward(inputs[1])
