@@ -28,8 +28,10 @@ struct EmbedParams {
     int32_t log2_tokens;                 // 1 << log2_tokens tokens per CTA, 128 >> log2_tokens threads each
 };
 
-// SEVERAL: tokens per CTA (else one)
-template <int BITS, bool GROUPED, bool SEVERAL>
+// SEVERAL: tokens per CTA (else one).  U: pieces of a thread that are requested together: 2 where it has more than one.  The table
+// comes from HBM, the rows of one prompt all over it (64 rows of 4096, the table not in L2, 3.6 -> 3.1 us, of 8192 5.2 -> 4.3; 2048 rows of 4096 11.5 both ways,
+// their scattered 64-byte reads and the writes are the bound there; with one piece per thread the second one's tests cost 0.1).
+template <int BITS, bool GROUPED, bool SEVERAL, int U = 1>
 __global__ void __launch_bounds__(128) embed_kernel(const EmbedParams p)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -50,30 +52,41 @@ __global__ void __launch_bounds__(128) embed_kernel(const EmbedParams p)
     const uint8_t* base = p.body + (int64_t)rsb * p.n_kc * p.block_bytes + rb * 512 + g * 64;
     uint32_t s2[2];                                                     // scales of the chunk's two groups, in both halves
     s2[0] = s2[1] = GROUPED ? 0u : 0x10001u * (uint32_t)__half_as_ushort(p.chan_scales[row]);
-    for (int piece = (int)first; piece < p.n_kc * 4; piece += lanes) {
-        const int kc = piece >> 2, c = piece & 3;
-        const uint8_t* blk = base + (int64_t)kc * p.block_bytes;
-        const uint4 w = *reinterpret_cast<const uint4*>(blk + c * 16);
-        if (GROUPED) {
-            const uint32_t s = *reinterpret_cast<const uint32_t*>(blk - (rb * 512 + g * 64) + kWeightBlockBytes + rb * 64 + g * 8 + 4 * hi);
-            s2[0] = __byte_perm(s, 0, 0x1010);
-            s2[1] = __byte_perm(s, 0, 0x3232);
+    for (int piece0 = (int)first; piece0 < p.n_kc * 4; piece0 += U * lanes) {
+        uint4 w[U];
+        uint32_t s[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const int piece = piece0 + j * (int)lanes;
+            if (piece >= p.n_kc * 4) break;
+            const uint8_t* blk = base + (int64_t)(piece >> 2) * p.block_bytes;
+            w[j] = *reinterpret_cast<const uint4*>(blk + (piece & 3) * 16);
+            if (GROUPED) s[j] = *reinterpret_cast<const uint32_t*>(blk - (rb * 512 + g * 64) + kWeightBlockBytes + rb * 64 + g * 8 + 4 * hi);
         }
-        const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-        constexpr int RUNS = BITS == 4 ? 2 : 1;                          // runs of 8 consecutive k in a piece: 16 bytes of output each
 #pragma unroll
-        for (int h = 0; h < RUNS; ++h) {
-            uint32_t o[4];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                uint32_t a[4];
-                if (BITS == 4) unpack_int4_word(ww[2 * h + i], a);
-                else unpack_int8_words(ww[2 * i], ww[2 * i + 1], a);
-                o[2 * i] = h2_mul(hi ? a[1] : a[0], s2[h]);              // registers hi and hi + 2 hold this row; one rounding
-                o[2 * i + 1] = h2_mul(hi ? a[3] : a[2], s2[h]);
+        for (int j = 0; j < U; ++j) {
+            const int piece = piece0 + j * (int)lanes, kc = piece >> 2, c = piece & 3;
+            if (piece >= p.n_kc * 4) break;
+            if (GROUPED) {
+                s2[0] = __byte_perm(s[j], 0, 0x1010);
+                s2[1] = __byte_perm(s[j], 0, 0x3232);
             }
-            const int k = kc * CHUNK_K + 32 * h + 8 * c;                 // (K is a multiple of 32: a run lies inside or outside)
-            if (k < p.K) *reinterpret_cast<uint4*>(yrow + k) = make_uint4(o[0], o[1], o[2], o[3]);
+            const uint32_t ww[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+            constexpr int RUNS = BITS == 4 ? 2 : 1;                      // runs of 8 consecutive k in a piece: 16 bytes of output each
+#pragma unroll
+            for (int h = 0; h < RUNS; ++h) {
+                uint32_t o[4];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    uint32_t a[4];
+                    if (BITS == 4) unpack_int4_word(ww[2 * h + i], a);
+                    else unpack_int8_words(ww[2 * i], ww[2 * i + 1], a);
+                    o[2 * i] = h2_mul(hi ? a[1] : a[0], s2[h]);          // registers hi and hi + 2 hold this row; one rounding
+                    o[2 * i + 1] = h2_mul(hi ? a[3] : a[2], s2[h]);
+                }
+                const int k = kc * CHUNK_K + 32 * h + 8 * c;             // (K is a multiple of 32: a run lies inside or outside)
+                if (k < p.K) *reinterpret_cast<uint4*>(yrow + k) = make_uint4(o[0], o[1], o[2], o[3]);
+            }
         }
     }
 }

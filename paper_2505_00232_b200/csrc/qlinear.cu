@@ -1576,6 +1576,7 @@ extern "C" ql_status qlinear_embed(qlinear_t h, const int32_t* ids, int32_t n, v
     // short rows: several tokens to a CTA where that leaves several CTAs per SM (a CTA costs more than what four threads of it do)
     while (L.n_kc * 4 <= 64 >> prm.log2_tokens && n >> (prm.log2_tokens + 1) >= 4 * h->num_sms) ++prm.log2_tokens;
     auto kern = L.bits == 8 ? embed_kernel<8, false, false> : L.grouped ? embed_kernel<4, true, false> : embed_kernel<4, false, false>;
+    if (L.n_kc * 4 > 128) kern = L.bits == 8 ? embed_kernel<8, false, false, 2> : L.grouped ? embed_kernel<4, true, false, 2> : embed_kernel<4, false, false, 2>;
     if (prm.log2_tokens) kern = L.bits == 8 ? embed_kernel<8, false, true> : L.grouped ? embed_kernel<4, true, true> : embed_kernel<4, false, true>;
     const cudaError_t e = launch(kern, prm, dim3(((n - 1) >> prm.log2_tokens) + 1), dim3(128), 0, st, 1, h->pdl);
     if (e != cudaSuccess) cudaGetLastError();
