@@ -180,6 +180,18 @@ __global__ void __launch_bounds__(narrow_threads(G), 2) gemm_narrow_kernel(const
     const uint32_t tmem_base = *tmem_slot;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
+    // The per-channel scales of the four channels whose sums over the K parts this thread finishes: requested here unless the kernel before
+    // may be writing them, so that their latency does not follow the cluster's barrier (Llama q + k + v at 32 tokens 9.5 -> 9.2 us, o 8.2 -> 7.9, at
+    // 16 tokens 8.9 -> 8.45; a gated pair, twice the registers, 24.3 -> 24.6).
+    constexpr bool EARLY_SCALES = !GROUPED && !GATED;
+    [[maybe_unused]] uint2 early = make_uint2(0, 0);
+    [[maybe_unused]] auto load_early = [&] {
+        const int row = rsb * kRsbRows + lane * 4;                       // (N is a multiple of 8: the four channels exist together)
+        if (row < p.N[ly]) asm volatile("ld.global.cg.v2.u32 {%0,%1}, [%2];" : "=r"(early.x), "=r"(early.y) : "l"(p.chan_scales[ly] + row) : "memory");
+    };
+    if constexpr (EARLY_SCALES)
+        if (p.cl > 1 && !p.late && warp >= kNarrowFirstWorker) load_early();
+
     bool ok = true;
     if (warp == 0) {
         // ------------------------------------------------------------------ weights
@@ -337,7 +349,12 @@ __global__ void __launch_bounds__(narrow_threads(G), 2) gemm_narrow_kernel(const
 #pragma unroll
             for (int r = 0; r < R; ++r)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) sc[r][i] = !GROUPED && row0 < N ? __half2float(ld_cg_half(p.chan_scales[GATED ? r : ly] + row0 + i)) : 1.f;
+                for (int i = 0; i < 4; ++i) sc[r][i] = !GROUPED && !EARLY_SCALES && row0 < N ? __half2float(ld_cg_half(p.chan_scales[GATED ? r : ly] + row0 + i)) : 1.f;
+            if constexpr (EARLY_SCALES) {
+                if (p.late) load_early();
+                const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&early.x)), hi = __half22float2(*reinterpret_cast<const __half2*>(&early.y));
+                sc[0][0] = lo.x; sc[0][1] = lo.y; sc[0][2] = hi.x; sc[0][3] = hi.y;
+            }
             for (int tok = crank + (t >> 5) * p.cl; tok < bn && m0 + tok < p.M; tok += 4 * G * p.cl) {
                 float v[R][4];
 #pragma unroll
