@@ -19,7 +19,7 @@
 // Measured, weights out of HBM, against the 256-token-tile kernel that served these sizes: Llama gate + up 25.9 us at 16 tokens (47.3 before),
 // 37.0 at 32 (48.9); down (33 MB) 13.7 (26.6), 18.9 (28.7); q + k + v (25 MB of int8) 8.9 (19.2), 12.4 (20.5); one 2304 x 2304 int8 layer 4.5
 // (11.7), 6.0 (13.7).  Against gemm_narrow.cuh: see gemm_route in qlinear.cu.  Value product of 1024 rows over 4096 positions,
-// d_h = 128: a pass over the probabilities for the scales and a single-CTA matmul on 8 CTAs 38.5 us, now 9.8.
+// d_h = 128: a pass over the probabilities for the scales and a single-CTA matmul on 8 CTAs 38.5 us, now 9.5; its tiles: value_tokens in qlinear.cu.
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
@@ -73,6 +73,9 @@ __global__ void __launch_bounds__(kMidThreads, 2) gemm_mid_kernel(const MidParam
     using S = MidSmem<BITS, GROUPED, NT>;
     constexpr int NS = S::kStages, CHUNK_K = BITS == 4 ? 64 : 32, BB = kWeightBlockBytes + (GROUPED ? kScaleBlockBytes : 0);
     constexpr int UNITS = S::kKStep / 8;                                 // 16-byte pieces of a token's stage
+    // Warps that share a tile's tokens, each with as many row-blocks: what a warp reads of x from shared memory halves.  (The value product, whose
+    // x needs arithmetic as well, 4096 rows of 4096 positions 22.8 -> 21.3 us; elsewhere the second unpacking of the weights costs more.)
+    constexpr int WT = KSCALE && NT >= 4 && NT % 2 == 0 ? 2 : 1, NTW = NT / WT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, c = lane & 3;
@@ -157,24 +160,31 @@ __global__ void __launch_bounds__(kMidThreads, 2) gemm_mid_kernel(const MidParam
         commit();
     }
 
-    float acc[NT][4];
+    const int rb0 = WT == 1 ? warp : WT * (warp & 3), n0 = WT == 1 ? 0 : (warp >> 2) * NTW;   // this warp's row-blocks and groups of 8 tokens
+    float acc[WT][NTW][4];
 #pragma unroll
-    for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+    for (int j = 0; j < WT; ++j)
+#pragma unroll
+        for (int n = 0; n < NTW; ++n) acc[j][n][0] = acc[j][n][1] = acc[j][n][2] = acc[j][n][3] = 0.f;
     auto lds128 = [](uint32_t addr) {
         uint4 v;
         asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
         return v;
     };
     // 32-k group G of the stage: this lane's piece of token 8 n + g
-    const uint32_t xl[2] = {(uint32_t)(g * S::kKStep * 2 + (g & 1) * 64 + c * 16), (uint32_t)(g * S::kKStep * 2 + ((g & 1) ^ 1) * 64 + c * 16)};
-    auto group = [&](uint32_t xs, int G, const uint32_t a0[4], const uint32_t a1[4], const uint4& f) {
+    const uint32_t x_warp = (uint32_t)(n0 * 8 * S::kKStep * 2);
+    const uint32_t xl[2] = {x_warp + (uint32_t)(g * S::kKStep * 2 + (g & 1) * 64 + c * 16), x_warp + (uint32_t)(g * S::kKStep * 2 + ((g & 1) ^ 1) * 64 + c * 16)};
+    auto group = [&](uint32_t xs, int G, const uint32_t a0[WT][4], const uint32_t a1[WT][4], const uint4& f) {
         const uint32_t xa = xs + xl[G & 1] + (G >> 1) * 128;
 #pragma unroll
-        for (int n = 0; n < NT; ++n) {
+        for (int n = 0; n < NTW; ++n) {
             uint4 b = lds128(xa + n * 8 * S::kKStep * 2);
             if (KSCALE) b = make_uint4(h2_mul(b.x, f.x), h2_mul(b.y, f.y), h2_mul(b.z, f.z), h2_mul(b.w, f.w));
-            mma_16816_pure(acc[n], a0, b.x, b.y);
-            mma_16816_pure(acc[n], a1, b.z, b.w);
+#pragma unroll
+            for (int j = 0; j < WT; ++j) {
+                mma_16816_pure(acc[j][n], a0[j], b.x, b.y);
+                mma_16816_pure(acc[j][n], a1[j], b.z, b.w);
+            }
         }
     };
     int stage = 0;
@@ -189,27 +199,31 @@ __global__ void __launch_bounds__(kMidThreads, 2) gemm_mid_kernel(const MidParam
         const uint32_t xs = smem0 + stage * S::kStage, ws = xs + S::kXBytes;
 #pragma unroll
         for (int ch = 0; ch < 2; ++ch) {
-            const uint4 w = lds128(ws + ch * kWeightBlockBytes + t * 16);
             if (BITS == 4) {
+                const uint4 w = lds128(ws + ch * kWeightBlockBytes + t * 16);
                 const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
                 uint2 sc = make_uint2(0, 0);
                 if (GROUPED) asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(sc.x), "=r"(sc.y) : "r"(ws + S::kWBytes + ch * kScaleBlockBytes + warp * 64 + g * 8));
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    uint32_t a0[4], a1[4];
-                    unpack_int4_word(ww[2 * h], a0);
-                    unpack_int4_word(ww[2 * h + 1], a1);
+                    uint32_t a0[WT][4], a1[WT][4];
+                    unpack_int4_word(ww[2 * h], a0[0]);
+                    unpack_int4_word(ww[2 * h + 1], a1[0]);
                     if (GROUPED) {
                         const uint32_t lo = __byte_perm(sc.x, 0, h ? 0x3232 : 0x1010), hi = __byte_perm(sc.y, 0, h ? 0x3232 : 0x1010);
-                        a0[0] = h2_mul(a0[0], lo); a0[1] = h2_mul(a0[1], hi); a0[2] = h2_mul(a0[2], lo); a0[3] = h2_mul(a0[3], hi);
-                        a1[0] = h2_mul(a1[0], lo); a1[1] = h2_mul(a1[1], hi); a1[2] = h2_mul(a1[2], lo); a1[3] = h2_mul(a1[3], hi);
+                        a0[0][0] = h2_mul(a0[0][0], lo); a0[0][1] = h2_mul(a0[0][1], hi); a0[0][2] = h2_mul(a0[0][2], lo); a0[0][3] = h2_mul(a0[0][3], hi);
+                        a1[0][0] = h2_mul(a1[0][0], lo); a1[0][1] = h2_mul(a1[0][1], hi); a1[0][2] = h2_mul(a1[0][2], lo); a1[0][3] = h2_mul(a1[0][3], hi);
                     }
                     group(xs, 2 * ch + h, a0, a1, make_uint4(0, 0, 0, 0));
                 }
             } else {
-                uint32_t a0[4], a1[4];
-                unpack_int8_words(w.x, w.y, a0);
-                unpack_int8_words(w.z, w.w, a1);
+                uint32_t a0[WT][4], a1[WT][4];
+#pragma unroll
+                for (int j = 0; j < WT; ++j) {
+                    const uint4 w = lds128(ws + ch * kWeightBlockBytes + (rb0 + j) * 512 + lane * 16);
+                    unpack_int8_words(w.x, w.y, a0[j]);
+                    unpack_int8_words(w.z, w.w, a1[j]);
+                }
                 uint4 f = make_uint4(0, 0, 0, 0);
                 if (KSCALE) f = lds128(ws + S::kWBytes + S::kSBytes + ch * CHUNK_K * 2 + c * 16);
                 group(xs, ch, a0, a1, f);
@@ -222,9 +236,11 @@ __global__ void __launch_bounds__(kMidThreads, 2) gemm_mid_kernel(const MidParam
 
     float* part = reinterpret_cast<float*>(smem_raw);                    // [token][channel]
 #pragma unroll
-    for (int n = 0; n < NT; ++n)
+    for (int j = 0; j < WT; ++j)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) part[(8 * n + 2 * c + (i & 1)) * S::kPartStride + warp * 16 + g + 8 * (i >> 1)] = acc[n][i];
+        for (int n = 0; n < NTW; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) part[(8 * (n0 + n) + 2 * c + (i & 1)) * S::kPartStride + (rb0 + j) * 16 + g + 8 * (i >> 1)] = acc[j][n][i];
     cg::cluster_group cluster = cg::this_cluster();
     if (p.cl > 1) {
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");

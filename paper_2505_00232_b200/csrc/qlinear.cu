@@ -654,16 +654,47 @@ bool takes_mid(const qlinear_s* const* hs, int n, int M, bool gated = false)
     return weights <= (M <= 48 || gated ? 48000000 : hs[0]->L.bits == 4 ? 30000000 : 24000000);
 }
 
+// Tokens per tile of the value product, in eights: 2, 3, 4 or 8, what an estimate of the launch says is fastest (us, consecutive launches over caches
+// in L2; 1350 measurements of 16 to 4096 rows, 256 to 16384 positions, heads of 64 to 256 with tiles of 16 to 64: 0.89 to 1.10 times this, 5th and
+// 95th percentile).  A step costs a CTA 0.22 us and 0.048 for every 8 tokens, so few rows want narrow tiles; beyond one CTA for 0.735 of
+// the SMs (14 clusters of 8 leave room for the next launch's) a launch slows down, and narrow tiles have more CTAs.  Against tiles of 64 to 64 rows, then of 32 while those
+// of 64 would leave an SM with one CTA, us before / now: 4096 positions, 48 rows 7.4 / 5.1, 64 8.4 / 5.1, 128 6.4 / 5.3, 256 6.5 / 5.8, 512 9.0 / 7.3, 1024
+// 9.7 / 9.5, 2048 14.6 / 13.8; 64 rows of 16384 positions 23.6 / 12.7; 13 % over all of them, the worst 0.95.
+int value_tokens(int units, int M, int n_steps, int num_sms)
+{
+    static const int widths[4] = {2, 3, 4, 8};
+    double best_us = 1e30;
+    int best = 2;
+    for (const int nt : widths) {
+        if (nt > 2 && M <= 8 * (nt == 8 ? 4 : nt - 1)) break;            // (a narrower one holds all rows as well)
+        const int tiles = units * ((M + 8 * nt - 1) / (8 * nt)), cl = mid_parts(tiles, n_steps, num_sms), ctas = tiles * cl;
+        if (ctas > 2 * num_sms && nt != 8) continue;                     // (more rounds than the estimate was made for)
+        const double u = ctas / (0.735 * num_sms);
+        const double load = 1.0 + 0.47 * std::min(1.0, std::max(0.0, (u - 1.0) / 0.12)) + 0.158 * std::max(0.0, u - 1.12);
+        const int steps = (n_steps + cl - 1) / cl, lg = log2_of(cl);
+        const double us = 0.88 + 0.137 * lg + load * (0.81 + nt * (0.142 + 0.0153 * lg) + steps * (0.221 + 0.0483 * nt));
+        if (us < best_us) { best_us = us; best = nt; }
+    }
+    return best;
+}
+
 template <int BITS, bool GROUPED, bool GATED, bool KSCALE = false>
 cudaError_t launch_mid(const qlinear_s* h, MidParams& prm, int units, bool pdl, cudaStream_t st)
 {
-    if (prm.M <= 16) return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, pdl, st);
-    if (prm.M <= 24) return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, pdl, st);
-    if (prm.M <= 32) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
-    // (more tokens than that: the value product.  Tiles of 32 tokens where those of 64 would leave every SM with one CTA.)
-    if (prm.M > 64 && units * ((prm.M + 63) / 64) * 8 <= 2 * h->num_sms) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
-    if (prm.M <= 48) return launch_mid_nt<BITS, GROUPED, 6, GATED, KSCALE>(h, prm, units, pdl, st);
-    return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
+    if constexpr (KSCALE) {
+        switch (value_tokens(units, prm.M, (prm.n_kc + 1) / 2, h->num_sms)) {
+            case 2: return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, pdl, st);
+            case 3: return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, pdl, st);
+            case 4: return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
+            default: return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
+        }
+    } else {
+        if (prm.M <= 16) return launch_mid_nt<BITS, GROUPED, 2, GATED, KSCALE>(h, prm, units, pdl, st);
+        if (prm.M <= 24) return launch_mid_nt<BITS, GROUPED, 3, GATED, KSCALE>(h, prm, units, pdl, st);
+        if (prm.M <= 32) return launch_mid_nt<BITS, GROUPED, 4, GATED, KSCALE>(h, prm, units, pdl, st);
+        if (prm.M <= 48) return launch_mid_nt<BITS, GROUPED, 6, GATED, KSCALE>(h, prm, units, pdl, st);
+        return launch_mid_nt<BITS, GROUPED, 8, GATED, KSCALE>(h, prm, units, pdl, st);
+    }
 }
 
 // n layers that share K and scheme, layer i on xs[i]; act >= 0: the gated form (n == 2, equal shapes, ys[0] the output);
