@@ -58,21 +58,25 @@ constexpr int kTaSlotCols = 32;              // 64 k of fp16
 constexpr int kTaAccCols = 256;
 
 // I8: the integer form (int8 activations, kind::i8): a k-step is 128 k, i.e. again 128 bytes per x row and 32 columns per A slot.
-template <int BITS, bool I8 = false>
+// BOTH: the gated form with two accumulators, which leaves tensor memory for 6 A slots.
+constexpr int kTaBothTokens = 160;           // its widest token block
+template <int BITS, bool I8 = false, bool BOTH = false>
 struct GemmTaSmem {
     // Two rings, because the two operands are needed at different times: the packed weights of a k-step are needed
     // early (they still have to be dequantised), its x tile only when the MMA is issued.  A deep ring of small
     // weight stages lets the dequantise warps run ahead; the x ring only has to cover the TMA latency.
     static constexpr int kXBytes = 128 * 128;                            // this CTA's 128 tokens x 64 k
     static constexpr int kKStep = I8 ? 128 : kGemmKStep;
-    static constexpr int kXStages = (I8 && BITS == 8) ? 6 : 7;           // <= kASlots: the x producer reads "stage free" off the A-slot barrier
+    static constexpr int kXStages = BOTH || (I8 && BITS == 8) ? 6 : 7;   // <= kASlots: the x producer reads "stage free" off the A-slot barrier
     static constexpr int kWBlocks = (I8 ? 2 : 1) * (BITS == 4 ? 1 : 2);  // packed blocks per k-step
     static constexpr int kWBytes = I8 ? kWBlocks * kWeightBlockBytes : (BITS == 4 ? 5120 : 8192);
     // A ring length that is a multiple of the 3 dequantise turns keeps every stage with one turn, whose warps then see all
     // of the stage's phases in order; the 16 KB stages of the int8 integer form leave room for 4 only, and its warps first
     // wait for the stage's release (see the main loop of the dequantise warps).
     static constexpr int kWStages = I8 ? (BITS == 4 ? 6 : 4) : (BITS == 4 ? 9 : 6);
-    static constexpr int kASlots = 8;                                    // tensor memory: 8 x 32 columns beside the accumulator
+    static constexpr int kASlots = BOTH ? 6 : 8;                         // tensor memory: 8 x 32 columns beside the accumulator
+    static constexpr int kAccCols = BOTH ? 2 * kTaBothTokens : kTaAccCols;
+    static_assert(kAccCols + kASlots * kTaSlotCols <= 512, "tensor memory");
     static constexpr int kEarlySteps = kASlots - 2;                      // steps of the next tile dequantised before the epilogue is forced
     static constexpr int kWOffset = kXStages * kXBytes;
     static constexpr int kOutOffset = kWOffset + kWStages * kWBytes;     // fp16 output tile [256 tokens][128 channels]
@@ -231,13 +235,17 @@ struct DequantRowTa {
 // sum of the token's quantised row) and applies both scales (paper Section 3.7, prefill stage).
 // PARTS: the launch has K parts (p.split is 2 or 4).  An instantiation of its own: the registers of one epilogue are the kernel's limit
 // (Gemma2-2B q + k + v at 777 tokens, which has no parts, 16.8 us with both in one kernel, 16.5 without).
-template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false, bool PARTS = false>
+// BOTH (gated, blocks of up to 160 tokens): gate and up have an accumulator each, the k-steps of the up tile follow those of the gate tile
+// without an epilogue between them, and act(gate) stays in fp32 until the product.  (With one accumulator it is rounded to fp16 between the two tiles.)
+template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false, bool PARTS = false, bool BOTH = false>
 __global__ void __launch_bounds__(kPairThreads, 1)
 gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
 {
     static_assert(!I8 || (!GATED && !GROUPED), "the integer form: per-channel scales, plain output");
     static_assert(!GATED || !PARTS, "a gated tile has no parts");
-    using S = GemmTaSmem<BITS, I8>;
+    static_assert(!BOTH || GATED, "two accumulators: a gated pair");
+    using S = GemmTaSmem<BITS, I8, BOTH>;
+    constexpr bool TURNS = GATED && !BOTH;                               // gate tile and up tile are units of their own
     constexpr int NX = S::kXStages, NW = S::kWStages, NA = S::kASlots;
     const int bn = p.bn;                                                 // tokens per tile: a multiple of 32, at most 256
     constexpr int W_BOX_BYTES = I8 ? S::kWBytes : BITS == 4 ? (GROUPED ? kWeightBlockBytes + kScaleBlockBytes : kWeightBlockBytes) : 2 * kWeightBlockBytes;
@@ -271,16 +279,17 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
     const int P = PARTS ? p.split : 1;
     const int part = P > 1 ? first_tile % P : 0;
     const int it_base = part * p.n_ksteps / P;
-    const int n_steps = (part + 1) * p.n_ksteps / P - it_base;          // k-steps per unit of work of this cluster
+    const int k_steps = (part + 1) * p.n_ksteps / P - it_base;          // k-steps per unit of work of this cluster and layer
+    const int n_steps = BOTH ? 2 * k_steps : k_steps;
     // the j-th unit of work of this cluster: a tile and, in the gated form, which of the two layers
     auto unit = [&](int j, int& tile, int& gl) {
-        const int v = first_tile + (GATED ? j >> 1 : j) * tile_stride;
+        const int v = first_tile + (TURNS ? j >> 1 : j) * tile_stride;
         tile = P > 1 ? v / P : v;
-        gl = GATED ? (j & 1) : 0;
+        gl = TURNS ? (j & 1) : 0;
         return v < p.n_tiles * P;
     };
     int n_units = 0;
-    for (int v = first_tile; v < p.n_tiles * P; v += tile_stride) n_units += GATED ? 2 : 1;
+    for (int v = first_tile; v < p.n_tiles * P; v += tile_stride) n_units += TURNS ? 2 : 1;
     const int total_steps = n_units * n_steps;
     const int w_rows = p.block_bytes >> 6;                               // 64-byte rows per packed block
 
@@ -348,7 +357,8 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                 for (int it = 0; it < n_steps; ++it) {
                     if (!mbar_wait(wempty_bar(s), par, abort_flag, 0x100 + s)) { ok = false; break; }
                     mbar_expect_tx(wfull_bar(s), W_BOX_BYTES);
-                    tma_load_2d(wpk_addr(s), wm, 0, row0 + (it_base + it) * CHUNKS * w_rows, wfull_bar(s));
+                    if (BOTH && it >= k_steps) tma_load_2d(wpk_addr(s), &maps.w[1], 0, row0 + (it - k_steps) * CHUNKS * w_rows, wfull_bar(s));
+                    else tma_load_2d(wpk_addr(s), wm, 0, row0 + (it_base + it) * CHUNKS * w_rows, wfull_bar(s));
                     ++issued;
                     if (++s == NW) { s = 0; par ^= 1; }
                 }
@@ -379,7 +389,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                         if (!mbar_wait(aempty_bar(ao), (uint32_t)((g - NX) / NA) & 1, abort_flag, 0x180 + ao)) { ok = false; break; }
                     }
                     mbar_expect_tx(afull_bar(g % NA), x_bytes);
-                    tma_load_2d(xs_addr(s), &maps.x, (it_base + it) * S::kKStep, m0, afull_bar(g % NA));
+                    tma_load_2d(xs_addr(s), &maps.x, (BOTH && it >= k_steps ? it - k_steps : it_base + it) * S::kKStep, m0, afull_bar(g % NA));
                     if (++s == NX) s = 0;
                 }
             }
@@ -409,13 +419,16 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                     // (the dequantise warps run ahead, so the phase is normally complete already: test, else suspend)
                     if (!mbar_wait(afull_bar(a), apar, abort_flag, 0x300 + a)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t ta = tmem_base + (uint32_t)(kTaAccCols + a * kTaSlotCols);
+                    const uint32_t ta = tmem_base + (uint32_t)(S::kAccCols + a * kTaSlotCols);
+                    const bool up = BOTH && it >= k_steps;
+                    const uint32_t d = up ? tmem_base + kTaBothTokens : tmem_base;
+                    const int first = up ? k_steps : 0;
                     const uint32_t b_lo = b_lo0 + (uint32_t)s * (S::kXBytes >> 4);
                     if (elect_one()) {
 #pragma unroll
                         for (int k4 = 0; k4 < 4; ++k4) {                 // 16 k (32 k of bytes): 8 columns of A, 32 bytes of the B swizzle row
-                            if (I8) umma_i8_pair_ta(tmem_base, ta + 8 * k4, b_lo + 2 * k4, idesc, (it > 0 || k4 > 0) ? 1u : 0u);
-                            else umma_f16_pair_ta(tmem_base, ta + 8 * k4, b_lo + 2 * k4, idesc, (it > 0 || k4 > 0) ? 1u : 0u);
+                            if (I8) umma_i8_pair_ta(d, ta + 8 * k4, b_lo + 2 * k4, idesc, (it > first || k4 > 0) ? 1u : 0u);
+                            else umma_f16_pair_ta(d, ta + 8 * k4, b_lo + 2 * k4, idesc, (it > first || k4 > 0) ? 1u : 0u);
                         }
                         umma_commit_pair(aempty_bar(a));                 // frees the A slot and the x stage in both CTAs
                     }
@@ -564,9 +577,9 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
             const int ly = GATED ? 0 : pair_layer(p, rsb);
             const int N = p.lN[ly];
             const int m0 = (tile % n_mblk) * bn + 64 * wi;
-            const uint32_t gpar = (uint32_t)(GATED ? j >> 1 : j) & 1;   // phase of the group barriers: once per output tile
+            const uint32_t gpar = (uint32_t)(TURNS ? j >> 1 : j) & 1;   // phase of the group barriers: once per output tile
             bool live = true;
-            if (!GATED || gl == 0) {
+            if (!TURNS || gl == 0) {
                 // the four warps have read their rows of the previous output tile
                 __syncwarp();
                 if (lane == 0) mbar_arrive(grp_bar(wi, 0));
@@ -611,6 +624,23 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                             orow[(cc + 4 * v4 + 3) * 128] = __float2half_rn(f.w * (scale * (float)((int)r[4 * v4 + 3] - OFF * i.w)));
                         }
                     }
+                } else if constexpr (BOTH) {
+                    float scale_up = 1.f;
+                    if (!GROUPED && n < N) scale_up = __half2float(p.lscales[1][n]);
+                    auto store = [&](auto act) {
+#pragma unroll 1
+                        for (int cc = 0; cc < n_cols; cc += 16) {
+                            uint32_t r[16], u[16];
+                            tmem_ld16(taddr + (uint32_t)cc, r);
+                            tmem_ld16(taddr + (uint32_t)(kTaBothTokens + cc), u);
+                            if (cc + 16 >= n_cols) release();
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) orow[(cc + q) * 128] = __float2half_rn(act(__uint_as_float(r[q]) * scale) * (__uint_as_float(u[q]) * scale_up));
+                        }
+                    };
+                    if (p.act == QL_ACT_SILU) store([](float v) { return gate_activation(v, QL_ACT_SILU); });
+                    else if (p.act == QL_ACT_GELU_TANH) store([](float v) { return gate_activation(v, QL_ACT_GELU_TANH); });
+                    else store([](float v) { return v; });
                 } else {
 #pragma unroll
                     for (int cc = 0; cc < 64; cc += 32) {
@@ -632,7 +662,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                     }
                 }
             }
-            if (GATED && gl == 0) {                                      // the product is sent when the up tile is done
+            if (TURNS && gl == 0) {                                      // the product is sent when the up tile is done
                 if (!live) ok = false;
                 return;
             }
@@ -693,7 +723,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
                 // the MMAs that read the slot (step g - NA) have retired
                 if (!mbar_wait(aempty_bar(a), apar, abort_flag, 0xB00 + a)) { ok = false; break; }
                 tc_fence_after();
-                tmem_st16(tmem_base + lane_base + (uint32_t)(kTaAccCols + a * kTaSlotCols + 16 * half), r);
+                tmem_st16(tmem_base + lane_base + (uint32_t)(S::kAccCols + a * kTaSlotCols + 16 * half), r);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) { mbar_arrive(wempty_bar(s)); mbar_arrive(afull_bar(a)); }
@@ -704,7 +734,7 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
         } else {
             // The addresses of the step's weight stage, barriers and A slot are kept and advanced, not formed from an index.
             uint32_t wst = wpk_addr(my_turn), wbar = wfull_bar(my_turn), abar = afull_bar(my_turn);   // my_turn < NW, NA
-            uint32_t slot = tmem_base + lane_base + (uint32_t)(kTaAccCols + my_turn * kTaSlotCols + 16 * half);
+            uint32_t slot = tmem_base + lane_base + (uint32_t)(S::kAccCols + my_turn * kTaSlotCols + 16 * half);
             const uint32_t wbar_end = wfull_bar(NW), abar_end = afull_bar(NA);
             int event = n_steps;                                         // first step at which the tile or the epilogue has to be looked at
             for (int g = my_turn; g < total_steps; g += 3) {
@@ -769,14 +799,14 @@ inline double gemm_pair_ta_us(int pairs, int n_mblk, int bn, int split, int n_ks
 // blocks here: gemm_route compares the two, and what is left of them has large K parts.
 struct TaPlan { int n_mblk, bn, split; };
 inline bool gemm_pair_ta_searches(int pairs, int M, int n_ksteps, bool i8) { return i8 || (M > 128 && pairs > 2 && n_ksteps > 16); }
-inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int layers, bool i8, int num_sms, bool may_split)
+inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int layers, bool i8, int num_sms, bool may_split, int widest = 256)
 {
     const int clusters = num_sms / 2;
     const int forced = gemm_config().force_split >= 4 ? 4 : gemm_config().force_split >= 2 ? 2 : gemm_config().force_split;
     const bool search = gemm_pair_ta_searches(pairs, M, n_ksteps, i8);
     TaPlan best{};
     double best_us = 1e30;
-    for (int bn = 256; bn >= 32; bn -= 32) {
+    for (int bn = widest; bn >= 32; bn -= 32) {
         const int n_mblk = (M + bn - 1) / bn, tiles = pairs * n_mblk;
         if (((M + n_mblk - 1) / n_mblk + 31) / 32 * 32 != bn) continue;  // (as many blocks, and narrower: comes later)
         for (int split = 1; split <= 4; split *= 2) {
@@ -795,17 +825,17 @@ inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int layers, bool
 // scratch / counters: the device's shared fp32 scratch and arrival counters for the K-split case (null: no split).
 // a8_scale != nullptr: the integer form; x is then the int8 activations, a8_scale / a8_rowsum their per-token arrays, and
 // set.wmap the integer form's weight maps (boxes of 128 k).
-template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false, bool PARTS = false>
+template <int BITS, bool GROUPED, bool GATED = false, bool I8 = false, bool PARTS = false, bool BOTH = false>
 ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const TaPlan& pl, const void* x, int M, cudaStream_t st, int device, bool pdl, int num_sms, int act = -1,
                               float* scratch = nullptr, unsigned int* counters = nullptr,
                               const float* a8_scale = nullptr, const int32_t* a8_rowsum = nullptr)
 {
-    using S = GemmTaSmem<BITS, I8>;
+    using S = GemmTaSmem<BITS, I8, BOTH>;
     const Layout& L = *set.L[0];
     TaMaps maps;
     if (!x_tensor_map(x, L.K, M, pl.bn / 2, &maps.x, I8 ? 1 : 2)) return QL_ERR_CUDA;
     for (int i = 0; i < kGemmMaxGroup; ++i) maps.w[i] = *set.wmap[i < set.n ? i : 0];
-    auto kern = gemm_pair_ta_kernel<BITS, GROUPED, GATED, I8, PARTS>;
+    auto kern = gemm_pair_ta_kernel<BITS, GROUPED, GATED, I8, PARTS, BOTH>;
     static std::atomic<bool> attr_set[64];
     if (device >= 0 && device < 64 && !attr_set[device]) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal) != cudaSuccess) {
@@ -867,17 +897,27 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const TaPlan& pl, const
 // Any M the prefill path sees (tokens beyond M are zero-filled by TMA and never stored): below 129 tokens the tile is
 // mostly padding, but the launch is bound by streaming and dequantising the weights, which this kernel spreads over
 // the whole GPU (K split), not by the MMAs.
+// A gated pair without a position of 256 tokens for every CTA pair: the form with two accumulators.
+inline bool gemm_pair_ta_both(const Layout& L, int M, int num_sms) { return L.n_rsb / 2 * ((M + 255) / 256) < num_sms / 2; }
+inline TaPlan gemm_pair_ta_gated_plan(const Layout& L, int M, int num_sms)
+{
+    return gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, 2, false, num_sms, false, gemm_pair_ta_both(L, M, num_sms) ? kTaBothTokens : 256);
+}
+
 inline bool gemm_pair_ta_applicable(const GemmPairLayers& set, int M, int num_sms, bool gated = false)
 {
     if (!gemm_config().ta || !gemm_config().pair) return false;
     for (int i = 0; i < set.n; ++i)
         if (!set.wmap[i] || (set.L[i]->n_rsb % 2)) return false;
-    // The plain form takes every launch.  The gated one where a position is left for every CTA pair in blocks of 256 tokens, and from 3073
-    // channels on with as many blocks as the plan finds (us, shared-memory form or gemm_narrow.cuh / this one: 9216 x 2304 at 300 tokens
-    // 47 / 28, at 512 47 / 33; 14336 x 4096 at 200 72 / 45; 6144 x 1792 at 512 37 / 24).  (Time alone would draw that line lower, 3072 x 4096 at 1500
-    // tokens 68 / 54: there the shared-memory form keeps calls that reach it by rule, in the tests and in smoke().)
-    const int pairs = set.L[0]->n_rsb / 2;
-    return !gated || (M > 128 && (pairs > 12 || pairs * ((M + 255) / 256) >= num_sms / 2));
+    // The plain form takes every launch.  The gated one where a position is left for every CTA pair in blocks of 256 tokens; and from 3073
+    // channels on, with two accumulators, where blocks of up to 160 tokens are dealt out in one round, or the weights are int8 (us, the
+    // faster of shared-memory form and gemm_narrow.cuh / this one: int4 in groups 9216 x 2304 at 300 tokens 43.6 / 28.7, 6144 x 1792 at 400 36.5 / 23.8, 14336 x
+    // 4096 at 160 62.7 / 43.5, in two rounds 9216 x 2304 at 512 47.5 / 50.7; int8 14336 x 4096 at 256 98 / 78, 9216 x 2304 at 400 52 / 49).  (Time alone would
+    // take fewer channels as well: there the shared-memory form keeps calls that reach it by rule, in the tests and in smoke().)
+    if (!gated) return true;
+    const Layout& L = *set.L[0];
+    if (M <= 128 || !gemm_pair_ta_both(L, M, num_sms)) return M > 128;
+    return L.n_rsb / 2 > 12 && (L.bits == 8 || L.n_rsb / 2 * gemm_pair_ta_gated_plan(L, M, num_sms).n_mblk <= num_sms / 2);
 }
 
 inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, int M, cudaStream_t st, int device, bool pdl, int num_sms,
@@ -905,7 +945,12 @@ inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, 
 inline ql_status gemm_pair_ta_forward_gated(const GemmPairLayers& set, const void* x, int M, int act, cudaStream_t st, int device, bool pdl, int num_sms)
 {
     const Layout& L = *set.L[0];
-    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, 2, false, num_sms, false);
+    const TaPlan pl = gemm_pair_ta_gated_plan(L, M, num_sms);
+    if (gemm_pair_ta_both(L, M, num_sms)) {
+        if (L.bits == 8) return gemm_pair_ta_launch<8, false, true, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
+        if (L.grouped) return gemm_pair_ta_launch<4, true, true, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
+        return gemm_pair_ta_launch<4, false, true, false, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
+    }
     if (L.bits == 8) return gemm_pair_ta_launch<8, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);
     if (L.grouped) return gemm_pair_ta_launch<4, true, true>(set, pl, x, M, st, device, pdl, num_sms, act);
     return gemm_pair_ta_launch<4, false, true>(set, pl, x, M, st, device, pdl, num_sms, act);

@@ -873,13 +873,25 @@ double mid_us(const qlinear_s* const* hs, int n, int M, bool gated)      // up t
     return 0.96 + 0.093 * log2_of(cl) + sm_load((double)units * cl, cl, hs[0]->num_sms, 0.772, 0.252, 0.46) * cta;
 }
 
-double pair_ta_us(const Layout& L, int pairs, int M, int layers, bool split, double mb, int num_sms)
+double pair_ta_fewest_us(int bn, int rounds, int steps, int split, double mb)   // plans of the fewest blocks
 {
-    const int steps = (L.K + kGemmKStep - 1) / kGemmKStep;
-    const TaPlan pl = gemm_pair_ta_plan(pairs, M, steps, layers, false, num_sms, split);
-    if (gemm_pair_ta_searches(pairs, M, steps, false)) return gemm_pair_ta_us(pairs, pl.n_mblk, pl.bn, pl.split, steps, layers, false, num_sms) + (layers == 2 ? 0.0 : 0.286 * mb);
-    const double rounds = round_up((double)pairs * pl.n_mblk * pl.split / (num_sms / 2));
-    return 2.66 + 0.0058 * pl.bn + rounds * (layers * ((steps + pl.split - 1) / pl.split) * (0.236 + 0.0003 * pl.bn)) + (pl.split > 1 ? 6.2 + 0.0162 * pl.bn : 0.0) + 0.34 * mb;
+    return 2.66 + 0.0058 * bn + rounds * (((steps + split - 1) / split) * (0.236 + 0.0003 * bn)) + (split > 1 ? 6.2 + 0.0162 * bn : 0.0) + 0.34 * mb;
+}
+
+double pair_ta_us(const Layout& L, int pairs, int M, bool split, double mb, int num_sms)
+{
+    const int steps = (L.K + kGemmKStep - 1) / kGemmKStep, clusters = num_sms / 2;
+    const TaPlan pl = gemm_pair_ta_plan(pairs, M, steps, 1, false, num_sms, split);
+    if (gemm_pair_ta_searches(pairs, M, steps, false)) return gemm_pair_ta_us(pairs, pl.n_mblk, pl.bn, pl.split, steps, 1, false, num_sms) + 0.286 * mb;
+    return pair_ta_fewest_us(pl.bn, (pairs * pl.n_mblk * pl.split + clusters - 1) / clusters, steps, pl.split, mb);
+}
+
+double pair_ta_gated_us(const Layout& L, int M, double mb, int num_sms)
+{
+    const int steps = (L.K + kGemmKStep - 1) / kGemmKStep, pairs = L.n_rsb / 2, n_mblk = (M + 255) / 256, clusters = num_sms / 2;
+    if (!gemm_pair_ta_both(L, M, num_sms)) return pair_ta_fewest_us(((M + n_mblk - 1) / n_mblk + 31) / 32 * 32, (pairs * n_mblk + clusters - 1) / clusters, 2 * steps, 1, mb);
+    const TaPlan pl = gemm_pair_ta_gated_plan(L, M, num_sms);
+    return gemm_pair_ta_us(pairs, pl.n_mblk, pl.bn, 1, steps, 2, false, num_sms);
 }
 
 double single_us(const Layout& L, int M, double mb, int num_sms)
@@ -897,18 +909,18 @@ double prefill_us(ql_kernel kernel, const qlinear_s* const* hs, int n, int M, bo
     const double mb = out_mb(hs, gated ? 1 : n, M);
     if (kernel == QL_KERNEL_SINGLE) return single_us(L, M, mb, sms);
     if (kernel == QL_KERNEL_SEPARATE) {
-        if (gated && L.n_rsb % 2 == 0) return 4.2 + pair_ta_us(L, L.n_rsb, M, 1, false, 2 * mb, sms) + 0.92 * mb;
+        if (gated && L.n_rsb % 2 == 0) return 4.2 + pair_ta_us(L, L.n_rsb, M, false, 2 * mb, sms) + 0.92 * mb;
         double us = gated ? 1.7 + 0.92 * mb : 0.0;
         for (int i = 0; i < n; ++i) {
             const Layout& Li = hs[i]->L;
             const double m = out_mb(hs + i, 1, M);
-            us += Li.n_rsb % 2 ? single_us(Li, M, m, sms) : pair_ta_us(Li, Li.n_rsb / 2, M, 1, true, m, sms);
+            us += Li.n_rsb % 2 ? single_us(Li, M, m, sms) : pair_ta_us(Li, Li.n_rsb / 2, M, true, m, sms);
         }
         return us;
     }
     if (gated && kernel == QL_KERNEL_PAIR)
         return 5.5 + 0.044 * std::min(M, 256) + round_up((double)(L.n_rsb / 2) * ((M + 255) / 256) / (sms / 2)) * 0.84 * steps + 0.3 * mb;
-    return gated ? pair_ta_us(L, L.n_rsb / 2, M, 2, false, mb, sms) : pair_ta_us(L, total_rsb(hs, n) / 2, M, 1, true, mb, sms);
+    return gated ? pair_ta_gated_us(L, M, mb, sms) : pair_ta_us(L, total_rsb(hs, n) / 2, M, true, mb, sms);
 }
 
 ql_kernel prefill_kernel(const qlinear_s* const* hs, int n, int M, bool gated)
@@ -956,7 +968,8 @@ ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
     const ql_kernel other = batch ? QL_KERNEL_MID : prefill_kernel(hs, n, M, gated);
     if (!narrow_can(hs, n, M, gated, batch)) return other;
     if (config().narrow == 2) return QL_KERNEL_NARROW;
-    const double limit = batch ? mid_us(hs, n, M, gated) : prefill_us(other, hs, n, M, gated);
+    // (A gated pair that gemm_pair_ta.cuh serves with one accumulator: 7 % below, as its estimate was made with.)
+    const double limit = batch ? mid_us(hs, n, M, gated) : (gated && other == QL_KERNEL_PAIR_TA && !gemm_pair_ta_both(L, M, hs[0]->num_sms) ? 0.93 : 1.0) * prefill_us(other, hs, n, M, gated);
     return narrow_us(hs, n, M, gated) < limit ? QL_KERNEL_NARROW : other;
 }
 
@@ -1910,7 +1923,7 @@ extern "C" int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_
     if (kernel == QL_KERNEL_NARROW) { width = pl.bn; parts = pl.cl; }
     if (kernel == QL_KERNEL_SINGLE) width = gemm_pick_bn(L, M, num_sms);
     if (kernel == QL_KERNEL_PAIR_TA) {
-        const TaPlan pl = gemm_pair_ta_plan((gated ? L.n_rsb : rows) / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, gated ? 2 : 1, false, num_sms, !gated);
+        const TaPlan pl = gated ? gemm_pair_ta_gated_plan(L, M, num_sms) : gemm_pair_ta_plan(rows / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, 1, false, num_sms, true);
         width = pl.bn;
         parts = pl.split;
     }
