@@ -69,9 +69,14 @@ __device__ __forceinline__ uint32_t pack_s8x4(int b0, int b1, int b2, int b3)
 // Sum of the four signed bytes of a word.
 __device__ __forceinline__ int sum_s8x4(uint32_t w) { return __dp4a((int)w, 0x01010101, 0); }
 
+// What the planner counts on: the CTAs per SM that the registers allow, and a CTA's shared memory beside the dynamic part
+// (static arrays, and the 1 KB that the system keeps per CTA).
+constexpr int kGemvA8MaxResident = 4;
+constexpr int kGemvA8OtherSmem = 5 * 1024 + 1024;
+
 // T: 1, 2, 4 or 8, at least M: the quantisation steps are unrolled over the tokens that exist, not over all 8 columns.
 template <int BITS, bool GROUPED, int T>
-__global__ void __launch_bounds__(kGemvThreads, 4) gemv_a8_kernel(const GemvA8Params p)
+__global__ void __launch_bounds__(kGemvThreads, kGemvA8MaxResident) gemv_a8_kernel(const GemvA8Params p)
 {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -217,6 +217,7 @@ bool hold_range(const qlinear_s* const* hs, int n, cudaStream_t st, int32_t toke
 }
 
 constexpr int kGemvMaxSmem = 96 * 1024;
+constexpr int kSmSharedBytes = 228 * 1024;   // shared memory of one SM
 
 // n_rb: row-blocks of the launch (one layer, or all layers of a group that shares x).
 // gated: the launch needs both branches of a channel in one CTA: an even number of row-blocks per CTA, no cluster.
@@ -261,6 +262,21 @@ GemvPlan plan_gemv(const Layout& L, int n_rb, int M, int num_sms, bool gated = f
             // Larger launches keep their clusters: timed alone they look better without (Llama o, 16.8 MB: 5.9 / 4.6 us),
             // but inside the step the under-filled grid costs the launches around it more than it saves.
             if (cl > 1 && (double)n_rb * L.n_kc * 512.0 < 6.0e6) score -= 0.75;
+            if (a8 && cl > 1) {
+                // Every CTA of the int8-activation kernel reads all of x for the row maxima, so doubling the CTAs gives less
+                // here once every SM has one: a cluster then has to fill the chip almost as well again (0.9 of a doubling).
+                // And its quantised x lies in shared memory, which leaves room for fewer than kGemvA8MaxResident CTAs per SM
+                // when M or the range is large: the CTAs that don't fit run as a second wave, with a whole quantisation
+                // before it.  For three and more CTAs the last 5 % of the slots count as taken: a cluster needs its slots within one GPC.
+                // Seven launches of a block, before -> with both lines: Llama 3.1 8B 844 3 tokens 69.4 -> 62.4 us, 844g32 2 tokens
+                // 64.7 -> 59.9; Gemma 2 2B q8 1 token 39.0 -> 36.8, 6 tokens 72.0 -> 67.3, 844g32 8 tokens 80.0 -> 73.1;
+                // Llama q8 and 844 at 1 and 4 tokens within 1 %, none slower.  Without the condition on one CTA per SM the
+                // Llama cases at 1 to 3 tokens lose 1 to 5 % of it again (k and v, 1024 x 4096, are left with 64 CTAs).
+                const int resident = std::min(kGemvA8MaxResident, kSmSharedBytes / (smem + kGemvA8OtherSmem));
+                const int ctas = ((n_rb + kGemvWarps / ks_cta - 1) / (kGemvWarps / ks_cta)) * cl;
+                if (ctas > (cl > 2 ? 0.95 : 1.0) * num_sms * resident) score -= 2.0;
+                if (ctas > num_sms) score -= 0.9 * std::log2((double)cl);
+            }
             if (cfg.force_ks && !gated) score = (ks == cfg.force_ks) ? 0.0 : -1e29;
             if (score > best_score) {
                 best_score = score;

@@ -86,6 +86,17 @@ def test_a8_decode_rows_at_the_edge_of_what_registers_keep(P, torch, M, K, bits,
     assert_a8(y.cpu().numpy(), x, q, s, group)
 
 
+# the lines of the cluster rule: few CTAs, launches whose CTAs would not fit at once, and one that keeps its clusters
+@pytest.mark.parametrize("M,N,K,bits,group", [(1, 1024, 4096, 8, 0), (2, 4096, 14336, 4, 0), (8, 2304, 9216, 4, 32), (7, 2304, 9216, 8, 0),
+                                              (8, 1024, 4096, 4, 0), (1, 4096, 14336, 8, 0)])
+def test_a8_decode_plans_with_and_without_clusters(P, torch, M, N, K, bits, group):
+    q, s, x = rand_case(7500 + N + K + M, M, N, K, bits, group)
+    lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
+    y = lin.forward_a8(torch.from_numpy(x).cuda())
+    torch.cuda.synchronize()
+    assert_a8(y.cpu().numpy(), x, q, s, group)
+
+
 @pytest.mark.parametrize("M,K", [(1, 96), (1, 1056), (2, 1056), (4, 352), (8, 96), (8, 1056)])
 def test_a8_decode_takes_nothing_from_beyond_the_row(P, torch, M, K):
     """int4 with a last chunk that is half padding: the quantised activations there are zeros, so whatever the padding of the
