@@ -605,11 +605,14 @@ inline ql_status gemm_pair_forward(const GemmPairLayers& set, const void* x, int
     return gemm_pair_launch<4, false, 1>(set, x, M, st, device, pdl, num_sms, scratch, counters);
 }
 
-// Integer form (per-channel schemes, K a multiple of 128): xq int8 [M, K] with per-token scale and row sum.
+// Integer form (per-channel schemes, K a multiple of 128): xq int8 [M, K] with per-token scale and row sum.  What is left to it: QLINEAR_GEMM_TA=0,
+// and layers without the wide weight map.  Launched without the programmatic edge: the quantisation kernel before it releases its dependents at
+// its start, and this kernel's epilogue reads scale and row sum as constant data, which they are only when that kernel is complete.
 inline ql_status gemm_pair_forward_i8(const GemmPairLayers& set, const void* xq, const float* scale, const int32_t* rowsum, int M,
-                                      cudaStream_t st, int device, bool pdl, int num_sms)
+                                      cudaStream_t st, int device, int num_sms)
 {
     const Layout& L = *set.L[0];
+    constexpr bool pdl = false;
     if (L.bits == 8) return gemm_pair_launch<8, false, 1, false, true>(set, xq, M, st, device, pdl, num_sms, nullptr, nullptr, -1, scale, rowsum);
     return gemm_pair_launch<4, false, 1, false, true>(set, xq, M, st, device, pdl, num_sms, nullptr, nullptr, -1, scale, rowsum);
 }

@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(256) quantize_activations_kernel(const __half*
     __shared__ int wsum[8];
     __shared__ float recip;
     // the matmul behind it may set up and request its weights; it reads what is written here, in scratch that the matmul before may still be
-    // reading, past its own wait (its epilogue with loads that pass L1 by)
+    // reading, past its own wait (its epilogue with loads that pass L1 by; the form that reads it as constant data starts when this grid is complete)
     asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
     const int m = blockIdx.x;
     const uint4* row = reinterpret_cast<const uint4*>(x + (int64_t)m * K);

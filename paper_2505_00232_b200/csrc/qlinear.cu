@@ -1410,7 +1410,7 @@ extern "C" ql_status qlinear_forward_a8(qlinear_t h, const void* x, void* y, int
             float* scratch = used + parts <= gemm_pair_scratch_bytes(h->num_sms) ? reinterpret_cast<float*>(base + used) : nullptr;
             return gemm_pair_ta_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms, scratch, h->dev->gemm_counters);
         }
-        return gemm_pair_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms);
+        return gemm_pair_forward_i8(set, xq, sx, rs, M, st, h->device, h->num_sms);
     }
     const GemvPlan pl = plan_gemv(L, h->n_rb, M, h->num_sms, false, true);
     if (pl.grid <= 0) return QL_ERR_UNSUPPORTED;

@@ -230,6 +230,35 @@ def test_a8_prefill_back_to_back_launches_keep_their_bits(P, torch, bits):
     assert lins[0].device_status() == (0, 0)
 
 
+SHARED_MEMORY_FORM = [(129, 256, 128, 8), (300, 512, 1024, 4), (700, 1000, 1152, 8), (520, 4864, 384, 4)]
+SHARED_MEMORY_CHILD = """
+import sys
+sys.path.insert(0, {root!r})
+import torch
+import paper_2505_00232_b200 as P
+from tests.test_a8_gpu import SHARED_MEMORY_FORM, assert_a8, rand_case
+for M, N, K, bits in SHARED_MEMORY_FORM:
+    q, s, x = rand_case(7900 + N + K + M, M, N, K, bits, 0)
+    lin = P.QLinear.from_weights(q, s, bits, 0, device="cuda:0")
+    xs = [torch.from_numpy(x).cuda() * f for f in (1.0, 0.0625, 8.0)] + [torch.from_numpy(x[::-1].copy()).cuda()]
+    ys = [lin.forward_a8(xs[i % 4]) for i in range(40)]
+    assert lin.device_status() == (0, 0)
+    for i in range(4):
+        assert_a8(ys[i].cpu().numpy(), xs[i].cpu().numpy(), q, s, 0)
+    assert all(torch.equal(y, ys[i % 4]) for i, y in enumerate(ys))
+"""
+
+
+def test_a8_prefill_with_the_weights_in_shared_memory(_built_library):
+    """The form that QLINEAR_GEMM_TA=0 leaves: calls in a row whose quantised rows, scales and row sums (one scratch for all) differ
+    from call to call, each against the oracle: none may see those of the call before."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", SHARED_MEMORY_CHILD.format(root=root)], check=True, env=dict(os.environ, QLINEAR_GEMM_TA="0"), cwd=root, timeout=600)
+
+
 def test_a8_zero_input_and_guard_bands(P, torch):
     q, s, x = rand_case(7100, 3, 200, 352, 4, 32)
     lin = P.QLinear.from_weights(q, s, 4, 32, device="cuda:0")
