@@ -525,7 +525,6 @@ class KVCache:
         self.k = QLinear(kd, qlinear_pack(kd, np.zeros((cache_size, d_h), np.int8), np.zeros((cache_size, 1), np.float16)), device)
         self.v = QLinear(vd, qlinear_pack(vd, np.zeros((d_h, cache_size), np.int8), np.ones((d_h, 1), np.float16)), device)
         self.v_scale = torch.zeros((cache_size,), dtype=torch.float16, device=device)
-        self._v_scale_ptr = self.v_scale.data_ptr()
 
     def append(self, k_new, v_new, stream=None):
         """k_new, v_new: fp16 CUDA [n_new, d_h], written to positions length .. length + n_new - 1."""
@@ -554,7 +553,7 @@ class KVCache:
 
     def output(self, prob, stream=None):
         """prob fp16 [R, cache_size] -> fp16 [R, d_h]."""
-        y = _native.kv_output(self.v._native, self._v_scale_ptr, prob, _raw(stream))
+        y = _native.kv_output(self.v._native, self.v_scale.data_ptr(), prob, _raw(stream))
         if y is not None:
             return y
         if not _is_x(prob, self.cache_size):

@@ -32,6 +32,42 @@ def test_anything_but_plain_cuda_tensors_is_left_to_python(P):
         P.qlinear_residual_rmsnorm(x, None, x[0], 1e-5)
 
 
+def test_value_product_is_given_the_scales_that_the_cache_has_now(P, monkeypatch):
+    """`v_scale` may be replaced (a restored cache): the address is asked for at every call."""
+    import torch
+    seen = []
+
+    class Native:
+        def kv_output(self, *a):
+            seen.append(a)
+            return a[2]
+    monkeypatch.setattr(P.binding, "_native", Native())
+    kv, prob, kept = P.KVCache.__new__(P.KVCache), torch.zeros((1, 64), dtype=torch.float16), []
+    kv.v = type("V", (), {"_native": (1, 64, 32), "_h": None})()
+    for _ in range(3):
+        kv.v_scale = torch.ones((64,), dtype=torch.float16)
+        kept.append(kv.v_scale)
+        assert kv.output(prob) is prob and seen[-1][1] == kv.v_scale.data_ptr()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("R", [4, 64])
+def test_value_product_after_the_scales_were_replaced(P, R):
+    import torch
+    f16 = lambda *s: torch.randn(s, device="cuda").half()
+    d, T, k, prob = 64, 256, f16(5, 64), f16(R, 256)
+    kv, fresh = P.KVCache(T, d, "cuda:0"), P.KVCache(T, d, "cuda:0")
+    prob[:, 10:] = 0
+    old = kv.v_scale
+    for v in (f16(5, d), 30 * f16(5, d)):
+        kv.append(k, v)
+        fresh.append(k, v)
+        kv.output(prob)
+        kv.v_scale = kv.v_scale.clone()                                  # (the append writes to the new one from here on)
+    old.fill_(float("nan"))
+    assert torch.equal(kv.output(prob), fresh.output(prob))
+
+
 @pytest.mark.gpu
 def test_both_halves_agree(P, monkeypatch):
     import torch
