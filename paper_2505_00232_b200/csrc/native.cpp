@@ -64,14 +64,20 @@ at::Tensor half_like(const at::Tensor& x, at::IntArrayRef size) { return at::det
 // None: the current stream of the current device; otherwise a raw stream handle.
 void* stream_of(PyObject* o) { return o == Py_None ? static_cast<void*>(c10::cuda::getCurrentCUDAStream(c10::cuda::current_device()).stream()) : PyLong_AsVoidPtr(o); }
 
-// Runs `call` without the interpreter lock; false with the binding's exception set if its status is not QL_OK.
+// Runs `call`, which allocates its outputs (that may go to the driver) and calls the library, without the interpreter lock; false with the
+// binding's exception set if its status is not QL_OK.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }                         // (past a C++ exception as well)
+};
 template <typename F>
 bool done(F call, const char* where)
 {
     ql_status s;
-    Py_BEGIN_ALLOW_THREADS
-    s = call();
-    Py_END_ALLOW_THREADS
+    {
+        Unlocked unlocked;
+        s = call();
+    }
     if (s == QL_OK) return true;
     PyObject* r = PyObject_CallFunction(check_status, "is", (int)s, where);
     if (r) { Py_DECREF(r); PyErr_SetString(PyExc_RuntimeError, where); }  // (the check raises)
@@ -106,13 +112,16 @@ PyObject* one_layer(Fn fn, const char* where, PyObject* const* a)        // (lay
     const at::Tensor* x = plain(a[1], at::kHalf);
     if (!layer_of(a[0], &l) || !x || x->dim() != 2 || x->size(1) != l.K || x->size(0) > INT_MAX) Py_RETURN_NONE;
     const int64_t M = x->size(0);
+    const bool make = a[2] == Py_None;
     at::Tensor made;
-    const at::Tensor* out = &made;
-    if (a[2] == Py_None) made = half_like(*x, {M, l.N});
-    else if (!is_matrix(out = plain(a[2], at::kHalf), M, l.N)) Py_RETURN_NONE;
-    void *xp = x->data_ptr(), *yp = out->data_ptr(), *st = stream_of(a[3]);
-    if (!done([&] { return fn(l.h, xp, yp, (int32_t)M, st); }, where)) return nullptr;
-    return a[2] == Py_None ? THPVariable_Wrap(std::move(made)) : Py_NewRef(a[2]);
+    const at::Tensor* out = make ? &made : plain(a[2], at::kHalf);
+    if (!make && !is_matrix(out, M, l.N)) Py_RETURN_NONE;
+    void *xp = x->data_ptr(), *st = stream_of(a[3]);
+    if (!done([&] {
+            if (make) made = half_like(*x, {M, l.N});
+            return fn(l.h, xp, out->data_ptr(), (int32_t)M, st);
+        }, where)) return nullptr;
+    return make ? THPVariable_Wrap(std::move(made)) : Py_NewRef(a[2]);
 }
 PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t) { return guarded([&] { return one_layer(api.forward, "qlinear_forward", a); }); }
 PyObject* kv_scores_one(PyObject*, PyObject* const* a, Py_ssize_t) { return guarded([&] { return one_layer(api.forward, "qlinear_kv_scores", a); }); }
@@ -140,9 +149,11 @@ PyObject* forward_group(PyObject*, PyObject* const* a, Py_ssize_t)       // (lis
         }
         const int64_t M = x->size(0);
         at::Tensor outs[kMost];
-        for (Py_ssize_t i = 0; i < n; ++i) { outs[i] = half_like(*x, {M, N[i]}); ys[i] = outs[i].data_ptr(); }
         void *xp = x->data_ptr(), *st = stream_of(a[2]);
-        if (!done([&] { return api.forward_group(hs, (int32_t)n, xp, ys, (int32_t)M, st); }, "qlinear_forward_group")) return nullptr;
+        if (!done([&] {
+                for (Py_ssize_t i = 0; i < n; ++i) { outs[i] = half_like(*x, {M, N[i]}); ys[i] = outs[i].data_ptr(); }
+                return api.forward_group(hs, (int32_t)n, xp, ys, (int32_t)M, st);
+            }, "qlinear_forward_group")) return nullptr;
         PyObject* r = PyList_New(n);
         for (Py_ssize_t i = 0; r && i < n; ++i) PyList_SET_ITEM(r, i, THPVariable_Wrap(std::move(outs[i])));
         return r;
@@ -157,13 +168,16 @@ PyObject* forward_gated(PyObject*, PyObject* const* a, Py_ssize_t)       // (gat
         if (!layer_of(a[0], &g) || !layer_of(a[1], &u) || !x || x->dim() != 2 || x->size(1) != g.K || x->size(0) > INT_MAX) Py_RETURN_NONE;
         const int64_t M = x->size(0);
         const int act = (int)PyLong_AsLong(a[3]);
+        const bool make = a[4] == Py_None;
         at::Tensor made;
-        const at::Tensor* out = &made;
-        if (a[4] == Py_None) made = half_like(*x, {M, g.N});
-        else if (!is_matrix(out = plain(a[4], at::kHalf), M, g.N)) Py_RETURN_NONE;
-        void *xp = x->data_ptr(), *yp = out->data_ptr(), *st = stream_of(a[5]);
-        if (!done([&] { return api.forward_gated(g.h, u.h, xp, yp, (int32_t)M, act, st); }, "qlinear_forward_gated")) return nullptr;
-        return a[4] == Py_None ? THPVariable_Wrap(std::move(made)) : Py_NewRef(a[4]);
+        const at::Tensor* out = make ? &made : plain(a[4], at::kHalf);
+        if (!make && !is_matrix(out, M, g.N)) Py_RETURN_NONE;
+        void *xp = x->data_ptr(), *st = stream_of(a[5]);
+        if (!done([&] {
+                if (make) made = half_like(*x, {M, g.N});
+                return api.forward_gated(g.h, u.h, xp, out->data_ptr(), (int32_t)M, act, st);
+            }, "qlinear_forward_gated")) return nullptr;
+        return make ? THPVariable_Wrap(std::move(made)) : Py_NewRef(a[4]);
     });
 }
 
@@ -182,13 +196,16 @@ PyObject* residual_rmsnorm(PyObject*, PyObject* const* a, Py_ssize_t)    // (x, 
         const at::Tensor *h = nullptr, *y = &made_y;
         if (a[5] != Py_None) { if (!is_matrix(h = plain(a[5], at::kHalf), M, K) || !same(h)) Py_RETURN_NONE; }
         if (a[6] != Py_None) { if (!is_matrix(y = plain(a[6], at::kHalf), M, K) || !same(y)) Py_RETURN_NONE; }
-        else made_y = half_like(*x, {M, K});
         const int want_h = a[5] == Py_None ? PyObject_IsTrue(a[7]) : 0;
         if (want_h < 0) return nullptr;
-        if (want_h) { made_h = half_like(*x, {M, K}); h = &made_h; }
-        void *xp = x->data_ptr(), *rp = r ? r->data_ptr() : nullptr, *gp = g->data_ptr(), *hp = h ? h->data_ptr() : nullptr, *yp = y->data_ptr(), *st = stream_of(a[8]);
+        if (want_h) h = &made_h;
+        void *xp = x->data_ptr(), *rp = r ? r->data_ptr() : nullptr, *gp = g->data_ptr(), *st = stream_of(a[8]);
         const int dev = x->get_device();
-        if (!done([&] { return api.residual_rmsnorm(xp, rp, gp, (float)eps, (float)offset, hp, yp, (int32_t)M, (int32_t)K, dev, st); }, "qlinear_residual_rmsnorm")) return nullptr;
+        if (!done([&] {
+                if (y == &made_y) made_y = half_like(*x, {M, K});
+                if (want_h) made_h = half_like(*x, {M, K});
+                return api.residual_rmsnorm(xp, rp, gp, (float)eps, (float)offset, h ? h->data_ptr() : nullptr, y->data_ptr(), (int32_t)M, (int32_t)K, dev, st);
+            }, "qlinear_residual_rmsnorm")) return nullptr;
         PyObject* pair = PyTuple_New(2);
         if (!pair) return nullptr;
         PyTuple_SET_ITEM(pair, 0, want_h ? THPVariable_Wrap(std::move(made_h)) : Py_NewRef(a[5]));
@@ -213,13 +230,16 @@ PyObject* rope_qkv(PyObject*, PyObject* const* a, Py_ssize_t)            // (q, 
         const auto same = [&](const at::Tensor* t) { return t->get_device() == q->get_device(); };
         if (hq % hkv || d % 16 || T > INT_MAX || hq * d > INT_MAX || !is_matrix(q, T, hq * d) || !is_matrix(k, T, hkv * d) || !is_matrix(v, T, hkv * d) || pos->dim() != 1 || pos->size(0) != T ||
             cos->dim() != 2 || cos->size(0) > INT_MAX || cos->size(1) != d / 2 || !is_matrix(sin, cos->size(0), d / 2) || !same(k) || !same(v) || !same(pos) || !same(cos) || !same(sin)) Py_RETURN_NONE;
-        at::Tensor qo = half_like(*q, {B * hkv, S * (hq / hkv), d}), ko = half_like(*q, {B * hkv, S, d}), vo = half_like(*q, {B * hkv, S, d});
+        at::Tensor qo, ko, vo;
         const void* in[6] = {q->data_ptr(), k->data_ptr(), v->data_ptr(), pos->data_ptr(), cos->data_ptr(), sin->data_ptr()};
-        void *qp = qo.data_ptr(), *kp = ko.data_ptr(), *vp = vo.data_ptr(), *st = stream_of(a[11]);
+        void* st = stream_of(a[11]);
         const int dev = q->get_device();
         const int32_t n_pos = (int32_t)cos->size(0);
-        if (!done([&] { return api.rope_qkv(in[0], in[1], in[2], static_cast<const int32_t*>(in[3]), static_cast<const float*>(in[4]), static_cast<const float*>(in[5]), n_pos, qp, kp, vp,
-                                            (int32_t)B, (int32_t)S, (int32_t)hq, (int32_t)hkv, (int32_t)d, dev, st); }, "qlinear_rope_qkv")) return nullptr;
+        if (!done([&] {
+                qo = half_like(*q, {B * hkv, S * (hq / hkv), d}); ko = half_like(*q, {B * hkv, S, d}); vo = half_like(*q, {B * hkv, S, d});
+                return api.rope_qkv(in[0], in[1], in[2], static_cast<const int32_t*>(in[3]), static_cast<const float*>(in[4]), static_cast<const float*>(in[5]), n_pos,
+                                    qo.data_ptr(), ko.data_ptr(), vo.data_ptr(), (int32_t)B, (int32_t)S, (int32_t)hq, (int32_t)hkv, (int32_t)d, dev, st);
+            }, "qlinear_rope_qkv")) return nullptr;
         PyObject* r = PyTuple_New(3);
         if (!r) return nullptr;
         PyTuple_SET_ITEM(r, 0, THPVariable_Wrap(std::move(qo)));
@@ -236,10 +256,13 @@ PyObject* embed(PyObject*, PyObject* const* a, Py_ssize_t)               // (lay
         const at::Tensor* ids = plain(a[1], at::kInt);
         if (!layer_of(a[0], &l) || !ids || ids->dim() != 1 || ids->size(0) > INT_MAX || a[2] != Py_None) Py_RETURN_NONE;
         const int64_t n = ids->size(0);
-        at::Tensor out = half_like(*ids, {n, l.K});
+        at::Tensor out;
         const auto* ip = static_cast<const int32_t*>(ids->data_ptr());
-        void *yp = out.data_ptr(), *st = stream_of(a[3]);
-        if (!done([&] { return api.embed(l.h, ip, (int32_t)n, yp, st); }, "qlinear_embed")) return nullptr;
+        void* st = stream_of(a[3]);
+        if (!done([&] {
+                out = half_like(*ids, {n, l.K});
+                return api.embed(l.h, ip, (int32_t)n, out.data_ptr(), st);
+            }, "qlinear_embed")) return nullptr;
         return THPVariable_Wrap(std::move(out));
     });
 }
@@ -280,9 +303,12 @@ PyObject* kv_scores(PyObject*, PyObject* const* a, Py_ssize_t)           // (hea
         const at::Tensor* q = plain(a[1], at::kHalf);
         if (!heads_of(a[0], &h) || !is_of_heads(q, h, h.d)) Py_RETURN_NONE;
         const int64_t R = q->size(1);
-        at::Tensor out = half_like(*q, {h.n, R, h.T});
-        void *qp = q->data_ptr(), *yp = out.data_ptr(), *st = stream_of(a[2]);
-        if (!done([&] { return api.kv_scores_heads(h.hk, h.n, qp, yp, (int32_t)R, st); }, "qlinear_kv_scores_heads")) return nullptr;
+        at::Tensor out;
+        void *qp = q->data_ptr(), *st = stream_of(a[2]);
+        if (!done([&] {
+                out = half_like(*q, {h.n, R, h.T});
+                return api.kv_scores_heads(h.hk, h.n, qp, out.data_ptr(), (int32_t)R, st);
+            }, "qlinear_kv_scores_heads")) return nullptr;
         return THPVariable_Wrap(std::move(out));
     });
 }
@@ -294,10 +320,13 @@ PyObject* kv_output_heads(PyObject*, PyObject* const* a, Py_ssize_t)     // (hea
         const at::Tensor* p = plain(a[1], at::kHalf);
         if (!heads_of(a[0], &h) || !is_of_heads(p, h, h.T)) Py_RETURN_NONE;
         const int64_t R = p->size(1);
-        at::Tensor out = half_like(*p, {h.n, R, h.d});
-        void *pp = p->data_ptr(), *yp = out.data_ptr(), *st = stream_of(a[2]);
+        at::Tensor out;
+        void *pp = p->data_ptr(), *st = stream_of(a[2]);
         const auto* vs = reinterpret_cast<const void* const*>(h.vs);
-        if (!done([&] { return api.kv_output_heads(h.hv, h.n, pp, vs, yp, (int32_t)R, st); }, "qlinear_kv_output_heads")) return nullptr;
+        if (!done([&] {
+                out = half_like(*p, {h.n, R, h.d});
+                return api.kv_output_heads(h.hv, h.n, pp, vs, out.data_ptr(), (int32_t)R, st);
+            }, "qlinear_kv_output_heads")) return nullptr;
         return THPVariable_Wrap(std::move(out));
     });
 }
@@ -309,10 +338,14 @@ PyObject* kv_output(PyObject*, PyObject* const* a, Py_ssize_t)           // (V l
         const at::Tensor* p = plain(a[2], at::kHalf);
         if (!layer_of(a[0], &l) || !p || p->dim() != 2 || p->size(1) != l.K || p->size(0) > INT_MAX) Py_RETURN_NONE;
         const int64_t R = p->size(0);
-        at::Tensor out = half_like(*p, {R, l.N}), tmp;
-        void *vs = PyLong_AsVoidPtr(a[1]), *pp = p->data_ptr(), *yp = out.data_ptr(), *tp = yp, *st = stream_of(a[3]);
-        if (R < 1 || api.kv_output_uses_tmp(l.h, pp, vs, (int32_t)R)) { tmp = half_like(*p, p->sizes()); tp = tmp.data_ptr(); }
-        if (!done([&] { return api.kv_output(l.h, pp, vs, tp, yp, (int32_t)R, st); }, "qlinear_kv_output")) return nullptr;
+        at::Tensor out, tmp;
+        void *vs = PyLong_AsVoidPtr(a[1]), *pp = p->data_ptr(), *st = stream_of(a[3]);
+        const bool uses_tmp = R < 1 || api.kv_output_uses_tmp(l.h, pp, vs, (int32_t)R);
+        if (!done([&] {
+                out = half_like(*p, {R, l.N});
+                if (uses_tmp) tmp = half_like(*p, {R, l.K});
+                return api.kv_output(l.h, pp, vs, (uses_tmp ? tmp : out).data_ptr(), out.data_ptr(), (int32_t)R, st);
+            }, "qlinear_kv_output")) return nullptr;
         return THPVariable_Wrap(std::move(out));
     });
 }

@@ -68,6 +68,63 @@ def test_value_product_after_the_scales_were_replaced(P, R):
     assert torch.equal(kv.output(prob), fresh.output(prob))
 
 
+ALLOCATOR = """
+#include <cuda_runtime.h>
+#include <sys/types.h>
+extern "C" {
+int PyGILState_Check(void);
+int calls = 0, locked = 0;
+void* take(ssize_t size, int, cudaStream_t) { void* p = nullptr; ++calls; locked += PyGILState_Check(); return cudaMalloc(&p, size ? size : 1) == cudaSuccess ? p : nullptr; }
+void give(void* p, ssize_t, int, cudaStream_t) { cudaFree(p); }
+}
+"""
+LOCK_CHILD = """
+import ctypes, sys
+sys.path.insert(0, {root!r})
+import torch
+torch.cuda.memory.change_current_allocator(torch.cuda.memory.CUDAPluggableAllocator({lib!r}, "take", "give"))
+import paper_2505_00232_b200 as P
+from tests.test_native_binding import tensor_calls
+count = [ctypes.c_int.in_dll(ctypes.CDLL({lib!r}), n) for n in ("calls", "locked")]
+for name, call in tensor_calls(P).items():
+    before = [c.value for c in count]
+    kept = call()
+    after = [c.value for c in count]
+    assert after[0] > before[0] and after[1] == before[1], (name, before, after)
+torch.cuda.synchronize()
+"""
+
+
+def tensor_calls(P):
+    """One call of every kind that allocates its outputs."""
+    import torch
+    rng = np.random.default_rng(1)
+    f16 = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float16)).cuda()
+    mk = lambda N, K, bits, group: P.QLinear.from_weights(*C.layer_weights(5, C.LayerSpec("t", N, K, bits, group, *((-8, 7) if bits == 4 else (-128, 127)))), bits, group, device="cuda:0")
+    a, b, table, kv, wide = mk(256, 512, 8, 0), mk(256, 512, 8, 0), mk(1000, 128, 4, 32), P.KVHeads(2, 1280, 64), P.KVCache(4096, 1024)
+    kv.append(f16(2, 9, 64), f16(2, 9, 64))
+    x, g, ids, pos, ang = f16(5, 512), f16(512), torch.tensor([3, 999], device="cuda", dtype=torch.int32), torch.arange(6, device="cuda", dtype=torch.int32), torch.rand((16, 32), device="cuda")
+    q, k, v, rows, prob, many = f16(6, 256), f16(6, 128), f16(6, 128), f16(2, 4, 64), f16(2, 4, 1280), f16(1024, 4096)
+    return {"forward": lambda: a.forward(x), "forward_a8": lambda: a.forward_a8(x), "forward_group": lambda: P.qlinear_forward_group([a, b], x),
+            "forward_gated": lambda: P.qlinear_forward_gated(a, b, x), "residual_rmsnorm": lambda: P.qlinear_residual_rmsnorm(x, x, g, 1e-5),
+            "rope_qkv": lambda: P.qlinear_rope_qkv(q, k, v, pos, ang, ang, 1, 6, 4, 2, 64), "embed": lambda: table.embed(ids), "kv_scores": lambda: kv.scores(rows),
+            "kv_scores_one": lambda: kv.heads[1].scores(rows[1]), "kv_output_heads": lambda: kv.output(prob), "kv_output": lambda: kv.heads[0].output(prob[0]),
+            "kv_output, rows scaled by a pass of their own": lambda: wide.output(many)}
+
+
+@pytest.mark.gpu
+def test_outputs_are_allocated_without_the_interpreter_lock(P, tmp_path):
+    """An allocation may have to go to the driver; other Python threads run meanwhile."""
+    import os
+    import subprocess
+    import sys
+    root, src, lib = os.path.dirname(os.path.dirname(os.path.abspath(__file__))), tmp_path / "alloc.cpp", str(tmp_path / "alloc.so")
+    src.write_text(ALLOCATOR)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-shared", "-fPIC", f"-I{cuda}/include", str(src), "-o", lib, f"-L{cuda}/lib64", "-lcudart"], check=True)
+    subprocess.run([sys.executable, "-c", LOCK_CHILD.format(root=root, lib=lib)], check=True, cwd=root, timeout=600)
+
+
 @pytest.mark.gpu
 def test_both_halves_agree(P, monkeypatch):
     import torch
