@@ -8,6 +8,7 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
+#include <ATen/PythonTorchFunctionTLS.h>
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/cuda/CUDAFunctions.h>
@@ -39,12 +40,13 @@ PyObject* check_status = nullptr;                                        // bind
 
 using c10::DispatchKey;
 
-// Tracing, functionalisation and the function transforms see every operator, allocations among them: such calls are Python's.
+// Tracing, modes of both kinds, functionalisation and the function transforms see every operator, allocations among them: such calls are Python's.
 bool modes_are_on()
 {
     const auto on = c10::impl::tls_local_dispatch_key_set().included_;
     return on.has_any(c10::DispatchKeySet({DispatchKey::Python, DispatchKey::PythonTLSSnapshot, DispatchKey::FuncTorchDynamicLayerFrontMode, DispatchKey::FuncTorchDynamicLayerBackMode,
-                                           DispatchKey::FuncTorchVmapMode, DispatchKey::Functionalize}));
+                                           DispatchKey::FuncTorchVmapMode, DispatchKey::Functionalize, DispatchKey::Tracer})) ||
+           at::impl::PythonTorchFunctionTLS::stack_len() > 0;
 }
 
 // The tensor of a Python object, if it is a dense contiguous CUDA tensor of the type and no subclass or wrapper of one.

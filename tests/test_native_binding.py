@@ -125,6 +125,65 @@ def test_outputs_are_allocated_without_the_interpreter_lock(P, tmp_path):
     subprocess.run([sys.executable, "-c", LOCK_CHILD.format(root=root, lib=lib)], check=True, cwd=root, timeout=600)
 
 
+def _modes(torch, fn):
+    """Calls of fn(x) that an operator-level observer would see, by name."""
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    from torch.overrides import TorchFunctionMode
+    from torch.utils._python_dispatch import TorchDispatchMode
+
+    class Dispatch(TorchDispatchMode):
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            seen.append(str(func))
+            return func(*args, **(kwargs or {}))
+
+    class Function(TorchFunctionMode):
+        def __torch_function__(self, func, types, args=(), kwargs=None):
+            seen.append(getattr(func, "__name__", str(func)))
+            return func(*args, **(kwargs or {}))
+
+    def under(mode):
+        def call(x):
+            with mode():
+                return fn(x)
+        return call
+    seen = []
+    return seen, {"dispatch mode": under(Dispatch), "function mode": under(Function), "fake tensors": under(lambda: FakeTensorMode(allow_non_fake_inputs=True)), "vmap": lambda x: torch.vmap(lambda r: fn(r[None])[0])(x),
+                  "jvp": lambda x: torch.func.jvp(fn, (x,), (x,)), "vjp": lambda x: torch.func.vjp(fn, x)[0], "functionalize": lambda x: torch.func.functionalize(fn)(x),
+                  "trace": lambda x: torch.jit.trace(fn, (x,), check_trace=False).inlined_graph.findNode("aten::new_empty") is not None}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", ["dispatch mode", "function mode", "fake tensors", "vmap", "jvp", "vjp", "functionalize", "trace"])
+def test_calls_that_something_observes_are_left_to_python(P, monkeypatch, mode):
+    """Modes, transforms and tracing see the allocations of the Python half (or its error): the native half takes none of these calls."""
+    import torch
+    lin = P.QLinear.from_weights(*C.layer_weights(5, C.LayerSpec("t", 64, 512, 8, 0, -128, 127)), 8, 0, device="cuda:0")
+    x, native, answers = torch.ones((3, 512), device="cuda").half(), P.binding._bind_torch(), []
+
+    class Recorded:
+        def __getattr__(self, name):
+            def call(*a):
+                answers.append(getattr(native, name)(*a) if real else None)
+                return answers[-1]
+            return call
+    monkeypatch.setattr(P.binding, "_native", Recorded())
+
+    def outcome():
+        seen, calls = _modes(torch, lin.forward)
+        try:
+            y = calls[mode](x)
+        except Exception as e:
+            return type(e), str(e), seen
+        return [t.shape if isinstance(t, torch.Tensor) else t for t in (y if isinstance(y, tuple) else (y,))], seen
+    real = True
+    lin.forward(x)
+    assert answers.pop() is not None                                     # (the same call without an observer)
+    with_native = outcome()
+    assert answers and all(a is None for a in answers)
+    real = False
+    assert outcome() == with_native
+
+
 @pytest.mark.gpu
 def test_both_halves_agree(P, monkeypatch):
     import torch
