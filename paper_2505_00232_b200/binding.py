@@ -194,7 +194,9 @@ def _bind_torch():
     global _half, _raw_stream, _device, _native
     import torch
     if _native is None:
-        from . import _native as native                                  # (no fallback: the build makes it beside libqlinear.so)
+        from . import _native as native, build                           # (no fallback: the build makes it beside libqlinear.so)
+        if native.built_for != build.installed_torch()[1]:
+            raise ImportError(f"_native.so was built for {native.built_for}, not for {build.installed_torch()[1]}: run paper_2505_00232_b200/build.py")
         native.init(_check, *(ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in _NATIVE_API))
         _native = native
     # (a torch without CUDA has neither entry point: its own error comes from the calls that need a device)

@@ -23,19 +23,45 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(os.path.join(CSRC, d)) > t for d in deps)
 
 
-def build_native(force: bool = False) -> str:
-    """The extension module of the binding, against the installed torch (which has loaded these libraries when the module is imported)."""
+def installed_torch():
+    """(folder, what a module built against it is built for) of the installed torch, which is not imported for that; None if there is none."""
+    spec = importlib.util.find_spec("torch")
+    if spec is None:
+        return None
+    folder = spec.submodule_search_locations[0]
+    spec = importlib.util.spec_from_file_location("_torch_version", os.path.join(folder, "version.py"))
+    version = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(version)
+    return folder, f"torch {version.__version__} {version.git_version} cuda {version.cuda} python {sysconfig.get_config_var('SOABI')}"
+
+
+def build_native(force: bool = False):
+    """The extension module of the binding, against the installed torch (which has loaded these libraries when the module is imported).  It uses
+    C++ interfaces of torch and Python that change with their versions, so it holds their names and is built again when they differ.
+    Without torch there is nothing to build it against, and nothing that would load it: packing and the C library need neither."""
+    torch = installed_torch()
+    if torch is None:
+        return None
+    folder, built_for = torch
     if not (force or _stale(NATIVE, ["native.cpp", HEADER])):
-        return NATIVE
-    torch = importlib.util.find_spec("torch").submodule_search_locations[0]
-    include = [os.path.join(torch, "include"), os.path.join(torch, "include", "torch", "csrc", "api", "include"), os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), sysconfig.get_paths()["include"]]
-    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", *("-I" + i for i in include), os.path.join(CSRC, "native.cpp"),
-                           "-L" + os.path.join(torch, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-o", NATIVE])
+        with open(NATIVE, "rb") as f:
+            if built_for.encode() + b"\0" in f.read():
+                return NATIVE
+    abi = subprocess.check_output([sys.executable, "-c", "import torch; print(int(torch.compiled_with_cxx11_abi()))"], text=True).strip()
+    include = [os.path.join(folder, "include"), os.path.join(folder, "include", "torch", "csrc", "api", "include"), os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), sysconfig.get_paths()["include"]]
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-D_GLIBCXX_USE_CXX11_ABI=" + abi, f'-DQL_BUILT_FOR="{built_for}"',
+                           *("-I" + i for i in include), os.path.join(CSRC, "native.cpp"),
+                           "-L" + os.path.join(folder, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-o", NATIVE])
     return NATIVE
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_library(force, verbose)
     build_native(force)
+    return LIB
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     if not (force or _stale(LIB, DEPS)):
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
