@@ -780,11 +780,14 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
 // quantisation before it): `layers` tiles (gated: 2) of n_ksteps steps in each of pairs * n_mblk positions of bn tokens, K in `split` parts.  A launch on
 // at most half of the CTA pairs leaves the others to the next one's start.  Fitted to 240 (integer form: 240) combinations of layer and
 // tokens (256 x 1024 to 14336 x 4096, 129 to 1400 tokens) with up to 15 plans each.
-inline double gemm_pair_ta_us(int pairs, int n_mblk, int bn, int split, int n_ksteps, int layers, bool i8, int num_sms)
+// A gated pair with one accumulator (layers == 2, not both): fitted to 385 random pairs of 129 to 2048 tokens with up to 6 widths each; of the
+// widths that run, measured / estimate 0.94 and 1.12 (5th and 95th percentile; 0.92 and 1.20 at the ends).
+inline double gemm_pair_ta_us(int pairs, int n_mblk, int bn, int split, int n_ksteps, int layers, bool both, bool i8, int num_sms)
 {
     const int units = pairs * n_mblk * split, clusters = num_sms / 2, rounds = (units + clusters - 1) / clusters, steps = (n_ksteps + split - 1) / split;
     const double more = units * 2 > clusters ? 1.0 : 0.0;
     if (i8) return 5.94 + 0.00896 * bn + rounds * steps * (0.2494 + 0.00006 * bn) + (split == 4 ? 2.09 + 0.0273 * bn : split == 2 ? 1.58 + 0.0116 * bn : 0.0) + 0.8 * more + 1.83 * (rounds - 1);
+    if (layers == 2 && !both) return 6.31 + 0.0021 * bn + (rounds - 1) * (2.63 - 0.0063 * bn) + rounds * 2 * steps * (0.1846 + 0.00042 * bn);
     if (layers == 2) return 5.48 + rounds * (0.0206 * bn - 1.35 + steps * (0.4395 + 0.00083 * bn));   // (the store included)
     return 3.01 + 0.0003 * bn + rounds * steps * (0.1966 + 0.00038 * bn) + (split == 4 ? 2.77 + 0.023 * bn : split == 2 ? 2.13 + 0.013 * bn : 0.0) + 1.22 * more - 0.51 * (rounds - 1);
 }
@@ -799,20 +802,20 @@ inline double gemm_pair_ta_us(int pairs, int n_mblk, int bn, int split, int n_ks
 // blocks here: gemm_route compares the two, and what is left of them has large K parts.
 struct TaPlan { int n_mblk, bn, split; };
 inline bool gemm_pair_ta_searches(int pairs, int M, int n_ksteps, bool i8) { return i8 || (M > 128 && pairs > 2 && n_ksteps > 16); }
-inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int layers, bool i8, int num_sms, bool may_split, int widest = 256)
+inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int layers, bool i8, int num_sms, bool may_split, bool both = false)
 {
     const int clusters = num_sms / 2;
     const int forced = gemm_config().force_split >= 4 ? 4 : gemm_config().force_split >= 2 ? 2 : gemm_config().force_split;
     const bool search = gemm_pair_ta_searches(pairs, M, n_ksteps, i8);
     TaPlan best{};
     double best_us = 1e30;
-    for (int bn = widest; bn >= 32; bn -= 32) {
+    for (int bn = both ? kTaBothTokens : 256; bn >= 32; bn -= 32) {
         const int n_mblk = (M + bn - 1) / bn, tiles = pairs * n_mblk;
         if (((M + n_mblk - 1) / n_mblk + 31) / 32 * 32 != bn) continue;  // (as many blocks, and narrower: comes later)
         for (int split = 1; split <= 4; split *= 2) {
             // one unit per CTA pair, which bounds the scratch
             if (split > 1 && (!may_split || tiles * split > clusters || n_ksteps / split < (search ? 2 : 8))) break;
-            double us = search ? gemm_pair_ta_us(pairs, n_mblk, bn, split, n_ksteps, layers, i8, num_sms) : 1.0 / split;
+            double us = search ? gemm_pair_ta_us(pairs, n_mblk, bn, split, n_ksteps, layers, both, i8, num_sms) : 1.0 / split;
             if (forced && split != forced) us += 1e6 / split;            // (the parts asked for, or the most that the launch can have)
             if (us < best_us) { best_us = us; best = TaPlan{n_mblk, bn, split}; }
         }
@@ -901,7 +904,7 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const TaPlan& pl, const
 inline bool gemm_pair_ta_both(const Layout& L, int M, int num_sms) { return L.n_rsb / 2 * ((M + 255) / 256) < num_sms / 2; }
 inline TaPlan gemm_pair_ta_gated_plan(const Layout& L, int M, int num_sms)
 {
-    return gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, 2, false, num_sms, false, gemm_pair_ta_both(L, M, num_sms) ? kTaBothTokens : 256);
+    return gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + kGemmKStep - 1) / kGemmKStep, 2, false, num_sms, false, gemm_pair_ta_both(L, M, num_sms));
 }
 
 inline bool gemm_pair_ta_applicable(const GemmPairLayers& set, int M, int num_sms, bool gated = false)

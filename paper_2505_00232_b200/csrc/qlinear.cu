@@ -898,16 +898,15 @@ double pair_ta_us(const Layout& L, int pairs, int M, bool split, double mb, int 
 {
     const int steps = (L.K + kGemmKStep - 1) / kGemmKStep, clusters = num_sms / 2;
     const TaPlan pl = gemm_pair_ta_plan(pairs, M, steps, 1, false, num_sms, split);
-    if (gemm_pair_ta_searches(pairs, M, steps, false)) return gemm_pair_ta_us(pairs, pl.n_mblk, pl.bn, pl.split, steps, 1, false, num_sms) + 0.286 * mb;
+    if (gemm_pair_ta_searches(pairs, M, steps, false)) return gemm_pair_ta_us(pairs, pl.n_mblk, pl.bn, pl.split, steps, 1, false, false, num_sms) + 0.286 * mb;
     return pair_ta_fewest_us(pl.bn, (pairs * pl.n_mblk * pl.split + clusters - 1) / clusters, steps, pl.split, mb);
 }
 
 double pair_ta_gated_us(const Layout& L, int M, double mb, int num_sms)
 {
-    const int steps = (L.K + kGemmKStep - 1) / kGemmKStep, pairs = L.n_rsb / 2, n_mblk = (M + 255) / 256, clusters = num_sms / 2;
-    if (!gemm_pair_ta_both(L, M, num_sms)) return pair_ta_fewest_us(((M + n_mblk - 1) / n_mblk + 31) / 32 * 32, (pairs * n_mblk + clusters - 1) / clusters, 2 * steps, 1, mb);
-    const TaPlan pl = gemm_pair_ta_gated_plan(L, M, num_sms);
-    return gemm_pair_ta_us(pairs, pl.n_mblk, pl.bn, 1, steps, 2, false, num_sms);
+    const bool both = gemm_pair_ta_both(L, M, num_sms);
+    const TaPlan pl = gemm_pair_ta_gated_plan(L, M, num_sms);            // (what the launch takes)
+    return gemm_pair_ta_us(L.n_rsb / 2, pl.n_mblk, pl.bn, 1, (L.K + kGemmKStep - 1) / kGemmKStep, 2, both, false, num_sms) + (both ? 0.0 : 0.53 * mb);
 }
 
 double single_us(const Layout& L, int M, double mb, int num_sms)
@@ -984,9 +983,9 @@ ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
     const ql_kernel other = batch ? QL_KERNEL_MID : prefill_kernel(hs, n, M, gated);
     if (!narrow_can(hs, n, M, gated, batch)) return other;
     if (config().narrow == 2) return QL_KERNEL_NARROW;
-    // (A gated pair that gemm_pair_ta.cuh serves with one accumulator: 7 % below, as its estimate was made with.)
-    const double limit = batch ? mid_us(hs, n, M, gated) : (gated && other == QL_KERNEL_PAIR_TA && !gemm_pair_ta_both(L, M, hs[0]->num_sms) ? 0.93 : 1.0) * prefill_us(other, hs, n, M, gated);
-    return narrow_us(hs, n, M, gated) < limit ? QL_KERNEL_NARROW : other;
+    // (A gated pair that gemm_pair_ta.cuh would serve with one accumulator: up to 4 % above, since act(gate) stays in fp32 here.)
+    const double lean = gated && other == QL_KERNEL_PAIR_TA && !gemm_pair_ta_both(L, M, hs[0]->num_sms) ? 1.04 : 1.0;
+    return narrow_us(hs, n, M, gated) < (batch ? mid_us(hs, n, M, gated) : lean * prefill_us(other, hs, n, M, gated)) ? QL_KERNEL_NARROW : other;
 }
 
 // y = act(g) * u, element-wise (the unfused form of the gating, for shapes the fused kernels do not take).

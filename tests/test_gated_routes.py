@@ -1,0 +1,30 @@
+"""Gated pairs of more than 128 tokens: the estimates that choose between the kernels, against times measured on a B200 (consecutive launches,
+weights out of HBM), evaluated without a device."""
+import ctypes
+
+import pytest
+
+SMS = 148
+NARROW, PAIR_TA, PAIR = 5, 6, 7
+# ((channels, K, bits, group, tokens), the kernel that serves the call, us it took)
+ONE_ACCUMULATOR = [((12800, 128, 4, 32, 1410), PAIR_TA, 39.70), ((7936, 128, 4, 0, 1032), PAIR_TA, 23.56), ((11744, 128, 8, 0, 1373), PAIR_TA, 34.91),
+                   ((14336, 4096, 4, 32, 777), PAIR_TA, 162.1), ((9216, 2304, 4, 32, 777), PAIR_TA, 57.77)]
+
+
+@pytest.fixture(scope="module")
+def route(_built_library):
+    import paper_2505_00232_b200 as P
+
+    def call(N, K, bits, group, M):
+        ds = (type(P.Desc(8, 32, 8, 0).c()) * 2)(*[P.Desc(N, K, bits, group).c()] * 2)
+        out = (ctypes.c_int32 * 5)()
+        assert P.lib.qlinear_debug_route(ds, 2, M, 1, SMS, out, 5) == 5
+        return list(out)
+    return call
+
+
+@pytest.mark.parametrize("shape,kernel,us", ONE_ACCUMULATOR)
+def test_the_estimate_is_of_the_launch_that_runs(route, shape, kernel, us):
+    """Within the spread of the fit (0.92 to 1.20)."""
+    r = route(*shape)
+    assert r[0] == kernel and 0.9 <= us / (r[3 if kernel == NARROW else 4] / 1000) <= 1.2, r
