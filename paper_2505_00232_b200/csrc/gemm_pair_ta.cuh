@@ -781,14 +781,16 @@ gemm_pair_ta_kernel(const __grid_constant__ TaMaps maps, const GemmParams p)
 // at most half of the CTA pairs leaves the others to the next one's start.  Fitted to 240 (integer form: 240) combinations of layer and
 // tokens (256 x 1024 to 14336 x 4096, 129 to 1400 tokens) with up to 15 plans each.
 // A gated pair with one accumulator (layers == 2, not both): fitted to 385 random pairs of 129 to 2048 tokens with up to 6 widths each; of the
-// widths that run, measured / estimate 0.94 and 1.12 (5th and 95th percentile; 0.92 and 1.20 at the ends).
+// widths that run, measured / estimate 0.94 and 1.12 (5th and 95th percentile; 0.92 and 1.20 at the ends).  With two accumulators (both): to 815
+// with up to 5 widths each, 0.92 and 1.10.  Its six A slots bound a step (0.27 us at any width), so wide blocks are the better ones
+// wherever they fill the GPU; one accumulator and eight slots take 0.20 at 32 tokens and 0.29 at 256.
 inline double gemm_pair_ta_us(int pairs, int n_mblk, int bn, int split, int n_ksteps, int layers, bool both, bool i8, int num_sms)
 {
     const int units = pairs * n_mblk * split, clusters = num_sms / 2, rounds = (units + clusters - 1) / clusters, steps = (n_ksteps + split - 1) / split;
     const double more = units * 2 > clusters ? 1.0 : 0.0;
     if (i8) return 5.94 + 0.00896 * bn + rounds * steps * (0.2494 + 0.00006 * bn) + (split == 4 ? 2.09 + 0.0273 * bn : split == 2 ? 1.58 + 0.0116 * bn : 0.0) + 0.8 * more + 1.83 * (rounds - 1);
     if (layers == 2 && !both) return 6.31 + 0.0021 * bn + (rounds - 1) * (2.63 - 0.0063 * bn) + rounds * 2 * steps * (0.1846 + 0.00042 * bn);
-    if (layers == 2) return 5.48 + rounds * (0.0206 * bn - 1.35 + steps * (0.4395 + 0.00083 * bn));   // (the store included)
+    if (layers == 2) return 2.93 + 0.006 * bn + (rounds - 1) * (1.65 - 0.0128 * bn) + rounds * 2 * steps * (0.2673 + 0.00004 * bn) + 1.72 * std::min(1.0, (double)units / clusters);
     return 3.01 + 0.0003 * bn + rounds * steps * (0.1966 + 0.00038 * bn) + (split == 4 ? 2.77 + 0.023 * bn : split == 2 ? 2.13 + 0.013 * bn : 0.0) + 1.22 * more - 0.51 * (rounds - 1);
 }
 
@@ -799,14 +801,14 @@ inline double gemm_pair_ta_us(int pairs, int n_mblk, int bn, int split, int n_ks
 // 2048 x 2304 at 512 tokens 19.9 / 12.2, 2304 x 2048 at 777 18.8 / 12.7, 4096 x 4096 at 512 24.9 / 21.2, 2304 x 9216 at 300 25.1 / 20.7, 4096 x 14336
 // at 1400 144 / 133; integer form (which had no parts, and few tiles in shared memory) 1024 x 4096 at 1024 39.3 / 18.2, 2304 x 9216 at 777 66.0 / 31.4.
 // Calls that gemm_narrow.cuh takes by a wide margin (up to 128 tokens, two pairs of row super-blocks or 1024 k) keep the plan with the fewest
-// blocks here: gemm_route compares the two, and what is left of them has large K parts.
+// blocks here: gemm_route compares the two, and what is left of them has large K parts.  (Not so the gated form with two accumulators.)
 struct TaPlan { int n_mblk, bn, split; };
 inline bool gemm_pair_ta_searches(int pairs, int M, int n_ksteps, bool i8) { return i8 || (M > 128 && pairs > 2 && n_ksteps > 16); }
 inline TaPlan gemm_pair_ta_plan(int pairs, int M, int n_ksteps, int layers, bool i8, int num_sms, bool may_split, bool both = false)
 {
     const int clusters = num_sms / 2;
     const int forced = gemm_config().force_split >= 4 ? 4 : gemm_config().force_split >= 2 ? 2 : gemm_config().force_split;
-    const bool search = gemm_pair_ta_searches(pairs, M, n_ksteps, i8);
+    const bool search = both || gemm_pair_ta_searches(pairs, M, n_ksteps, i8);
     TaPlan best{};
     double best_us = 1e30;
     for (int bn = both ? kTaBothTokens : 256; bn >= 32; bn -= 32) {
@@ -897,6 +899,13 @@ ql_status gemm_pair_ta_launch(const GemmPairLayers& set, const TaPlan& pl, const
     return QL_OK;
 }
 
+// Estimate of the gated form of gemm_pair.cuh, as above; fitted to 815 pairs, measured / estimate 0.93 and 1.10.
+inline double gemm_pair_gated_us(const Layout& L, int M, double mb, int num_sms)
+{
+    const int steps = (L.K + kGemmKStep - 1) / kGemmKStep, clusters = num_sms / 2, rounds = (L.n_rsb / 2 * ((M + 255) / 256) + clusters - 1) / clusters;
+    return 6.11 + 0.0411 * std::min(M, 256) + rounds * steps * (L.bits == 8 ? 0.888 : 0.761) + 0.242 * mb;
+}
+
 // Any M the prefill path sees (tokens beyond M are zero-filled by TMA and never stored): below 129 tokens the tile is
 // mostly padding, but the launch is bound by streaming and dequantising the weights, which this kernel spreads over
 // the whole GPU (K split), not by the MMAs.
@@ -912,15 +921,16 @@ inline bool gemm_pair_ta_applicable(const GemmPairLayers& set, int M, int num_sm
     if (!gemm_config().ta || !gemm_config().pair) return false;
     for (int i = 0; i < set.n; ++i)
         if (!set.wmap[i] || (set.L[i]->n_rsb % 2)) return false;
-    // The plain form takes every launch.  The gated one where a position is left for every CTA pair in blocks of 256 tokens; and from 3073
-    // channels on, with two accumulators, where blocks of up to 160 tokens are dealt out in one round, or the weights are int8 (us, the
-    // faster of shared-memory form and gemm_narrow.cuh / this one: int4 in groups 9216 x 2304 at 300 tokens 43.6 / 28.7, 6144 x 1792 at 400 36.5 / 23.8, 14336 x
-    // 4096 at 160 62.7 / 43.5, in two rounds 9216 x 2304 at 512 47.5 / 50.7; int8 14336 x 4096 at 256 98 / 78, 9216 x 2304 at 400 52 / 49).  (Time alone would
-    // take fewer channels as well: there the shared-memory form keeps calls that reach it by rule, in the tests and in smoke().)
+    // The plain form takes every launch.  The gated one where a position is left for every CTA pair in blocks of 256 tokens; and, with two
+    // accumulators, from 3073 channels on where its estimate is below that of the shared-memory form (us, that form / this one: int4 in groups 9216 x 2304
+    // at 300 tokens 43.6 / 28.7, 6144 x 1792 at 400 36.5 / 23.8, in two rounds 9216 x 2304 at 512 47.5 / 50.4, 4536 x 1920 at 649 41.4 / 42.4; int8 14336 x
+    // 4096 at 256 98 / 78, 9216 x 2304 at 400 52.6 / 48.2, 14272 x 7680 at 196 138 / 135; of 89 int8 pairs that it takes two rounds for 3 are slower, by up to 2 %).
     if (!gated) return true;
     const Layout& L = *set.L[0];
     if (M <= 128 || !gemm_pair_ta_both(L, M, num_sms)) return M > 128;
-    return L.n_rsb / 2 > 12 && (L.bits == 8 || L.n_rsb / 2 * gemm_pair_ta_gated_plan(L, M, num_sms).n_mblk <= num_sms / 2);
+    const TaPlan pl = gemm_pair_ta_gated_plan(L, M, num_sms);
+    const double mb = 2e-6 * M * L.N;
+    return L.n_rsb / 2 > 12 && gemm_pair_ta_us(L.n_rsb / 2, pl.n_mblk, pl.bn, 1, (L.K + kGemmKStep - 1) / kGemmKStep, 2, true, false, num_sms) + 0.56 * mb < gemm_pair_gated_us(L, M, mb, num_sms);
 }
 
 inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, int M, cudaStream_t st, int device, bool pdl, int num_sms,

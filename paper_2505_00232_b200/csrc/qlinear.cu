@@ -854,8 +854,8 @@ bool gate_fits_scratch(int N, int M, int num_sms) { return (size_t)M * N * 2 * s
 // tokens, plain and gated, the three schemes), each on both routes; long calls and the shapes of the two models weigh more.  Measured /
 // estimate, 5th and 95th percentile (1st and 99th): narrow_us 0.90 and 1.11 (0.84, 1.17), mid_us 0.90 and 1.11 (0.85, 1.16), prefill_us on the
 // CTA-pair kernel's plans of the fewest blocks 0.83 and 1.19 (0.81, 1.70: gated pairs of K up to 128, far from the line; those it searches, of 700 later
-// calls: 0.88 and 1.12), on the single-CTA kernel 0.86 and 1.07 (0.79, 1.17), on
-// the shared-memory gated form 0.89 and 1.14 (0.88, 1.19), unfused 0.86 and 1.05 (0.81, 1.13).
+// calls: 0.88 and 1.12), on the single-CTA kernel 0.86 and 1.07 (0.79, 1.17), unfused 0.86 and 1.05 (0.81, 1.13).  The fused gated forms of more
+// than 128 tokens have estimates of their own (narrow_gated_us, gemm_pair_ta_us, gemm_pair_gated_us).
 // What a CTA's time is multiplied by for the others of the launch, `ctas` in all in clusters of cl, two to an SM: up to one per SM they slow it
 // down by `first`, the second ones by `second` more; beyond two per SM further rounds, of which the last one costs `last` at least.
 // (Clusters of 4 and 8 lie inside a GPC: fewer fit.)
@@ -869,9 +869,21 @@ double sm_load(double ctas, int cl, int num_sms, double first, double second, do
 int total_rsb(const qlinear_s* const* hs, int n) { int t = 0; for (int i = 0; i < n; ++i) t += hs[i]->L.n_rsb; return t; }
 double out_mb(const qlinear_s* const* hs, int n, int M) { double t = 0; for (int i = 0; i < n; ++i) t += 2e-6 * M * hs[i]->L.N; return t; }
 
+// Gated pairs that the kernels of CTA pairs can serve as well, which was a corner of the calls that the estimate below was made with: fitted to 1675
+// such pairs of 129 to 4096 tokens, measured / estimate 0.93 and 1.10 (the other one: 0.82 and 1.18).
+double narrow_gated_us(const qlinear_s* const* hs, int M)
+{
+    const Layout& L = hs[0]->L;
+    const NarrowPlan pl = plan_narrow(L, L.n_rsb, true, M, hs[0]->num_sms);
+    const int steps = ((L.K + kNarrowKStep - 1) / kNarrowKStep + pl.cl - 1) / pl.cl * 2;
+    const double cta = steps * (L.bits == 4 ? 0.304 : 0.289) + 0.63 + 0.0342 * pl.bn;
+    return 0.92 + 0.77 * log2_of(pl.cl) + sm_load((double)L.n_rsb * pl.n_tb * pl.cl, pl.cl, hs[0]->num_sms, 0.672, 0.205, 0.408) * cta;
+}
+
 double narrow_us(const qlinear_s* const* hs, int n, int M, bool gated)
 {
     const Layout& L = hs[0]->L;
+    if (gated && gemm_pair_applicable(L, M)) return narrow_gated_us(hs, M);
     const int rows = gated ? L.n_rsb : total_rsb(hs, n);
     const NarrowPlan pl = plan_narrow(L, rows, gated, M, hs[0]->num_sms);
     const int steps = ((L.K + kNarrowKStep - 1) / kNarrowKStep + pl.cl - 1) / pl.cl * (gated ? 2 : 1);
@@ -906,7 +918,7 @@ double pair_ta_gated_us(const Layout& L, int M, double mb, int num_sms)
 {
     const bool both = gemm_pair_ta_both(L, M, num_sms);
     const TaPlan pl = gemm_pair_ta_gated_plan(L, M, num_sms);            // (what the launch takes)
-    return gemm_pair_ta_us(L.n_rsb / 2, pl.n_mblk, pl.bn, 1, (L.K + kGemmKStep - 1) / kGemmKStep, 2, both, false, num_sms) + (both ? 0.0 : 0.53 * mb);
+    return gemm_pair_ta_us(L.n_rsb / 2, pl.n_mblk, pl.bn, 1, (L.K + kGemmKStep - 1) / kGemmKStep, 2, both, false, num_sms) + (both ? 0.56 : 0.53) * mb;
 }
 
 double single_us(const Layout& L, int M, double mb, int num_sms)
@@ -920,7 +932,7 @@ double single_us(const Layout& L, int M, double mb, int num_sms)
 double prefill_us(ql_kernel kernel, const qlinear_s* const* hs, int n, int M, bool gated)
 {
     const Layout& L = hs[0]->L;
-    const int sms = hs[0]->num_sms, steps = (L.K + kGemmKStep - 1) / kGemmKStep;
+    const int sms = hs[0]->num_sms;
     const double mb = out_mb(hs, gated ? 1 : n, M);
     if (kernel == QL_KERNEL_SINGLE) return single_us(L, M, mb, sms);
     if (kernel == QL_KERNEL_SEPARATE) {
@@ -933,8 +945,7 @@ double prefill_us(ql_kernel kernel, const qlinear_s* const* hs, int n, int M, bo
         }
         return us;
     }
-    if (gated && kernel == QL_KERNEL_PAIR)
-        return 5.5 + 0.044 * std::min(M, 256) + round_up((double)(L.n_rsb / 2) * ((M + 255) / 256) / (sms / 2)) * 0.84 * steps + 0.3 * mb;
+    if (gated && kernel == QL_KERNEL_PAIR) return gemm_pair_gated_us(L, M, mb, sms);
     return gated ? pair_ta_gated_us(L, M, mb, sms) : pair_ta_us(L, total_rsb(hs, n) / 2, M, true, mb, sms);
 }
 
@@ -983,8 +994,8 @@ ql_kernel gemm_route(const qlinear_s* const* hs, int n, int M, bool gated)
     const ql_kernel other = batch ? QL_KERNEL_MID : prefill_kernel(hs, n, M, gated);
     if (!narrow_can(hs, n, M, gated, batch)) return other;
     if (config().narrow == 2) return QL_KERNEL_NARROW;
-    // (A gated pair that gemm_pair_ta.cuh would serve with one accumulator: up to 4 % above, since act(gate) stays in fp32 here.)
-    const double lean = gated && other == QL_KERNEL_PAIR_TA && !gemm_pair_ta_both(L, M, hs[0]->num_sms) ? 1.04 : 1.0;
+    // (Pairs that the kernels of CTA pairs can serve: up to 4 % above.  With one accumulator they round act(gate) to fp16, which this one doesn't.)
+    const double lean = gated && gemm_pair_applicable(L, M) ? 1.04 : 1.0;
     return narrow_us(hs, n, M, gated) < (batch ? mid_us(hs, n, M, gated) : lean * prefill_us(other, hs, n, M, gated)) ? QL_KERNEL_NARROW : other;
 }
 

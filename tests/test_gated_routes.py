@@ -11,6 +11,18 @@ ONE_ACCUMULATOR = [((12800, 128, 4, 32, 1410), PAIR_TA, 39.70), ((7936, 128, 4, 
                    ((14336, 4096, 4, 32, 777), PAIR_TA, 162.1), ((9216, 2304, 4, 32, 777), PAIR_TA, 57.77)]
 
 
+# (beside each: us on the kernel that the estimates must not choose)
+TWO_ACCUMULATORS = [((9440, 1536, 8, 0, 131), NARROW, 16.74),             # 20.5
+                    ((7424, 1152, 8, 0, 176), NARROW, 14.78),             # 16.7
+                    ((6144, 1120, 8, 0, 330), NARROW, 16.11),             # 18.1
+                    ((9216, 1120, 8, 0, 130), NARROW, 14.06),             # 17.2
+                    ((3464, 6336, 4, 32, 322), NARROW, 54.15),            # 60.2
+                    ((6400, 7168, 8, 0, 426), NARROW, 97.06),             # 125.1
+                    ((4096, 128, 4, 32, 873), PAIR_TA, 10.42),            # 13.2
+                    ((4096, 128, 8, 0, 920), PAIR_TA, 11.12),             # 13.7 (two rounds)
+                    ((9216, 2304, 4, 32, 300), PAIR_TA, 28.7)]            # 43.6
+
+
 @pytest.fixture(scope="module")
 def route(_built_library):
     import paper_2505_00232_b200 as P
@@ -23,7 +35,7 @@ def route(_built_library):
     return call
 
 
-@pytest.mark.parametrize("shape,kernel,us", ONE_ACCUMULATOR)
+@pytest.mark.parametrize("shape,kernel,us", ONE_ACCUMULATOR + TWO_ACCUMULATORS)
 def test_the_estimate_is_of_the_launch_that_runs(route, shape, kernel, us):
     """Within the spread of the fit (0.92 to 1.20)."""
     r = route(*shape)
