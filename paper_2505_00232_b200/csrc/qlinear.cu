@@ -975,7 +975,7 @@ bool narrow_can(const qlinear_s* const* hs, int n, int M, bool gated, bool batch
 // estimate is below that of gemm_mid.cuh, the CTA-pair kernel or the three other forms (single CTA, shared-memory gating, unfused gating).  No line is always right with these errors.  Of the calls above and 3110 others, 80 run more than 3 %
 // slower this way than on the other route: 54 of 4821 against gemm_mid.cuh (two of them by 46 and 26 %, the others by 24 % at most), 9
 // of 5488 against the other forms (9 %).  Against the CTA-pair kernel with its plans searched, 700 calls take 0.3 % more than on the faster route each,
-// the worst 21 %.  Measured, us, the route otherwise / gemm_narrow.cuh:
+// the worst 21 %.  1676 gated pairs of 129 to 4096 tokens, timed on every form and width: 1.3 % more than on the fastest, the worst 26 %.  Measured, us, the route otherwise / gemm_narrow.cuh:
 //   weights                        16 tokens     24           32           48           64
 //     0.3 M (512 x 512)             2.8 /  3.7   3.0 /  3.8   3.3 /  4.0   3.8 /  4.2   4.1 /  4.5
 //     1 M (1024 x 1024, int8)       3.2 /  4.3   3.5 /  4.5   4.0 /  4.6   4.6 /  5.0   5.2 /  5.3

@@ -20,7 +20,11 @@ TWO_ACCUMULATORS = [((9440, 1536, 8, 0, 131), NARROW, 16.74),             # 20.5
                     ((6400, 7168, 8, 0, 426), NARROW, 97.06),             # 125.1
                     ((4096, 128, 4, 32, 873), PAIR_TA, 10.42),            # 13.2
                     ((4096, 128, 8, 0, 920), PAIR_TA, 11.12),             # 13.7 (two rounds)
-                    ((9216, 2304, 4, 32, 300), PAIR_TA, 28.7)]            # 43.6
+                    ((9216, 2304, 4, 32, 300), PAIR_TA, 28.7),            # 43.6
+                    ((1792, 1984, 4, 32, 1518), PAIR_TA, 25.95),          # 39.1
+                    ((3040, 2624, 8, 0, 848), PAIR_TA, 30.68),            # 54.5
+                    ((768, 4608, 8, 0, 3800), PAIR_TA, 47.31),            # 79.7
+                    ((1000, 512, 8, 0, 257), NARROW, 7.73), ((3072, 4096, 4, 32, 1500), PAIR, 69.3)]   # 8.7, 81.9
 
 
 @pytest.fixture(scope="module")
