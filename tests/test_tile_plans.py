@@ -14,6 +14,10 @@ PAIR_TA = 6
 PLAIN = [(300, 2304, 9216, 4, 32, 160, 4), (257, 2800, 8224, 8, 0, 96, 2), (641, 4096, 2176, 4, 0, 192, 1), (1409, 2560, 1152, 4, 128, 224, 1), (1030, 4864, 1152, 8, 0, 160, 1)]
 GATED = [(300, 8400, 1088, 4, 32, 160), (240, 17352, 960, 8, 0, 128), (168, 16640, 448, 8, 0, 96), (259, 13312, 1088, 4, 0, 160)]
 GATED_ON_NARROW = [(330, 6144, 1120, 8, 0), (130, 9216, 1120, 8, 0)]      # (us, gemm_narrow.cuh / two accumulators: 16.1 / 18.1, 14.1 / 17.2)
+# Two accumulators (the position's second one, at blocks of 160, 128, 96 and 64): one round and two, one k-step to many, few channels, the three activations
+TWO_ACCUMULATORS = [(240, 17352, 960, 8, 0, 128, "gelu_tanh"), (161, 17152, 384, 4, 32, 96, "identity"), (391, 9216, 192, 4, 32, 160, "gelu_tanh"), (183, 17664, 128, 4, 32, 96, "silu"),
+                    (415, 7424, 128, 8, 0, 160, "identity"), (1518, 1792, 1984, 4, 32, 160, "gelu_tanh"), (1100, 504, 224, 8, 0, 96, "silu"), (2000, 248, 32, 8, 0, 96, "gelu_tanh"),
+                    (1029, 248, 160, 8, 0, 64, "identity"), (228, 10752, 192, 4, 0, 128, "silu")]
 # integer form (its plan is not asked for): one pair of row super-blocks to many, one k-step to many, parts and narrow blocks
 A8 = [(129, 256, 128, 4), (130, 200, 8192, 8), (200, 1024, 4096, 4), (333, 2296, 9216, 8), (700, 1024, 2304, 4), (1030, 4096, 1152, 8), (641, 9216, 256, 4)]
 
@@ -38,6 +42,9 @@ def route(P, Ns, K, bits, group, M, gated):
 def test_the_calls_below_get_these_plans(P):
     assert [route(P, [N], K, b, g, M, 0)[:3] for M, N, K, b, g, _, _ in PLAIN] == [[PAIR_TA, w, p] for *_, w, p in PLAIN]
     assert [route(P, [N, N], K, b, g, M, 1)[:3] for M, N, K, b, g, _ in GATED] == [[PAIR_TA, w, 1] for *_, w in GATED]
+    assert [route(P, [N, N], K, b, g, M, 1)[:3] for M, N, K, b, g, *_ in TWO_ACCUMULATORS] == [[PAIR_TA, w, 1] for *_, w, _ in TWO_ACCUMULATORS]
+    rounds = {-(-(-(-N // 256) * -(-M // w)) // (SMS // 2)) for M, N, *_, w, _ in TWO_ACCUMULATORS}
+    assert rounds == {1, 2} and all(-(-N // 256) * -(-M // 256) < SMS // 2 for M, N, *_ in TWO_ACCUMULATORS)
 
 
 @pytest.mark.gpu
@@ -70,6 +77,23 @@ def test_gated(P, M, N, K, bits, group):
     assert torch.equal(y, P.qlinear_forward_gated(lg, lu, xd, "silu")) and lg.device_status() == (0, 0)
     rows = np.r_[0:300, N - 300:N]
     assert_gated(y.cpu().numpy()[:, rows], x, (gw[0][rows], gw[1][rows]), (uw[0][rows], uw[1][rows]), group, "silu")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,bits,group,width,act", TWO_ACCUMULATORS)
+def test_two_accumulators(P, M, N, K, bits, group, width, act):
+    import torch
+    from tests.test_gated_gpu import assert_gated
+    gw, uw = (C.layer_weights(8400 + M + i, spec(N, K, bits, group)) for i in range(2))
+    x = C.layer_activations(8400 + M, spec(N, K, bits, group), M)
+    lg, lu = (P.QLinear.from_weights(q, s, bits, group, device="cuda:0") for q, s in (gw, uw))
+    xd = torch.from_numpy(x).cuda()
+    guard = torch.full((M + 2, N), -7.0, dtype=torch.float16, device="cuda")
+    y = P.qlinear_forward_gated(lg, lu, xd, act, out=guard[1:-1])
+    again = [P.qlinear_forward_gated(lg, lu, xd, act) for _ in range(20)]
+    assert all(torch.equal(y, a) for a in again) and lg.device_status() == (0, 0) and (guard[0] == -7.0).all() and (guard[-1] == -7.0).all()
+    rows = np.r_[0:300, N // 2:N // 2 + 100, N - 300:N] if N > 700 else np.r_[0:N]
+    assert_gated(y.cpu().numpy()[:, rows], x, (gw[0][rows], gw[1][rows]), (uw[0][rows], uw[1][rows]), group, act)
 
 
 @pytest.mark.gpu
