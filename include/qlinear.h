@@ -382,6 +382,8 @@ uint32_t qlinear_version(void);
  * qlinear_debug_route evaluates, without a device, the dispatch of a call beyond the decode stage on layers like these (n = 1: forward, more:
  * a group, gated: a pair) on a GPU of num_sms SMs; up to n_out of {the kernel (ql_kernel); its tokens per tile and K parts (NARROW, PAIR_TA, SINGLE;
  * else 0 and 1); the estimates behind the choice in ns: NARROW, the kernel that takes the call otherwise}; returns how many it wrote (0 on bad arguments).
+ * qlinear_debug_plan_a8 does the same for qlinear_forward_a8 on a layer like this: {QL_KERNEL_DECODE; CTAs; CTAs per cluster; K slices per CTA} or
+ * {PAIR_TA or PAIR; tokens per tile; K parts; token blocks}, 0 numbers where the call is refused.
  * qlinear_debug_kv_hold gives the tokens [*first, *end) of n caches that a decode reader of theirs on this stream would leave until the
  * kernel before it is complete: those of the last append if that was enqueued on the same stream and in the same capture, all of
  * them (an *end beyond any cache) if it was enqueued elsewhere, none for layers that nothing was appended to. */
@@ -400,6 +402,7 @@ typedef enum {
     QL_KERNEL_SEPARATE = 9   /* a group: one call per layer; a gated pair: two projections and an element-wise product */
 } ql_kernel;
 int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_t M, int32_t gated, int32_t num_sms, int32_t* out, int32_t n_out);
+int32_t qlinear_debug_plan_a8(const qlinear_desc* d, int32_t M, int32_t num_sms, int32_t* out, int32_t n_out);
 ql_status qlinear_debug_kv_hold(const qlinear_t* hs, int32_t n, void* stream, int32_t* first, int32_t* end);
 uint32_t qlinear_debug_config_reads(void);
 

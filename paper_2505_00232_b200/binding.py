@@ -24,7 +24,7 @@ ACTIVATIONS = {"identity": QL_ACT_IDENTITY, "silu": QL_ACT_SILU, "gelu_tanh": QL
 EXPORTS = (
     "qlinear_packed_size", "qlinear_pack", "qlinear_unpack", "qlinear_create", "qlinear_forward", "qlinear_forward_group", "qlinear_forward_batch", "qlinear_forward_gated", "qlinear_forward_a8", "qlinear_quantize_activations", "qlinear_kv_append", "qlinear_kv_scores", "qlinear_kv_output", "qlinear_kv_output_uses_tmp", "qlinear_kv_append_heads", "qlinear_kv_scores_heads", "qlinear_kv_output_heads", "qlinear_embed", "qlinear_residual_rmsnorm", "qlinear_rope_qkv",
     "qlinear_path_for", "qlinear_debug_unpack_device", "qlinear_debug_expire_wait", "qlinear_debug_null_launch", "qlinear_device_status", "qlinear_decode_static", "qlinear_destroy",
-    "qlinear_status_string", "qlinear_version", "qlinear_debug_plan", "qlinear_debug_plan_kv_output", "qlinear_debug_takes_batch_kernel", "qlinear_debug_kv_hold", "qlinear_debug_route", "qlinear_debug_config_reads",
+    "qlinear_status_string", "qlinear_version", "qlinear_debug_plan", "qlinear_debug_plan_kv_output", "qlinear_debug_takes_batch_kernel", "qlinear_debug_kv_hold", "qlinear_debug_route", "qlinear_debug_plan_a8", "qlinear_debug_config_reads",
 )
 
 
@@ -113,6 +113,8 @@ def _load() -> ctypes.CDLL:
     lib.qlinear_debug_kv_hold.argtypes = [ctypes.POINTER(vp), i32, vp, ctypes.POINTER(i32), ctypes.POINTER(i32)]
     lib.qlinear_debug_route.argtypes = [vp, i32, i32, i32, i32, ctypes.POINTER(i32), i32]
     lib.qlinear_debug_route.restype = i32
+    lib.qlinear_debug_plan_a8.argtypes = [vp, i32, i32, ctypes.POINTER(i32), i32]
+    lib.qlinear_debug_plan_a8.restype = i32
     lib.qlinear_debug_kv_hold.restype = ctypes.c_int
     lib.qlinear_debug_config_reads.restype = ctypes.c_uint32
     return lib

@@ -977,11 +977,15 @@ inline bool gemm_pair_ta_i8_applicable(const GemmPairLayers& set, int M)
 {
     return gemm_config().ta && M > 128 && set.wmap[0];
 }
+inline TaPlan gemm_pair_ta_i8_plan(const Layout& L, int M, int num_sms, bool may_split)
+{
+    return gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + 127) / 128, 1, true, num_sms, may_split);
+}
 inline ql_status gemm_pair_ta_forward_i8(const GemmPairLayers& set, const void* xq, const float* scale, const int32_t* rowsum, int M,
                                          cudaStream_t st, int device, bool pdl, int num_sms, float* scratch, unsigned int* counters)
 {
     const Layout& L = *set.L[0];
-    const TaPlan pl = gemm_pair_ta_plan(L.n_rsb / 2, M, (L.K + 127) / 128, 1, true, num_sms, scratch && counters);
+    const TaPlan pl = gemm_pair_ta_i8_plan(L, M, num_sms, scratch && counters);
     if (pl.split > 1)
         return L.bits == 8 ? gemm_pair_ta_launch<8, false, false, true, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, scratch, counters, scale, rowsum)
                            : gemm_pair_ta_launch<4, false, false, true, true>(set, pl, xq, M, st, device, pdl, num_sms, -1, scratch, counters, scale, rowsum);

@@ -1390,6 +1390,25 @@ cudaError_t launch_quantize(const __half* x, signed char* xq, float* scale, int3
 }
 }  // namespace
 
+// Bytes of the device's scratch that a prompt with int8 activations uses: the quantised rows, the per-token arrays behind them (padded to
+// whole 256-token tiles) and, where the scratch holds them as well, the K parts of launches of few tiles.
+namespace {
+struct A8Scratch {
+    size_t xq, arr;
+    bool fits, parts;
+};
+A8Scratch a8_scratch(int M, int K, int num_sms)
+{
+    A8Scratch s;
+    s.xq = (((size_t)M * K + 255) / 256) * 256;
+    s.arr = (size_t)((M + 255) / 256) * 256 * 4;
+    const size_t used = s.xq + 2 * s.arr, all = gemm_pair_scratch_bytes(num_sms);
+    s.fits = used <= all;
+    s.parts = used + (size_t)(num_sms / 2) * 2 * 256 * 128 * sizeof(float) <= all;
+    return s;
+}
+}  // namespace
+
 extern "C" ql_status qlinear_forward_a8(qlinear_t h, const void* x, void* y, int32_t M, void* stream)
 {
     if (!h || !x || !y || M < 1) return QL_ERR_INVALID_ARG;
@@ -1401,23 +1420,20 @@ extern "C" ql_status qlinear_forward_a8(qlinear_t h, const void* x, void* y, int
         // Built for the per-channel schemes on the CTA-pair kernel; the quantised activations live in the device's
         // shared scratch (calls must be ordered against other users of it).
         if (L.grouped || (L.K % 128) || !gemm_pair_applicable(L, M)) return QL_ERR_UNSUPPORTED;
-        const size_t xq_bytes = (((size_t)M * L.K + 255) / 256) * 256;
-        const size_t arr = (size_t)((M + 255) / 256) * 256 * 4;             // per-token arrays padded to whole 256-token tiles
-        if (xq_bytes + 2 * arr > gemm_pair_scratch_bytes(h->num_sms)) return QL_ERR_UNSUPPORTED;
+        const A8Scratch sc = a8_scratch(M, L.K, h->num_sms);
+        if (!sc.fits) return QL_ERR_UNSUPPORTED;
         DeviceGuard guard(h->device);
         if (!guard.ok) { cudaGetLastError(); return QL_ERR_CUDA; }
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         unsigned char* base = reinterpret_cast<unsigned char*>(h->dev->gemm_scratch);
         signed char* xq = reinterpret_cast<signed char*>(base);
-        float* sx = reinterpret_cast<float*>(base + xq_bytes);
-        int32_t* rs = reinterpret_cast<int32_t*>(base + xq_bytes + arr);
+        float* sx = reinterpret_cast<float*>(base + sc.xq);
+        int32_t* rs = reinterpret_cast<int32_t*>(base + sc.xq + sc.arr);
         if (launch_quantize(static_cast<const __half*>(x), xq, sx, rs, M, L.K, st, h->pdl) != cudaSuccess) { cudaGetLastError(); return QL_ERR_CUDA; }
         GemmPairLayers set{};
         set.n = 1; set.L[0] = &h->L; set.blob[0] = h->blob; set.y[0] = y; set.wmap[0] = h->wmap_wide_ok ? &h->wmap_wide : nullptr;
         if (gemm_pair_ta_i8_applicable(set, M)) {
-            // the K parts of few tiles meet behind the activations, where the scratch holds both
-            const size_t used = xq_bytes + 2 * arr, parts = (size_t)(h->num_sms / 2) * 2 * 256 * 128 * sizeof(float);
-            float* scratch = used + parts <= gemm_pair_scratch_bytes(h->num_sms) ? reinterpret_cast<float*>(base + used) : nullptr;
+            float* scratch = sc.parts ? reinterpret_cast<float*>(base + sc.xq + 2 * sc.arr) : nullptr;
             return gemm_pair_ta_forward_i8(set, xq, sx, rs, M, st, h->device, h->early(), h->num_sms, scratch, h->dev->gemm_counters);
         }
         return gemm_pair_forward_i8(set, xq, sx, rs, M, st, h->device, h->num_sms);
@@ -1956,6 +1972,27 @@ extern "C" int32_t qlinear_debug_route(const qlinear_desc* ds, int32_t n, int32_
     const double other = takes_mid(hs, n, M, gated) ? mid_us(hs, n, M, gated) : prefill_us(prefill_kernel(hs, n, M, gated), hs, n, M, gated);
     const int32_t v[5] = {kernel, width, parts, (int32_t)(1000 * narrow_us(hs, n, M, gated)), (int32_t)(1000 * other)};
     const int k = n_out < 5 ? n_out : 5;
+    for (int i = 0; i < k; ++i) out[i] = v[i];
+    return k;
+}
+
+extern "C" int32_t qlinear_debug_plan_a8(const qlinear_desc* d, int32_t M, int32_t num_sms, int32_t* out, int32_t n_out)
+{
+    Layout L;
+    if (!d || M < 1 || num_sms < 2 || !out || !make_layout(d->N, d->K, d->bits, d->group, &L)) return 0;
+    int32_t v[4];
+    if (M <= config().gemv_max_m) {
+        const GemvPlan pl = plan_gemv(L, (L.N + kRbRows - 1) / kRbRows, M, num_sms, false, true);
+        if (pl.grid <= 0) return 0;
+        v[0] = QL_KERNEL_DECODE; v[1] = pl.grid; v[2] = pl.cl; v[3] = pl.ks_cta;
+    } else {
+        const A8Scratch sc = a8_scratch(M, L.K, num_sms);
+        if (L.grouped || (L.K % 128) || !gemm_pair_applicable(L, M) || !sc.fits) return 0;
+        const bool ta = gemm_config().ta && w_map_fits(L, true);
+        const TaPlan pl = ta ? gemm_pair_ta_i8_plan(L, M, num_sms, sc.parts) : TaPlan{(M + 255) / 256, 256, 1};
+        v[0] = ta ? QL_KERNEL_PAIR_TA : QL_KERNEL_PAIR; v[1] = pl.bn; v[2] = pl.split; v[3] = pl.n_mblk;
+    }
+    const int k = std::min(n_out, 4);
     for (int i = 0; i < k; ++i) out[i] = v[i];
     return k;
 }

@@ -185,6 +185,50 @@ def test_calls_that_something_observes_are_left_to_python(P, monkeypatch, mode):
 
 
 @pytest.mark.gpu
+def test_common_calls_are_taken_by_the_native_half(P, monkeypatch):
+    """None means "Python's": without this check a native half that takes nothing would go unnoticed.  Same bits from both, the product over
+    more than 256 channels (whose scaled rows need a buffer) and single caches between appends among them."""
+    import torch
+    native, taken = P.binding._bind_torch(), []
+
+    class Recorded:
+        def __getattr__(self, name):
+            def call(*a):
+                taken.append((name, getattr(native, name)(*a) if real else None))
+                return taken[-1][1]
+            return call
+    monkeypatch.setattr(P.binding, "_native", Recorded())
+    real = True
+    calls = tensor_calls(P)
+    out = []
+    for name, call in calls.items():
+        taken.clear()
+        out.append(call())
+        assert len(taken) == 1 and taken[0][1] is not None, name
+    assert {n for n in dir(native) if not n.startswith("_")} - {"init", "built_for", "kv_append"} == {n.split(",")[0] for n in calls}
+
+    def cache():
+        g = torch.Generator(device="cuda").manual_seed(3)
+        f16 = lambda *s: torch.randn(s, generator=g, device="cuda").half()
+        kv, heads, y = P.KVCache(256, 64), P.KVHeads(2, 256, 64), []
+        for n in (5, 1, 70):
+            kv.append(f16(n, 64), f16(n, 64))
+            heads.append(f16(2, n, 64), f16(2, n, 64))
+            for R in (2, 40):
+                prob = f16(2, R, 256)
+                prob[:, :, kv.length:] = 0
+                y += [kv.scores(f16(R, 64)), kv.output(prob[0]), heads.scores(f16(2, R, 64))] + ([heads.output(prob)] if R <= 8 else [])
+        return y
+    fast = cache()
+    assert taken and all(r is not None for _, r in taken) and {"kv_append", "kv_output", "kv_output_heads", "kv_scores_one"} <= {n for n, _ in taken}
+    real = False
+    slow = cache() + [call() for call in calls.values()]
+    flat = lambda ys: [t for y in ys for t in (y if isinstance(y, (list, tuple)) else [y])]
+    fast, slow = flat(fast + out), flat(slow)
+    assert len(fast) == len(slow) and all(torch.equal(a, b) for a, b in zip(fast, slow))
+
+
+@pytest.mark.gpu
 def test_both_halves_agree(P, monkeypatch):
     import torch
     native = P.binding._bind_torch()

@@ -21,6 +21,13 @@ TWO_ACCUMULATORS = [(240, 17352, 960, 8, 0, 128, "gelu_tanh"), (161, 17152, 384,
 # integer form (its plan is not asked for): one pair of row super-blocks to many, one k-step to many, parts and narrow blocks
 A8 = [(129, 256, 128, 4), (130, 200, 8192, 8), (200, 1024, 4096, 4), (333, 2296, 9216, 8), (700, 1024, 2304, 4), (1030, 4096, 1152, 8), (641, 9216, 256, 4)]
 
+# its plan: tokens per tile, K parts, token blocks.  int4 in 4 parts, remainders in tokens and channels
+A8_PARTS = [((150, 256, 8192, 4), (32, 4, 5)), ((333, 504, 9216, 4), (64, 4, 6)), ((129, 2296, 8192, 4), (96, 4, 2)), ((257, 1000, 9216, 8), (96, 4, 3)), ((200, 1024, 14336, 4), (64, 4, 4)),
+            ((200, 1024, 4096, 4), (64, 2, 4)), ((1030, 4096, 1152, 8), (128, 1, 9))]
+# int8-activation decode: CTAs, CTAs per cluster
+A8_DECODE = [((1, 1024, 4096, 8, 0), (128, 2)), ((2, 4096, 14336, 4, 0), (256, 1)), ((8, 2304, 9216, 4, 32), (288, 2)), ((7, 2304, 9216, 8, 0), (288, 2)), ((8, 1024, 4096, 4, 0), (128, 2)),
+             ((1, 4096, 14336, 8, 0), (512, 2)), ((1, 256, 4096, 8, 0), (64, 4)), ((3, 264, 14336, 4, 32), (119, 7)), ((8, 64, 16384, 8, 0), (32, 8)), ((1, 14336, 4096, 4, 0), (448, 1))]
+
 
 @pytest.fixture(scope="module")
 def P(_built_library):
@@ -45,6 +52,18 @@ def test_the_calls_below_get_these_plans(P):
     assert [route(P, [N, N], K, b, g, M, 1)[:3] for M, N, K, b, g, *_ in TWO_ACCUMULATORS] == [[PAIR_TA, w, 1] for *_, w, _ in TWO_ACCUMULATORS]
     rounds = {-(-(-(-N // 256) * -(-M // w)) // (SMS // 2)) for M, N, *_, w, _ in TWO_ACCUMULATORS}
     assert rounds == {1, 2} and all(-(-N // 256) * -(-M // 256) < SMS // 2 for M, N, *_ in TWO_ACCUMULATORS)
+
+
+def test_calls_with_int8_activations_get_these_plans(P):
+    out = (ctypes.c_int32 * 4)()
+
+    def plan(M, N, K, bits, group=0):
+        n = P.lib.qlinear_debug_plan_a8(ctypes.byref(P.Desc(N, K, bits, group).c()), M, SMS, out, 4)
+        return list(out)[:n]
+    assert [plan(*c) for c, _ in A8_PARTS] == [[PAIR_TA, *p] for _, p in A8_PARTS]
+    assert [plan(*c)[:3] for c, _ in A8_DECODE] == [[1, *p] for _, p in A8_DECODE]
+    # refused: 9 to 128 tokens, K no multiple of 128, an odd number of row super-blocks, groups, rows that the scratch does not hold
+    assert [plan(*c) for c in ((100, 256, 256, 8), (300, 256, 160, 8), (300, 128, 256, 8), (300, 256, 256, 4, 32), (5000, 256, 16384, 8))] == [[]] * 5
 
 
 @pytest.mark.gpu
@@ -97,7 +116,7 @@ def test_two_accumulators(P, M, N, K, bits, group, width, act):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("M,N,K,bits", A8)
+@pytest.mark.parametrize("M,N,K,bits", A8 + [c for c, _ in A8_PARTS])
 def test_integer_form(P, M, N, K, bits):
     import torch
     from tests.test_a8_gpu import assert_a8
@@ -110,3 +129,17 @@ def test_integer_form(P, M, N, K, bits):
     assert all(torch.equal(y, a) for a in again) and lin.device_status() == (0, 0)
     rows = np.r_[0:128, N - 128:N] if N > 2304 else np.r_[0:N]
     assert_a8(y.cpu().numpy()[:, rows], x, q[rows], s[rows], 0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,bits,group", [c for c, _ in A8_DECODE[6:]])
+def test_integer_decode_in_clusters_of_each_size(P, M, N, K, bits, group):
+    import torch
+    from tests.test_a8_gpu import assert_a8
+    q, s = C.layer_weights(8500 + M + N, spec(N, K, bits, group))
+    x = C.layer_activations(8500 + M + N, spec(N, K, bits, group), M)
+    lin = P.QLinear.from_weights(q, s, bits, group, device="cuda:0")
+    xd = torch.from_numpy(x).cuda()
+    y = lin.forward_a8(xd)
+    assert all(torch.equal(y, lin.forward_a8(xd)) for _ in range(10))
+    assert_a8(y.cpu().numpy(), x, q, s, group)
