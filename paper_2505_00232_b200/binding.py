@@ -184,8 +184,8 @@ def qlinear_unpack(desc: Desc, packed: np.ndarray):
 # A small layer takes the GPU a few microseconds, less than these calls took the host.  So every call on tensors first goes to the module built
 # from csrc/native.cpp, which checks the arguments, allocates the outputs and calls the library; it returns None for everything
 # that is not the common form of the call (subclasses, tracing, wrong shapes, ...), and the Python below it then does the call, or raises.
-# Measured, us per call of the host: QLinear.forward at one token 6.7 -> 3.9, qlinear_forward_group of three layers 14.0 -> 6.1,
-# qlinear_residual_rmsnorm 11.1 -> 4.7, qlinear_rope_qkv 15.5 -> 5.2, KVCache.output 11.0 -> 5.4.
+# Measured, us per call of the host: QLinear.forward at one token 6.7 -> 3.5 to 4.0 (by machine), qlinear_forward_group of three layers 14.0 -> 5.8,
+# qlinear_residual_rmsnorm 11.1 -> 4.3, qlinear_rope_qkv 15.5 -> 4.8, KVCache.output 11.0 -> 5.3.
 _half = _raw_stream = _device = _native = None
 _NATIVE_API = ("qlinear_forward", "qlinear_forward_a8", "qlinear_forward_group", "qlinear_forward_gated", "qlinear_residual_rmsnorm", "qlinear_rope_qkv", "qlinear_embed",
                "qlinear_kv_append_heads", "qlinear_kv_scores_heads", "qlinear_kv_output_heads", "qlinear_kv_output", "qlinear_kv_output_uses_tmp")

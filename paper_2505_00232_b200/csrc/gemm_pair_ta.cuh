@@ -9,8 +9,8 @@
 //
 // Layout consequences:
 //   * tensor memory (512 columns): one 256-column fp32 accumulator + 8 A slots of 32 columns (64 k of fp16); there
-//     is no room for a second accumulator, so the epilogue is not hidden under the next tile.  It is kept short
-//     instead: 16 warps take the accumulator out together (64 columns each) as soon as they see the tile complete,
+//     is no room for a second accumulator of that width, so the epilogue is not hidden under the next tile (nor is it in the
+//     gated form with two of 160 columns, BOTH, whose second one holds the up tile).  It is kept short instead: 16 warps take the accumulator out together (64 columns each) as soon as they see the tile complete,
 //     free it, and leave fp16 values in a shared output tile, from which the four warps of 64 tokens store whole rows;
 //     meanwhile up to 6 A slots of the next tile are already filled, so the MMA restarts at once;
 //   * a thread of a dequantise warp owns ONE tile row (its TMEM lane): it needs 32 consecutive k of that row, which
@@ -38,7 +38,8 @@
 // included; Llama gate + up, fused, 2048 tokens 363 -> 347 us, 777 tokens 185 -> 165, Gemma2-2B's 777 tokens 64.0 -> 58.7).
 //
 // Forms of the kernel (template flags): the plain product, whole tiles dealt out round-robin or, for launches with
-// few tiles, 2 or 4 K parts per tile that meet in the device scratch; GATED (y = act(gate) * up, Section 3.6); I8
+// few tiles, 2 or 4 K parts per tile that meet in the device scratch (PARTS); GATED (y = act(gate) * up, Section 3.6), one tile after the
+// other through one accumulator, or, for few positions, with an accumulator each (BOTH: blocks of up to 160 tokens, 6 A slots); I8
 // (int8 activations, kind::i8 on the stored weight bytes, Section 3.7).
 //
 // Protocol between the two CTAs: own loads only; the leader issues; commits are multicast to both CTAs; the peer relays

@@ -1,6 +1,7 @@
 // The calls of the Python binding whose host work a small layer would otherwise wait for: the arguments of a call are checked, its outputs
 // allocated and the C entry point called in native code.  Bound: a layer of a few million weights takes the GPU 3 us, and the launch itself
-// the host 2.3; QLinear.forward at one token took 6.7 us through Python and ctypes and takes 3.9 through here (other calls: binding.py).
+// the host 2.3; QLinear.forward at one token took 6.7 us through Python and ctypes and takes 3.5 to 4.0 through here, by machine (other calls:
+// binding.py).
 //
 // Every function takes the common form of its call (plain tensors of the documented types, shapes and layout) and returns None for anything
 // else, whatever is wrong with it; the caller in binding.py then does the call in Python, with Python's own errors.  A status

@@ -972,7 +972,7 @@ bool narrow_can(const qlinear_s* const* hs, int n, int M, bool gated, bool batch
 }
 
 // The kernel of a call beyond the decode stage: one layer, n > 1 layers that share x, or (gated) a pair.  gemm_narrow.cuh where its
-// estimate is below that of gemm_mid.cuh, the CTA-pair kernel or the three other forms (single CTA, shared-memory gating, unfused gating).  No line is always right with these errors.  Of the calls above and 3110 others, 80 run more than 3 %
+// estimate is below that of gemm_mid.cuh, the CTA-pair kernel or the three other forms (single CTA, shared-memory gating, unfused gating).  No line is always right with these errors.  Of the calls above and 3110 others, 63 run more than 3 %
 // slower this way than on the other route: 54 of 4821 against gemm_mid.cuh (two of them by 46 and 26 %, the others by 24 % at most), 9
 // of 5488 against the other forms (9 %).  Against the CTA-pair kernel with its plans searched, 700 calls take 0.3 % more than on the faster route each,
 // the worst 21 %.  1676 gated pairs of 129 to 4096 tokens, timed on every form and width: 1.3 % more than on the fastest, the worst 26 %.  Measured, us, the route otherwise / gemm_narrow.cuh:
