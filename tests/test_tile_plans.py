@@ -18,10 +18,10 @@ GATED_ON_NARROW = [(330, 6144, 1120, 8, 0), (130, 9216, 1120, 8, 0)]      # (us,
 TWO_ACCUMULATORS = [(240, 17352, 960, 8, 0, 128, "gelu_tanh"), (161, 17152, 384, 4, 32, 96, "identity"), (391, 9216, 192, 4, 32, 160, "gelu_tanh"), (183, 17664, 128, 4, 32, 96, "silu"),
                     (415, 7424, 128, 8, 0, 160, "identity"), (1518, 1792, 1984, 4, 32, 160, "gelu_tanh"), (1100, 504, 224, 8, 0, 96, "silu"), (2000, 248, 32, 8, 0, 96, "gelu_tanh"),
                     (1029, 248, 160, 8, 0, 64, "identity"), (228, 10752, 192, 4, 0, 128, "silu")]
-# integer form (its plan is not asked for): one pair of row super-blocks to many, one k-step to many, parts and narrow blocks
+# integer form: one pair of row super-blocks to many, one k-step to many, parts and narrow blocks
 A8 = [(129, 256, 128, 4), (130, 200, 8192, 8), (200, 1024, 4096, 4), (333, 2296, 9216, 8), (700, 1024, 2304, 4), (1030, 4096, 1152, 8), (641, 9216, 256, 4)]
 
-# its plan: tokens per tile, K parts, token blocks.  int4 in 4 parts, remainders in tokens and channels
+# and with its plan (tokens per tile, K parts, token blocks): int4 in 4 parts, remainders in tokens and channels
 A8_PARTS = [((150, 256, 8192, 4), (32, 4, 5)), ((333, 504, 9216, 4), (64, 4, 6)), ((129, 2296, 8192, 4), (96, 4, 2)), ((257, 1000, 9216, 8), (96, 4, 3)), ((200, 1024, 14336, 4), (64, 4, 4)),
             ((200, 1024, 4096, 4), (64, 2, 4)), ((1030, 4096, 1152, 8), (128, 1, 9))]
 # int8-activation decode: CTAs, CTAs per cluster
