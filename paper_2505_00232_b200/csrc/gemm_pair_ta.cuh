@@ -927,13 +927,13 @@ inline bool gemm_pair_ta_applicable(const GemmPairLayers& set, int M, int num_sm
     // 1792 x 1984 at 1518 39.1 / 26.0, in two rounds 9216 x 2304 at 512 47.5 / 50.4, 3072 x 4096 at 1500 69.3 / 81.9; int8 3040 x 2624 at 848 54.5 / 30.7, 14336 x
     // 4096 at 256 98 / 78, 768 x 4608 at 3800 79.7 / 47.3, 14272 x 7680 at 196 138 / 135; of 89 int8 pairs that it takes two rounds for 3 are slower, by up to 2 %).
     // Up to 1024 channels and 1024 tokens these forms are not the ones that count: gemm_narrow.cuh takes such pairs, and is 0.03 % from the fastest on
-    // average (116 of K from 512 on; of smaller K, calls of 5 to 8 us, 75: 5.6 %).
+    // average (116 of K from 512 on; of smaller K, calls of 5 to 8 us, 75: 5.6 %).  Unless its weight map does not fit the layer: 256 x 32 at 184 19.5 / 5.4.
     if (!gated) return true;
     const Layout& L = *set.L[0];
     if (M <= 128 || !gemm_pair_ta_both(L, M, num_sms)) return M > 128;
     const TaPlan pl = gemm_pair_ta_gated_plan(L, M, num_sms);
     const double mb = 2e-6 * M * L.N;
-    return (L.n_rsb / 2 > 4 || M > 1024) && gemm_pair_ta_us(L.n_rsb / 2, pl.n_mblk, pl.bn, 1, (L.K + kGemmKStep - 1) / kGemmKStep, 2, true, false, num_sms) + 0.56 * mb < gemm_pair_gated_us(L, M, mb, num_sms);
+    return (L.n_rsb / 2 > 4 || M > 1024 || !w_map_fits(L, true)) && gemm_pair_ta_us(L.n_rsb / 2, pl.n_mblk, pl.bn, 1, (L.K + kGemmKStep - 1) / kGemmKStep, 2, true, false, num_sms) + 0.56 * mb < gemm_pair_gated_us(L, M, mb, num_sms);
 }
 
 inline ql_status gemm_pair_ta_forward(const GemmPairLayers& set, const void* x, int M, cudaStream_t st, int device, bool pdl, int num_sms,

@@ -17,7 +17,7 @@ GATED_ON_NARROW = [(330, 6144, 1120, 8, 0), (130, 9216, 1120, 8, 0)]      # (us,
 # Two accumulators (the position's second one, at blocks of 160, 128, 96 and 64): one round and two, one k-step to many, few channels, the three activations
 TWO_ACCUMULATORS = [(240, 17352, 960, 8, 0, 128, "gelu_tanh"), (161, 17152, 384, 4, 32, 96, "identity"), (391, 9216, 192, 4, 32, 160, "gelu_tanh"), (183, 17664, 128, 4, 32, 96, "silu"),
                     (415, 7424, 128, 8, 0, 160, "identity"), (1518, 1792, 1984, 4, 32, 160, "gelu_tanh"), (1100, 504, 224, 8, 0, 96, "silu"), (2000, 248, 32, 8, 0, 96, "gelu_tanh"),
-                    (1029, 248, 160, 8, 0, 64, "identity"), (228, 10752, 192, 4, 0, 128, "silu")]
+                    (1029, 248, 160, 8, 0, 64, "identity"), (184, 256, 32, 8, 0, 32, "silu"), (228, 10752, 192, 4, 0, 128, "silu")]
 # integer form: one pair of row super-blocks to many, one k-step to many, parts and narrow blocks
 A8 = [(129, 256, 128, 4), (130, 200, 8192, 8), (200, 1024, 4096, 4), (333, 2296, 9216, 8), (700, 1024, 2304, 4), (1030, 4096, 1152, 8), (641, 9216, 256, 4)]
 
