@@ -557,7 +557,7 @@ class KVCache:
 
     def output(self, prob, stream=None):
         """prob fp16 [R, cache_size] -> fp16 [R, d_h]."""
-        y = _native.kv_output(self.v._native, self.v_scale.data_ptr(), prob, _raw(stream))
+        y = _native.kv_output(self.v._native, self.v_scale, prob, _raw(stream))
         if y is not None:
             return y
         if not _is_x(prob, self.cache_size):

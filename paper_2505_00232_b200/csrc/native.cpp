@@ -334,15 +334,15 @@ PyObject* kv_output_heads(PyObject*, PyObject* const* a, Py_ssize_t)     // (hea
     });
 }
 
-PyObject* kv_output(PyObject*, PyObject* const* a, Py_ssize_t)           // (V layer, address of the V scales, prob, stream)
+PyObject* kv_output(PyObject*, PyObject* const* a, Py_ssize_t)           // (V layer, V scales, prob, stream)
 {
     return guarded([&]() -> PyObject* {
         Layer l;
-        const at::Tensor* p = plain(a[2], at::kHalf);
-        if (!layer_of(a[0], &l) || !p || p->dim() != 2 || p->size(1) != l.K || p->size(0) > INT_MAX) Py_RETURN_NONE;
+        const at::Tensor *p = plain(a[2], at::kHalf), *scales = plain(a[1], at::kHalf);
+        if (!layer_of(a[0], &l) || !p || !scales || p->dim() != 2 || p->size(1) != l.K || p->size(0) > INT_MAX) Py_RETURN_NONE;
         const int64_t R = p->size(0);
         at::Tensor out, tmp;
-        void *vs = PyLong_AsVoidPtr(a[1]), *pp = p->data_ptr(), *st = stream_of(a[3]);
+        void *vs = scales->data_ptr(), *pp = p->data_ptr(), *st = stream_of(a[3]);
         const bool uses_tmp = R < 1 || api.kv_output_uses_tmp(l.h, pp, vs, (int32_t)R);
         if (!done([&] {
                 out = half_like(*p, {R, l.N});
